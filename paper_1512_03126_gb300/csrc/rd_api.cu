@@ -133,6 +133,17 @@ namespace rdapi {
 
 int check_err(rdsplit_mesh* h, const char* where) { return check_err_impl(h, where); }
 
+// Both parities' inbox words (S <= 2) or masks back to zero.
+static cudaError_t clear_inboxes(rdsplit_mesh* h) {
+    const size_t T = (size_t)h->T;
+    cudaError_t ce = cudaSuccess;
+    for (int p = 0; p < 2 && ce == cudaSuccess; ++p)
+        ce = h->imask[p] ? cudaMemsetAsync(h->imask[p], 0, 4 * T * mask_bytes(h->S), h->stream)
+                         : cudaMemsetAsync(h->inbox[p], 0, 4 * T * inbox_stride(h->S) * sizeof(int32_t), h->stream);
+    if (ce == cudaSuccess) h->inbox_dirty = false;
+    return ce;
+}
+
 // The period loop of Algorithm 1 for one handle.  Step 1: the last period is
 // shortened so that it ends on t_end.  Step 2-3 run in k_period, which also
 // applies the previous period's transfers; the closing k_gather applies the
@@ -151,9 +162,10 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
             return fail(RDSPLIT_ECUDA, "rdsplit_run: %s", cudaGetErrorString(ce));
         }
     }
+    if (h->inbox_dirty) CUDA_TRY(clear_inboxes(h));
     int64_t j = 0;
-    const int32_t* prev = nullptr;
     while (h->t < t_end && (max_periods < 0 || j < max_periods)) {
+        h->inbox_dirty = true;   // until the closing transfer
         if (h->period >= (int64_t)0xffffffffll)
             return fail(RDSPLIT_EOVERFLOW, "rdsplit_run: period index exceeds 2^32-1");
         double tau_k = h->tau;
@@ -167,8 +179,9 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
             launch_thresholds(h->T, h->mp, h->g, h->G, tau_k, h->thr_last, h->stream);
             thr = h->thr_last;
         }
-        int32_t* cur = h->inbox[j & 1];
-        PeriodArgs a{(uint32_t)h->period, tau_k, (float)tau_k, seed, j == 0 ? 1 : 0, thr, prev, cur};
+        const int q = (int)(j & 1);
+        PeriodArgs a{(uint32_t)h->period, tau_k, (float)tau_k, seed, j == 0 ? 1 : 0, thr,
+                     h->inbox[q ^ 1], h->inbox[q], h->imask[q ^ 1], h->imask[q]};
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (h->timing_stride > 0 && j % h->timing_stride == 0) {
             e0 = next_event(h);
@@ -178,14 +191,20 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
         if (split) launch_period_split(m, h->mp, s, a, h->dq, h->dqn, (int32_t)(j & 1), block, h->stream);
         else launch_period(m, h->mp, s, a, block, h->stream);
         if (e0 && e1) cudaEventRecord(e1, h->stream);
-        prev = cur;
         h->t = last ? t_end : h->t + h->tau;
         h->period += 1;
         j += 1;
     }
-    if (j > 0) launch_gather(m, h->S, s, prev, h->stream);
+    if (j > 0) {
+        const int q = (int)((j - 1) & 1);
+        PeriodArgs a{};
+        a.in_prev = h->inbox[q];
+        a.mask_prev = h->imask[q];
+        launch_gather(m, h->S, s, a, h->stream);
+    }
     int rc = launch_check("rdsplit_run");
     if (rc) return rc;
+    h->inbox_dirty = false;
     rc = check_err(h, "rdsplit_run");
     collect_timing(h);
     return rc;
@@ -515,6 +534,8 @@ int rdsplit_set_model(rdsplit_mesh_t h, int32_t S, const double* D, int32_t R, c
         (rc = alloc_into(&h->cnt, T * S, "counts")) || (rc = alloc_into(&h->rem, T * S, "remainders")) ||
         (rc = alloc_into(&h->inbox[0], T * 4 * inbox_stride(S), "inboxes")) ||
         (rc = alloc_into(&h->inbox[1], T * 4 * inbox_stride(S), "inboxes")) ||
+        (S > 2 && ((rc = alloc_into(&h->imask[0], 4 * T * mask_bytes(S), "inbox masks")) ||
+                   (rc = alloc_into(&h->imask[1], 4 * T * mask_bytes(S), "inbox masks")))) ||
         (rc = alloc_into(&h->thr, T * S, "thresholds")) || (rc = alloc_into(&h->thr_last, T * S, "thresholds")) ||
         (rc = alloc_into(&h->staging, T * S, "staging")) || (rc = alloc_into(&h->avv, T, "avv")) ||
         (rc = alloc_into(&h->dq, T, "deferred-tet queue")) || (rc = alloc_into(&h->dqn, 2, "queue counters"))) {
@@ -544,9 +565,12 @@ int rdsplit_set_model(rdsplit_mesh_t h, int32_t S, const double* D, int32_t R, c
     launch_tau(h->D, S, h->gmax, tau_scale, h->d_tau, st);
     CUDA_TRY(cudaMemcpyAsync(&h->tau, h->d_tau, sizeof(double), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaMemsetAsync(h->cnt, 0, T * S * sizeof(int32_t), st));
-    // boundary slots of the inboxes are never written and must read as zero
-    CUDA_TRY(cudaMemsetAsync(h->inbox[0], 0, T * 4 * inbox_stride(S) * sizeof(int32_t), st));
-    CUDA_TRY(cudaMemsetAsync(h->inbox[1], 0, T * 4 * inbox_stride(S) * sizeof(int32_t), st));
+    // no inbox word is valid (from three species on the masks say which are)
+    for (int p = 0; p < 2; ++p) {
+        if (S > 2) CUDA_TRY(cudaMemsetAsync(h->imask[p], 0, 4 * T * mask_bytes(S), st));
+        else CUDA_TRY(cudaMemsetAsync(h->inbox[p], 0, T * 4 * inbox_stride(S) * sizeof(int32_t), st));
+    }
+    h->inbox_dirty = false;
     CUDA_TRY(cudaMemsetAsync(h->rem, 0, T * S * sizeof(int32_t), st));
     CUDA_TRY(cudaStreamSynchronize(st));
     if (std::isfinite(h->tau)) launch_thresholds(h->T, mp, h->g, h->G, h->tau, h->thr, st);
@@ -675,11 +699,14 @@ int rdsplit_partition_step(rdsplit_mesh_t h, double t_end, uint64_t seed, int32_
             thr = h->thr_last;
         }
         const int64_t j = h->part_j;
+        if (j == 0 && h->inbox_dirty) CUDA_TRY(rdapi::clear_inboxes(h));
         if (j == 0 && two_pass(h)) {
             CUDA_TRY(cudaMemsetAsync(h->dqn, 0, 2 * sizeof(int32_t), h->stream));
         }
         PeriodArgs a{(uint32_t)h->period, tau_k, (float)tau_k, seed, j == 0 ? 1 : 0, thr,
-                     h->inbox[(j + 1) & 1], h->inbox[j & 1], h->part_lo, h->part_hi};
+                     h->inbox[(j + 1) & 1], h->inbox[j & 1], h->imask[(j + 1) & 1], h->imask[j & 1],
+                     h->part_lo, h->part_hi, 1};
+        h->inbox_dirty = true;   // slots of other ranks' tets are written here and cleared by nobody
         const int block = period_block(h, sm_count());
         if (two_pass(h)) launch_period_split(h->dev_mesh(), h->mp, h->dev_state(), a, h->dq, h->dqn, (int32_t)(j & 1),
                                              block, h->stream);
@@ -699,8 +726,12 @@ int rdsplit_partition_end(rdsplit_mesh_t h) {
     const char* where = "rdsplit_partition_end";
     if (!h) return fail(RDSPLIT_EINVAL, "%s: NULL handle", where);
     if (h->part_j > 0) {
-        launch_gather(h->dev_mesh(), h->S, h->dev_state(), h->inbox[(h->part_j - 1) & 1], h->stream, h->part_lo,
-                      h->part_hi);
+        PeriodArgs a{};
+        a.in_prev = h->inbox[(h->part_j - 1) & 1];
+        a.mask_prev = h->imask[(h->part_j - 1) & 1];
+        a.t_lo = h->part_lo;
+        a.t_hi = h->part_hi;
+        launch_gather(h->dev_mesh(), h->S, h->dev_state(), a, h->stream);
         h->part_j = 0;
         int rc = launch_check(where);
         if (rc) return rc;
@@ -714,8 +745,9 @@ static int inbox_copy(rdsplit_mesh_t h, const int32_t* d_slots, int32_t n, int32
     if (n < 0) return fail(RDSPLIT_EINVAL, "%s: n < 0", where);
     if (h->part_j == 0) return fail(RDSPLIT_ESTATE, "%s: no partition step since the last begin or end", where);
     int32_t* box = h->inbox[(h->part_j - 1) & 1];
-    if (out) launch_inbox_export(h->S, box, d_slots, n, d_buf, h->stream);
-    else launch_inbox_import(h->S, box, d_slots, n, d_buf, h->stream);
+    uint8_t* mask = h->imask[(h->part_j - 1) & 1];
+    if (out) launch_inbox_export(h->S, box, mask, d_slots, n, d_buf, h->stream);
+    else launch_inbox_import(h->S, box, mask, d_slots, n, d_buf, h->stream);
     int rc = launch_check(where);
     if (rc) return rc;
     CUDA_TRY(cudaStreamSynchronize(h->stream));

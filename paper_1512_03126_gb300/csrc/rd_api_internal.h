@@ -31,8 +31,10 @@ struct rdsplit_mesh {
     double* D = nullptr;
     double* d_tau = nullptr;
     int32_t* cnt = nullptr;
-    int32_t* rem = nullptr;
+    int32_t* rem = nullptr;                   // the batched engine's second count buffer
     int32_t* inbox[2] = {nullptr, nullptr};   // [T][4][Sp] transfer inboxes by period parity
+    uint8_t* imask[2] = {nullptr, nullptr};   // their masks (three species or more)
+    bool inbox_dirty = false;                 // a run or partition run left inbox words or masks set
     uint4* thr = nullptr;
     uint4* thr_last = nullptr;
     int32_t* staging = nullptr;
@@ -61,12 +63,13 @@ struct rdsplit_mesh {
     int64_t period = 0;
 
     rdk::DevMesh dev_mesh() const { return rdk::DevMesh{T, src, g, G, vol, mask, avv, perm}; }
-    rdk::DevState dev_state() const { return rdk::DevState{cnt, rem, err}; }
+    rdk::DevState dev_state() const { return rdk::DevState{cnt, err}; }
 
     void free_model() {
-        void* ps[] = {D, d_tau, cnt, rem, inbox[0], inbox[1], thr, thr_last, staging, mask, avv, dq, dqn};
+        void* ps[] = {D, d_tau, cnt, rem, inbox[0], inbox[1], imask[0], imask[1], thr, thr_last, staging, mask, avv, dq, dqn};
         for (void* p : ps) rdapi::dev_free(p);
         D = nullptr; d_tau = nullptr; cnt = nullptr; rem = nullptr; inbox[0] = inbox[1] = nullptr;
+        imask[0] = imask[1] = nullptr;
         thr = nullptr; thr_last = nullptr; staging = nullptr; mask = nullptr; avv = nullptr;
         dq = nullptr; dqn = nullptr;
         has_model = false;
@@ -89,11 +92,13 @@ inline bool two_pass(const rdsplit_mesh* h) { return h->period_mode == 2; }
 // the 2.4 M-tet bar: 310 us per period against 339 us with 256), smaller
 // for a small mesh so that it still spreads over the SMs (at least 4 blocks
 // per SM when the tets allow it; a power of two down to 32).
-inline int period_block(const rdsplit_mesh* h, int sms) {
-    if (h->period_block > 0) return h->period_block;
+inline int period_block(int64_t T, int sms) {
     int b = 128;
-    while (b > 32 && (int64_t)h->T < (int64_t)4 * sms * b) b >>= 1;
+    while (b > 32 && T < (int64_t)4 * sms * b) b >>= 1;
     return b;
+}
+inline int period_block(const rdsplit_mesh* h, int sms) {
+    return h->period_block > 0 ? h->period_block : period_block(h->T, sms);
 }
 int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed);
 int check_err(rdsplit_mesh* h, const char* where);

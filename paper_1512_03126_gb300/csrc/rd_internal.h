@@ -71,8 +71,7 @@ struct DevMesh {
 __device__ __forceinline__ int key_of(const DevMesh& m, int t) { return m.perm ? __ldg(m.perm + t) : t; }
 
 struct DevState {
-    int32_t* cnt;           // [S][T] counts between runs
-    int32_t* rem;           // [S][T] molecules that stayed in the last period
+    int32_t* cnt;           // [S][T] counts, in place over the periods of a run
     uint32_t* err;          // error word
 };
 
@@ -102,8 +101,12 @@ void launch_counts_out(int32_t T, int32_t S, const int32_t* st_major, int32_t* t
 // per species, the molecules that the neighbour across face r of tet u sent
 // to u in one period; a tet t writes its leavers through face f into slot
 // src[t].f = 4 u + r of its neighbour u (each interior slot has exactly one
-// writer per period, boundary slots are never written and stay zero), and
-// reads its own four slots, contiguous, in the next period.
+// writer per period) and reads its own four slots, contiguous, in the next
+// period.  Only nonzero words are written.  With one or two species a word
+// itself says whether something came, and the reader sets it back to zero;
+// from three on a mask per slot ([T][4], 8 bits up to eight species, else 16)
+// has a bit per valid word, and the reader clears the masks.  Between runs
+// all words (S <= 2) and masks are zero, in both parities.
 __host__ __device__ inline int32_t inbox_stride(int32_t S) { return S <= 2 ? S : (S + 3) & ~3; }
 
 struct PeriodArgs {
@@ -113,25 +116,31 @@ struct PeriodArgs {
     uint64_t seed;
     int32_t first;          // 1: counts come from cnt (no pending transfer)
     const uint4* thr;       // [S][T] cumulative 32-bit face thresholds for tau_k
-    const int32_t* in_prev; // [T][4][Sp] inboxes filled by the previous period
+    int32_t* in_prev;       // [T][4][Sp] inboxes filled by the previous period
     int32_t* in_cur;        // [T][4][Sp] inboxes this period fills
+    uint8_t* mask_prev;     // their masks (S >= 3)
+    uint8_t* mask_cur;
     int32_t t_lo = 0;       // the period advances the stored tets [t_lo, t_hi) (a
     int32_t t_hi = 0;       // rank's range; 0, 0: all tets)
+    int32_t dense = 0;      // 1: write every slot of the own tets' faces, zeros too (partitioned runs)
 };
 void launch_period(const DevMesh& m, const ModelParams& mp, const DevState& s, const PeriodArgs& a, int block,
                    cudaStream_t st);
-void launch_gather(const DevMesh& m, int32_t S, const DevState& s, const int32_t* in_last, cudaStream_t st,
-                   int32_t t_lo = 0, int32_t t_hi = 0);
+// The closing transfer: a.in_prev / a.mask_prev hold the last period's.
+void launch_gather(const DevMesh& m, int32_t S, const DevState& s, const PeriodArgs& a, cudaStream_t st);
+// Bytes of a slot's mask (0: none).
+__host__ __device__ inline int32_t mask_bytes(int32_t S) { return S <= 2 ? 0 : (S <= 8 ? 1 : 2); }
 // Copy inbox slots out of / into a packed buffer int32 [n][S] (the transfers
 // across the cut faces of a partitioned mesh).
-void launch_inbox_export(int32_t S, const int32_t* inbox, const int32_t* slots, int32_t n, int32_t* buf,
-                         cudaStream_t st);
-void launch_inbox_import(int32_t S, int32_t* inbox, const int32_t* slots, int32_t n, const int32_t* buf,
-                         cudaStream_t st);
-// The period in two passes (light pass, then the deferred tets): queue holds
-// T entries, qcount two counters (both zero before the first period of a
-// run; parity alternates 0, 1, 0, ... over the run's periods); `block` is the
-// light pass's block size (32..256, a multiple of 32).
+void launch_inbox_export(int32_t S, const int32_t* inbox, const uint8_t* mask, const int32_t* slots, int32_t n,
+                         int32_t* buf, cudaStream_t st);
+void launch_inbox_import(int32_t S, int32_t* inbox, uint8_t* mask, const int32_t* slots, int32_t n,
+                         const int32_t* buf, cudaStream_t st);
+// The period in two passes (first all tets but those whose reactions have to
+// run, then these): queue holds T entries, qcount two counters (both zero
+// before the first period of a run; parity alternates 0, 1, 0, ... over the
+// run's periods); `block` is the first pass's block size (32..256, a multiple
+// of 32).
 void launch_period_split(const DevMesh& m, const ModelParams& mp, const DevState& s, const PeriodArgs& a,
                          int32_t* queue, int32_t* qcount, int32_t parity, int block, cudaStream_t st);
 

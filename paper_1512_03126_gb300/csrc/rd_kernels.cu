@@ -7,20 +7,18 @@
 //   k_thresholds   cumulative 32-bit face thresholds of zeta * w_f
 //   k_count_ge     tets with G >= x (rank selection for the outlier option)
 //   k_zeta_hist    histogram of zeta over the tets (diagnostic, Fig. 1d)
-//   k_period       per tet: gather of the previous period's transfers, SSA
-//                  reactions with occupancy (Step 2), mean-corrected binomial
-//                  count and multinomial split (Step 3)
-//   k_period_light / k_period_slow
-//                  the same period in two passes for large meshes: the
-//                  common tets without the double-precision samplers, then
-//                  the deferred ones with them
+//   k_period       per tet: the previous period's transfers, SSA reactions
+//                  with occupancy (Step 2), mean-corrected binomial count and
+//                  multinomial split (Step 3); in one pass, or in two with
+//                  the tets whose reactions have to run in the second
 //   k_gather       the closing synchronous transfer of a run
 //
-// Layout: counts and remainders are species-major int32 [S][T] (coalesced);
-// transfers go through inboxes int32 [T][4][Sp]: a tet writes what leaves
-// through face f into the neighbour's slot (a scattered store that nothing
-// waits for) and reads its own four slots, contiguous, in the next period
-// (a coalesced load), instead of gathering from its neighbours.
+// Layout: counts are species-major int32 [S][T] (coalesced), updated in
+// place; transfers go through inboxes int32 [T][4][Sp]: a tet writes what
+// leaves through face f into the neighbour's slot (a scattered store that
+// nothing waits for) and reads its own four slots, contiguous, in the next
+// period, instead of gathering from its neighbours.  Only what is not zero
+// is written, and the reader clears it.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -28,6 +26,7 @@
 #include "rd_device.cuh"
 #include "rd_internal.h"
 #include "rd_period.cuh"
+#include "rd_warp.cuh"
 
 namespace rdk {
 
@@ -37,6 +36,16 @@ constexpr int kBlock = 256;
 
 inline int grid_for(int64_t n) { return (int)((n + kBlock - 1) / kBlock); }
 }  // namespace
+
+int sm_count() {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) {
+        cudaGetLastError();
+        n = 1;
+    }
+    return n;
+}
 
 int64_t launches() { return g_launches.load(); }
 void note_launch() { ++g_launches; }
@@ -258,281 +267,282 @@ void launch_avv(int32_t T, const double* vol, float2* avv, cudaStream_t st) {
     ++g_launches;
 }
 
-// A tet's counts at the start of a period: its molecules that stayed in the
-// previous period plus what its neighbours sent (its inbox), or the counts
-// of the handle in a run's first period.  Returns error bits.
-template <int SA>
-__device__ __forceinline__ uint32_t gather_counts(const DevState& s, const PeriodArgs& a, int t, int T, int S, int Sp,
-                                                  int32_t* N) {
+// A tet's molecules that arrived in the previous period, added to its column
+// (clamped at 2^31-1), and its inbox words cleared for their next use.  Up to
+// two species a nonzero word is the message; from three on a byte (16 bits
+// from nine species on) a face says which species' words are valid, so a tet
+// reads 4 or 8 bytes unless something came: 256 of the 356 bytes a
+// tet-period of eight species moved were inbox words, nearly all zero.
+// Returns error bits.
+__device__ __forceinline__ uint32_t take_inbox(const PeriodArgs& a, int t, int S, int lane, int32_t* N,
+                                               uint32_t* dirty) {
+    const int Sp = inbox_stride(S);
     uint32_t bad = 0;
-    int64_t n[SA];
-#pragma unroll
-    for (int sp = 0; sp < SA; ++sp) {
-        if (sp >= S) break;
-        n[sp] = a.first ? s.cnt[(int64_t)sp * T + t] : s.rem[(int64_t)sp * T + t];
+    auto add = [&](int sp, int64_t v) {
+        int64_t n = N[32 * sp + lane] + v;
+        if (n > 2147483647) { bad |= kErrOverflow; n = 2147483647; }
+        if (n < 0) { bad |= kErrNegative; n = 0; }
+        N[32 * sp + lane] = (int32_t)n;
+        *dirty |= 1u << sp;
+    };
+    if (S <= 2) {
+        int4* p = reinterpret_cast<int4*>(a.in_prev + (int64_t)t * 4 * Sp);
+        const int4 x = __ldcg(p);
+        int4 y = make_int4(0, 0, 0, 0);
+        if (S == 2) y = __ldcg(p + 1);
+        if (x.x | x.y | x.z | x.w) {
+            *p = make_int4(0, 0, 0, 0);
+            if (S == 1) add(0, (int64_t)x.x + x.y + x.z + x.w);
+        }
+        if (S == 2) {
+            if (y.x | y.y | y.z | y.w) p[1] = make_int4(0, 0, 0, 0);
+            if (x.x | x.z | y.x | y.z) add(0, (int64_t)x.x + x.z + y.x + y.z);
+            if (x.y | x.w | y.y | y.w) add(1, (int64_t)x.y + x.w + y.y + y.w);
+        }
+        return bad;
     }
-    if (!a.first) add_inbox<SA>(a.in_prev, t, S, Sp, n);
-#pragma unroll
-    for (int sp = 0; sp < SA; ++sp) {
-        if (sp >= S) break;
-        int64_t v = n[sp];
-        if (v > 2147483647) { bad |= kErrOverflow; v = 2147483647; }
-        if (v < 0) { bad |= kErrNegative; v = 0; }
-        N[sp] = (int32_t)v;
+    uint64_t bits;
+    if (S <= 8) {
+        uint32_t* p = reinterpret_cast<uint32_t*>(a.mask_prev) + t;
+        bits = __ldcg(p);
+        if (bits) *p = 0u;
+    } else {
+        unsigned long long* p = reinterpret_cast<unsigned long long*>(a.mask_prev) + t;
+        bits = __ldcg(p);
+        if (bits) *p = 0ull;
+    }
+    const int shift = S <= 8 ? 3 : 4;   // log2 of the bits a face
+    while (bits) {
+        const int i = __ffsll((long long)bits) - 1;
+        bits &= bits - 1ull;
+        const int f = i >> shift, sp = i & ((1 << shift) - 1);
+        add(sp, __ldcg(a.in_prev + ((int64_t)t * 4 + f) * Sp + sp));
     }
     return bad;
 }
 
-// One period for one tet: apply the previous period's transfers, run the
-// reaction phase, draw the diffusion out-counts.  S_ > 0 fixes the species
-// count at compile time so that counts live in registers; S_ = 0 reads it
-// from the model (up to kMaxS).
-template <int S_, bool kReact>
-__global__ void __launch_bounds__(kBlock) k_period(DevMesh m, ModelParams mp, DevState s, PeriodArgs a) {
-    constexpr int SA = S_ > 0 ? S_ : kMaxS;
-    const int S = S_ > 0 ? S_ : mp.S;
-    const int t_hi = a.t_hi > 0 ? a.t_hi : m.T;
-    const int t = a.t_lo + blockIdx.x * blockDim.x + threadIdx.x;
-    const bool valid = t < t_hi;         // every lane stays for the warp draw
-    const int T = m.T;
-    const int Sp = inbox_stride(S);
-    int32_t N[SA];
-    int4 o[SA];
-    int4 sr = make_int4(-1, -1, -1, -1);
-    uint32_t bad = 0, heavy = 0;
-    if (valid) {
-        sr = m.src[t];
-        bad |= gather_counts<SA>(s, a, t, T, S, Sp, N);
-        bad |= step_tet<SA, kReact>(m, mp, a.period, a.tau_k, a.tau_kf, a.seed, a.thr, t, S, N, o, &heavy, s.err);
+// What a tet's emit writes: leavers into its neighbours' inbox words, and
+// the valid bits of each face's slot at the end (one writer a slot).
+struct Sender {
+    const PeriodArgs& a;
+    const int4* src;
+    int t, S;
+    int4 sr;
+    bool have;
+    uint64_t bits;
+
+    __device__ __forceinline__ Sender(const PeriodArgs& a_, const int4* src_, int t_, int S_)
+        : a(a_), src(src_), t(t_), S(S_), sr(make_int4(-1, -1, -1, -1)), have(false), bits(0) {}
+
+    __device__ __forceinline__ void load() {
+        if (!have) sr = __ldg(src + t);
+        have = true;
     }
-    warp_split<SA>(heavy, a.seed, a.period, t, valid ? key_of(m, t) : 0, a.thr, T, N, o);
-    if (valid) {
-        push_inbox<SA>(a.in_cur, sr, S, Sp, o);
+    // Partitioned runs export slots of tets the rank never reads (and so
+    // never clears): there every slot is written in full.
+    __device__ __forceinline__ void clear_all() {
+        load();
+        const int slot[4] = {sr.x, sr.y, sr.z, sr.w};
+        if (S <= 2)
+            for (int f = 0; f < 4; ++f)
+                if (slot[f] >= 0)
+                    for (int s = 0; s < S; ++s) a.in_cur[(int64_t)slot[f] * S + s] = 0;
+    }
+    __device__ __forceinline__ void operator()(int sp, const int4& o) {
+        load();
+        const int slot[4] = {sr.x, sr.y, sr.z, sr.w}, n[4] = {o.x, o.y, o.z, o.w};
+        const int Sp = inbox_stride(S);
 #pragma unroll
-        for (int sp = 0; sp < SA; ++sp) {
-            if (sp >= S) break;
-            s.rem[(int64_t)sp * T + t] = N[sp];
+        for (int f = 0; f < 4; ++f) {
+            if (n[f] <= 0 || slot[f] < 0) continue;
+            a.in_cur[(int64_t)slot[f] * Sp + sp] = n[f];
+            bits |= 1ull << (16 * f + sp);
         }
-        if (bad) atomicOr(s.err, bad);
     }
+    __device__ __forceinline__ void finish(bool all) {
+        if (S <= 2 || (!all && bits == 0)) return;
+        const int slot[4] = {sr.x, sr.y, sr.z, sr.w};
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            const uint32_t b = (uint32_t)(bits >> (16 * f)) & 0xffffu;
+            if (slot[f] < 0 || (!all && b == 0u)) continue;
+            if (S <= 8) a.mask_cur[slot[f]] = (uint8_t)b;
+            else reinterpret_cast<uint16_t*>(a.mask_cur)[slot[f]] = (uint16_t)b;
+        }
+    }
+};
+
+// Passes of a period: all in one kernel, or a first pass that defers the tets
+// whose reaction phase has to run to a queue and a second one over the queue.
+enum { kPassAll = 0, kPassFirst = 1, kPassQueue = 2 };
+
+// One period for every tet, one a lane: the previous period's transfers, the
+// reaction phase, the diffusion draws, leavers pushed to the neighbours'
+// inboxes (rd_warp.cuh).  Counts stay in place in cnt (only their own
+// tet reads or writes them) and are written back where they changed.
+// S_ > 0 fixes the species count at compile time.
+template <int S_, bool kReact, int kPass>
+__global__ void __launch_bounds__(kBlock, kPass == kPassFirst ? 4 : 3)
+k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp, DevState s,
+         const __grid_constant__ PeriodArgs a, int32_t* __restrict__ queue, int32_t* qcount, int32_t parity) {
+    extern __shared__ int32_t sm[];
+    const int S = S_ > 0 ? S_ : mp.S;
+    const int lane = threadIdx.x & 31;
+    const WarpMem w(sm + (threadIdx.x >> 5) * warp_words(S, kReact), S, kReact);
+    const int64_t T = m.T;
+    const PeriodView v{a.period, a.tau_k, a.tau_kf, a.seed, a.thr, 1};
+    const int hi = kPass == kPassQueue ? qcount[parity] : (a.t_hi > 0 ? a.t_hi : m.T);
+    const int lo = kPass == kPassQueue ? 0 : a.t_lo;
+    if (kPass == kPassFirst && blockIdx.x == 0 && threadIdx.x == 0) qcount[parity ^ 1] = 0;
+    for (int64_t base = lo + (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < hi;
+         base += (int64_t)gridDim.x * blockDim.x) {
+        bool live = base + lane < hi;
+        const int t = !live ? 0 : (kPass == kPassQueue ? queue[base + lane] : (int)(base + lane));
+        uint32_t bad = 0, dirty = 0;
+        if (live) {
+            for (int s0 = 0; s0 < S; s0 += 8) {
+                int32_t n[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (s0 + k < S) n[k] = s.cnt[(int64_t)(s0 + k) * T + t];
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (s0 + k < S) w.N[32 * (s0 + k) + lane] = n[k];
+            }
+            if (kPass != kPassQueue && !a.first) bad |= take_inbox(a, t, S, lane, w.N, &dirty);
+        }
+        Sender send(a, m.src, t, S);
+        if (a.dense && live) send.clear_all();
+        bool deferred = false;
+        bad |= warp_step<kReact, kPass == kPassFirst>(m, mp, S, w, v, t, live, &dirty, &deferred, s.err, send);
+        if (live && !deferred) send.finish(a.dense != 0);
+        if (kPass == kPassFirst) {
+            const unsigned dm = __ballot_sync(0xffffffffu, deferred);
+            if (dm) {
+                const int leader = __ffs(dm) - 1;
+                int at = 0;
+                if (lane == leader) at = atomicAdd(qcount + parity, __popc(dm));
+                at = __shfl_sync(0xffffffffu, at, leader);
+                if (deferred) queue[at + __popc(dm & ((1u << lane) - 1u))] = t;
+            }
+        }
+        if (live)
+            for (uint32_t bits = dirty; bits; bits &= bits - 1u) {
+                const int sp = __ffs(bits) - 1;
+                s.cnt[(int64_t)sp * T + t] = w.N[32 * sp + lane];
+            }
+        if (bad) atomicOr(s.err, bad);
+        __syncwarp();
+    }
+}
+
+template <int S_, bool kReact, int kPass>
+void launch_pass(const DevMesh& m, const ModelParams& mp, const DevState& s, const PeriodArgs& a, int32_t* queue,
+                 int32_t* qcount, int32_t parity, int grid, int block, cudaStream_t st) {
+    const size_t smem = (size_t)(block / 32) * warp_words(mp.S, kReact) * sizeof(int32_t);
+    if (smem > 48u * 1024u)   // large blocks of many species
+        cudaFuncSetAttribute(k_period<S_, kReact, kPass>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_period<S_, kReact, kPass><<<grid, block, smem, st>>>(m, mp, s, a, queue, qcount, parity);
+    ++g_launches;
 }
 
 template <int S_>
 void launch_period_s(const DevMesh& m, const ModelParams& mp, const DevState& s, const PeriodArgs& a, int block,
-                     cudaStream_t st) {
+                     int32_t* queue, int32_t* qcount, int32_t parity, bool split, cudaStream_t st) {
     const int64_t n = (a.t_hi > 0 ? a.t_hi : m.T) - a.t_lo;
     const int grid = (int)((n + block - 1) / block);
-    if (mp.any_reaction) k_period<S_, true><<<grid, block, 0, st>>>(m, mp, s, a);
-    else k_period<S_, false><<<grid, block, 0, st>>>(m, mp, s, a);
+    if (!mp.any_reaction) {
+        // nothing to defer: without reactions one pass is both
+        launch_pass<S_, false, kPassAll>(m, mp, s, a, nullptr, nullptr, 0, grid, block, st);
+    } else if (!split) {
+        launch_pass<S_, true, kPassAll>(m, mp, s, a, nullptr, nullptr, 0, grid, block, st);
+    } else {
+        launch_pass<S_, true, kPassFirst>(m, mp, s, a, queue, qcount, parity, grid, block, st);
+        launch_pass<S_, true, kPassQueue>(m, mp, s, a, queue, qcount, parity,
+                                          std::min(grid_for(n), 2 * sm_count()), kBlock, st);
+    }
+}
+
+static void launch_any(const DevMesh& m, const ModelParams& mp, const DevState& s, const PeriodArgs& a, int block,
+                       int32_t* queue, int32_t* qcount, int32_t parity, bool split, cudaStream_t st) {
+    if (mp.S == 1) launch_period_s<1>(m, mp, s, a, block, queue, qcount, parity, split, st);
+    else launch_period_s<0>(m, mp, s, a, block, queue, qcount, parity, split, st);
 }
 
 void launch_period(const DevMesh& m, const ModelParams& mp, const DevState& s, const PeriodArgs& a, int block,
                    cudaStream_t st) {
-    switch (mp.S) {
-        case 1: launch_period_s<1>(m, mp, s, a, block, st); break;
-        case 2: launch_period_s<2>(m, mp, s, a, block, st); break;
-        case 3: launch_period_s<3>(m, mp, s, a, block, st); break;
-        case 4: launch_period_s<4>(m, mp, s, a, block, st); break;
-        case 8: launch_period_s<8>(m, mp, s, a, block, st); break;
-        default: launch_period_s<0>(m, mp, s, a, block, st); break;
-    }
-    ++g_launches;
-}
-
-// The same period split in two passes, for large meshes.  The light pass
-// runs every tet that needs neither the reaction phase (no reaction
-// possible, or one proved impossible by the single-precision test) nor the
-// double-precision binomial (all counts below kMoleculeCut): it is compiled
-// without the non-inlined samplers, so it holds fewer registers and more
-// warps per SM.  It defers every other tet to a queue, with its gathered
-// counts stored in rem; the slow pass runs the queued tets with the full
-// step.  Every draw is keyed by (tet, period), so the result equals the
-// fused kernel's.  queue holds T entries; qcount[parity] counts this
-// period's, and the light pass clears the other parity's for the next.
-template <int S_, bool kReact>
-__global__ void __launch_bounds__(kBlock, 3) k_period_light(DevMesh m, ModelParams mp, DevState s, PeriodArgs a,
-                                                            int32_t* __restrict__ queue, int32_t* qcount,
-                                                            int32_t parity) {
-    constexpr int SA = S_ > 0 ? S_ : kMaxS;
-    const int S = S_ > 0 ? S_ : mp.S;
-    const int t_hi = a.t_hi > 0 ? a.t_hi : m.T;
-    const int t = a.t_lo + blockIdx.x * blockDim.x + threadIdx.x;
-    const bool valid = t < t_hi;         // every lane stays for the warp draw
-    const int T = m.T;
-    const int lane = threadIdx.x & 31;
-    if (blockIdx.x == 0 && threadIdx.x == 0) qcount[parity ^ 1] = 0;
-    const int Sp = inbox_stride(S);
-    int32_t N[SA];
-    int4 o[SA];
-    int4 sr = make_int4(-1, -1, -1, -1);
-    uint32_t bad = 0, heavy = 0;
-    bool light = false;
-    if (valid) {
-        sr = m.src[t];
-        bad |= gather_counts<SA>(s, a, t, T, S, Sp, N);
-        light = step_is_light<SA, kReact>(m, mp, a.period, a.tau_kf, a.seed, t, S, N);
-        if (light) {
-            bad |= step_tet<SA, false, false>(m, mp, a.period, a.tau_k, a.tau_kf, a.seed, a.thr, t, S, N, o, &heavy,
-                                              s.err);
-        } else {
-#pragma unroll
-            for (int sp = 0; sp < SA; ++sp) {
-                if (sp >= S) break;
-                s.rem[(int64_t)sp * T + t] = N[sp];
-            }
-        }
-    }
-    // deferred tets: one queue slot reservation per warp
-    const unsigned dm = __ballot_sync(0xffffffffu, valid && !light);
-    if (dm) {
-        const int leader = __ffs(dm) - 1;
-        int at = 0;
-        if (lane == leader) at = atomicAdd(qcount + parity, __popc(dm));
-        at = __shfl_sync(0xffffffffu, at, leader);
-        if (valid && !light) queue[at + __popc(dm & ((1u << lane) - 1u))] = t;
-    }
-    warp_split<SA>(heavy, a.seed, a.period, t, valid ? key_of(m, t) : 0, a.thr, T, N, o);
-    if (valid && light) {
-        push_inbox<SA>(a.in_cur, sr, S, Sp, o);
-#pragma unroll
-        for (int sp = 0; sp < SA; ++sp) {
-            if (sp >= S) break;
-            s.rem[(int64_t)sp * T + t] = N[sp];
-        }
-    }
-    if (bad) atomicOr(s.err, bad);
-}
-
-// The queued tets of one period with the full step (reaction phase and the
-// double-precision samplers), warp by warp over the queue.
-template <int S_, bool kReact>
-__global__ void __launch_bounds__(kBlock) k_period_slow(DevMesh m, ModelParams mp, DevState s, PeriodArgs a,
-                                                        const int32_t* __restrict__ queue, const int32_t* qcount,
-                                                        int32_t parity) {
-    constexpr int SA = S_ > 0 ? S_ : kMaxS;
-    const int S = S_ > 0 ? S_ : mp.S;
-    const int T = m.T;
-    const int n = qcount[parity];
-    const int lane = threadIdx.x & 31;
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t base = gw * 32; base < n; base += nw * 32) {
-        const bool live = base + lane < n;
-        const int t = live ? queue[base + lane] : 0;
-        int32_t N[SA];
-        int4 o[SA];
-        uint32_t bad = 0, heavy = 0;
-        if (live) {
-#pragma unroll
-            for (int sp = 0; sp < SA; ++sp) {
-                if (sp >= S) break;
-                N[sp] = s.rem[(int64_t)sp * T + t];
-            }
-            bad |= step_tet<SA, kReact>(m, mp, a.period, a.tau_k, a.tau_kf, a.seed, a.thr, t, S, N, o, &heavy, s.err);
-        }
-        warp_split<SA>(heavy, a.seed, a.period, t, live ? key_of(m, t) : 0, a.thr, T, N, o);
-        if (live) {
-            push_inbox<SA>(a.in_cur, m.src[t], S, inbox_stride(S), o);
-#pragma unroll
-            for (int sp = 0; sp < SA; ++sp) {
-                if (sp >= S) break;
-                s.rem[(int64_t)sp * T + t] = N[sp];
-            }
-        }
-        if (bad) atomicOr(s.err, bad);
-    }
-}
-
-int sm_count() {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) {
-        cudaGetLastError();
-        n = 1;
-    }
-    return n;
-}
-
-template <int S_>
-void launch_split_s(const DevMesh& m, const ModelParams& mp, const DevState& s, const PeriodArgs& a,
-                    int32_t* queue, int32_t* qcount, int32_t parity, int block, cudaStream_t st) {
-    const int64_t n = (a.t_hi > 0 ? a.t_hi : m.T) - a.t_lo;
-    const int grid = (int)((n + block - 1) / block);
-    const int grid_slow = std::min(grid_for(m.T), 2 * sm_count());
-    if (mp.any_reaction) {
-        k_period_light<S_, true><<<grid, block, 0, st>>>(m, mp, s, a, queue, qcount, parity);
-        k_period_slow<S_, true><<<grid_slow, kBlock, 0, st>>>(m, mp, s, a, queue, qcount, parity);
-    } else {
-        k_period_light<S_, false><<<grid, block, 0, st>>>(m, mp, s, a, queue, qcount, parity);
-        k_period_slow<S_, false><<<grid_slow, kBlock, 0, st>>>(m, mp, s, a, queue, qcount, parity);
-    }
+    launch_any(m, mp, s, a, block, nullptr, nullptr, 0, false, st);
 }
 
 void launch_period_split(const DevMesh& m, const ModelParams& mp, const DevState& s, const PeriodArgs& a,
                          int32_t* queue, int32_t* qcount, int32_t parity, int block, cudaStream_t st) {
-    switch (mp.S) {
-        case 1: launch_split_s<1>(m, mp, s, a, queue, qcount, parity, block, st); break;
-        case 2: launch_split_s<2>(m, mp, s, a, queue, qcount, parity, block, st); break;
-        case 3: launch_split_s<3>(m, mp, s, a, queue, qcount, parity, block, st); break;
-        case 4: launch_split_s<4>(m, mp, s, a, queue, qcount, parity, block, st); break;
-        case 8: launch_split_s<8>(m, mp, s, a, queue, qcount, parity, block, st); break;
-        default: launch_split_s<0>(m, mp, s, a, queue, qcount, parity, block, st); break;
-    }
-    g_launches += 2;
+    launch_any(m, mp, s, a, block, queue, qcount, parity, true, st);
 }
 
-__global__ void k_gather(DevMesh m, int32_t S, DevState s, const int32_t* __restrict__ in_last, int32_t t_lo,
-                         int32_t t_hi) {
-    int t = t_lo + blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= t_hi) return;
-    const int T = m.T;
-    const int Sp = inbox_stride(S);
-    const int32_t* box = in_last + (int64_t)t * 4 * Sp;
-    uint32_t bad = 0;
-    for (int sp = 0; sp < S; ++sp) {
-        int64_t n = s.rem[(int64_t)sp * T + t];
-        for (int f = 0; f < 4; ++f) n += box[f * Sp + sp];
-        if (n > 2147483647) { bad |= kErrOverflow; n = 2147483647; }
-        if (n < 0) { bad |= kErrNegative; n = 0; }
-        s.cnt[(int64_t)sp * T + t] = (int32_t)n;
+// The closing synchronous transfer of a run, in place; leaves every inbox
+// word and mask of its tets cleared.
+__global__ void k_gather(int32_t T, int32_t S, DevState s, PeriodArgs a) {
+    extern __shared__ int32_t sm[];
+    const int t = a.t_lo + blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (a.t_hi > 0 ? a.t_hi : T)) return;
+    const int lane = threadIdx.x & 31;
+    int32_t* N = sm + (threadIdx.x >> 5) * 32 * S;
+    for (int sp = 0; sp < S; ++sp) N[32 * sp + lane] = s.cnt[(int64_t)sp * T + t];
+    uint32_t dirty = 0;
+    const uint32_t bad = take_inbox(a, t, S, lane, N, &dirty);
+    for (uint32_t bits = dirty; bits; bits &= bits - 1u) {
+        const int sp = __ffs(bits) - 1;
+        s.cnt[(int64_t)sp * T + t] = N[32 * sp + lane];
     }
     if (bad) atomicOr(s.err, bad);
 }
 
-void launch_gather(const DevMesh& m, int32_t S, const DevState& s, const int32_t* in_last, cudaStream_t st,
-                   int32_t t_lo, int32_t t_hi) {
-    if (t_hi <= 0) t_hi = m.T;
-    k_gather<<<grid_for(t_hi - t_lo), kBlock, 0, st>>>(m, S, s, in_last, t_lo, t_hi);
+void launch_gather(const DevMesh& m, int32_t S, const DevState& s, const PeriodArgs& a, cudaStream_t st) {
+    const int64_t n = (a.t_hi > 0 ? a.t_hi : m.T) - a.t_lo;
+    k_gather<<<grid_for(n), kBlock, (size_t)kBlock * S * sizeof(int32_t), st>>>(m.T, S, s, a);
     ++g_launches;
 }
 
-__global__ void k_inbox_export(int32_t S, const int32_t* __restrict__ inbox, const int32_t* __restrict__ slots,
-                               int32_t n, int32_t* __restrict__ buf) {
+// Inbox slots packed as int32 [n][S] (words without a valid bit are zero).
+__global__ void k_inbox_export(int32_t S, const int32_t* __restrict__ inbox, const uint8_t* __restrict__ mask,
+                               const int32_t* __restrict__ slots, int32_t n, int32_t* __restrict__ buf) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)n * S) return;
-    const int64_t k = i / S, sp = i - k * S;
-    buf[i] = inbox[(int64_t)slots[k] * inbox_stride(S) + sp];
+    const int64_t k = i / S;
+    const int sp = (int)(i - k * S);
+    const int64_t slot = slots[k];
+    bool valid = true;
+    if (S > 8) valid = (reinterpret_cast<const uint16_t*>(mask)[slot] >> sp) & 1;
+    else if (S > 2) valid = (mask[slot] >> sp) & 1;
+    buf[i] = valid ? inbox[slot * inbox_stride(S) + sp] : 0;
 }
 
-__global__ void k_inbox_import(int32_t S, int32_t* __restrict__ inbox, const int32_t* __restrict__ slots,
-                               int32_t n, const int32_t* __restrict__ buf) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)n * S) return;
-    const int64_t k = i / S, sp = i - k * S;
-    inbox[(int64_t)slots[k] * inbox_stride(S) + sp] = buf[i];
+__global__ void k_inbox_import(int32_t S, int32_t* __restrict__ inbox, uint8_t* __restrict__ mask,
+                               const int32_t* __restrict__ slots, int32_t n, const int32_t* __restrict__ buf) {
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const int64_t slot = slots[k];
+    uint32_t bits = 0;
+    for (int sp = 0; sp < S; ++sp) {
+        const int32_t v = buf[k * S + sp];
+        inbox[slot * inbox_stride(S) + sp] = v;
+        if (v != 0) bits |= 1u << sp;
+    }
+    if (S > 8) reinterpret_cast<uint16_t*>(mask)[slot] = (uint16_t)bits;
+    else if (S > 2) mask[slot] = (uint8_t)bits;
 }
 
-void launch_inbox_export(int32_t S, const int32_t* inbox, const int32_t* slots, int32_t n, int32_t* buf,
-                         cudaStream_t st) {
+void launch_inbox_export(int32_t S, const int32_t* inbox, const uint8_t* mask, const int32_t* slots, int32_t n,
+                         int32_t* buf, cudaStream_t st) {
     if (n <= 0) return;
-    k_inbox_export<<<grid_for((int64_t)n * S), kBlock, 0, st>>>(S, inbox, slots, n, buf);
+    k_inbox_export<<<grid_for((int64_t)n * S), kBlock, 0, st>>>(S, inbox, mask, slots, n, buf);
     ++g_launches;
 }
 
-void launch_inbox_import(int32_t S, int32_t* inbox, const int32_t* slots, int32_t n, const int32_t* buf,
-                         cudaStream_t st) {
+void launch_inbox_import(int32_t S, int32_t* inbox, uint8_t* mask, const int32_t* slots, int32_t n,
+                         const int32_t* buf, cudaStream_t st) {
     if (n <= 0) return;
-    k_inbox_import<<<grid_for((int64_t)n * S), kBlock, 0, st>>>(S, inbox, slots, n, buf);
+    k_inbox_import<<<grid_for(n), kBlock, 0, st>>>(S, inbox, mask, slots, n, buf);
     ++g_launches;
 }
 

@@ -184,15 +184,23 @@ extern "C" int rdsplit_run_static(int32_t n_tets, const int32_t* d_adj, const do
     float2* avv = (float2*)(base + L.avv);
     uint32_t* mask32 = d_rxn_tet_mask ? (uint32_t*)(base + L.mask) : nullptr;
     int32_t* cnt = (int32_t*)(base + L.cnt);
-    int32_t* rem = (int32_t*)(base + L.rem);
+    // inbox masks of both parities, in the space the layout has for a second
+    // count array (from three species on 4 S T bytes hold them)
+    uint8_t* mask[2] = {nullptr, nullptr};
+    if (n_species > 2) {
+        mask[0] = base + L.rem;
+        mask[1] = mask[0] + 4 * T * (size_t)mask_bytes(n_species);
+    }
     int32_t* out[2] = {(int32_t*)(base + L.out0), (int32_t*)(base + L.out1)};
     uint4* thr = (uint4*)(base + L.thr);
 
     // The array keeps the previous call's contents: clear what must start at
-    // 0 (the control words, and both inboxes, whose boundary slots are never
-    // written).
+    // 0 (the control words, and the masks of the inboxes, or up to two
+    // species their words).
     cudaError_t ce = cudaMemsetAsync(base, 0, 3 * 256, st);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(base + L.out0, 0, L.thr - L.out0, st);
+    if (ce == cudaSuccess)
+        ce = n_species > 2 ? cudaMemsetAsync(mask[0], 0, 8 * T * (size_t)mask_bytes(n_species), st)
+                           : cudaMemsetAsync(base + L.out0, 0, L.thr - L.out0, st);
     if (ce != cudaSuccess) {
         cudaGetLastError();
         return rdapi::fail(RDSPLIT_ECUDA, "%s: memset failed: %s", where, cudaGetErrorString(ce));
@@ -211,16 +219,16 @@ extern "C" int rdsplit_run_static(int32_t n_tets, const int32_t* d_adj, const do
     if ((rc = read_err(base, L, st, where))) return rc;
 
     DevMesh m{n_tets, src, g, G, d_vol, mask32, avv, nullptr};
-    DevState s{cnt, rem, err};
+    DevState s{cnt, err};
     launch_counts_in(n_tets, n_species, d_counts, cnt, err, nullptr, st);
     if (std::isfinite(tau)) launch_thresholds(n_tets, mp, g, G, tau, thr, st);
 
     // Algorithm 1: Step 1 aligns the last period to t_end, Steps 2-3 run in
     // the period kernel, Step 4 advances t.
+    const int sms = sm_count();
     double tn = *t;
     int64_t pk = *period;
     int64_t j = 0;
-    const int32_t* prev = nullptr;
     while (tn < t_end) {
         if (pk >= (int64_t)0xffffffffll) return rdapi::fail(RDSPLIT_EOVERFLOW, "%s: period index exceeds 2^32-1", where);
         double tau_k = tau;
@@ -230,15 +238,21 @@ extern "C" int rdsplit_run_static(int32_t n_tets, const int32_t* d_adj, const do
             last = true;
         }
         if (last) launch_thresholds(n_tets, mp, g, G, tau_k, thr, st);
-        int32_t* cur = out[j & 1];
-        PeriodArgs a{(uint32_t)pk, tau_k, (float)tau_k, seed, j == 0 ? 1 : 0, thr, prev, cur};
-        launch_period(m, mp, s, a, 256, st);
-        prev = cur;
+        const int q = (int)(j & 1);
+        PeriodArgs a{(uint32_t)pk, tau_k, (float)tau_k, seed, j == 0 ? 1 : 0, thr, out[q ^ 1], out[q],
+                     mask[q ^ 1], mask[q]};
+        launch_period(m, mp, s, a, rdapi::period_block(n_tets, sms), st);
         tn = last ? t_end : tn + tau;
         pk += 1;
         j += 1;
     }
-    if (j > 0) launch_gather(m, n_species, s, prev, st);
+    if (j > 0) {
+        const int q = (int)((j - 1) & 1);
+        PeriodArgs a{};
+        a.in_prev = out[q];
+        a.mask_prev = mask[q];
+        launch_gather(m, n_species, s, a, st);
+    }
     launch_counts_out(n_tets, n_species, cnt, d_counts, nullptr, st);
     ce = cudaGetLastError();
     if (ce != cudaSuccess) return rdapi::fail(RDSPLIT_ECUDA, "%s: launch failed: %s", where, cudaGetErrorString(ce));

@@ -1,0 +1,486 @@
+// One period (Algorithm 1 of arXiv:1512.03126, Steps 2 and 3) for the 32 tets
+// of a warp, one per lane, with the tets' counts in shared memory.
+//
+// What bounds a period of a small mesh is the serial chain of its slowest
+// tet, and of a large one the instructions and bytes spent on tets where
+// nothing happens.  Three things follow from that here:
+//
+//  * Counts live in shared-memory columns ([species][lane]), so that loops
+//    over species and reactions index them at run time without a register
+//    array per species count (no local memory, one code path for 1 to 16
+//    species, fewer registers).
+//  * The diffusion draws of all lanes and species form one list of Philox
+//    blocks (four molecules each) that the warp works off 32 at a time
+//    (draw_all).
+//  * The reaction phase runs in single precision with error bounds that
+//    certify every decision (react_fast); only a decision inside its bound
+//    repeats the tet in double precision (react_exact).
+//
+// Measured on GB300 against a kernel with the counts in registers, one
+// whole-warp pass per tet of ten molecules or more, and the reaction phase in
+// double precision (a run of periods, counts in and out): 3,072-tet point
+// source, 217 periods, 5.09 -> 2.21 ms; 48,000-tet A/B/C cube, 200 periods,
+// 4.15 -> 2.91 ms; six species, 68,034 tets, 100 periods, 9.29 -> 3.55 ms;
+// 2.4 M-tet bar, 24 periods, 9.48 -> 7.12 ms.
+//
+// Every draw uses the words of the same keyed stream as the sequential
+// definition, so the counts are the same whole numbers.
+#pragma once
+#include "rd_device.cuh"
+#include "rd_internal.h"
+#include "rd_period.cuh"
+
+namespace rdk {
+
+constexpr unsigned kAllLanes = 0xffffffffu;
+// A species with more draws than this is drawn by the whole warp together
+// (at least a full round of 32 Philox blocks); below it its blocks go to the
+// shared list.
+constexpr int32_t kCoopMin = 128;
+constexpr int kListWords = 64;   // draw list of a warp (a round takes 32 entries)
+
+// Shared memory of one warp: N, D (draws of species a reaction touched) and
+// acc[0], acc[1] (leavers per face, two 16-bit counts a word) as columns
+// [species][32], and the draw list.
+__host__ __device__ inline int warp_words(int S, bool react) { return 32 * S * (react ? 4 : 3) + kListWords; }
+
+struct WarpMem {
+    int32_t* N;
+    int32_t* D;
+    uint32_t* acc0;
+    uint32_t* acc1;
+    uint32_t* list;
+    __device__ __forceinline__ WarpMem(int32_t* base, int S, bool react) {
+        N = base;
+        acc0 = reinterpret_cast<uint32_t*>(N + 32 * S);
+        acc1 = acc0 + 32 * S;
+        list = acc1 + 32 * S;
+        D = react ? reinterpret_cast<int32_t*>(list + kListWords) : N;
+    }
+};
+
+// What a period pass needs beside the mesh and the model.
+struct PeriodView {
+    uint32_t period;
+    double tau_k;
+    float tau_kf;
+    uint64_t seed;
+    const uint4* thr;    // thresholds of (species s, tet t) at (s T + t) * thr_stride
+    int thr_stride;
+};
+
+// Reactions of `on` whose reactants are present in the lane's column.
+__device__ __forceinline__ uint32_t possible_in_column(const ModelParams& mp, const int32_t* Ncol, int S, uint32_t on) {
+    uint32_t m = on;
+    for (int s = 0; s < S; ++s) {
+        const int32_t n = Ncol[32 * s];
+        if (n <= 0) m &= ~mp.needs[s];
+        else if (n == 1) m &= ~mp.needs2[s];
+    }
+    return m;
+}
+
+// Propensity of reaction r in single precision (relative error below
+// 8 * 2^-24: three roundings in the rate, three in the combinations, one in
+// their product).
+__device__ __forceinline__ float propensity_f(const ModelParams& mp, int r, const int32_t* Ncol, float2 avf) {
+    const int a = mp.rs1[r], b = mp.rs2[r], o = mp.order[r];
+    float c = mp.kf[r];
+    if (o == 0) return c * avf.x;
+    if (o == 2) c = c * avf.y;
+    const int32_t na = Ncol[32 * a];
+    if (b < 0) return c * (float)na;
+    if (a == b) return c * (0.5f * (float)na * (float)(na - 1));
+    return c * ((float)na * (float)Ncol[32 * b]);
+}
+
+enum : int { kReactNone = 0, kReactDone = 1, kReactDoubt = 2 };
+
+// The reaction phase of one tet (Gillespie's direct method over one period,
+// Step 2 and 2.1) in single precision.  Time is x = t / tau_k.  The mean
+// occupancy telescopes: with N_end the final count and dn_i the change at
+// event time x_i, N-bar = N_end - sum_i dn_i x_i, so the stochastically
+// rounded N* = ceil(N-bar - u) is N_end - floor(sum_i dn_i x_i + u), whose
+// error does not grow with the counts.
+//
+// Bounds, in units of e = 2^-24 (the reference values are the double-precision
+// ones, whose own error is below 1e-12 of these): propensities 8, their sum
+// (at most 32 terms) 39, -log u1 by log1pf or logf (1 ulp each, condition
+// at most 1.45) 4, times tau and divided 3; so a waiting time is off by at
+// most 46 e of itself and, with one rounding per event, an event time by
+// (46 + k) e after k events.  Every comparison with tau_k or tau_k / 2 keeps
+// (128 + 4 k) e away from its limit, the choice of the reaction 128 e of the
+// total propensity, and the rounding of N-bar (256 + 8 k) e per molecule made
+// or consumed (+ 2^-20 for the double-precision sums of counts below 2^20);
+// inside a margin the function undoes its changes and answers kReactDoubt.
+// Waiting times beyond the period are first ruled out by -log u >= 1 - u
+// without a logarithm.
+// Replaces a double-precision chain of one logarithm (24 dependent operations
+// and a division) and three further divisions an event: at 64 cycles an FP64
+// operation it set the period of every small mesh with reactions.
+// On kReactDone: Ncol holds the counts after the phase, *touched the species
+// that changed, and Dcol, for those, N* (mean rule) or the mid-period count
+// (half-step rule).  scratch: the lane's column of one word per species.
+__device__ __forceinline__ int react_fast(const ModelParams& mp, int S, int key, const PeriodView& v, uint32_t on,
+                                          uint32_t poss, float2 avf, int32_t* Ncol, int32_t* Dcol, uint32_t* scratch,
+                                          uint32_t* touched_out) {
+    constexpr float e = 5.9604644775390625e-08f;   // 2^-24
+    constexpr int kMaxEvents = 64;
+    const bool mid = mp.rule == kRuleMid;
+    rdd::Stream st(v.seed, (uint32_t)key, v.period, rdd::kPurposeReaction, 0);
+    float x = 0.0f, dsum = 0.0f;
+    uint32_t touched = 0;
+    int k = 0;
+    bool past = false, doubt = !(v.tau_kf < 1e6f);   // (keeps underflowed rates below 1e-13 a period)
+    while (!doubt) {
+        if (k > 0) poss = possible_in_column(mp, Ncol, S, on);
+        if (!poss) break;                          // total propensity 0
+        const uint64_t x1 = st.bits53();
+        float a0 = 0.0f;
+        for (uint32_t bits = poss; bits; bits &= bits - 1u) a0 += propensity_f(mp, __ffs(bits) - 1, Ncol, avf);
+        const float at = a0 * v.tau_kf;
+        const float eps = (float)(128 + 4 * k) * e;
+        const uint64_t y = 9007199254740991ull - x1;                    // (1 - u1) 2^53
+        const float ylo = (float)(uint32_t)(y >> 29) * e;               // at most 1 - u1
+        if (!(at < 1e30f)) { doubt = true; break; }
+        if (ylo > 0.0f && ylo >= at * ((1.0f + eps) - x) * 1.0001f) break;   // no event before tau_k
+        if (!(at > 1e-6f)) { doubt = true; break; }
+        float E;
+        if (y <= 4503599627370496ull) E = -log1pf(-(float)y * 1.1102230246251565e-16f);
+        else E = -logf((float)(x1 + 1ull) * 1.1102230246251565e-16f);
+        const float xn = x + E / at;
+        if (xn >= 1.0f + eps) break;
+        if (xn > 1.0f - eps) { doubt = true; break; }
+        if (mid && !past) {
+            if (xn >= 0.5f + eps) {
+                for (int s = 0; s < S; ++s) Dcol[32 * s] = Ncol[32 * s];
+                past = true;
+            } else if (xn > 0.5f - eps) {
+                doubt = true;
+                break;
+            }
+        }
+        // the first reaction whose cumulated propensity exceeds u2 a0
+        const float target = (float)st.bits53() * 1.1102230246251565e-16f * a0;
+        const float margin = 128.0f * e * a0;
+        int mu = -1;
+        float cum = 0.0f;
+        for (uint32_t bits = poss; bits; bits &= bits - 1u) {
+            const int r = __ffs(bits) - 1;
+            cum += propensity_f(mp, r, Ncol, avf);
+            if (target < cum - margin) { mu = r; break; }
+            if (target <= cum + margin) break;
+        }
+        if (mu < 0) { doubt = true; break; }
+        float dmax = 0.0f;
+        for (int s = 0; s < S; ++s) {
+            const int dn = mp.delta[mu][s];
+            if (dn == 0) continue;
+            const int32_t n = Ncol[32 * s];
+            if (n >= (1 << 20)) doubt = true;
+            if (!((touched >> s) & 1u)) {
+                scratch[32 * s] = (uint32_t)n;     // to undo
+                if (!mid) Dcol[32 * s] = __float_as_int(0.0f);
+                touched |= 1u << s;
+            }
+            if (!mid) Dcol[32 * s] = __float_as_int(__int_as_float(Dcol[32 * s]) + (float)dn * xn);
+            Ncol[32 * s] = n + dn;
+            dmax = fmaxf(dmax, fabsf((float)dn));
+        }
+        dsum += dmax;
+        x = xn;
+        if (++k > kMaxEvents) doubt = true;
+    }
+    if (!doubt && touched) {
+        const float eps = dsum * ((float)(256 + 8 * k) * e) + 9.5367431640625e-07f;
+        for (uint32_t bits = touched; bits; bits &= bits - 1u) {
+            const int s = __ffs(bits) - 1;
+            if (mid) {
+                if (!past) Dcol[32 * s] = Ncol[32 * s];
+            } else if (mp.rule == kRuleMean) {
+                rdd::Stream rs(v.seed, (uint32_t)key, v.period, rdd::kPurposeRounding, (uint32_t)s);
+                const float w = __int_as_float(Dcol[32 * s]) + (float)rs.bits53() * 1.1102230246251565e-16f;
+                const float fl = floorf(w);
+                if (w - fl < eps || (fl + 1.0f) - w < eps) { doubt = true; break; }
+                Dcol[32 * s] = Ncol[32 * s] - (int32_t)fl;
+            }
+        }
+    }
+    if (doubt) {
+        for (uint32_t bits = touched; bits; bits &= bits - 1u) {
+            const int s = __ffs(bits) - 1;
+            Ncol[32 * s] = (int32_t)scratch[32 * s];
+        }
+        return kReactDoubt;
+    }
+    *touched_out = touched;
+    return touched ? kReactDone : kReactNone;
+}
+
+// The same phase by the double-precision definition, for a tet whose
+// single-precision pass met a decision inside its error bound (or counts or
+// event numbers beyond it).  Returns the touched species, error bits in the
+// upper half.
+static __device__ __noinline__ uint32_t react_exact(const ModelParams& mp, int key, uint32_t period, double tau_k,
+                                                    uint64_t seed, double vol_t, uint32_t on, float2 avf,
+                                                    int32_t* Ncol, int32_t* Dcol, uint32_t* err) {
+    int64_t N64[kMaxS], nmid[kMaxS];
+    double occ[kMaxS], tl[kMaxS];
+    for (int s = 0; s < mp.S; ++s) {
+        N64[s] = Ncol[32 * s];
+        occ[s] = 0.0;
+        tl[s] = 0.0;
+    }
+    uint32_t touched = 0, bad = 0;
+    react_tet(mp, key, period, tau_k, seed, vol_t, on, avf, N64, occ, tl, touched, nmid, err);
+    for (int s = 0; s < mp.S; ++s) {
+        if (!((touched >> s) & 1u)) continue;
+        int64_t n = N64[s];
+        if (n < 0) { bad |= kErrNegative; n = 0; }
+        if (n > 2147483647) { bad |= kErrOverflow; n = 2147483647; }
+        Ncol[32 * s] = (int32_t)n;
+        int64_t star = nmid[s];
+        if (mp.rule != kRuleMid) {
+            rdd::Stream rs(seed, (uint32_t)key, period, rdd::kPurposeRounding, (uint32_t)s);
+            const double nbar = occ[s] / tau_k;
+            const double fl = floor(nbar);
+            star = (int64_t)fl + (rs.u01() < nbar - fl ? 1 : 0);
+        }
+        if (star > 2147483647) star = 2147483647;
+        Dcol[32 * s] = (int32_t)star;
+    }
+    return touched | (bad << 16);
+}
+
+// Step 3 for N* >= kMoleculeCut: min(Binomial(N*, zeta), N) split over the
+// faces by conditional binomials (double precision).
+static __device__ __noinline__ int4 diffuse_binomial(const double* __restrict__ G, const double* __restrict__ gface,
+                                                     int t, int key, int s, double Dsp, uint32_t period, double tau_k,
+                                                     uint64_t seed, int64_t Nt, int64_t Nstar) {
+    const double z = zeta_of(tau_k, Dsp, G[t]);
+    int4 o = make_int4(0, 0, 0, 0);
+    if (!(z > 0.0)) return o;
+    rdd::Stream ds(seed, (uint32_t)key, period, rdd::kPurposeDiffusion, (uint32_t)s);
+    int64_t n = rdd::binomial(Nstar, z, ds);
+    if (n > Nt) n = Nt;
+    if (n == 0) return o;
+    double g[4], suf[4], acc = 0.0;
+    for (int f = 0; f < 4; ++f) g[f] = gface[4 * (int64_t)t + f];
+    for (int f = 3; f >= 0; --f) { acc = g[f] + acc; suf[f] = acc; }
+    int last = -1;
+    for (int f = 0; f < 4; ++f)
+        if (g[f] > 0.0) last = f;
+    int64_t rest = n, nf[4] = {0, 0, 0, 0};
+    for (int f = 0; f < 4; ++f) {
+        if (!(g[f] > 0.0)) continue;
+        if (f == last) { nf[f] = rest; break; }
+        const int64_t x = rdd::binomial(rest, g[f] / suf[f], ds);
+        nf[f] = x;
+        rest -= x;
+    }
+    return make_int4((int)nf[0], (int)nf[1], (int)nf[2], (int)nf[3]);
+}
+
+// The molecule-by-molecule draw that stops once all Nt molecules have left:
+// only where N* exceeds the count and more than Nt of the N* draws leave.
+static __device__ __noinline__ int4 draw_capped(uint64_t seed, uint32_t period, int key, int s, int32_t Nstar,
+                                                int32_t Nt, uint4 C) {
+    int4 o = make_int4(0, 0, 0, 0);
+    rdd::Stream ds(seed, (uint32_t)key, period, rdd::kPurposeDiffusion, (uint32_t)s);
+    int32_t moved = 0;
+    for (int32_t i = 0; i < Nstar && moved < Nt; ++i) {
+        const uint32_t u = ds.u32();
+        if (rdd::below(u, C.x)) { o.x += 1; ++moved; }
+        else if (rdd::below(u, C.y)) { o.y += 1; ++moved; }
+        else if (rdd::below(u, C.z)) { o.z += 1; ++moved; }
+        else if (rdd::below(u, C.w)) { o.w += 1; ++moved; }
+    }
+    return o;
+}
+
+// Leavers per face among the first m words of a Philox block, two 16-bit
+// counts a word.  The thresholds are cumulative (C.x <= ... <= C.w), so
+// a word is below C_f for every face from its own on: faces are counted by
+// differences.  0xffffffff means "always".
+__device__ __forceinline__ void count_block(const uint4& w, int m, const uint4& C, uint32_t& a0, uint32_t& a1) {
+    const uint32_t u0 = w.x;
+    const uint32_t u1 = m > 1 ? w.y : 0xffffffffu;
+    const uint32_t u2 = m > 2 ? w.z : 0xffffffffu;
+    const uint32_t u3 = m > 3 ? w.w : 0xffffffffu;
+    if (min(min(u0, u1), min(u2, u3)) >= C.w && C.w != 0xffffffffu) return;
+    auto under = [&](uint32_t c) -> uint32_t {
+        const uint32_t n = (u0 < c) + (u1 < c) + (u2 < c) + (u3 < c);
+        return c == 0xffffffffu ? (uint32_t)m : n;
+    };
+    const uint32_t nx = under(C.x), ny = under(C.y), nz = under(C.z), nw = under(C.w);
+    a0 += nx | ((ny - nx) << 16);
+    a1 += (nz - ny) | ((nw - nz) << 16);
+}
+
+// The diffusion draws of a warp's tets (Step 3; Eq. 2-3): every (lane,
+// species) with molecules contributes ceil(n / 4) Philox blocks to one list,
+// filled block index by block index with a ballot (so neighbouring entries
+// belong to different lanes), and 32 entries make a round with one block a
+// lane.  The cost follows the number of blocks, not the largest count of
+// a lane or the species present in any lane.  big(sp, N*) handles a lane's
+// binomial draws.  Returns the species whose acc words hold leavers-to-be.
+// All lanes must call it.  The per-lane loop with a whole-warp pass per
+// species and tet from 10 molecules on took one serial pass a tet: 600 cycles
+// each, up to 32 a warp.
+template <class Big>
+__device__ __forceinline__ uint32_t draw_all(const ModelParams& mp, int S, int64_t T, const WarpMem& w,
+                                             const PeriodView& v, int t, int key, uint32_t present, uint32_t touched,
+                                             Big big) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const uint32_t k0 = (uint32_t)v.seed, k1 = (uint32_t)(v.seed >> 32);
+    uint32_t drawn = 0;
+    int cnt = 0;
+    // species after species; one turn more flushes the list
+    for (int sp = 0; sp <= S; ++sp) {
+        int n = 0;
+        if (sp < S && mp.D[sp] != 0.0) {
+            if ((present >> sp) & 1u) {
+                n = ((touched >> sp) & 1u) ? w.D[32 * sp + lane] : w.N[32 * sp + lane];
+                if (n >= (int32_t)kMoleculeCut) {
+                    big(sp, n);
+                    n = 0;
+                }
+                if (n > 0) {
+                    w.acc0[32 * sp + lane] = 0u;
+                    w.acc1[32 * sp + lane] = 0u;
+                    drawn |= 1u << sp;
+                }
+            }
+            unsigned cm = __ballot_sync(kAllLanes, n > kCoopMin);
+            while (cm) {
+                const int src = __ffs(cm) - 1;
+                cm &= cm - 1u;
+                const int nn = __shfl_sync(kAllLanes, n, src);
+                const int tt = __shfl_sync(kAllLanes, t, src), kk = __shfl_sync(kAllLanes, key, src);
+                const uint4 C = __ldg(v.thr + ((int64_t)sp * T + tt) * v.thr_stride);
+                uint32_t a0 = 0, a1 = 0;
+                for (int blk = lane; 4 * blk < nn; blk += 32)
+                    count_block(rdd::philox_block((uint32_t)blk, (uint32_t)kk, v.period,
+                                                  (rdd::kPurposeDiffusion << 16) | (uint32_t)sp, k0, k1),
+                                min(4, nn - 4 * blk), C, a0, a1);
+                a0 = __reduce_add_sync(kAllLanes, a0);
+                a1 = __reduce_add_sync(kAllLanes, a1);
+                if (lane == src) {
+                    w.acc0[32 * sp + lane] = a0;
+                    w.acc1[32 * sp + lane] = a1;
+                    n = 0;
+                }
+            }
+        }
+        const int nb = (n + 3) >> 2;
+        for (int b = 0;; ++b) {
+            const unsigned act = __ballot_sync(kAllLanes, b < nb);
+            if (b < nb)
+                w.list[cnt + __popc(act & lt)] =
+                    (uint32_t)lane | ((uint32_t)(min(4, n - 4 * b) - 1) << 5) | ((uint32_t)sp << 7) | ((uint32_t)b << 11);
+            cnt += __popc(act);
+            if (cnt >= 32 || (sp == S && cnt > 0)) {
+                // one round: the last min(32, cnt) entries, one a lane
+                __syncwarp();
+                const int take = min(cnt, 32);
+                cnt -= take;
+                const bool mine = lane < take;
+                const uint32_t en = mine ? w.list[cnt + lane] : (uint32_t)lane;
+                const int owner = (int)(en & 31u);
+                const int tu = __shfl_sync(kAllLanes, t, owner), ku = __shfl_sync(kAllLanes, key, owner);
+                if (mine) {
+                    const int su = (int)((en >> 7) & 15u);
+                    const uint4 C = __ldg(v.thr + ((int64_t)su * T + tu) * v.thr_stride);
+                    uint32_t a0 = 0, a1 = 0;
+                    count_block(rdd::philox_block(en >> 11, (uint32_t)ku, v.period,
+                                                  (rdd::kPurposeDiffusion << 16) | (uint32_t)su, k0, k1),
+                                (int)((en >> 5) & 3u) + 1, C, a0, a1);
+                    if (a0) atomicAdd(w.acc0 + 32 * su + owner, a0);
+                    if (a1) atomicAdd(w.acc1 + 32 * su + owner, a1);
+                }
+                __syncwarp();
+            }
+            if (act == 0u) break;
+        }
+    }
+    return drawn;
+}
+
+// Steps 2 and 3 for the warp's tets: column N of each live lane holds its
+// counts.  After it N holds what stays; emit(sp, o) was called by a lane for
+// each species of which molecules leave (o: per face).  Bits of the species
+// whose count changed are added to *dirty.  With kDefer, a lane whose tet
+// needs the reaction phase leaves it undone and answers true in *deferred.
+// Returns error bits.  All lanes must call it.
+template <bool kReact, bool kDefer, class Emit>
+__device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParams& mp, int S, const WarpMem& w,
+                                              const PeriodView& v, int t, bool live, uint32_t* dirty, bool* deferred,
+                                              uint32_t* err, Emit& emit) {
+    const int lane = threadIdx.x & 31;
+    const int key = live ? key_of(m, t) : 0;
+    uint32_t bad = 0, touched = 0;
+    if (kReact) {
+        if (live) {
+            const uint32_t all = mp.has_mask ? m.mask[t] : 0xffffffffu;
+            const uint32_t on = all & mp.kpos;
+            const uint32_t poss = possible_in_column(mp, w.N + lane, S, on);
+            if (poss) {
+                const float2 avf = m.avv[t];
+                if (kDefer) {
+                    // only the first waiting time, by its bound
+                    float a0 = 0.0f;
+                    for (uint32_t bits = poss; bits; bits &= bits - 1u)
+                        a0 += propensity_f(mp, __ffs(bits) - 1, w.N + lane, avf);
+                    rdd::Stream st(v.seed, (uint32_t)key, v.period, rdd::kPurposeReaction, 0);
+                    const uint64_t y = 9007199254740991ull - st.bits53();
+                    const float need = a0 * v.tau_kf * 1.0001f * 1.0001f;
+                    *deferred = !(need < 3.0e38f) || !((float)(uint32_t)(y >> 29) * 5.9604644775390625e-08f >= need) ||
+                                (y >> 29) == 0ull;
+                    if (*deferred) live = false;
+                } else {
+                    uint32_t tch = 0;
+                    int r = react_fast(mp, S, key, v, on, poss, avf, w.N + lane, w.D + lane, w.acc0 + lane, &tch);
+                    if (r == kReactDoubt) {
+                        tch = react_exact(mp, key, v.period, v.tau_k, v.seed, m.vol[t], all, avf, w.N + lane,
+                                          w.D + lane, err);
+                        bad |= tch >> 16;
+                        tch &= 0xffffu;
+                    }
+                    *dirty |= tch;
+                    if (mp.rule != kRuleEnd) touched = tch;   // first order: the draw uses N(tau_k)
+                }
+            }
+        }
+    }
+    uint32_t present = 0;
+    if (live)
+        for (int s = 0; s < S; ++s)
+            if (w.N[32 * s + lane] > 0) present |= 1u << s;
+    const uint32_t drawn = draw_all(mp, S, m.T, w, v, t, key, present, touched, [&](int sp, int32_t star) {
+        const int32_t Nt = w.N[32 * sp + lane];
+        const int4 o = diffuse_binomial(m.G, m.g, t, key, sp, mp.D[sp], v.period, v.tau_k, v.seed, Nt, star);
+        const int32_t all = o.x + o.y + o.z + o.w;
+        if (all > 0) {
+            w.N[32 * sp + lane] = Nt - all;
+            *dirty |= 1u << sp;
+            emit(sp, o);
+        }
+    });
+    for (uint32_t bits = drawn; bits; bits &= bits - 1u) {
+        const int sp = __ffs(bits) - 1;
+        const uint32_t a = w.acc0[32 * sp + lane], b = w.acc1[32 * sp + lane];
+        if ((a | b) == 0u) continue;
+        int4 o = make_int4((int)(a & 0xffffu), (int)(a >> 16), (int)(b & 0xffffu), (int)(b >> 16));
+        const int32_t Nt = w.N[32 * sp + lane];
+        if (o.x + o.y + o.z + o.w > Nt)
+            o = draw_capped(v.seed, v.period, key, sp, w.D[32 * sp + lane], Nt,
+                            __ldg(v.thr + ((int64_t)sp * m.T + t) * v.thr_stride));
+        w.N[32 * sp + lane] = Nt - (o.x + o.y + o.z + o.w);
+        *dirty |= 1u << sp;
+        emit(sp, o);
+    }
+    return bad;
+}
+
+}  // namespace rdk

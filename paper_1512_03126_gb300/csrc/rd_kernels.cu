@@ -158,28 +158,57 @@ void launch_zeta_hist(int32_t T, const double* G, double tau, double D, int32_t 
 
 // C_f = floor(2^32 zeta (g_0 + ... + g_f) / G): a molecule leaves through the
 // first face f whose threshold exceeds its 32-bit draw, and stays if none does.
-__global__ void k_thresholds(int32_t T, ModelParams mp, const double* __restrict__ g,
-                             const double* __restrict__ G, double tau_k, uint4* __restrict__ thr) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)T * mp.S) return;
-    int s = (int)(i / T);
-    int t = (int)(i - (int64_t)s * T);
-    double Gt = G[t];
-    double z = zeta_of(tau_k, mp.D[s], Gt);
+// By the definition's operations:
+static __device__ __noinline__ uint4 thresholds_by_definition(double tau_k, double D, double Gt, const double* cum) {
+    const double z = zeta_of(tau_k, D, Gt);
     uint32_t C[4] = {0, 0, 0, 0};
-    if (z > 0.0) {
-        double cum = 0.0;
+    if (z > 0.0)
+        for (int f = 0; f < 4; ++f) C[f] = rdd::threshold_of(z * (cum[f] / Gt));
+    return make_uint4(C[0], C[1], C[2], C[3]);
+}
+
+// One tet a thread, all species.  Below zeta = 1 the G's cancel: 2^32 zeta
+// cum_f / G = (2^32 tau D) cum_f, off by at most 6 * 2^-53 of itself from the
+// definition's value (its five roundings and one here), so by less than
+// 2^-18.  Its floor is the definition's unless it lies within 4 * 2^-20 of a
+// whole number (8 are kept); such a face (one in 65,536), and every tet whose zeta is not
+// clearly below 1, takes the definition's operations.  FP64 (64 cycles an
+// operation, 562 a division) is what bounds this kernel: two operations a
+// face instead of a division and four.  2.4 M tets of 8 species: 2060 us with
+// one thread a (species, tet) and the divisions.
+__global__ void k_thresholds(int32_t T, const __grid_constant__ ModelParams mp, const double* __restrict__ g,
+                             const double* __restrict__ G, double tau_k, uint4* __restrict__ thr) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= T) return;
+    const double2 g01 = reinterpret_cast<const double2*>(g)[2 * (int64_t)t];
+    const double2 g23 = reinterpret_cast<const double2*>(g)[2 * (int64_t)t + 1];
+    double cum[4];
+    cum[0] = 0.0 + g01.x;
+    cum[1] = cum[0] + g01.y;
+    cum[2] = cum[1] + g23.x;
+    cum[3] = cum[2] + g23.y;
+    const double Gt = G[t];
+    for (int s = 0; s < mp.S; ++s) {
+        const double scale = tau_k * mp.D[s] * 4503599627370496.0;   // 2^52 tau D
+        uint32_t C[4];
+        // 2^52 zeta, clearly below 2^52 (and finite)
+        bool sure = scale * Gt < 4503599627370496.0 * 0.999;
+#pragma unroll
         for (int f = 0; f < 4; ++f) {
-            cum = cum + g[4 * t + f];
-            C[f] = rdd::threshold_of(z * (cum / Gt));
+            const unsigned long long y = (unsigned long long)(scale * cum[f]);   // 2^20 units of a threshold step
+            const uint32_t frac = (uint32_t)y & 0xfffffu;
+            sure = sure && (y == 0ull || frac - 8u < 0xfffffu - 16u);
+            C[f] = (uint32_t)(y >> 20);
         }
+        uint4 c = make_uint4(C[0], C[1], C[2], C[3]);
+        if (!sure) c = thresholds_by_definition(tau_k, mp.D[s], Gt, cum);
+        thr[(int64_t)s * T + t] = c;
     }
-    thr[i] = make_uint4(C[0], C[1], C[2], C[3]);
 }
 
 void launch_thresholds(int32_t T, const ModelParams& mp, const double* g, const double* G, double tau_k,
                        uint4* thr, cudaStream_t st) {
-    k_thresholds<<<grid_for((int64_t)T * mp.S), kBlock, 0, st>>>(T, mp, g, G, tau_k, thr);
+    k_thresholds<<<grid_for(T), kBlock, 0, st>>>(T, mp, g, G, tau_k, thr);
     ++g_launches;
 }
 
@@ -201,35 +230,66 @@ void launch_pack_mask(int32_t T, int32_t R, const uint8_t* mask8, uint32_t* mask
 }
 
 // Counts between the caller's canonical [T][S] order and the stored [S][T]
-// (stored tet t is canonical tet perm[t], or t without a reordering).
+// (stored tet t is canonical tet perm[t], or t without a reordering).  A block
+// takes 256 tets: species by species on the stored side, and the caller's
+// side through shared memory so that both are contiguous (no alignment is
+// asked of the caller's array).
 __global__ void k_counts_in(int32_t T, int32_t S, const int32_t* __restrict__ ts, int32_t* __restrict__ sm,
                             uint32_t* err, const int32_t* __restrict__ perm) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)T * S) return;
-    int t = (int)(i / S), s = (int)(i - (int64_t)t * S);
-    const int64_t c = perm ? perm[t] : t;
-    int32_t v = ts[c * S + s];
-    if (v < 0) { atomicOr(err, kErrNegative); v = 0; }
-    sm[(int64_t)s * T + t] = v;
+    extern __shared__ int32_t tile[];   // [256][S + 1 - S % 2]: an odd stride, free of bank conflicts
+    const int ld = S | 1;
+    const int64_t t0 = (int64_t)blockIdx.x * kBlock;
+    const int n = (int)min((int64_t)kBlock, T - t0);
+    if (!perm) {
+        for (int i = threadIdx.x; i < n * S; i += kBlock) {
+            const int r = i / S;
+            tile[r * ld + (i - r * S)] = ts[t0 * S + i];
+        }
+        __syncthreads();
+    }
+    const int r = threadIdx.x;
+    if (r >= n) return;
+    const int64_t c = perm ? perm[t0 + r] : 0;
+    uint32_t bad = 0;
+    for (int s = 0; s < S; ++s) {
+        int32_t v = perm ? ts[c * S + s] : tile[r * ld + s];
+        if (v < 0) { bad |= kErrNegative; v = 0; }
+        sm[(int64_t)s * T + t0 + r] = v;
+    }
+    if (bad) atomicOr(err, bad);
 }
 
 __global__ void k_counts_out(int32_t T, int32_t S, const int32_t* __restrict__ sm, int32_t* __restrict__ ts,
                              const int32_t* __restrict__ perm) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)T * S) return;
-    int t = (int)(i / S), s = (int)(i - (int64_t)t * S);
-    const int64_t c = perm ? perm[t] : t;
-    ts[c * S + s] = sm[(int64_t)s * T + t];
+    extern __shared__ int32_t tile[];
+    const int ld = S | 1;
+    const int64_t t0 = (int64_t)blockIdx.x * kBlock;
+    const int n = (int)min((int64_t)kBlock, T - t0);
+    const int r = threadIdx.x;
+    if (r < n) {
+        const int64_t c = perm ? perm[t0 + r] : 0;
+        for (int s = 0; s < S; ++s) {
+            const int32_t v = sm[(int64_t)s * T + t0 + r];
+            if (perm) ts[c * S + s] = v;
+            else tile[r * ld + s] = v;
+        }
+    }
+    if (perm) return;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n * S; i += kBlock) {
+        const int q = i / S;
+        ts[t0 * S + i] = tile[q * ld + (i - q * S)];
+    }
 }
 
 void launch_counts_in(int32_t T, int32_t S, const int32_t* ts, int32_t* sm, uint32_t* err, const int32_t* perm,
                       cudaStream_t st) {
-    k_counts_in<<<grid_for((int64_t)T * S), kBlock, 0, st>>>(T, S, ts, sm, err, perm);
+    k_counts_in<<<grid_for(T), kBlock, kBlock * (S | 1) * sizeof(int32_t), st>>>(T, S, ts, sm, err, perm);
     ++g_launches;
 }
 
 void launch_counts_out(int32_t T, int32_t S, const int32_t* sm, int32_t* ts, const int32_t* perm, cudaStream_t st) {
-    k_counts_out<<<grid_for((int64_t)T * S), kBlock, 0, st>>>(T, S, sm, ts, perm);
+    k_counts_out<<<grid_for(T), kBlock, kBlock * (S | 1) * sizeof(int32_t), st>>>(T, S, sm, ts, perm);
     ++g_launches;
 }
 

@@ -43,8 +43,8 @@ extern "C" {
 #define RDSPLIT_EINVAL (-1)    /* bad argument, malformed mesh or model */
 #define RDSPLIT_ENOMEM (-2)    /* device allocation failed or budget exceeded */
 #define RDSPLIT_ECUDA (-3)     /* a CUDA runtime call failed */
-#define RDSPLIT_ETIMEOUT (-4)  /* reserved: no call returns it (the kernels wait
-                                  only at hardware barriers, never on a flag) */
+#define RDSPLIT_ETIMEOUT (-4)  /* a run's grid barrier was waited for in vain (two
+                                  minutes; not expected: its blocks are resident) */
 #define RDSPLIT_EOVERFLOW (-5) /* a count would exceed INT32_MAX, or a
                                   period would exceed the per-tet event cap */
 #define RDSPLIT_ESTATE (-6)    /* call out of order (e.g. run before set_model) */
@@ -202,17 +202,20 @@ int rdsplit_get_shape(rdsplit_mesh_t mesh, int32_t* n_tets, int32_t* n_species);
  * Kernel form of the period (Algorithm 1, Steps 2-3), a tuning choice with no
  * effect on results (every draw is keyed by tet and period):
  *   mode 1  one pass: gather, reactions and draws of each tet in one kernel
- *   mode 2  two passes: a light pass runs the tets that need neither the
- *           reaction phase nor the double-precision binomial (compiled
- *           without those samplers, so it keeps more warps per SM) and
- *           defers the others to a slow pass with the full step
- *   mode 0  automatic (default): one pass
- *   block   threads per block of the period kernel (of the light pass in
+ *   mode 2  two passes: the first runs the tets in which no reaction has to
+ *           be followed (compiled without the reaction phase, so it keeps
+ *           more warps per SM) and defers the others to the second
+ *   mode 0  automatic (default): while all tets of the mesh are resident on
+ *           the GPU at once (up to 24 warps of 32 tets per multiprocessor),
+ *           many periods per launch with a grid barrier between them; else
+ *           one pass per period
+ *   block   threads per block of the period kernel (of the first pass in
  *           mode 2): a multiple of 32 in 32..256, or 0 (default) for a size
  *           chosen from the mesh (smaller blocks for small meshes, so that
  *           their tets spread over all SMs)
  * rdsplit_get_period_kernel reports whether runs use two passes and the
- * block size they use.
+ * block size of a one-period launch.  A block size, or timing
+ * (rdsplit_set_timing), asks for one-period launches.
  */
 int rdsplit_set_period_kernel(rdsplit_mesh_t mesh, int32_t mode, int32_t block);
 int rdsplit_get_period_kernel(rdsplit_mesh_t mesh, int32_t* two_passes, int32_t* block);

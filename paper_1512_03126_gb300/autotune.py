@@ -89,7 +89,8 @@ def _timed(fn, stream) -> float:
     return e0.elapsed_time(e1)
 
 
-DENSE_CANDIDATES = [(1, 32), (1, 64), (1, 128), (1, 256), (2, 64), (2, 256)]
+# (0, 0): automatic, which keeps a small mesh resident over many periods a launch
+DENSE_CANDIDATES = [(0, 0), (1, 32), (1, 64), (1, 128), (1, 256), (2, 64), (2, 256)]
 
 
 def tune_period(rd, w, stream, periods: int = 48, candidates=None, use_cache: bool = True) -> dict:
@@ -98,7 +99,7 @@ def tune_period(rd, w, stream, periods: int = 48, candidates=None, use_cache: bo
     also the batched engine on the same periods.  Returns {"best": {...},
     "results": [...]} with "best" the fastest dense form (the engine's time
     is reported for the single-mesh choice)."""
-    key = f"{_device_name()}|period|{bucket(w.mesh.n_tets, w.model.n_species, w.model.n_reactions)}"
+    key = f"{_device_name()}|dense run|{bucket(w.mesh.n_tets, w.model.n_species, w.model.n_reactions)}"
     if use_cache:
         hit = cache_get(key)
         if hit:

@@ -92,6 +92,7 @@ int check_err_impl(rdsplit_mesh* h, const char* where) {
     if (e & kErrAdjAsym) return fail(RDSPLIT_EINVAL, "%s: adjacency is not symmetric", where);
     if (e & kErrVolume) return fail(RDSPLIT_EINVAL, "%s: a tet volume is not finite and positive", where);
     if (e & kErrFace) return fail(RDSPLIT_EINVAL, "%s: a face area or centroid distance is invalid", where);
+    if (e & kErrTimeout) return fail(RDSPLIT_ETIMEOUT, "%s: a grid barrier's wait ran out", where);
     if (e & kErrOverflow) return fail(RDSPLIT_EOVERFLOW, "%s: a count exceeded INT32_MAX", where);
     if (e & kErrEventCap) return fail(RDSPLIT_EOVERFLOW, "%s: SSA event cap per tet and period exceeded", where);
     if (e & kErrNegative) return fail(RDSPLIT_EINVAL, "%s: negative count", where);
@@ -145,16 +146,22 @@ static cudaError_t clear_inboxes(rdsplit_mesh* h) {
 }
 
 // The period loop of Algorithm 1 for one handle.  Step 1: the last period is
-// shortened so that it ends on t_end.  Step 2-3 run in k_period, which also
-// applies the previous period's transfers; the closing k_gather applies the
-// last one.  Step 4: t += tau.
+// shortened so that it ends on t_end.  Steps 2-3 run in the kernels, which
+// also apply the previous period's transfers; the closing transfer applies the
+// last one.  Step 4: t += tau.  Meshes whose tets are all resident at once
+// take many periods a launch (unless a kernel form was asked for or launches
+// are being timed), others one.
 int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) {
     if (!h->has_model) return fail(RDSPLIT_ESTATE, "rdsplit_run: no model attached");
     if (std::isnan(t_end)) return fail(RDSPLIT_EINVAL, "rdsplit_run: t_end is NaN");
     DevMesh m = h->dev_mesh();
     DevState s = h->dev_state();
+    const int sms = sm_count();
     const bool split = two_pass(h);
-    const int block = period_block(h, sm_count());
+    const int block = period_block(h, sms);
+    int warps = 0;
+    bool resident = h->period_mode == 0 && h->period_block == 0 && h->timing_stride == 0 &&
+                    run_shape(h->T, sms, &warps) > 0;
     if (split && h->t < t_end && max_periods != 0) {
         cudaError_t ce = cudaMemsetAsync(h->dqn, 0, 2 * sizeof(int32_t), h->stream);
         if (ce != cudaSuccess) {
@@ -163,24 +170,48 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
         }
     }
     if (h->inbox_dirty) CUDA_TRY(clear_inboxes(h));
-    int64_t j = 0;
+    int64_t j = 0;        // periods done
+    int64_t jl = 0;       // of them in single launches since the last closing transfer
     while (h->t < t_end && (max_periods < 0 || j < max_periods)) {
         h->inbox_dirty = true;   // until the closing transfer
-        if (h->period >= (int64_t)0xffffffffll)
-            return fail(RDSPLIT_EOVERFLOW, "rdsplit_run: period index exceeds 2^32-1");
-        double tau_k = h->tau;
+        // the next stretch: one period, or as many as a resident launch takes
+        int n = 0;
         bool last = false;
-        if (h->t + h->tau > t_end) {
-            tau_k = t_end - h->t;
-            last = true;
+        double t = h->t, tau_k = h->tau;
+        const int64_t room = 0xffffffffll - h->period;
+        if (room <= 0) return fail(RDSPLIT_EOVERFLOW, "rdsplit_run: period index exceeds 2^32-1");
+        int64_t most = std::min<int64_t>(resident ? kRunPeriods : 1, room);
+        if (max_periods >= 0) most = std::min<int64_t>(most, max_periods - j);
+        while (n < most && t < t_end) {
+            if (t + h->tau > t_end) {
+                tau_k = t_end - t;
+                last = true;
+                t = t_end;
+            } else {
+                t = t + h->tau;
+            }
+            ++n;
         }
-        const uint4* thr = h->thr;
-        if (last) {
-            launch_thresholds(h->T, h->mp, h->g, h->G, tau_k, h->thr_last, h->stream);
-            thr = h->thr_last;
+        if (last) launch_thresholds(h->T, h->mp, h->g, h->G, tau_k, h->thr_last, h->stream);
+        if (resident) {
+            RunArgs r{(uint32_t)h->period, n, last ? 1 : 0, h->tau, tau_k, (float)h->tau, (float)tau_k, seed, h->thr,
+                      h->thr_last, {h->inbox[0], h->inbox[1]}, {h->imask[0], h->imask[1]}, h->barrier,
+                      h->barrier_base};
+            int grid = 0;
+            if (launch_run(m, h->mp, s, r, sms, &grid, h->stream)) {
+                h->barrier_base += (uint32_t)grid * (uint32_t)n;
+                h->inbox_dirty = false;
+                h->t = t;
+                h->period += n;
+                j += n;
+                continue;
+            }
+            resident = false;
+            continue;
         }
-        const int q = (int)(j & 1);
-        PeriodArgs a{(uint32_t)h->period, tau_k, (float)tau_k, seed, j == 0 ? 1 : 0, thr,
+        const uint4* thr = last ? h->thr_last : h->thr;
+        const int q = (int)(jl & 1);
+        PeriodArgs a{(uint32_t)h->period, tau_k, (float)tau_k, seed, jl == 0 ? 1 : 0, thr,
                      h->inbox[q ^ 1], h->inbox[q], h->imask[q ^ 1], h->imask[q]};
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (h->timing_stride > 0 && j % h->timing_stride == 0) {
@@ -188,15 +219,16 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
             e1 = next_event(h);
         }
         if (e0 && e1) cudaEventRecord(e0, h->stream);
-        if (split) launch_period_split(m, h->mp, s, a, h->dq, h->dqn, (int32_t)(j & 1), block, h->stream);
+        if (split) launch_period_split(m, h->mp, s, a, h->dq, h->dqn, (int32_t)(jl & 1), block, h->stream);
         else launch_period(m, h->mp, s, a, block, h->stream);
         if (e0 && e1) cudaEventRecord(e1, h->stream);
-        h->t = last ? t_end : h->t + h->tau;
+        h->t = t;
         h->period += 1;
         j += 1;
+        jl += 1;
     }
-    if (j > 0) {
-        const int q = (int)((j - 1) & 1);
+    if (jl > 0) {
+        const int q = (int)((jl - 1) & 1);
         PeriodArgs a{};
         a.in_prev = h->inbox[q];
         a.mask_prev = h->imask[q];
@@ -206,6 +238,11 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
     if (rc) return rc;
     h->inbox_dirty = false;
     rc = check_err(h, "rdsplit_run");
+    if (rc == RDSPLIT_ETIMEOUT) {   // blocks left the launch early
+        h->inbox_dirty = true;
+        CUDA_TRY(cudaMemsetAsync(h->barrier, 0, sizeof(uint32_t), h->stream));
+        h->barrier_base = 0;
+    }
     collect_timing(h);
     return rc;
 }
@@ -327,7 +364,7 @@ int mesh_create_impl(const char* where, int32_t n_tets, const int32_t* adj, cons
         (rc = alloc_into(&d_dist, 4 * T, "dist")) || (rc = alloc_into(&h->vol, T, "vol")) ||
         (rc = alloc_into(&h->src, T, "src")) || (rc = alloc_into(&h->g, 4 * T, "g")) ||
         (rc = alloc_into(&h->G, T, "G")) || (rc = alloc_into(&h->gmax, 1, "gmax")) ||
-        (rc = alloc_into(&h->err, 1, "err")) || (reorder && (rc = alloc_into(&h->perm, T, "order"))))
+        (rc = alloc_into(&h->err, 1, "err")) || (rc = alloc_into(&h->barrier, 1, "barrier")) || (reorder && (rc = alloc_into(&h->perm, T, "order"))))
         return cleanup(rc);
     cudaStream_t st = h->stream;
     cudaError_t ce = cudaSuccess;
@@ -338,6 +375,7 @@ int mesh_create_impl(const char* where, int32_t n_tets, const int32_t* adj, cons
     if (reorder) ce = ce ? ce : cudaMemcpyAsync(h->perm, perm.data(), 4 * T, cudaMemcpyHostToDevice, st);
     ce = ce ? ce : cudaMemsetAsync(h->gmax, 0, sizeof(unsigned long long), st);
     ce = ce ? ce : cudaMemsetAsync(h->err, 0, sizeof(uint32_t), st);
+    ce = ce ? ce : cudaMemsetAsync(h->barrier, 0, sizeof(uint32_t), st);
     if (ce != cudaSuccess) {
         cudaGetLastError();
         return cleanup(fail(RDSPLIT_ECUDA, "%s: copy failed: %s", where, cudaGetErrorString(ce)));

@@ -34,6 +34,8 @@ struct rdsplit_mesh {
     int32_t* rem = nullptr;                   // the batched engine's second count buffer
     int32_t* inbox[2] = {nullptr, nullptr};   // [T][4][Sp] transfer inboxes by period parity
     uint8_t* imask[2] = {nullptr, nullptr};   // their masks (three species or more)
+    uint32_t* barrier = nullptr;              // grid-barrier counter of a run's launches
+    uint32_t barrier_base = 0;                // its value between runs
     bool inbox_dirty = false;                 // a run or partition run left inbox words or masks set
     uint4* thr = nullptr;
     uint4* thr_last = nullptr;
@@ -77,7 +79,7 @@ struct rdsplit_mesh {
     ~rdsplit_mesh() {
         for (cudaEvent_t e : ev_pool) cudaEventDestroy(e);
         free_model();
-        void* ps[] = {src, g, G, vol, gmax, err, bits[0], bits[1], packed, N2, perm};
+        void* ps[] = {src, g, G, vol, gmax, err, barrier, bits[0], bits[1], packed, N2, perm};
         for (void* p : ps) rdapi::dev_free(p);
     }
 };
@@ -100,6 +102,8 @@ inline int period_block(int64_t T, int sms) {
 inline int period_block(const rdsplit_mesh* h, int sms) {
     return h->period_block > 0 ? h->period_block : period_block(h->T, sms);
 }
+// Periods a launch of k_run takes at most (some milliseconds to tens of them).
+constexpr int kRunPeriods = 4096;
 int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed);
 int check_err(rdsplit_mesh* h, const char* where);
 }  // namespace rdapi

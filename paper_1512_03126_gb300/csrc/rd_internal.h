@@ -18,6 +18,7 @@ enum : uint32_t {
     kErrNegative = 1u << 4,      // negative count (input or invariant)
     kErrOverflow = 1u << 5,      // a count would exceed INT32_MAX
     kErrEventCap = 1u << 6,      // more SSA events in one tet-period than the cap
+    kErrTimeout = 1u << 7,       // a grid barrier's wait ran out
 };
 
 // Chemistry, passed by value to kernels (lives in the constant bank).
@@ -143,6 +144,28 @@ void launch_inbox_import(int32_t S, int32_t* inbox, uint8_t* mask, const int32_t
 // of 32).
 void launch_period_split(const DevMesh& m, const ModelParams& mp, const DevState& s, const PeriodArgs& a,
                          int32_t* queue, int32_t* qcount, int32_t parity, int block, cudaStream_t st);
+
+// A stretch of periods in one cooperative launch (k_run).
+struct RunArgs {
+    uint32_t period0;       // global index of the stretch's first period
+    int32_t periods;        // >= 1
+    int32_t last_short;     // the stretch's last period has length tau_last and thresholds thr_last
+    double tau, tau_last;
+    float tauf, tau_lastf;
+    uint64_t seed;
+    const uint4* thr;
+    const uint4* thr_last;
+    int32_t* inbox[2];
+    uint8_t* mask[2];
+    uint32_t* barrier;      // grid-barrier counter; holds barrier_base before the launch
+    uint32_t barrier_base;  // and barrier_base + grid * periods after it
+};
+// Launches it if the mesh's tets fit on the device at once (else, or when a
+// cooperative launch is refused, answers false with nothing launched); *grid
+// receives its blocks.
+bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int sms, int* grid,
+                cudaStream_t st);
+int run_shape(int64_t T, int sms, int* warps);
 
 int64_t launches();
 int sm_count();       // multiprocessors of the current device

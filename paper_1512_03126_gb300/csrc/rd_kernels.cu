@@ -11,6 +11,8 @@
 //                  with occupancy (Step 2), mean-corrected binomial count and
 //                  multinomial split (Step 3); in one pass, or in two with
 //                  the tets whose reactions have to run in the second
+//   k_run          many periods in one cooperative launch, for a mesh whose
+//                  tets are all resident at once
 //   k_gather       the closing synchronous transfer of a run
 //
 // Layout: counts are species-major int32 [S][T] (coalesced), updated in
@@ -494,6 +496,141 @@ k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams 
         if (bad) atomicOr(s.err, bad);
         __syncwarp();
     }
+}
+
+// Grid barrier of a cooperative launch: the counter only grows, by one per
+// block and barrier; the wait ends when it reaches `target` (modulo 2^32).
+// The launch holds every block resident, so the wait is as long as the slowest
+// block's period; past the limit (a period at the event cap takes seconds)
+// the block sets kErrTimeout and gives up, and the others follow it.
+__device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target, uint32_t* err, volatile int* gave_up) {
+    constexpr unsigned long long kLimitNs = 120ull * 1000000000ull;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();   // the block's inbox words before its arrival
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
+        unsigned long long start = 0ull;
+        for (uint32_t i = 1;; ++i) {
+            uint32_t c;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(counter) : "memory");
+            if ((int32_t)(c - target) >= 0) break;
+            if ((i & 1023u) == 0u) {
+                unsigned long long now;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+                if (start == 0ull) start = now;
+                if (now - start > kLimitNs || (__ldcg(err) & kErrTimeout)) {
+                    atomicOr(err, kErrTimeout);
+                    *gave_up = 1;
+                    break;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    return *gave_up == 0;
+}
+
+// A stretch of periods in one launch, for a mesh whose tets are all resident
+// at once (one lane each): counts stay in shared memory, the code, the
+// thresholds and the neighbour records in the SM's caches, and a grid barrier
+// takes the place of the launch between two periods.  Started alone, a
+// period of a small mesh is mostly cold instruction and constant fetches: the
+// 3,072-tet cube's took 10.2 us a launch and takes 6.5 here (217 periods, 2.21 ->
+// 1.40 ms; 48,000-tet A/B/C cube, 200 periods, 2.91 -> 2.20 ms).  Ends with the closing transfer, all
+// inbox words and masks cleared.
+template <int S_, bool kReact>
+__global__ void __launch_bounds__(kBlock, 3)
+k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp, DevState s,
+      const __grid_constant__ RunArgs r) {
+    extern __shared__ int32_t sm[];
+    __shared__ int gave_up;
+    const int S = S_ > 0 ? S_ : mp.S;
+    const int lane = threadIdx.x & 31;
+    const WarpMem w(sm + (threadIdx.x >> 5) * warp_words(S, kReact), S, kReact);
+    const int64_t T = m.T;
+    const int64_t tt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool live = tt < T;
+    const int t = live ? (int)tt : 0;
+    if (threadIdx.x == 0) gave_up = 0;
+    if (live)
+        for (int sp = 0; sp < S; ++sp) w.N[32 * sp + lane] = s.cnt[sp * T + t];
+    uint32_t bad = 0, dirty = 0, target = r.barrier_base;
+    for (int q = 0; q <= r.periods; ++q) {
+        PeriodArgs a{};
+        const int p = q & 1;
+        a.in_prev = r.inbox[p ^ 1];
+        a.in_cur = r.inbox[p];
+        a.mask_prev = r.mask[p ^ 1];
+        a.mask_cur = r.mask[p];
+        if (q > 0) {
+            target += gridDim.x;
+            if (!grid_barrier(r.barrier, target, s.err, &gave_up)) return;
+            if (live) bad |= take_inbox(a, t, S, lane, w.N, &dirty);
+        }
+        if (q == r.periods) break;
+        const bool last = r.last_short && q == r.periods - 1;
+        const PeriodView v{r.period0 + (uint32_t)q, last ? r.tau_last : r.tau, last ? r.tau_lastf : r.tauf, r.seed,
+                           last ? r.thr_last : r.thr, 1};
+        Sender send(a, m.src, t, S);
+        bool deferred = false;
+        bad |= warp_step<kReact, false>(m, mp, S, w, v, t, live, &dirty, &deferred, s.err, send);
+        if (live) send.finish(false);
+    }
+    if (live)
+        for (uint32_t bits = dirty; bits; bits &= bits - 1u) {
+            const int sp = __ffs(bits) - 1;
+            s.cnt[sp * T + t] = w.N[32 * sp + lane];
+        }
+    if (bad) atomicOr(s.err, bad);
+}
+
+// Warps a block and blocks of k_run for T tets, or 0 if they do not fit: the
+// 32-tet warps are spread over all SMs first (a warp that has an SM's issue
+// slots and caches to itself is fastest), in at most 3 blocks of 8 warps an SM.
+int run_shape(int64_t T, int sms, int* warps) {
+    const int64_t chunks = (T + 31) / 32;
+    const int64_t per_sm = (chunks + sms - 1) / sms;
+    if (per_sm > 24) return 0;
+    const int64_t blocks_per_sm = (per_sm + 7) / 8;
+    *warps = (int)((per_sm + blocks_per_sm - 1) / blocks_per_sm);
+    return (int)((chunks + *warps - 1) / *warps);
+}
+
+template <int S_, bool kReact>
+cudaError_t launch_run_s(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int grid,
+                         int warps, int sms, cudaStream_t st) {
+    auto kern = k_run<S_, kReact>;
+    const size_t smem = (size_t)warps * warp_words(mp.S, kReact) * sizeof(int32_t);
+    if (smem > 48u * 1024u)
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int fit = 0;
+    cudaError_t ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, 32 * warps, smem);
+    if (ce == cudaSuccess && (int64_t)fit * sms < grid) ce = cudaErrorCooperativeLaunchTooLarge;
+    if (ce != cudaSuccess) return ce;
+    DevMesh m_ = m;
+    ModelParams mp_ = mp;
+    DevState s_ = s;
+    RunArgs r_ = r;
+    void* args[] = {&m_, &mp_, &s_, &r_};
+    ce = cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(32 * warps), args, smem, st);
+    if (ce == cudaSuccess) ++g_launches;
+    return ce;
+}
+
+bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int sms, int* grid,
+                cudaStream_t st) {
+    int warps = 0;
+    *grid = run_shape(m.T, sms, &warps);
+    if (*grid == 0) return false;
+    cudaError_t ce;
+    if (mp.S == 1)
+        ce = mp.any_reaction ? launch_run_s<1, true>(m, mp, s, r, *grid, warps, sms, st)
+                             : launch_run_s<1, false>(m, mp, s, r, *grid, warps, sms, st);
+    else
+        ce = mp.any_reaction ? launch_run_s<0, true>(m, mp, s, r, *grid, warps, sms, st)
+                             : launch_run_s<0, false>(m, mp, s, r, *grid, warps, sms, st);
+    if (ce != cudaSuccess) cudaGetLastError();   // no room for a cooperative launch: one launch a period
+    return ce == cudaSuccess;
 }
 
 template <int S_, bool kReact, int kPass>

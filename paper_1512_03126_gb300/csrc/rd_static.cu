@@ -5,6 +5,7 @@
 // caller passes the mesh, the model and the counts, and gets the counts back
 // in place.  The kernels are the ones rdsplit_run launches, given pointers
 // into that array.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <mutex>
@@ -137,6 +138,7 @@ int read_err(unsigned char* base, const Layout& L, cudaStream_t st, const char* 
     if (e == 0) return RDSPLIT_OK;
     if (e & (kErrAdjRange | kErrAdjAsym | kErrVolume | kErrFace))
         return rdapi::fail(RDSPLIT_EINVAL, "%s: malformed mesh (error bits 0x%x)", where, e);
+    if (e & kErrTimeout) return rdapi::fail(RDSPLIT_ETIMEOUT, "%s: a grid barrier's wait ran out", where);
     if (e & (kErrOverflow | kErrEventCap)) return rdapi::fail(RDSPLIT_EOVERFLOW, "%s: count or event overflow", where);
     if (e & kErrNegative) return rdapi::fail(RDSPLIT_EINVAL, "%s: negative count", where);
     return rdapi::fail(RDSPLIT_ECUDA, "%s: device error bits 0x%x", where, e);
@@ -224,30 +226,56 @@ extern "C" int rdsplit_run_static(int32_t n_tets, const int32_t* d_adj, const do
     if (std::isfinite(tau)) launch_thresholds(n_tets, mp, g, G, tau, thr, st);
 
     // Algorithm 1: Step 1 aligns the last period to t_end, Steps 2-3 run in
-    // the period kernel, Step 4 advances t.
+    // the period kernels (many periods a launch while the tets are resident at
+    // once, see run_loop), Step 4 advances t.
     const int sms = sm_count();
     double tn = *t;
     int64_t pk = *period;
-    int64_t j = 0;
+    int64_t jl = 0;
+    uint32_t* barrier = (uint32_t*)(base + L.tau + 128);   // cleared above
+    uint32_t barrier_base = 0;
+    int warps = 0;
+    bool resident = run_shape(n_tets, sms, &warps) > 0;
     while (tn < t_end) {
         if (pk >= (int64_t)0xffffffffll) return rdapi::fail(RDSPLIT_EOVERFLOW, "%s: period index exceeds 2^32-1", where);
-        double tau_k = tau;
+        const int64_t most = std::min<int64_t>(resident ? rdapi::kRunPeriods : 1, 0xffffffffll - pk);
+        int n = 0;
         bool last = false;
-        if (tn + tau > t_end) {
-            tau_k = t_end - tn;
-            last = true;
+        double te = tn, tau_k = tau;
+        // one threshold array: a shortened last period goes into a launch of its own
+        while (n < most && te < t_end) {
+            if (te + tau > t_end) {
+                if (n > 0) break;
+                tau_k = t_end - te;
+                last = true;
+                te = t_end;
+            } else {
+                te = te + tau;
+            }
+            ++n;
         }
         if (last) launch_thresholds(n_tets, mp, g, G, tau_k, thr, st);
-        const int q = (int)(j & 1);
-        PeriodArgs a{(uint32_t)pk, tau_k, (float)tau_k, seed, j == 0 ? 1 : 0, thr, out[q ^ 1], out[q],
-                     mask[q ^ 1], mask[q]};
-        launch_period(m, mp, s, a, rdapi::period_block(n_tets, sms), st);
-        tn = last ? t_end : tn + tau;
-        pk += 1;
-        j += 1;
+        if (resident) {
+            RunArgs r{(uint32_t)pk, n, 0, tau_k, tau_k, (float)tau_k, (float)tau_k, seed, thr, thr,
+                      {out[0], out[1]}, {mask[0], mask[1]}, barrier, barrier_base};
+            int grid = 0;
+            if (!launch_run(m, mp, s, r, sms, &grid, st)) {
+                resident = false;
+                continue;
+            }
+            barrier_base += (uint32_t)grid * (uint32_t)n;
+        } else {
+            const int q = (int)(jl & 1);
+            PeriodArgs a{(uint32_t)pk, tau_k, (float)tau_k, seed, jl == 0 ? 1 : 0, thr, out[q ^ 1], out[q],
+                         mask[q ^ 1], mask[q]};
+            launch_period(m, mp, s, a, rdapi::period_block(n_tets, sms), st);
+            jl += 1;
+        }
+        tn = te;
+        pk += n;
     }
-    if (j > 0) {
-        const int q = (int)((j - 1) & 1);
+    if (jl > 0) {
+        const int q = (int)((jl - 1) & 1);
         PeriodArgs a{};
         a.in_prev = out[q];
         a.mask_prev = mask[q];

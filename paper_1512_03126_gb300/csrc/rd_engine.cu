@@ -683,7 +683,9 @@ void warm_kernels_sa(EngineLaunch& W) {
     warm_kernel<SA, true, 8>(W);
 }
 
-// head: int32[kGroups] of the engine being created (left zero); err and
+// head: int32[kGroups] of the engine being created (set to zero before, since a
+// fresh allocation may hold anything and a negative index would be taken for
+// an item, and left zero); err and
 // processed: its error word and entry counter (not written: no item runs).
 void warm_engine_kernels(int32_t* head, uint32_t* err, unsigned long long* processed, int sms) {
     static std::mutex mu;
@@ -695,6 +697,10 @@ void warm_engine_kernels(int32_t* head, uint32_t* err, unsigned long long* proce
     }
     std::lock_guard<std::mutex> lock(mu);
     if (std::find(warmed.begin(), warmed.end(), dev) != warmed.end()) return;
+    if (cudaMemsetAsync(head, 0, sizeof(int32_t) * 10, (cudaStream_t)0) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
     EngineLaunch W{nullptr, nullptr, nullptr, 0, head, err, processed, nullptr, (cudaStream_t)0, sms, 1};
     warm_kernels_sa<1>(W);
     warm_kernels_sa<2>(W);

@@ -29,6 +29,7 @@
 #include "rd_device.cuh"
 #include "rd_internal.h"
 #include "rd_period.cuh"
+#include "rd_warp.cuh"
 
 using namespace rdk;
 
@@ -42,8 +43,8 @@ struct SlotDesc {
     const uint4* thr_last;   // thresholds for the shortened last period
     int32_t* N[2];           // count buffers [S][T]; the slice starts in N[0]
     uint32_t* bits[2];       // active-tet bitmaps (bit t of word t/32), by period parity in the slice
-    const uint4* packed;     // one species: {src, thr} per tet (null: separate arrays)
-    int32_t* N2;             // one species: counts of both parities interleaved (null: N[2])
+    const uint4* packed;     // one species: {src, thr} per tet
+    int32_t* N2;             // one species: counts of both parities interleaved
     uint64_t seed;
     uint32_t period0;        // global period index of local period 0
     int32_t P;               // periods to run in total
@@ -54,12 +55,6 @@ struct SlotDesc {
     double tau, tau_last;
     float tauf, tau_lastf;
 };
-
-__device__ __forceinline__ bool zero_order_on(const SlotDesc& d, const ModelParams& mp, int t) {
-    if (!d.zero_order) return false;
-    uint32_t on = mp.has_mask ? d.m.mask[t] : 0xffffffffu;
-    return (on & d.zero_order) != 0u;
-}
 
 // Fire-and-forget integer add to global memory (no value comes back, so the
 // warp does not wait for the L2 round trip).
@@ -81,361 +76,248 @@ __device__ __forceinline__ void red_or(uint32_t* p, uint32_t v) {
 
 constexpr int kWarps = kRunBlock / 32;
 constexpr int kGroup = 8;                   // bitmap columns (32 words each) a warp loads at once
-constexpr int kQueue = 64;                  // deferred tets per warp
-constexpr int kListCap = 32 * 32 + 32;      // active tets one column can add, plus a partial round
-constexpr int kDynSmemBytes = kWarps * kListCap * 4;
 
-// Shared memory of the engine kernel, at file scope so that the period
-// functions below address it directly.
+// Dynamic shared memory of a warp, in words: the step's (rd_warp.cuh) and the
+// bitmap words of its current batch.
+__host__ __device__ inline int engine_warp_words(int S, bool react) { return warp_words(S, react) + 32 * kGroup; }
+
+// Position of set bit number k (from 0) of w, by halves.
+__device__ __forceinline__ int nth_set_bit(uint32_t w, int k) {
+    int p = 0;
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) {
+        const int c = __popc(w & ((1u << h) - 1u));
+        if (k >= c) {
+            k -= c;
+            p += h;
+            w >>= h;
+        }
+    }
+    return p;
+}
+
+// The bitmap word of lane `lane` in column kk of batch b of warp gw: column by
+// column 8 runs of 4 words, runs dealt round-robin over kW warps.
+__device__ __forceinline__ int word_of(int gw, int b, int kk, int lane, int kW) {
+    return (gw + ((b * kGroup + kk) * 8 + (lane >> 2)) * kW) * 4 + (lane & 3);
+}
+
+// Shared memory of the engine kernel.
 __shared__ int32_t s_item;                          // work-item index (first CTA of the cluster)
 __shared__ unsigned long long s_mass[3];            // [0] molecules of the simulation (all species) at the
                                                     // start of the period; [1], [2] net change by reactions
                                                     // in periods of even / odd parity (two's complement)
-__shared__ uint32_t s_wbuf[kWarps][kGroup * 32];    // per warp: the bitmap words of its current batch
-__shared__ int32_t s_slowq[kWarps][kQueue];         // per warp: tets deferred to the rounds with the full step
-extern __shared__ int32_t s_list[];                 // [kWarps][kListCap]: per warp, active tets not yet run
+__shared__ SlotDesc s_desc;                         // the simulation's descriptor and chemistry
+__shared__ ModelParams s_mp;
+extern __shared__ int32_t s_warp[];                 // [kWarps][engine_warp_words]
 
-// Where one period stands for one warp.  The light pass stops early when the
-// warp's queue of deferred tets could overflow, and resumes after the queue
-// has been run: at batch g0, column kk (the batch's words are kept in s_wbuf
-// when `loaded`), with `cnt` active tets still in the warp's list.
-struct LightState {
+// Counts of one period and the next: N[r] / N[r^1], or the two halves of the
+// interleaved pairs.
+template <bool kOne>
+struct CountView {
+    int32_t* cur;
+    int32_t* next;
+    int64_t T;
+    static constexpr int stride = kOne ? 2 : 1;
+    __device__ __forceinline__ CountView(const SlotDesc& d, int r) : T(d.m.T) {
+        cur = kOne ? d.N2 + r : d.N[r];
+        next = kOne ? d.N2 + (r ^ 1) : d.N[r ^ 1];
+    }
+};
+
+// Leavers of a tet into the next period's counts (fire-and-forget integer
+// adds).  An add that takes a count past 2^31-1 wraps it negative; as the
+// simulation's molecule total is kept below 2^32 (checked every period), the
+// next read of the count, or the check at the end of the slice, sees it
+// negative and reports the overflow, exactly when the dense gather would.
+template <bool kOne>
+struct Scatter {
+    const CountView<kOne>& c;
+    const int4* src;
+    int t;
+    int4 sr;
+    bool have;
+    uint32_t send;        // faces through which something leaves
     uint32_t bad;
-    int32_t n_slow;      // tets in the warp's queue
-    int32_t g0, kk;      // resume point (batch, column)
-    int32_t cnt;         // tets in the warp's list
-    int32_t loaded;      // the batch's words are in s_wbuf
-    int32_t finished;
-    unsigned long long done;
-};
+    long long sent;       // molecules that leave
 
-// Everything a period pass derives from the slot descriptor and the period.
-template <int kC>
-struct PeriodView {
-    int T, S, W, r, tstride;
-    bool use_packed, more;
-    double tau_k;
-    float tau_kf;
-    uint32_t period;
-    const uint4* thr;
-    int32_t* Ncur;
-    int32_t* Nnext;
-    uint32_t* bcur;
-    uint32_t* bnext;
-    int64_t cstride;
+    __device__ __forceinline__ Scatter(const CountView<kOne>& c_, const int4* src_, int t_, int4 sr_, bool have_)
+        : c(c_), src(src_), t(t_), sr(sr_), have(have_), send(0), bad(0), sent(0) {}
 
-    __device__ __forceinline__ PeriodView(const SlotDesc& d, int q) {
-        T = d.m.T;
-        S = d.S;
-        W = (T + 31) >> 5;
-        r = (q - d.q0) & 1;
-        const bool last = (q == d.P - 1) && d.last_short;
-        tau_k = last ? d.tau_last : d.tau;
-        tau_kf = last ? d.tau_lastf : d.tauf;
-        // thresholds: packed beside the reverse-face record (stride 2) except
-        // in a shortened last period
-        use_packed = d.packed != nullptr && !last;
-        thr = last ? d.thr_last : (use_packed ? d.packed + 1 : d.thr);
-        tstride = use_packed ? 2 : 1;
-        period = d.period0 + (uint32_t)q;
-        // counts of this period and the next: N[r] / N[r^1], or the two
-        // halves of the interleaved pairs
-        const bool inter = d.N2 != nullptr;
-        Ncur = inter ? d.N2 + r : d.N[r];
-        Nnext = inter ? d.N2 + (r ^ 1) : d.N[r ^ 1];
-        cstride = inter ? 2 : 1;
-        bcur = d.bits[r];
-        bnext = d.bits[r ^ 1];
-        more = q + 1 < d.q1;
-    }
-
-    // Transfer of one tet's molecules (kept and leaving) into the next
-    // counts (fire-and-forget integer adds), and its bits in the next bitmap
-    // (fire-and-forget ORs: a bit set twice is set once).  An add that takes
-    // a count past 2^31-1 wraps it negative; as the simulation's molecule
-    // total is kept below 2^32 (checked every period), the next read of the
-    // count, or the check at the end of the slice, sees it negative and
-    // reports the overflow, exactly when the dense gather would.
-    template <int SA, bool kReact>
-    __device__ __forceinline__ uint32_t scatter(const SlotDesc& d, const ModelParams& mp, int t, const int4& sr,
-                                                const int32_t* N, const int4* o) const {
-        uint32_t bad = 0;
-        const int nbr[4] = {sr.x, sr.y, sr.z, sr.w};
-        bool keep = kReact && zero_order_on(d, mp, t);
-        bool send[4] = {false, false, false, false};
+    __device__ __forceinline__ void operator()(int sp, const int4& o) {
+        if (!have) sr = __ldg(src + t);
+        have = true;
+        const int nbr[4] = {sr.x, sr.y, sr.z, sr.w}, n[4] = {o.x, o.y, o.z, o.w};
+        int32_t* Ns = kOne ? c.next : c.next + sp * c.T;
 #pragma unroll
-        for (int s = 0; s < SA; ++s) {
-            if (s >= S) break;
-            int32_t* Ns = Nnext + (int64_t)s * T * cstride;
-            if (N[s] > 0) {
-                red_add(Ns + (int64_t)t * cstride, N[s]);
-                keep = true;
-            }
-            const int ov[4] = {o[s].x, o[s].y, o[s].z, o[s].w};
-#pragma unroll
-            for (int f = 0; f < 4; ++f) {
-                if (ov[f] <= 0) continue;
-                if (nbr[f] < 0) { bad |= kErrNegative; continue; }
-                red_add(Ns + (int64_t)(nbr[f] >> 2) * cstride, ov[f]);
-                send[f] = true;
-            }
+        for (int f = 0; f < 4; ++f) {
+            if (n[f] <= 0) continue;
+            if (nbr[f] < 0) { bad |= kErrNegative; continue; }
+            red_add(Ns + (int64_t)(nbr[f] >> 2) * c.stride, n[f]);
+            send |= 1u << f;
         }
-        if (more) {
-            if (keep) red_or(bnext + (t >> 5), 1u << (t & 31));
-#pragma unroll
-            for (int f = 0; f < 4; ++f) {
-                if (!send[f]) continue;
-                const int u = nbr[f] >> 2;
-                red_or(bnext + (u >> 5), 1u << (u & 31));
-            }
-        }
-        return bad;
+        sent += (long long)o.x + o.y + o.z + o.w;
     }
 };
 
-// The light pass of one period for one warp.  The bitmap is dealt to the
+// One period of a simulation for one warp.  The bitmap is dealt to the
 // cluster's kW warps in runs of 4 words (128 tets): run r goes to warp
 // r mod kW, so the active tets of a region are spread over all warps (runs
-// of 4 measured faster than runs of 1, 2 or 8).  A column is 8 runs of a
-// warp (32 words, one per lane); a warp
-// loads kGroup of its columns at once, clears them for their next use, and
-// appends the set bits of each column to its list in shared memory
-// (a prefix sum of the lanes' popcounts gives each lane its place); whenever
-// the list holds 32 tets, one round takes them, one per lane.  A round runs
-// every tet that needs neither a non-inlined sampler (step_is_light) nor a
-// whole-warp draw (10 or more molecules of a species) with the call-free
-// step, and queues the others for the slow pass.  Kept out of
-// line, and free of calls, so that the compiler allocates its registers
-// without the double-precision samplers' demands.  Returns early, with a
-// resume point, when the next round could overflow the queue.
-template <int SA, bool kReact, int kC>
-__device__ __noinline__ LightState light_pass(const SlotDesc* __restrict__ dp, const ModelParams* __restrict__ mpp,
-                                              int q, uint32_t* err, LightState st) {
-    constexpr unsigned kAll = 0xffffffffu;
+// of 4 measured faster than runs of 1, 2 or 8).  A column is 8 runs of a warp
+// (32 words, one per lane); a warp loads kGroup of its columns at once and
+// clears them for their next use.  With a prefix sum of a column's popcounts
+// each lane finds a set bit of its own (a search over the sums and one inside
+// the word: a fixed 60 instructions, where writing the bits of a dense word
+// into a list took 32 turns of one lane); whenever 32 tets are at hand, one
+// round steps them (warp_step), and adds what stays and what leaves into the
+// next counts.
+template <bool kOne, bool kReact, int kC>
+__device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned long long* mass_delta,
+                                               unsigned long long* done) {
     constexpr int kW = kC * kWarps;
-    const SlotDesc& d = *dp;
-    const ModelParams& mp = *mpp;
-    const PeriodView<kC> v(d, q);
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
+    const SlotDesc& d = s_desc;
+    const ModelParams& mp = s_mp;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rank = kC > 1 ? (int)cooperative_groups::this_cluster().block_rank() : 0;
     const int gw = rank * kWarps + warp;
-    const unsigned lane_lt = (1u << lane) - 1u;
-    uint32_t* wb = s_wbuf[warp];
-    int32_t* list = s_list + warp * kListCap;
-    int32_t* slowq = s_slowq[warp];
-    st.bad = 0u;
-    st.n_slow = 0;
-    st.done = 0ull;
-
-    // one round: the tets t of the live lanes
-    auto round = [&](int t, bool live) {
-        uint32_t heavy = 0;
-        int32_t N[SA];
-        int4 o[SA];
-        int4 sr = make_int4(-1, -1, -1, -1);
-        uint4 pre = make_uint4(0u, 0u, 0u, 0u);
-        bool light = false;
-        if (live) {
-            // the tet's record and counts, loaded together
-            sr = d.packed ? *reinterpret_cast<const int4*>(d.packed + 2 * t) : d.m.src[t];
-            if (v.use_packed) pre = d.packed[2 * t + 1];
-#pragma unroll
-            for (int s = 0; s < SA; ++s) {
-                if (s >= v.S) break;
-                N[s] = v.Ncur[((int64_t)s * v.T + t) * v.cstride];
-                if (N[s] < 0) {          // wrapped past 2^31-1 by the previous period's adds
-                    st.bad |= kErrOverflow;
-                    N[s] = 0;
-                }
-            }
-            light = step_is_light<SA, kReact>(d.m, mp, v.period, v.tau_kf, d.seed, t, v.S, N);
-            // tets whose draws need the whole warp (warp_split) go to the slow
-            // pass too, which keeps the light pass free of that loop
-#pragma unroll
-            for (int s = 0; s < SA; ++s) {
-                if (s >= v.S) break;
-                if (N[s] >= kWarpSplitMin) light = false;
-            }
-        }
-        const unsigned slow_mask = __ballot_sync(kAll, live && !light);
-        if (live && !light) slowq[st.n_slow + __popc(slow_mask & lane_lt)] = t;
-        st.n_slow += __popc(slow_mask);
-        if (light) {
-#pragma unroll
-            for (int s = 0; s < SA; ++s) {
-                if (s >= v.S) break;
-                v.Ncur[((int64_t)s * v.T + t) * v.cstride] = 0;
-            }
-            if (SA == 1 && !kReact && v.use_packed && N[0] <= 4) {
-                // one species, at most four molecules: the first Philox
-                // block of the tet's diffusion stream holds all their draws
-                // (the words split_molecules would take, in its order)
-                const uint32_t key = (uint32_t)key_of(d.m, t);
-                const uint4 w = rdd::philox_block(0u, key, v.period, rdd::kPurposeDiffusion << 16,
-                                                  (uint32_t)d.seed, (uint32_t)(d.seed >> 32));
-                const uint32_t u[4] = {w.x, w.y, w.z, w.w};
-                int c0 = 0, c1 = 0, c2 = 0, c3 = 0;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    if (i >= N[0]) break;
-                    if (rdd::below(u[i], pre.x)) ++c0;
-                    else if (rdd::below(u[i], pre.y)) ++c1;
-                    else if (rdd::below(u[i], pre.z)) ++c2;
-                    else if (rdd::below(u[i], pre.w)) ++c3;
-                }
-                o[0] = make_int4(c0, c1, c2, c3);
-                N[0] -= c0 + c1 + c2 + c3;
-            } else {
-                st.bad |= step_tet<SA, false, false>(d.m, mp, v.period, v.tau_k, v.tau_kf, d.seed, v.thr, t, v.S, N,
-                                                     o, &heavy, err, v.tstride, v.use_packed, pre);
-            }
-        }
-        if (light) st.bad |= v.template scatter<SA, kReact>(d, mp, t, sr, N, o);
-    };
-
-    // the word of lane `lane` in column kk of batch b: run j of this warp
-    // (4 words), runs dealt round-robin over the warps
-    auto word_of = [&](int b, int kk) {
-        const int j = (b * kGroup + kk) * 8 + (lane / 4);
-        return (gw + j * kW) * 4 + (lane % 4);
-    };
-    int b = st.g0;
-    for (;; ++b) {
-        if (!st.loaded) {
-            if ((gw + b * kGroup * 8 * kW) * 4 >= v.W) break;
+    const int S = kOne ? 1 : d.S;
+    int32_t* base_mem = s_warp + warp * engine_warp_words(S, kReact);
+    const WarpMem w(base_mem, S, kReact);
+    uint32_t* wb = reinterpret_cast<uint32_t*>(base_mem + warp_words(S, kReact));
+    const int W = (d.m.T + 31) >> 5;
+    const int r = (q - d.q0) & 1;
+    const bool last = (q == d.P - 1) && d.last_short;
+    // thresholds: packed beside the reverse-face record (stride 2) except in a
+    // shortened last period
+    const PeriodView v{d.period0 + (uint32_t)q, last ? d.tau_last : d.tau, last ? d.tau_lastf : d.tauf, d.seed,
+                       last ? d.thr_last : (kOne ? d.packed + 1 : d.thr), kOne && !last ? 2 : 1};
+    const CountView<kOne> c(d, r);
+    uint32_t* bcur = d.bits[r];
+    uint32_t* bnext = d.bits[r ^ 1];
+    const bool more = q + 1 < d.q1;
+    uint32_t bad = 0;
+    int pend = 0, cnt = 0;      // tets not yet run: lane i < cnt holds one
+    unsigned long long visited = 0;
+    for (int b = 0;; ++b) {
+        const bool flush = (gw + b * kGroup * 8 * kW) * 4 >= W;   // past the last batch: run what is left
+        int columns = 1;
+        if (!flush) {
             uint32_t wds[kGroup];
 #pragma unroll
             for (int kk = 0; kk < kGroup; ++kk) {
-                const int wi = word_of(b, kk);
-                wds[kk] = wi < v.W ? v.bcur[wi] : 0u;
+                const int wi = word_of(gw, b, kk, lane, kW);
+                wds[kk] = wi < W ? __ldcg(bcur + wi) : 0u;
             }
+            uint32_t any = 0;
 #pragma unroll
             for (int kk = 0; kk < kGroup; ++kk) {
-                const int wi = word_of(b, kk);
-                if (wds[kk]) v.bcur[wi] = 0u;
+                if (wds[kk]) bcur[word_of(gw, b, kk, lane, kW)] = 0u;
                 wb[kk * 32 + lane] = wds[kk];
+                any |= wds[kk] ? 1u << kk : 0u;
             }
-            __syncwarp();
-            st.loaded = 1;
-            st.kk = 0;
+            columns = (int)__reduce_or_sync(kAllLanes, any);
         }
-        for (int kk = st.kk; kk < kGroup; ++kk) {
-            // full rounds first, so that one more column always fits the list
-            while (st.cnt >= 32) {
-                if (st.n_slow > kQueue - 32) {
-                    st.g0 = b;
-                    st.kk = kk;
-                    st.finished = 0;
-                    return st;
+        // the columns that hold a set bit (flush: one turn without any)
+        while (columns) {
+            const int kk = __ffs(columns) - 1;
+            columns &= columns - 1;
+            const uint32_t word = flush ? 0u : wb[kk * 32 + lane];
+            const int own = __popc(word);
+            int inc = own;
+#pragma unroll
+            for (int dd = 1; dd < 32; dd <<= 1) {
+                const int y = __shfl_up_sync(kAllLanes, inc, dd);
+                if (lane >= dd) inc += y;
+            }
+            const int total = __shfl_sync(kAllLanes, inc, 31);
+            int off = cnt, avail = cnt + total;
+            visited += (unsigned long long)total;
+            for (;;) {
+                // the lane's tet: one that was left over, or the column's set bit number lane - off
+                const int e = lane - off;
+                int from = 0;
+#pragma unroll
+                for (int step = 16; step > 0; step >>= 1)
+                    if (__shfl_sync(kAllLanes, inc, from + step - 1) <= e) from += step;
+                const int k = e - __shfl_sync(kAllLanes, inc - own, from);
+                const int bit = nth_set_bit(__shfl_sync(kAllLanes, word, from), k);
+                const int t_new = word_of(gw, b, kk, from, kW) * 32 + bit;
+                const int t_lane = e < 0 ? pend : t_new;
+                if (avail < 32 && !(flush && avail > 0)) {
+                    pend = t_lane;
+                    cnt = avail;
+                    break;
                 }
-                const int t = list[st.cnt - 32 + lane];
+                const bool live = lane < avail;
+                const int t = live ? t_lane : 0;
+                off -= 32;
+                avail = max(avail - 32, 0);
+                int4 sr = make_int4(-1, -1, -1, -1);
+                uint4 pre = make_uint4(0u, 0u, 0u, 0u);
+                long long held = 0;
+                if (live) {
+                    if (kOne) {
+                        // the record and the count, loaded together
+                        sr = __ldg(reinterpret_cast<const int4*>(d.packed + 2 * (int64_t)t));
+                        pre = __ldg(v.thr + (int64_t)t * v.thr_stride);
+                    }
+                    for (int s0 = 0; s0 < S; s0 += 4) {
+                        int32_t n[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (s0 + k < S) n[k] = __ldcg(c.cur + ((s0 + k) * c.T + t) * c.stride);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            if (s0 + k >= S) continue;
+                            if (n[k] != 0) c.cur[((s0 + k) * c.T + t) * c.stride] = 0;
+                            if (n[k] < 0) {          // wrapped past 2^31-1 by the previous period's adds
+                                bad |= kErrOverflow;
+                                n[k] = 0;
+                            }
+                            w.N[32 * (s0 + k) + lane] = n[k];
+                            if (kReact) held += n[k];
+                        }
+                    }
+                }
+                Scatter<kOne> scatter(c, d.m.src, t, sr, kOne);
+                uint32_t dirty = 0;
+                bool deferred = false;
+                bad |= warp_step<kOne, kReact, false, kOne>(d.m, mp, S, w, v, t, live, &dirty, &deferred, err, scatter,
+                                                            pre);
+                bad |= scatter.bad;
+                long long delta = 0;
+                if (live) {
+                    bool keep = false;
+                    if (kReact && d.zero_order) keep = ((mp.has_mask ? d.m.mask[t] : 0xffffffffu) & d.zero_order) != 0u;
+                    for (int s = 0; s < S; ++s) {
+                        const int32_t n = w.N[32 * s + lane];
+                        if (n > 0) {
+                            red_add(c.next + (s * c.T + t) * c.stride, n);
+                            keep = true;
+                            if (kReact) delta += n;
+                        }
+                    }
+                    if (kReact) delta += scatter.sent - held;
+                    if (more) {
+                        if (keep) red_or(bnext + (t >> 5), 1u << (t & 31));
+                        const int nbr[4] = {scatter.sr.x, scatter.sr.y, scatter.sr.z, scatter.sr.w};
+#pragma unroll
+                        for (int f = 0; f < 4; ++f) {
+                            if (!((scatter.send >> f) & 1u)) continue;
+                            const int u = nbr[f] >> 2;
+                            red_or(bnext + (u >> 5), 1u << (u & 31));
+                        }
+                    }
+                }
+                // net molecules made by reactions: all that stays and leaves
+                // minus what was held
+                if (kReact && delta != 0) atomicAdd(mass_delta, (unsigned long long)delta);
                 __syncwarp();
-                st.cnt -= 32;
-                round(t, true);
-            }
-            uint32_t w = wb[kk * 32 + lane];
-            if (__any_sync(kAll, w != 0u)) {
-                const uint32_t c = (uint32_t)__popc(w);
-                uint32_t inc = c;
-#pragma unroll
-                for (int dd = 1; dd < 32; dd <<= 1) {
-                    const uint32_t y = __shfl_up_sync(kAll, inc, dd);
-                    if (lane >= dd) inc += y;
-                }
-                const int total = (int)__shfl_sync(kAll, inc, 31);
-                int at = st.cnt + (int)(inc - c);
-                const int base = word_of(b, kk) * 32;
-                while (w) {
-                    const int bit = __ffs(w) - 1;
-                    list[at++] = base + bit;
-                    w &= w - 1u;
-                }
-                __syncwarp();
-                st.cnt += total;
-                st.done += (unsigned long long)total;
             }
         }
-        st.loaded = 0;
-        st.kk = 0;
+        if (flush) break;
     }
-    // the rest of the list, in rounds of up to 32
-    while (st.cnt > 0) {
-        if (st.n_slow > kQueue - 32) {
-            st.g0 = b;
-            st.finished = 0;
-            return st;
-        }
-        const int n = st.cnt < 32 ? st.cnt : 32;
-        const int t = lane < n ? list[st.cnt - n + lane] : 0;
-        __syncwarp();
-        st.cnt -= n;
-        round(t, lane < n);
-    }
-    st.g0 = b;
-    st.finished = 1;
-    return st;
-}
-
-// The deferred tets of one warp's queue (n of them), in rounds of 32, with
-// the full per-tet step: reactions and the non-inlined samplers.
-template <int SA, bool kReact, int kC>
-__device__ __noinline__ uint32_t slow_pass(const SlotDesc* __restrict__ dp, const ModelParams* __restrict__ mpp, int q,
-                                           uint32_t* err, int n, unsigned long long* mass_delta) {
-    const SlotDesc& d = *dp;
-    const ModelParams& mp = *mpp;
-    const PeriodView<kC> v(d, q);
-    const int lane = threadIdx.x & 31;
-    const int32_t* slowq = s_slowq[threadIdx.x >> 5];
-    uint32_t bad = 0;
-    for (int k0 = 0; k0 < n; k0 += 32) {
-        const bool live = k0 + lane < n;
-        const int t = live ? slowq[k0 + lane] : 0;
-        uint32_t heavy = 0;
-        int32_t N[SA];
-        int4 o[SA];
-        int4 sr = make_int4(-1, -1, -1, -1);
-        uint4 pre = make_uint4(0u, 0u, 0u, 0u);
-        long long before = 0;
-        if (live) {
-            sr = d.packed ? *reinterpret_cast<const int4*>(d.packed + 2 * t) : d.m.src[t];
-            if (v.use_packed) pre = d.packed[2 * t + 1];
-#pragma unroll
-            for (int s = 0; s < SA; ++s) {
-                if (s >= v.S) break;
-                int32_t* p = v.Ncur + ((int64_t)s * v.T + t) * v.cstride;
-                N[s] = *p;
-                *p = 0;
-                if (N[s] < 0) {          // wrapped past 2^31-1 by the previous period's adds
-                    bad |= kErrOverflow;
-                    N[s] = 0;
-                }
-                before += N[s];
-            }
-            bad |= step_tet<SA, kReact, true>(d.m, mp, v.period, v.tau_k, v.tau_kf, d.seed, v.thr, t, v.S, N, o,
-                                              &heavy, err, v.tstride, v.use_packed, pre);
-        }
-        warp_split<SA>(heavy, d.seed, v.period, t, live ? key_of(d.m, t) : 0, v.thr, v.T, N, o, v.tstride,
-                       v.use_packed, pre);
-        if (live) bad |= v.template scatter<SA, kReact>(d, mp, t, sr, N, o);
-        if (kReact) {
-            // net molecules made by this tet's reactions: all it keeps and
-            // sends minus what it held
-            long long delta = 0;
-            if (live) {
-                delta = -before;
-#pragma unroll
-                for (int s = 0; s < SA; ++s) {
-                    if (s >= v.S) break;
-                    delta += (long long)N[s] + o[s].x + o[s].y + o[s].z + o[s].w;
-                }
-            }
-#pragma unroll
-            for (int dd = 16; dd > 0; dd >>= 1) delta += __shfl_xor_sync(0xffffffffu, delta, dd);
-            if (lane == 0 && delta != 0) atomicAdd(mass_delta, (unsigned long long)delta);
-        }
-    }
-    __syncwarp();   // the queue is refilled by the next light pass
+    *done += visited;
     return bad;
 }
 
@@ -453,15 +335,15 @@ __device__ __noinline__ uint32_t slow_pass(const SlotDesc* __restrict__ dp, cons
 // Count adds are fire-and-forget reductions.  A count that an add takes past
 // 2^31-1 wraps negative and is reported when read (next period, or the check
 // at the end of the slice); the molecule total of the simulation, tracked per
-// period (the slow pass adds what reactions make or consume), is kept below
-// 2^32 - 1 so that no count can wrap all the way round unseen.
-template <int SA, bool kReact, int kC>
-__global__ void __launch_bounds__(kRunBlock, 1)
+// period (each round adds what its reactions make or consume), is kept
+// below 2^32 - 1 so that no count can wrap all the way round unseen.
+template <int S_, bool kReact, int kC>
+__global__ void __launch_bounds__(kRunBlock, 2)
 k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__ mps, const int32_t* __restrict__ order,
              int32_t n_items, int32_t* head, uint32_t* err, unsigned long long* processed,
              unsigned long long* times) {
     namespace cg = cooperative_groups;
-    constexpr unsigned kAll = 0xffffffffu;
+    constexpr bool kOne = S_ == 1;
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = kC > 1 ? (int)cluster.block_rank() : 0;
     int32_t* item = kC > 1 ? cluster.map_shared_rank(&s_item, 0) : &s_item;
@@ -490,12 +372,20 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
             times[4 * slot + 2] = 0ull;
         }
         unsigned long long item_done = 0;
-        const SlotDesc& d = descs[slot];   // read-only; fields are loaded where used
-        const ModelParams& mp = mps[slot];
+        {
+            const uint32_t* from = reinterpret_cast<const uint32_t*>(descs + slot);
+            for (int i = threadIdx.x; i < (int)(sizeof(SlotDesc) / 4); i += kRunBlock)
+                reinterpret_cast<uint32_t*>(&s_desc)[i] = from[i];
+            from = reinterpret_cast<const uint32_t*>(mps + slot);
+            for (int i = threadIdx.x; i < (int)(sizeof(ModelParams) / 4); i += kRunBlock)
+                reinterpret_cast<uint32_t*>(&s_mp)[i] = from[i];
+        }
+        __syncthreads();
+        const SlotDesc& d = s_desc;
         const int T = d.m.T;
-        const int S = d.S;
+        const int S = kOne ? 1 : d.S;
         const int W = (T + 31) >> 5;
-        const bool inter = d.N2 != nullptr;   // one species, interleaved counts
+        constexpr bool inter = kOne;   // interleaved counts
         uint32_t bad = 0;
         // initial bitmap: occupied tets and tets with a zero-order reaction on
         // (whole words, written by the first lane of each 32-tet run); and the
@@ -505,7 +395,8 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
             const int t = base + threadIdx.x;
             bool occ = false;
             if (t < T) {
-                occ = kReact && zero_order_on(d, mp, t);
+                if (kReact && d.zero_order)
+                    occ = ((s_mp.has_mask ? d.m.mask[t] : 0xffffffffu) & d.zero_order) != 0u;
                 for (int s = 0; s < S; ++s) {
                     const int32_t c = d.N[0][(int64_t)s * T + t];
                     occ = occ || c > 0;
@@ -514,15 +405,15 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
                     if (inter) reinterpret_cast<int2*>(d.N2)[t] = make_int2(c, 0);
                 }
             }
-            const uint32_t word = __ballot_sync(kAll, occ);
+            const uint32_t word = __ballot_sync(kAllLanes, occ);
             if (lane == 0 && (t >> 5) < W) d.bits[0][t >> 5] = word;
         }
 #pragma unroll
-        for (int dd = 16; dd > 0; dd >>= 1) mine += __shfl_xor_sync(kAll, mine, dd);
+        for (int dd = 16; dd > 0; dd >>= 1) mine += __shfl_xor_sync(kAllLanes, mine, dd);
         if (lane == 0 && mine) atomicAdd(&mass[0], mine);
         // The molecule total after a period, kept below 2^32 - 1: then no
-        // int32 count can wrap past 2^32 unseen (see PeriodView::scatter).
-        // Reactions change it; the slow pass adds their net change.
+        // int32 count can wrap past 2^32 unseen (see Scatter).  Reactions
+        // change it; each round adds their net change.
         auto account = [&](int q) {
             if (rank == 0 && threadIdx.x == 0) {
                 unsigned long long* dq = &mass[1 + (q & 1)];
@@ -534,15 +425,7 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
         for (int q = d.q0; q < d.q1; ++q) {
             csync();   // the previous period's adds and bits are complete
             if (q > d.q0) account(q - 1);
-            LightState st{0u, 0, 0, 0, 0, 0, 0, 0ull};
-            for (;;) {
-                st = light_pass<SA, kReact, kC>(descs + slot, mps + slot, q, err, st);
-                bad |= st.bad;
-                item_done += st.done;
-                if (st.n_slow > 0)
-                    bad |= slow_pass<SA, kReact, kC>(descs + slot, mps + slot, q, err, st.n_slow, &mass[1 + (q & 1)]);
-                if (st.finished) break;
-            }
+            bad |= run_period<kOne, kReact, kC>(q, err, &mass[1 + (q & 1)], &item_done);
         }
         csync();   // every add of the slice is complete
         account(d.q1 - 1);
@@ -553,12 +436,12 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
                 if (inter) {
                     // the slice's counts are in the pairs' half (q1 - q0) & 1;
                     // hand them back in N[0]
-                    const int32_t c = d.N2[2 * t + half];
+                    const int32_t c = __ldcg(d.N2 + 2 * (int64_t)t + half);
                     if (c < 0) bad |= kErrOverflow;
                     d.N[0][t] = c;
                 } else {
                     for (int s = 0; s < S; ++s)
-                        if (d.N[half][(int64_t)s * T + t] < 0) bad |= kErrOverflow;
+                        if (__ldcg(d.N[half] + (int64_t)s * T + t) < 0) bad |= kErrOverflow;
                 }
             }
         }
@@ -602,6 +485,7 @@ struct EngineLaunch {
     cudaStream_t st;
     int sms;
     int clusters;
+    int S;                // largest species count of the group's simulations
     int used = 0;         // clusters launched
     int max_active = 0;   // clusters resident at once (occupancy query)
     bool query_only = false;   // fill max_active, launch nothing
@@ -610,9 +494,11 @@ struct EngineLaunch {
 template <int SA, bool R, int C>
 cudaError_t launch_cluster(EngineLaunch& L) {
     auto kern = k_engine_run<SA, R, C>;
-    cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemBytes);
+    // the attribute covers every group of this kernel, whatever its species
+    const size_t most = (size_t)kWarps * engine_warp_words(SA == 1 ? 1 : kMaxS, R) * sizeof(int32_t);
+    cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (ce != cudaSuccess) return ce;
-    const size_t dyn = (size_t)kDynSmemBytes;
+    const size_t dyn = (size_t)kWarps * engine_warp_words(L.S, R) * sizeof(int32_t);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C, 1, 1);
     cfg.blockDim = dim3(kRunBlock, 1, 1);
@@ -701,12 +587,9 @@ void warm_engine_kernels(int32_t* head, uint32_t* err, unsigned long long* proce
         cudaGetLastError();
         return;
     }
-    EngineLaunch W{nullptr, nullptr, nullptr, 0, head, err, processed, nullptr, (cudaStream_t)0, sms, 1};
+    EngineLaunch W{nullptr, nullptr, nullptr, 0, head, err, processed, nullptr, (cudaStream_t)0, sms, 1, 1};
     warm_kernels_sa<1>(W);
-    warm_kernels_sa<2>(W);
-    warm_kernels_sa<4>(W);
-    warm_kernels_sa<8>(W);
-    warm_kernels_sa<kMaxS>(W);
+    warm_kernels_sa<0>(W);
     cudaMemsetAsync(head, 0, sizeof(int32_t) * 10, (cudaStream_t)0);
     cudaStreamSynchronize((cudaStream_t)0);
     cudaGetLastError();
@@ -742,6 +625,7 @@ struct rdsplit_engine {
     cudaEvent_t ev_fork = nullptr;
     cudaEvent_t ev_join[10] = {};
     int32_t cluster = 2;                      // CTAs per simulation (1, 2, 4 or 8)
+    bool cluster_auto = false;                // chosen at each step by the number of simulations
     std::vector<rdsplit_mesh_t> slot_mesh;    // null = free
     std::vector<SlotDesc> h_desc;
     std::vector<int32_t> slot_q;              // local periods done
@@ -894,11 +778,9 @@ int rdsplit_engine_add(rdsplit_engine_t e, rdsplit_mesh_t h, double t_end, uint6
         return rdapi::fail(RDSPLIT_ECUDA, "%s: memset failed: %s", where, cudaGetErrorString(ce));
     }
     if (last_short) launch_thresholds(h->T, h->mp, h->g, h->G, tau_last, h->thr_last, st);
-    // one species without a zero-order reaction: packed per-tet records and
-    // interleaved counts (fewer cache lines per active tet)
-    bool zero = false;
-    for (int r = 0; r < h->R; ++r) zero = zero || (h->mp.order[r] == 0 && h->mp.k[r] > 0.0);
-    const bool pack = h->S == 1 && !zero && std::isfinite(h->tau);
+    // one species: packed per-tet records and interleaved counts (fewer cache
+    // lines per active tet)
+    const bool pack = h->S == 1;
     if (pack && !h->packed) {
         h->packed = (uint4*)rdapi::dev_alloc(32 * T);
         h->N2 = (int2*)rdapi::dev_alloc(8 * T);
@@ -970,10 +852,9 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
         max_adv = std::max<int64_t>(max_adv, d.q1 - d.q0);
     }
     if (items.empty()) return engine_err(e, where);
-    // Simulations are launched in groups of one kernel instantiation each:
-    // species class (1, 2, up to 4, up to 8, more) and with or without
-    // reactions, so that a one-species simulation does not run the code
-    // sized for eight.  Groups run concurrently on their own streams, the
+    // Simulations are launched in groups by species class (1, 2, up to 4, up
+    // to 8, more: it sets the shared memory of a warp) and with or without
+    // reactions.  Groups run concurrently on their own streams, the
     // resident clusters shared among them by work; largest first in each.
     auto cls_of = [&](int s) {
         const rdsplit_mesh* h = e->slot_mesh[s];
@@ -1011,6 +892,20 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
         cudaGetLastError();
         return rdapi::fail(RDSPLIT_ECUDA, "%s: upload failed: %s", where, cudaGetErrorString(ce));
     }
+    // The largest cluster of which as many fit as there are simulations: an
+    // ensemble of fewer than the GPU's clusters would leave SMs idle.
+    if (e->cluster_auto) {
+        for (int c = 8; c >= 1; c >>= 1) {
+            e->cluster = c;
+            EngineLaunch Q{e->d_desc, e->d_mp, e->d_order, 1, e->d_head, e->err, e->processed, nullptr, st, e->sms, 0, 1};
+            Q.query_only = true;
+            const int g = cls_of(order.back());
+            Q.S = g >> 1 ? (g >> 1 == 1 ? 2 : g >> 1 == 2 ? 4 : g >> 1 == 3 ? 8 : kMaxS) : 1;
+            const cudaError_t qe = g >> 1 ? launch_run_sa<0>((g & 1) != 0, c, Q) : launch_run_sa<1>((g & 1) != 0, c, Q);
+            if (qe == cudaSuccess && Q.max_active >= (int)items.size()) break;
+        }
+        if (e->cluster == 1) e->cluster = 2;
+    }
     const int csize = e->cluster;
     if (e->timing && !e->ev[0]) {
         cudaEventCreate(&e->ev[0]);
@@ -1019,13 +914,9 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
     if (e->timing) cudaEventRecord(e->ev[0], st);
     auto launch_group = [&](int g, EngineLaunch& L) -> cudaError_t {
         const bool react = (g & 1) != 0;
-        switch (g >> 1) {
-            case 0: return launch_run_sa<1>(react, csize, L);
-            case 1: return launch_run_sa<2>(react, csize, L);
-            case 2: return launch_run_sa<4>(react, csize, L);
-            case 3: return launch_run_sa<8>(react, csize, L);
-            default: return launch_run_sa<kMaxS>(react, csize, L);
-        }
+        const int most[5] = {1, 2, 4, 8, kMaxS};
+        L.S = most[g >> 1];
+        return g >> 1 ? launch_run_sa<0>(react, csize, L) : launch_run_sa<1>(react, csize, L);
     };
     int used = 0, fit = 0;
     if (n_groups == 1) {
@@ -1034,13 +925,13 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
         // default: as many clusters as can be resident at once (one CTA per
         // SM where the GPCs allow it)
         EngineLaunch L{e->d_desc, e->d_mp, e->d_order, g_count[g], e->d_head, e->err, e->processed,
-                       e->timing ? e->d_times : nullptr, st, e->sms, e->concurrency};
+                       e->timing ? e->d_times : nullptr, st, e->sms, e->concurrency, 1};
         ce = launch_group(g, L);
         used = L.used;
         fit = L.max_active;
     } else {
         // the clusters that fit, shared by work (at least one per group)
-        EngineLaunch Q{e->d_desc, e->d_mp, e->d_order, 1, e->d_head, e->err, e->processed, nullptr, st, e->sms, 0};
+        EngineLaunch Q{e->d_desc, e->d_mp, e->d_order, 1, e->d_head, e->err, e->processed, nullptr, st, e->sms, 0, 1};
         Q.query_only = true;
         ce = launch_group(7, Q);
         fit = Q.max_active;
@@ -1075,7 +966,7 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
             if (!g_count[g]) continue;
             ce = cudaStreamWaitEvent(e->aux[g], e->ev_fork, 0);
             EngineLaunch L{e->d_desc, e->d_mp, e->d_order + g_begin[g], g_count[g], e->d_head + g, e->err,
-                           e->processed, e->timing ? e->d_times : nullptr, e->aux[g], e->sms, share[g]};
+                           e->processed, e->timing ? e->d_times : nullptr, e->aux[g], e->sms, share[g], 1};
             if (ce == cudaSuccess) ce = launch_group(g, L);
             used += L.used;
             if (ce == cudaSuccess) ce = cudaEventRecord(e->ev_join[g], e->aux[g]);
@@ -1223,6 +1114,7 @@ int rdsplit_ensemble_run(int32_t n, const rdsplit_mesh_t* meshes, const double* 
     int rc = rdsplit_engine_create(n, tets, &e);
     if (rc) return rc;
     e->stream = meshes[0]->stream;
+    e->cluster_auto = true;
     for (int i = 0; i < n && rc == RDSPLIT_OK; ++i) rc = rdsplit_engine_add(e, meshes[i], t_end[i], seeds[i], nullptr);
     if (rc == RDSPLIT_OK) rc = rdsplit_engine_step(e, INT64_MAX / 4);
     rdsplit_engine_destroy(e);

@@ -476,7 +476,7 @@ k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams 
         Sender send(a, m.src, t, S);
         if (a.dense && live) send.clear_all();
         bool deferred = false;
-        bad |= warp_step<kReact, kPass == kPassFirst>(m, mp, S, w, v, t, live, &dirty, &deferred, s.err, send);
+        bad |= warp_step<S_ == 1, kReact, kPass == kPassFirst>(m, mp, S, w, v, t, live, &dirty, &deferred, s.err, send);
         if (live && !deferred) send.finish(a.dense != 0);
         if (kPass == kPassFirst) {
             const unsigned dm = __ballot_sync(0xffffffffu, deferred);
@@ -573,7 +573,7 @@ k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp,
                            last ? r.thr_last : r.thr, 1};
         Sender send(a, m.src, t, S);
         bool deferred = false;
-        bad |= warp_step<kReact, false>(m, mp, S, w, v, t, live, &dirty, &deferred, s.err, send);
+        bad |= warp_step<S_ == 1, kReact, false>(m, mp, S, w, v, t, live, &dirty, &deferred, s.err, send);
         if (live) send.finish(false);
     }
     if (live)

@@ -327,10 +327,13 @@ __device__ __forceinline__ void count_block(const uint4& w, int m, const uint4& 
 // All lanes must call it.  The per-lane loop with a whole-warp pass per
 // species and tet from 10 molecules on took one serial pass a tet: 600 cycles
 // each, up to 32 a warp.
-template <class Big>
+// With one species (kOne) every lane draws its own first block, without the
+// list, and only counts above four go on to it.  pre: the lane's thresholds
+// of species 0, when kPre says that they are loaded.
+template <bool kOne, bool kPre, class Big>
 __device__ __forceinline__ uint32_t draw_all(const ModelParams& mp, int S, int64_t T, const WarpMem& w,
                                              const PeriodView& v, int t, int key, uint32_t present, uint32_t touched,
-                                             Big big) {
+                                             uint4 pre, Big big) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const uint32_t k0 = (uint32_t)v.seed, k1 = (uint32_t)(v.seed >> 32);
@@ -347,8 +350,14 @@ __device__ __forceinline__ uint32_t draw_all(const ModelParams& mp, int S, int64
                     n = 0;
                 }
                 if (n > 0) {
-                    w.acc0[32 * sp + lane] = 0u;
-                    w.acc1[32 * sp + lane] = 0u;
+                    uint32_t a0 = 0, a1 = 0;
+                    if (kOne && n <= kCoopMin) {
+                        const uint4 C = kPre ? pre : __ldg(v.thr + (int64_t)t * v.thr_stride);
+                        count_block(rdd::philox_block(0u, (uint32_t)key, v.period, rdd::kPurposeDiffusion << 16, k0, k1),
+                                    min(4, n), C, a0, a1);
+                    }
+                    w.acc0[32 * sp + lane] = a0;
+                    w.acc1[32 * sp + lane] = a1;
                     drawn |= 1u << sp;
                 }
             }
@@ -374,7 +383,7 @@ __device__ __forceinline__ uint32_t draw_all(const ModelParams& mp, int S, int64
             }
         }
         const int nb = (n + 3) >> 2;
-        for (int b = 0;; ++b) {
+        for (int b = kOne ? 1 : 0;; ++b) {
             const unsigned act = __ballot_sync(kAllLanes, b < nb);
             if (b < nb)
                 w.list[cnt + __popc(act & lt)] =
@@ -413,10 +422,10 @@ __device__ __forceinline__ uint32_t draw_all(const ModelParams& mp, int S, int64
 // whose count changed are added to *dirty.  With kDefer, a lane whose tet
 // needs the reaction phase leaves it undone and answers true in *deferred.
 // Returns error bits.  All lanes must call it.
-template <bool kReact, bool kDefer, class Emit>
+template <bool kOne, bool kReact, bool kDefer, bool kPre = false, class Emit>
 __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParams& mp, int S, const WarpMem& w,
                                               const PeriodView& v, int t, bool live, uint32_t* dirty, bool* deferred,
-                                              uint32_t* err, Emit& emit) {
+                                              uint32_t* err, Emit& emit, uint4 pre = make_uint4(0u, 0u, 0u, 0u)) {
     const int lane = threadIdx.x & 31;
     const int key = live ? key_of(m, t) : 0;
     uint32_t bad = 0, touched = 0;
@@ -457,7 +466,7 @@ __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParam
     if (live)
         for (int s = 0; s < S; ++s)
             if (w.N[32 * s + lane] > 0) present |= 1u << s;
-    const uint32_t drawn = draw_all(mp, S, m.T, w, v, t, key, present, touched, [&](int sp, int32_t star) {
+    const uint32_t drawn = draw_all<kOne, kPre>(mp, S, m.T, w, v, t, key, present, touched, pre, [&](int sp, int32_t star) {
         const int32_t Nt = w.N[32 * sp + lane];
         const int4 o = diffuse_binomial(m.G, m.g, t, key, sp, mp.D[sp], v.period, v.tau_k, v.seed, Nt, star);
         const int32_t all = o.x + o.y + o.z + o.w;

@@ -42,7 +42,8 @@ struct SlotDesc {
     const uint4* thr;        // thresholds for tau
     const uint4* thr_last;   // thresholds for the shortened last period
     int32_t* N[2];           // count buffers [S][T]; the slice starts in N[0]
-    uint32_t* bits[2];       // active-tet bitmaps (bit t of word t/32), by period parity in the slice
+    uint32_t* bits[2];       // active-tet bitmaps of 2^wshift words, by period parity in the slice
+    int32_t wshift;          // tet t is bit t >> wshift of word t & (2^wshift - 1)
     const uint4* packed;     // one species: {src, thr} per tet
     int32_t* N2;             // one species: counts of both parities interleaved
     uint64_t seed;
@@ -74,6 +75,11 @@ __device__ __forceinline__ void red_or(uint32_t* p, uint32_t v) {
     asm volatile("red.relaxed.gpu.global.or.b32 [%0], %1;" ::"l"(p), "r"(v));
 }
 
+// Fire-and-forget AND.
+__device__ __forceinline__ void red_and(uint32_t* p, uint32_t v) {
+    asm volatile("red.relaxed.gpu.global.and.b32 [%0], %1;" ::"l"(p), "r"(v));
+}
+
 constexpr int kWarps = kRunBlock / 32;
 constexpr int kGroup = 8;                   // bitmap columns (32 words each) a warp loads at once
 
@@ -94,12 +100,6 @@ __device__ __forceinline__ int nth_set_bit(uint32_t w, int k) {
         }
     }
     return p;
-}
-
-// The bitmap word of lane `lane` in column kk of batch b of warp gw: column by
-// column 8 runs of 4 words, runs dealt round-robin over kW warps.
-__device__ __forceinline__ int word_of(int gw, int b, int kk, int lane, int kW) {
-    return (gw + ((b * kGroup + kk) * 8 + (lane >> 2)) * kW) * 4 + (lane & 3);
 }
 
 // Shared memory of the engine kernel.
@@ -160,17 +160,19 @@ struct Scatter {
     }
 };
 
-// One period of a simulation for one warp.  The bitmap is dealt to the
-// cluster's kW warps in runs of 4 words (128 tets): run r goes to warp
-// r mod kW, so the active tets of a region are spread over all warps (runs
-// of 4 measured faster than runs of 1, 2 or 8).  A column is 8 runs of a warp
-// (32 words, one per lane); a warp loads kGroup of its columns at once and
-// clears them for their next use.  With a prefix sum of a column's popcounts
-// each lane finds a set bit of its own (a search over the sums and one inside
-// the word: a fixed 60 instructions, where writing the bits of a dense word
-// into a list took 32 turns of one lane); whenever 32 tets are at hand, one
-// round steps them (warp_step), and adds what stays and what leaves into the
-// next counts.
+// One period of a simulation for one warp.  A bitmap word holds 32 tets a
+// power of two apart, so that every word has its share of a compact cloud of
+// molecules and of its crowded tets: dealing runs of 128 consecutive tets
+// left warps waiting at the period barrier for the one that held the source
+// (15 of 24 stall cycles an instruction).  The words go to the cluster's kW
+// warps in equal contiguous parts (fewer words than warps: several warps share
+// a word by bit position).  A column is 32 words, one per lane; a warp loads
+// kGroup of its columns at once and clears them for their next use.  With a
+// prefix sum of a column's popcounts each lane finds a set bit of its own (a
+// search over the sums and one inside the word: a fixed 60 instructions, where
+// writing the bits of a dense word into a list took 32 turns of one lane);
+// whenever 32 tets are at hand, one round steps them (warp_step), and adds
+// what stays and what leaves into the next counts.
 template <bool kOne, bool kReact, int kC>
 __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned long long* mass_delta,
                                                unsigned long long* done) {
@@ -184,7 +186,19 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
     int32_t* base_mem = s_warp + warp * engine_warp_words(S, kReact);
     const WarpMem w(base_mem, S, kReact);
     uint32_t* wb = reinterpret_cast<uint32_t*>(base_mem + warp_words(S, kReact));
-    const int W = (d.m.T + 31) >> 5;
+    const int ws = d.wshift, W = 1 << ws;
+    // this warp's words: `per` from word0 on, or its bits of one shared word
+    constexpr int kWShift = kC == 1 ? 4 : (kC == 2 ? 5 : (kC == 4 ? 6 : 7));
+    static_assert((1 << kWShift) == kW, "warps of a cluster");
+    const bool shared = ws < kWShift;
+    const int per = shared ? 1 : W >> kWShift;
+    const int word0 = shared ? gw & (W - 1) : gw * per;
+    uint32_t part = 0xffffffffu;
+    if (shared) {
+        const int split = min(kW >> ws, 32), sub = gw >> ws;
+        part = 0u;
+        for (int i = sub; i < 32; i += split) part |= sub < split ? 1u << i : 0u;
+    }
     const int r = (q - d.q0) & 1;
     const bool last = (q == d.P - 1) && d.last_short;
     // thresholds: packed beside the reverse-face record (stride 2) except in a
@@ -199,19 +213,22 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
     int pend = 0, cnt = 0;      // tets not yet run: lane i < cnt holds one
     unsigned long long visited = 0;
     for (int b = 0;; ++b) {
-        const bool flush = (gw + b * kGroup * 8 * kW) * 4 >= W;   // past the last batch: run what is left
+        const int at = b * kGroup * 32 + lane;
+        const bool flush = b * kGroup * 32 >= per;   // past the last batch: run what is left
         int columns = 1;
         if (!flush) {
             uint32_t wds[kGroup];
 #pragma unroll
             for (int kk = 0; kk < kGroup; ++kk) {
-                const int wi = word_of(gw, b, kk, lane, kW);
-                wds[kk] = wi < W ? __ldcg(bcur + wi) : 0u;
+                wds[kk] = at + kk * 32 < per ? __ldcg(bcur + word0 + at + kk * 32) & part : 0u;
             }
             uint32_t any = 0;
 #pragma unroll
             for (int kk = 0; kk < kGroup; ++kk) {
-                if (wds[kk]) bcur[word_of(gw, b, kk, lane, kW)] = 0u;
+                if (wds[kk]) {
+                    if (shared) red_and(bcur + word0, ~part);
+                    else bcur[word0 + at + kk * 32] = 0u;
+                }
                 wb[kk * 32 + lane] = wds[kk];
                 any |= wds[kk] ? 1u << kk : 0u;
             }
@@ -241,7 +258,7 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
                     if (__shfl_sync(kAllLanes, inc, from + step - 1) <= e) from += step;
                 const int k = e - __shfl_sync(kAllLanes, inc - own, from);
                 const int bit = nth_set_bit(__shfl_sync(kAllLanes, word, from), k);
-                const int t_new = word_of(gw, b, kk, from, kW) * 32 + bit;
+                const int t_new = (bit << ws) + word0 + (b * kGroup + kk) * 32 + from;
                 const int t_lane = e < 0 ? pend : t_new;
                 if (avail < 32 && !(flush && avail > 0)) {
                     pend = t_lane;
@@ -299,13 +316,13 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
                     }
                     if (kReact) delta += scatter.sent - held;
                     if (more) {
-                        if (keep) red_or(bnext + (t >> 5), 1u << (t & 31));
+                        if (keep) red_or(bnext + (t & (W - 1)), 1u << (t >> ws));
                         const int nbr[4] = {scatter.sr.x, scatter.sr.y, scatter.sr.z, scatter.sr.w};
 #pragma unroll
                         for (int f = 0; f < 4; ++f) {
                             if (!((scatter.send >> f) & 1u)) continue;
                             const int u = nbr[f] >> 2;
-                            red_or(bnext + (u >> 5), 1u << (u & 31));
+                            red_or(bnext + (u & (W - 1)), 1u << (u >> ws));
                         }
                     }
                 }
@@ -384,17 +401,17 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
         const SlotDesc& d = s_desc;
         const int T = d.m.T;
         const int S = kOne ? 1 : d.S;
-        const int W = (T + 31) >> 5;
+        const int W = 1 << d.wshift;
         constexpr bool inter = kOne;   // interleaved counts
         uint32_t bad = 0;
         // initial bitmap: occupied tets and tets with a zero-order reaction on
-        // (whole words, written by the first lane of each 32-tet run); and the
-        // simulation's molecule total
+        // (a thread a word; its tets are W apart, so a warp's loads are
+        // contiguous); and the simulation's molecule total
         unsigned long long mine = 0;
-        for (int base = rank * kRunBlock; base < W * 32; base += kC * kRunBlock) {
-            const int t = base + threadIdx.x;
-            bool occ = false;
-            if (t < T) {
+        for (int wi = rank * kRunBlock + threadIdx.x; wi < W; wi += kC * kRunBlock) {
+            uint32_t word = 0;
+            for (int t = wi, bit = 0; t < T; t += W, ++bit) {
+                bool occ = false;
                 if (kReact && d.zero_order)
                     occ = ((s_mp.has_mask ? d.m.mask[t] : 0xffffffffu) & d.zero_order) != 0u;
                 for (int s = 0; s < S; ++s) {
@@ -404,9 +421,9 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
                     if (c < 0) bad |= kErrNegative;
                     if (inter) reinterpret_cast<int2*>(d.N2)[t] = make_int2(c, 0);
                 }
+                if (occ) word |= 1u << bit;
             }
-            const uint32_t word = __ballot_sync(kAllLanes, occ);
-            if (lane == 0 && (t >> 5) < W) d.bits[0][t >> 5] = word;
+            d.bits[0][wi] = word;
         }
 #pragma unroll
         for (int dd = 16; dd > 0; dd >>= 1) mine += __shfl_xor_sync(kAllLanes, mine, dd);
@@ -763,7 +780,9 @@ int rdsplit_engine_add(rdsplit_engine_t e, rdsplit_mesh_t h, double t_end, uint6
     if (h->period + P > (int64_t)0xffffffffll) return rdapi::fail(RDSPLIT_EOVERFLOW, "%s: period index exceeds 2^32-1", where);
     if (P > 0x7fffffffll) return rdapi::fail(RDSPLIT_EINVAL, "%s: too many periods", where);
     const size_t T = (size_t)h->T;
-    const size_t W = (T + 31) / 32;
+    int wshift = 0;
+    while (((size_t)32 << wshift) < T) ++wshift;
+    const size_t W = (size_t)1 << wshift;
     if (!h->bits[0]) {
         h->bits[0] = (uint32_t*)rdapi::dev_alloc(4 * W);
         h->bits[1] = (uint32_t*)rdapi::dev_alloc(4 * W);
@@ -795,6 +814,7 @@ int rdsplit_engine_add(rdsplit_engine_t e, rdsplit_mesh_t h, double t_end, uint6
     d.N[1] = h->rem;
     d.bits[0] = h->bits[0];
     d.bits[1] = h->bits[1];
+    d.wshift = wshift;
     d.packed = pack ? h->packed : nullptr;
     d.N2 = pack ? reinterpret_cast<int32_t*>(h->N2) : nullptr;
     d.seed = seed;

@@ -184,7 +184,7 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
     const int gw = rank * kWarps + warp;
     const int S = kOne ? 1 : d.S;
     int32_t* base_mem = s_warp + warp * engine_warp_words(S, kReact);
-    const WarpMem w(base_mem, S, kReact);
+    const WarpMem w(base_mem, S, kReact, s_mp.rx);
     uint32_t* wb = reinterpret_cast<uint32_t*>(base_mem + warp_words(S, kReact));
     const int ws = d.wshift, W = 1 << ws;
     // this warp's words: `per` from word0 on, or its bits of one shared word
@@ -272,6 +272,8 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
                 int4 sr = make_int4(-1, -1, -1, -1);
                 uint4 pre = make_uint4(0u, 0u, 0u, 0u);
                 long long held = 0;
+                Presence pr;
+                const uint32_t mask = kReact && mp.has_mask && live ? __ldg(d.m.mask + t) : 0xffffffffu;
                 if (live) {
                     if (kOne) {
                         // the record and the count, loaded together
@@ -292,6 +294,7 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
                                 n[k] = 0;
                             }
                             w.N[32 * (s0 + k) + lane] = n[k];
+                            pr.set(s0 + k, n[k]);
                             if (kReact) held += n[k];
                         }
                     }
@@ -299,20 +302,18 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
                 Scatter<kOne> scatter(c, d.m.src, t, sr, kOne);
                 uint32_t dirty = 0;
                 bool deferred = false;
-                bad |= warp_step<kOne, kReact, false, kOne>(d.m, mp, S, w, v, t, live, &dirty, &deferred, err, scatter,
-                                                            pre);
+                bad |= warp_step<kOne, kReact, false, kOne>(d.m, mp, S, w, v, t, live, mask, pr, &dirty, &deferred,
+                                                            err, scatter, pre);
                 bad |= scatter.bad;
                 long long delta = 0;
                 if (live) {
-                    bool keep = false;
-                    if (kReact && d.zero_order) keep = ((mp.has_mask ? d.m.mask[t] : 0xffffffffu) & d.zero_order) != 0u;
-                    for (int s = 0; s < S; ++s) {
+                    bool keep = pr.any != 0u;
+                    if (kReact && d.zero_order) keep = keep || (mask & d.zero_order) != 0u;
+                    for (uint32_t bits = pr.any; bits; bits &= bits - 1u) {
+                        const int s = __ffs(bits) - 1;
                         const int32_t n = w.N[32 * s + lane];
-                        if (n > 0) {
-                            red_add(c.next + (s * c.T + t) * c.stride, n);
-                            keep = true;
-                            if (kReact) delta += n;
-                        }
+                        red_add(c.next + (s * c.T + t) * c.stride, n);
+                        if (kReact) delta += n;
                     }
                     if (kReact) delta += scatter.sent - held;
                     if (more) {

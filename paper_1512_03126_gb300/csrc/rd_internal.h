@@ -41,6 +41,11 @@ struct ModelParams {
     // is absent (or, for 2A, present only once).
     uint32_t needs[kMaxS];
     uint32_t needs2[kMaxS];
+    // Per reaction, for the warp's reaction phase: k as float bits, and
+    // reactant a | reactant b << 4 | kind << 8 | changed species << 16 (kind 0:
+    // no reactant, 1: a, 2: a + b, 3: 2a).
+    uint2 rx[kMaxR];
+    uint32_t moves;       // species with D > 0
     // Transfer rule of the diffusion draw (Sec. II.C): kRuleMean (N-bar,
     // Eq. 3, the method), kRuleEnd (N at tau_k, first-order splitting) or
     // kRuleMid (N at tau_k / 2).

@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <cstring>
 
 #include "rd_device.cuh"
 #include "rd_internal.h"
@@ -298,6 +299,9 @@ void launch_counts_out(int32_t T, int32_t S, const int32_t* sm, int32_t* ts, con
 // ---------------------------------------------------------------- period ---
 void finish_model_params(ModelParams& mp) {
     mp.kpos = 0;
+    mp.moves = 0;
+    for (int s = 0; s < mp.S; ++s)
+        if (mp.D[s] > 0.0) mp.moves |= 1u << s;
     for (int s = 0; s < kMaxS; ++s) mp.needs[s] = mp.needs2[s] = 0u;
     for (int r = 0; r < mp.R; ++r) {
         mp.rs1[r] = mp.rs2[r] = -1;
@@ -314,6 +318,12 @@ void finish_model_params(ModelParams& mp) {
             if (mp.lhs[r][s] >= 1) mp.needs[s] |= 1u << r;
             if (mp.lhs[r][s] >= 2) mp.needs2[s] |= 1u << r;
         }
+        uint32_t changed = 0;
+        for (int s = 0; s < mp.S; ++s) changed |= mp.delta[r][s] != 0 ? 1u << s : 0u;
+        const int a = mp.rs1[r], b = mp.rs2[r];
+        const uint32_t kind = a < 0 ? 0u : (b < 0 ? 1u : (a == b ? 3u : 2u));
+        std::memcpy(&mp.rx[r].x, &mp.kf[r], sizeof(float));
+        mp.rx[r].y = (uint32_t)std::max(a, 0) | (uint32_t)std::max(b, 0) << 4 | kind << 8 | changed << 16;
     }
 }
 
@@ -337,7 +347,7 @@ void launch_avv(int32_t T, const double* vol, float2* avv, cudaStream_t st) {
 // tet-period of eight species moved were inbox words, nearly all zero.
 // Returns error bits.
 __device__ __forceinline__ uint32_t take_inbox(const PeriodArgs& a, int t, int S, int lane, int32_t* N,
-                                               uint32_t* dirty) {
+                                               Presence& pr, uint32_t* dirty) {
     const int Sp = inbox_stride(S);
     uint32_t bad = 0;
     auto add = [&](int sp, int64_t v) {
@@ -345,6 +355,7 @@ __device__ __forceinline__ uint32_t take_inbox(const PeriodArgs& a, int t, int S
         if (n > 2147483647) { bad |= kErrOverflow; n = 2147483647; }
         if (n < 0) { bad |= kErrNegative; n = 0; }
         N[32 * sp + lane] = (int32_t)n;
+        pr.set(sp, (int32_t)n);
         *dirty |= 1u << sp;
     };
     if (S <= 2) {
@@ -450,7 +461,12 @@ k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams 
     extern __shared__ int32_t sm[];
     const int S = S_ > 0 ? S_ : mp.S;
     const int lane = threadIdx.x & 31;
-    const WarpMem w(sm + (threadIdx.x >> 5) * warp_words(S, kReact), S, kReact);
+    __shared__ uint2 rx[kReact ? kMaxR : 1];
+    const WarpMem w(sm + (threadIdx.x >> 5) * warp_words(S, kReact), S, kReact, rx);
+    if (kReact) {
+        if (threadIdx.x < kMaxR) rx[threadIdx.x] = mp.rx[threadIdx.x];
+        __syncthreads();
+    }
     const int64_t T = m.T;
     const PeriodView v{a.period, a.tau_k, a.tau_kf, a.seed, a.thr, 1};
     const int hi = kPass == kPassQueue ? qcount[parity] : (a.t_hi > 0 ? a.t_hi : m.T);
@@ -461,6 +477,8 @@ k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams 
         bool live = base + lane < hi;
         const int t = !live ? 0 : (kPass == kPassQueue ? queue[base + lane] : (int)(base + lane));
         uint32_t bad = 0, dirty = 0;
+        Presence pr;
+        const uint32_t mask = kReact && mp.has_mask && live ? __ldg(m.mask + t) : 0xffffffffu;
         if (live) {
             for (int s0 = 0; s0 < S; s0 += 8) {
                 int32_t n[8];
@@ -469,14 +487,17 @@ k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams 
                     if (s0 + k < S) n[k] = s.cnt[(int64_t)(s0 + k) * T + t];
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
-                    if (s0 + k < S) w.N[32 * (s0 + k) + lane] = n[k];
+                    if (s0 + k < S) {
+                        w.N[32 * (s0 + k) + lane] = n[k];
+                        pr.set(s0 + k, n[k]);
+                    }
             }
-            if (kPass != kPassQueue && !a.first) bad |= take_inbox(a, t, S, lane, w.N, &dirty);
+            if (kPass != kPassQueue && !a.first) bad |= take_inbox(a, t, S, lane, w.N, pr, &dirty);
         }
         Sender send(a, m.src, t, S);
         if (a.dense && live) send.clear_all();
         bool deferred = false;
-        bad |= warp_step<S_ == 1, kReact, kPass == kPassFirst>(m, mp, S, w, v, t, live, &dirty, &deferred, s.err, send);
+        bad |= warp_step<S_ == 1, kReact, kPass == kPassFirst>(m, mp, S, w, v, t, live, mask, pr, &dirty, &deferred, s.err, send);
         if (live && !deferred) send.finish(a.dense != 0);
         if (kPass == kPassFirst) {
             const unsigned dm = __ballot_sync(0xffffffffu, deferred);
@@ -546,14 +567,25 @@ k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp,
     __shared__ int gave_up;
     const int S = S_ > 0 ? S_ : mp.S;
     const int lane = threadIdx.x & 31;
-    const WarpMem w(sm + (threadIdx.x >> 5) * warp_words(S, kReact), S, kReact);
+    __shared__ uint2 rx[kReact ? kMaxR : 1];
+    const WarpMem w(sm + (threadIdx.x >> 5) * warp_words(S, kReact), S, kReact, rx);
+    if (kReact) {
+        if (threadIdx.x < kMaxR) rx[threadIdx.x] = mp.rx[threadIdx.x];
+        __syncthreads();
+    }
     const int64_t T = m.T;
     const int64_t tt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool live = tt < T;
     const int t = live ? (int)tt : 0;
     if (threadIdx.x == 0) gave_up = 0;
+    Presence pr;
+    const uint32_t mask = kReact && mp.has_mask && live ? __ldg(m.mask + t) : 0xffffffffu;
     if (live)
-        for (int sp = 0; sp < S; ++sp) w.N[32 * sp + lane] = s.cnt[sp * T + t];
+        for (int sp = 0; sp < S; ++sp) {
+            const int32_t n = s.cnt[sp * T + t];
+            w.N[32 * sp + lane] = n;
+            pr.set(sp, n);
+        }
     uint32_t bad = 0, dirty = 0, target = r.barrier_base;
     for (int q = 0; q <= r.periods; ++q) {
         PeriodArgs a{};
@@ -565,7 +597,7 @@ k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp,
         if (q > 0) {
             target += gridDim.x;
             if (!grid_barrier(r.barrier, target, s.err, &gave_up)) return;
-            if (live) bad |= take_inbox(a, t, S, lane, w.N, &dirty);
+            if (live) bad |= take_inbox(a, t, S, lane, w.N, pr, &dirty);
         }
         if (q == r.periods) break;
         const bool last = r.last_short && q == r.periods - 1;
@@ -573,7 +605,7 @@ k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp,
                            last ? r.thr_last : r.thr, 1};
         Sender send(a, m.src, t, S);
         bool deferred = false;
-        bad |= warp_step<S_ == 1, kReact, false>(m, mp, S, w, v, t, live, &dirty, &deferred, s.err, send);
+        bad |= warp_step<S_ == 1, kReact, false>(m, mp, S, w, v, t, live, mask, pr, &dirty, &deferred, s.err, send);
         if (live) send.finish(false);
     }
     if (live)
@@ -686,7 +718,8 @@ __global__ void k_gather(int32_t T, int32_t S, DevState s, PeriodArgs a) {
     int32_t* N = sm + (threadIdx.x >> 5) * 32 * S;
     for (int sp = 0; sp < S; ++sp) N[32 * sp + lane] = s.cnt[(int64_t)sp * T + t];
     uint32_t dirty = 0;
-    const uint32_t bad = take_inbox(a, t, S, lane, N, &dirty);
+    Presence pr;
+    const uint32_t bad = take_inbox(a, t, S, lane, N, pr, &dirty);
     for (uint32_t bits = dirty; bits; bits &= bits - 1u) {
         const int sp = __ffs(bits) - 1;
         s.cnt[(int64_t)sp * T + t] = N[32 * sp + lane];

@@ -50,7 +50,8 @@ struct WarpMem {
     uint32_t* acc0;
     uint32_t* acc1;
     uint32_t* list;
-    __device__ __forceinline__ WarpMem(int32_t* base, int S, bool react) {
+    const uint2* rx;      // reaction table (ModelParams::rx) in shared memory
+    __device__ __forceinline__ WarpMem(int32_t* base, int S, bool react, const uint2* rx_) : rx(rx_) {
         N = base;
         acc0 = reinterpret_cast<uint32_t*>(N + 32 * S);
         acc1 = acc0 + 32 * S;
@@ -69,29 +70,39 @@ struct PeriodView {
     int thr_stride;
 };
 
-// Reactions of `on` whose reactants are present in the lane's column.
-__device__ __forceinline__ uint32_t possible_in_column(const ModelParams& mp, const int32_t* Ncol, int S, uint32_t on) {
+// Which species of a lane's tet have molecules, and which more than one: kept
+// beside the column, so that loops run over set bits only.
+struct Presence {
+    uint32_t any = 0, two = 0;
+    __device__ __forceinline__ void set(int s, int32_t n) {
+        const uint32_t bit = 1u << s;
+        any = n > 0 ? any | bit : any & ~bit;
+        two = n > 1 ? two | bit : two & ~bit;
+    }
+};
+
+// Reactions of `on` whose reactants are present.
+__device__ __forceinline__ uint32_t possible_by_presence(const ModelParams& mp, const Presence& pr, int S, uint32_t on) {
     uint32_t m = on;
     for (int s = 0; s < S; ++s) {
-        const int32_t n = Ncol[32 * s];
-        if (n <= 0) m &= ~mp.needs[s];
-        else if (n == 1) m &= ~mp.needs2[s];
+        if (!((pr.any >> s) & 1u)) m &= ~mp.needs[s];
+        if (!((pr.two >> s) & 1u)) m &= ~mp.needs2[s];
     }
     return m;
 }
 
-// Propensity of reaction r in single precision (relative error below
-// 8 * 2^-24: three roundings in the rate, three in the combinations, one in
-// their product).
-__device__ __forceinline__ float propensity_f(const ModelParams& mp, int r, const int32_t* Ncol, float2 avf) {
-    const int a = mp.rs1[r], b = mp.rs2[r], o = mp.order[r];
-    float c = mp.kf[r];
-    if (o == 0) return c * avf.x;
-    if (o == 2) c = c * avf.y;
-    const int32_t na = Ncol[32 * a];
-    if (b < 0) return c * (float)na;
-    if (a == b) return c * (0.5f * (float)na * (float)(na - 1));
-    return c * ((float)na * (float)Ncol[32 * b]);
+// Propensity of a reaction of the table in single precision (relative error
+// below 8 * 2^-24: three roundings in the rate, three in the combinations, one
+// in their product).
+__device__ __forceinline__ float propensity_f(const uint2 rx, const int32_t* Ncol, float2 avf) {
+    float c = __uint_as_float(rx.x);
+    const uint32_t kind = (rx.y >> 8) & 3u;
+    if (kind == 0u) return c * avf.x;
+    const int32_t na = Ncol[32 * (rx.y & 15u)];
+    if (kind == 1u) return c * (float)na;
+    c = c * avf.y;
+    if (kind == 3u) return c * (0.5f * (float)na * (float)(na - 1));
+    return c * ((float)na * (float)Ncol[32 * ((rx.y >> 4) & 15u)]);
 }
 
 enum : int { kReactNone = 0, kReactDone = 1, kReactDoubt = 2 };
@@ -121,23 +132,25 @@ enum : int { kReactNone = 0, kReactDone = 1, kReactDoubt = 2 };
 // On kReactDone: Ncol holds the counts after the phase, *touched the species
 // that changed, and Dcol, for those, N* (mean rule) or the mid-period count
 // (half-step rule).  scratch: the lane's column of one word per species.
-__device__ __forceinline__ int react_fast(const ModelParams& mp, int S, int key, const PeriodView& v, uint32_t on,
-                                          uint32_t poss, float2 avf, int32_t* Ncol, int32_t* Dcol, uint32_t* scratch,
-                                          uint32_t* touched_out) {
+__device__ __forceinline__ int react_fast(const ModelParams& mp, const uint2* rx, int S, int key, const PeriodView& v,
+                                          uint32_t on, uint32_t poss, float2 avf, int32_t* Ncol, int32_t* Dcol,
+                                          uint32_t* scratch, Presence& pr, uint32_t* touched_out) {
     constexpr float e = 5.9604644775390625e-08f;   // 2^-24
     constexpr int kMaxEvents = 64;
     const bool mid = mp.rule == kRuleMid;
-    rdd::Stream st(v.seed, (uint32_t)key, v.period, rdd::kPurposeReaction, 0);
+    const uint32_t k0 = (uint32_t)v.seed, k1 = (uint32_t)(v.seed >> 32);
     float x = 0.0f, dsum = 0.0f;
     uint32_t touched = 0;
     int k = 0;
     bool past = false, doubt = !(v.tau_kf < 1e6f);   // (keeps underflowed rates below 1e-13 a period)
     while (!doubt) {
-        if (k > 0) poss = possible_in_column(mp, Ncol, S, on);
+        if (k > 0) poss = possible_by_presence(mp, pr, S, on);
         if (!poss) break;                          // total propensity 0
-        const uint64_t x1 = st.bits53();
+        // block k of the tet's reaction stream: u1 and u2 of event k
+        const uint4 rw = rdd::philox_block((uint32_t)k, (uint32_t)key, v.period, rdd::kPurposeReaction << 16, k0, k1);
+        const uint64_t x1 = ((uint64_t)(rw.x >> 5) << 26) | (rw.y >> 6);
         float a0 = 0.0f;
-        for (uint32_t bits = poss; bits; bits &= bits - 1u) a0 += propensity_f(mp, __ffs(bits) - 1, Ncol, avf);
+        for (uint32_t bits = poss; bits; bits &= bits - 1u) a0 += propensity_f(rx[__ffs(bits) - 1], Ncol, avf);
         const float at = a0 * v.tau_kf;
         const float eps = (float)(128 + 4 * k) * e;
         const uint64_t y = 9007199254740991ull - x1;                    // (1 - u1) 2^53
@@ -161,21 +174,21 @@ __device__ __forceinline__ int react_fast(const ModelParams& mp, int S, int key,
             }
         }
         // the first reaction whose cumulated propensity exceeds u2 a0
-        const float target = (float)st.bits53() * 1.1102230246251565e-16f * a0;
+        const float target = (float)(((uint64_t)(rw.z >> 5) << 26) | (rw.w >> 6)) * 1.1102230246251565e-16f * a0;
         const float margin = 128.0f * e * a0;
         int mu = -1;
         float cum = 0.0f;
         for (uint32_t bits = poss; bits; bits &= bits - 1u) {
             const int r = __ffs(bits) - 1;
-            cum += propensity_f(mp, r, Ncol, avf);
+            cum += propensity_f(rx[r], Ncol, avf);
             if (target < cum - margin) { mu = r; break; }
             if (target <= cum + margin) break;
         }
         if (mu < 0) { doubt = true; break; }
         float dmax = 0.0f;
-        for (int s = 0; s < S; ++s) {
+        for (uint32_t bits = rx[mu].y >> 16; bits; bits &= bits - 1u) {
+            const int s = __ffs(bits) - 1;
             const int dn = mp.delta[mu][s];
-            if (dn == 0) continue;
             const int32_t n = Ncol[32 * s];
             if (n >= (1 << 20)) doubt = true;
             if (!((touched >> s) & 1u)) {
@@ -185,6 +198,7 @@ __device__ __forceinline__ int react_fast(const ModelParams& mp, int S, int key,
             }
             if (!mid) Dcol[32 * s] = __float_as_int(__int_as_float(Dcol[32 * s]) + (float)dn * xn);
             Ncol[32 * s] = n + dn;
+            pr.set(s, n + dn);
             dmax = fmaxf(dmax, fabsf((float)dn));
         }
         dsum += dmax;
@@ -210,6 +224,7 @@ __device__ __forceinline__ int react_fast(const ModelParams& mp, int S, int key,
         for (uint32_t bits = touched; bits; bits &= bits - 1u) {
             const int s = __ffs(bits) - 1;
             Ncol[32 * s] = (int32_t)scratch[32 * s];
+            pr.set(s, Ncol[32 * s]);
         }
         return kReactDoubt;
     }
@@ -318,160 +333,176 @@ __device__ __forceinline__ void count_block(const uint4& w, int m, const uint4& 
 }
 
 // The diffusion draws of a warp's tets (Step 3; Eq. 2-3): every (lane,
-// species) with molecules contributes ceil(n / 4) Philox blocks to one list,
-// filled block index by block index with a ballot (so neighbouring entries
-// belong to different lanes), and 32 entries make a round with one block a
-// lane.  The cost follows the number of blocks, not the largest count of
-// a lane or the species present in any lane.  big(sp, N*) handles a lane's
-// binomial draws.  Returns the species whose acc words hold leavers-to-be.
-// All lanes must call it.  The per-lane loop with a whole-warp pass per
-// species and tet from 10 molecules on took one serial pass a tet: 600 cycles
-// each, up to 32 a warp.
+// species) with molecules contributes ceil(n / 4) Philox blocks to one list;
+// in each turn every lane adds its next block (of its next species when one is
+// done), so neighbouring entries belong to different lanes, and 32 entries
+// make a round with one block a lane.  The cost follows the number of blocks,
+// not the largest count of a lane or the species present in any lane.
+// Species with more than kCoopMin draws are drawn by the whole warp first,
+// and those from kMoleculeCut on by big(sp, N*).  Returns the species whose
+// acc words hold leavers-to-be.  All lanes must call it.  The per-lane loop
+// with a whole-warp pass per species and tet from 10 molecules on took one
+// serial pass a tet: 600 cycles each, up to 32 a warp.
 // With one species (kOne) every lane draws its own first block, without the
 // list, and only counts above four go on to it.  pre: the lane's thresholds
 // of species 0, when kPre says that they are loaded.
 template <bool kOne, bool kPre, class Big>
-__device__ __forceinline__ uint32_t draw_all(const ModelParams& mp, int S, int64_t T, const WarpMem& w,
-                                             const PeriodView& v, int t, int key, uint32_t present, uint32_t touched,
-                                             uint4 pre, Big big) {
+__device__ __forceinline__ uint32_t draw_all(int S, int64_t T, const WarpMem& w, const PeriodView& v, int t, int key,
+                                             uint32_t present, uint32_t touched, uint4 pre, Big big) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const uint32_t k0 = (uint32_t)v.seed, k1 = (uint32_t)(v.seed >> 32);
-    uint32_t drawn = 0;
+    auto draws_of = [&](int sp) -> int {
+        return ((touched >> sp) & 1u) ? w.D[32 * sp + lane] : w.N[32 * sp + lane];
+    };
+    // the species of each lane with draws of a usual number, and the others
+    uint32_t drawn = 0, heavy = 0;
+    for (uint32_t bits = present; bits; bits &= bits - 1u) {
+        const int sp = __ffs(bits) - 1;
+        const int n = draws_of(sp);
+        if (n > kCoopMin) heavy |= 1u << sp;
+        else if (n > 0) drawn |= 1u << sp;
+    }
+    uint32_t todo = drawn;
+    for (;;) {
+        const unsigned hm = __ballot_sync(kAllLanes, heavy != 0u);
+        if (hm == 0u) break;
+        const int src = __ffs(hm) - 1;
+        const int sp_own = heavy ? __ffs(heavy) - 1 : 0;
+        const int sp = __shfl_sync(kAllLanes, sp_own, src);
+        const int nn = __shfl_sync(kAllLanes, heavy ? draws_of(sp_own) : 0, src);
+        if (lane == src) heavy &= heavy - 1u;
+        if (nn >= (int)kMoleculeCut) {
+            if (lane == src) big(sp, nn);
+            __syncwarp();
+            continue;
+        }
+        const int tt = __shfl_sync(kAllLanes, t, src), kk = __shfl_sync(kAllLanes, key, src);
+        const uint4 C = __ldg(v.thr + ((int64_t)sp * T + tt) * v.thr_stride);
+        uint32_t a0 = 0, a1 = 0;
+        for (int blk = lane; 4 * blk < nn; blk += 32)
+            count_block(rdd::philox_block((uint32_t)blk, (uint32_t)kk, v.period,
+                                          (rdd::kPurposeDiffusion << 16) | (uint32_t)sp, k0, k1),
+                        min(4, nn - 4 * blk), C, a0, a1);
+        a0 = __reduce_add_sync(kAllLanes, a0);
+        a1 = __reduce_add_sync(kAllLanes, a1);
+        if (lane == src) {
+            w.acc0[32 * sp + lane] = a0;
+            w.acc1[32 * sp + lane] = a1;
+            drawn |= 1u << sp;
+        }
+    }
+    int sp = 0, n = 0, b = 0, nb = 0;
+    if (kOne && todo) {
+        n = draws_of(0);
+        uint32_t a0 = 0, a1 = 0;
+        const uint4 C = kPre ? pre : __ldg(v.thr + (int64_t)t * v.thr_stride);
+        count_block(rdd::philox_block(0u, (uint32_t)key, v.period, rdd::kPurposeDiffusion << 16, k0, k1), min(4, n), C,
+                    a0, a1);
+        w.acc0[lane] = a0;
+        w.acc1[lane] = a1;
+        nb = (n + 3) >> 2;
+        b = 1;
+    }
     int cnt = 0;
-    // species after species; one turn more flushes the list
-    for (int sp = 0; sp <= S; ++sp) {
-        int n = 0;
-        if (sp < S && mp.D[sp] != 0.0) {
-            if ((present >> sp) & 1u) {
-                n = ((touched >> sp) & 1u) ? w.D[32 * sp + lane] : w.N[32 * sp + lane];
-                if (n >= (int32_t)kMoleculeCut) {
-                    big(sp, n);
-                    n = 0;
-                }
-                if (n > 0) {
-                    uint32_t a0 = 0, a1 = 0;
-                    if (kOne && n <= kCoopMin) {
-                        const uint4 C = kPre ? pre : __ldg(v.thr + (int64_t)t * v.thr_stride);
-                        count_block(rdd::philox_block(0u, (uint32_t)key, v.period, rdd::kPurposeDiffusion << 16, k0, k1),
-                                    min(4, n), C, a0, a1);
-                    }
-                    w.acc0[32 * sp + lane] = a0;
-                    w.acc1[32 * sp + lane] = a1;
-                    drawn |= 1u << sp;
-                }
-            }
-            unsigned cm = __ballot_sync(kAllLanes, n > kCoopMin);
-            while (cm) {
-                const int src = __ffs(cm) - 1;
-                cm &= cm - 1u;
-                const int nn = __shfl_sync(kAllLanes, n, src);
-                const int tt = __shfl_sync(kAllLanes, t, src), kk = __shfl_sync(kAllLanes, key, src);
-                const uint4 C = __ldg(v.thr + ((int64_t)sp * T + tt) * v.thr_stride);
+    for (;;) {
+        if (!kOne && b >= nb && todo) {
+            sp = __ffs(todo) - 1;
+            todo &= todo - 1u;
+            n = draws_of(sp);
+            nb = (n + 3) >> 2;
+            b = 0;
+            w.acc0[32 * sp + lane] = 0u;
+            w.acc1[32 * sp + lane] = 0u;
+        }
+        const unsigned act = __ballot_sync(kAllLanes, b < nb);
+        if (b < nb)
+            w.list[cnt + __popc(act & lt)] =
+                (uint32_t)lane | ((uint32_t)(min(4, n - 4 * b) - 1) << 5) | ((uint32_t)sp << 7) | ((uint32_t)b << 11);
+        ++b;
+        cnt += __popc(act);
+        if (cnt >= 32 || (act == 0u && cnt > 0)) {
+            // one round: the last min(32, cnt) entries, one a lane
+            __syncwarp();
+            const int take = min(cnt, 32);
+            cnt -= take;
+            const bool mine = lane < take;
+            const uint32_t en = mine ? w.list[cnt + lane] : (uint32_t)lane;
+            const int owner = (int)(en & 31u);
+            const int tu = __shfl_sync(kAllLanes, t, owner), ku = __shfl_sync(kAllLanes, key, owner);
+            if (mine) {
+                const int su = kOne ? 0 : (int)((en >> 7) & 15u);
+                const uint4 C = __ldg(v.thr + ((int64_t)su * T + tu) * v.thr_stride);
                 uint32_t a0 = 0, a1 = 0;
-                for (int blk = lane; 4 * blk < nn; blk += 32)
-                    count_block(rdd::philox_block((uint32_t)blk, (uint32_t)kk, v.period,
-                                                  (rdd::kPurposeDiffusion << 16) | (uint32_t)sp, k0, k1),
-                                min(4, nn - 4 * blk), C, a0, a1);
-                a0 = __reduce_add_sync(kAllLanes, a0);
-                a1 = __reduce_add_sync(kAllLanes, a1);
-                if (lane == src) {
-                    w.acc0[32 * sp + lane] = a0;
-                    w.acc1[32 * sp + lane] = a1;
-                    n = 0;
-                }
+                count_block(rdd::philox_block(en >> 11, (uint32_t)ku, v.period,
+                                              (rdd::kPurposeDiffusion << 16) | (uint32_t)su, k0, k1),
+                            (int)((en >> 5) & 3u) + 1, C, a0, a1);
+                if (a0) atomicAdd(w.acc0 + 32 * su + owner, a0);
+                if (a1) atomicAdd(w.acc1 + 32 * su + owner, a1);
             }
+            __syncwarp();
         }
-        const int nb = (n + 3) >> 2;
-        for (int b = kOne ? 1 : 0;; ++b) {
-            const unsigned act = __ballot_sync(kAllLanes, b < nb);
-            if (b < nb)
-                w.list[cnt + __popc(act & lt)] =
-                    (uint32_t)lane | ((uint32_t)(min(4, n - 4 * b) - 1) << 5) | ((uint32_t)sp << 7) | ((uint32_t)b << 11);
-            cnt += __popc(act);
-            if (cnt >= 32 || (sp == S && cnt > 0)) {
-                // one round: the last min(32, cnt) entries, one a lane
-                __syncwarp();
-                const int take = min(cnt, 32);
-                cnt -= take;
-                const bool mine = lane < take;
-                const uint32_t en = mine ? w.list[cnt + lane] : (uint32_t)lane;
-                const int owner = (int)(en & 31u);
-                const int tu = __shfl_sync(kAllLanes, t, owner), ku = __shfl_sync(kAllLanes, key, owner);
-                if (mine) {
-                    const int su = (int)((en >> 7) & 15u);
-                    const uint4 C = __ldg(v.thr + ((int64_t)su * T + tu) * v.thr_stride);
-                    uint32_t a0 = 0, a1 = 0;
-                    count_block(rdd::philox_block(en >> 11, (uint32_t)ku, v.period,
-                                                  (rdd::kPurposeDiffusion << 16) | (uint32_t)su, k0, k1),
-                                (int)((en >> 5) & 3u) + 1, C, a0, a1);
-                    if (a0) atomicAdd(w.acc0 + 32 * su + owner, a0);
-                    if (a1) atomicAdd(w.acc1 + 32 * su + owner, a1);
-                }
-                __syncwarp();
-            }
-            if (act == 0u) break;
-        }
+        if (act == 0u) break;
     }
     return drawn;
 }
 
 // Steps 2 and 3 for the warp's tets: column N of each live lane holds its
-// counts.  After it N holds what stays; emit(sp, o) was called by a lane for
-// each species of which molecules leave (o: per face).  Bits of the species
-// whose count changed are added to *dirty.  With kDefer, a lane whose tet
-// needs the reaction phase leaves it undone and answers true in *deferred.
-// Returns error bits.  All lanes must call it.
+// counts and `pr` says which are not zero (all clear for a lane that is not
+// live); mask: the tet's reaction mask.  After it N and pr hold what stays;
+// emit(sp, o) was called by a lane for each species of which molecules leave
+// (o: per face).  Bits of the species whose count changed are added to
+// *dirty.  With kDefer, a lane whose tet needs the reaction phase leaves it
+// undone and answers true in *deferred.  Returns error bits.  All lanes must
+// call it.
 template <bool kOne, bool kReact, bool kDefer, bool kPre = false, class Emit>
 __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParams& mp, int S, const WarpMem& w,
-                                              const PeriodView& v, int t, bool live, uint32_t* dirty, bool* deferred,
-                                              uint32_t* err, Emit& emit, uint4 pre = make_uint4(0u, 0u, 0u, 0u)) {
+                                              const PeriodView& v, int t, bool live, uint32_t mask, Presence& pr,
+                                              uint32_t* dirty, bool* deferred, uint32_t* err, Emit& emit,
+                                              uint4 pre = make_uint4(0u, 0u, 0u, 0u)) {
     const int lane = threadIdx.x & 31;
     const int key = live ? key_of(m, t) : 0;
     uint32_t bad = 0, touched = 0;
     if (kReact) {
-        if (live) {
-            const uint32_t all = mp.has_mask ? m.mask[t] : 0xffffffffu;
-            const uint32_t on = all & mp.kpos;
-            const uint32_t poss = possible_in_column(mp, w.N + lane, S, on);
-            if (poss) {
-                const float2 avf = m.avv[t];
-                if (kDefer) {
-                    // only the first waiting time, by its bound
-                    float a0 = 0.0f;
-                    for (uint32_t bits = poss; bits; bits &= bits - 1u)
-                        a0 += propensity_f(mp, __ffs(bits) - 1, w.N + lane, avf);
-                    rdd::Stream st(v.seed, (uint32_t)key, v.period, rdd::kPurposeReaction, 0);
-                    const uint64_t y = 9007199254740991ull - st.bits53();
-                    const float need = a0 * v.tau_kf * 1.0001f * 1.0001f;
-                    *deferred = !(need < 3.0e38f) || !((float)(uint32_t)(y >> 29) * 5.9604644775390625e-08f >= need) ||
-                                (y >> 29) == 0ull;
-                    if (*deferred) live = false;
-                } else {
-                    uint32_t tch = 0;
-                    int r = react_fast(mp, S, key, v, on, poss, avf, w.N + lane, w.D + lane, w.acc0 + lane, &tch);
-                    if (r == kReactDoubt) {
-                        tch = react_exact(mp, key, v.period, v.tau_k, v.seed, m.vol[t], all, avf, w.N + lane,
-                                          w.D + lane, err);
-                        bad |= tch >> 16;
-                        tch &= 0xffffu;
-                    }
-                    *dirty |= tch;
-                    if (mp.rule != kRuleEnd) touched = tch;   // first order: the draw uses N(tau_k)
+        const uint32_t on = mask & mp.kpos;
+        const uint32_t poss = live ? possible_by_presence(mp, pr, S, on) : 0u;
+        if (poss) {
+            const float2 avf = __ldg(m.avv + t);
+            if (kDefer) {
+                // only the first waiting time, by its bound
+                float a0 = 0.0f;
+                for (uint32_t bits = poss; bits; bits &= bits - 1u)
+                    a0 += propensity_f(w.rx[__ffs(bits) - 1], w.N + lane, avf);
+                rdd::Stream st(v.seed, (uint32_t)key, v.period, rdd::kPurposeReaction, 0);
+                const uint64_t y = 9007199254740991ull - st.bits53();
+                const float need = a0 * v.tau_kf * 1.0001f * 1.0001f;
+                *deferred = !(need < 3.0e38f) || !((float)(uint32_t)(y >> 29) * 5.9604644775390625e-08f >= need) ||
+                            (y >> 29) == 0ull;
+                if (*deferred) pr = Presence{};
+            } else {
+                uint32_t tch = 0;
+                int r = react_fast(mp, w.rx, S, key, v, on, poss, avf, w.N + lane, w.D + lane, w.acc0 + lane, pr, &tch);
+                if (r == kReactDoubt) {
+                    tch = react_exact(mp, key, v.period, v.tau_k, v.seed, m.vol[t], mask, avf, w.N + lane, w.D + lane,
+                                      err);
+                    bad |= tch >> 16;
+                    tch &= 0xffffu;
+                    for (uint32_t bits = tch; bits; bits &= bits - 1u)
+                        pr.set(__ffs(bits) - 1, w.N[32 * (__ffs(bits) - 1) + lane]);
                 }
+                *dirty |= tch;
+                if (mp.rule != kRuleEnd) touched = tch;   // first order: the draw uses N(tau_k)
             }
         }
     }
-    uint32_t present = 0;
-    if (live)
-        for (int s = 0; s < S; ++s)
-            if (w.N[32 * s + lane] > 0) present |= 1u << s;
-    const uint32_t drawn = draw_all<kOne, kPre>(mp, S, m.T, w, v, t, key, present, touched, pre, [&](int sp, int32_t star) {
+    const uint32_t drawn = draw_all<kOne, kPre>(S, m.T, w, v, t, key, pr.any & mp.moves, touched, pre,
+                                                [&](int sp, int32_t star) {
         const int32_t Nt = w.N[32 * sp + lane];
         const int4 o = diffuse_binomial(m.G, m.g, t, key, sp, mp.D[sp], v.period, v.tau_k, v.seed, Nt, star);
         const int32_t all = o.x + o.y + o.z + o.w;
         if (all > 0) {
             w.N[32 * sp + lane] = Nt - all;
+            pr.set(sp, Nt - all);
             *dirty |= 1u << sp;
             emit(sp, o);
         }
@@ -485,7 +516,9 @@ __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParam
         if (o.x + o.y + o.z + o.w > Nt)
             o = draw_capped(v.seed, v.period, key, sp, w.D[32 * sp + lane], Nt,
                             __ldg(v.thr + ((int64_t)sp * m.T + t) * v.thr_stride));
-        w.N[32 * sp + lane] = Nt - (o.x + o.y + o.z + o.w);
+        const int32_t left = Nt - (o.x + o.y + o.z + o.w);
+        w.N[32 * sp + lane] = left;
+        pr.set(sp, left);
         *dirty |= 1u << sp;
         emit(sp, o);
     }

@@ -559,8 +559,8 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target,
 // 3,072-tet cube's took 10.2 us a launch and takes 6.5 here (217 periods, 2.21 ->
 // 1.40 ms; 48,000-tet A/B/C cube, 200 periods, 2.91 -> 2.20 ms).  Ends with the closing transfer, all
 // inbox words and masks cleared.
-template <int S_, bool kReact>
-__global__ void __launch_bounds__(kBlock, 3)
+template <int S_, bool kReact, int kBlocks>
+__global__ void __launch_bounds__(kBlock, kBlocks)
 k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp, DevState s,
       const __grid_constant__ RunArgs r) {
     extern __shared__ int32_t sm[];
@@ -619,6 +619,9 @@ k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp,
 // Warps a block and blocks of k_run for T tets, or 0 if they do not fit: the
 // 32-tet warps are spread over all SMs first (a warp that has an SM's issue
 // slots and caches to itself is fastest), in at most 3 blocks of 8 warps an SM.
+// Up to 2 blocks an SM (77,824 tets on 152 SMs) the kernel has 128 registers,
+// above it 80 (eleven species on 12,870 tets, 60 periods: 1.27 ms with 128,
+// 1.36 with 80; 3,072-tet cube, 217 periods, 1.30 and 1.47).
 int run_shape(int64_t T, int sms, int* warps) {
     const int64_t chunks = (T + 31) / 32;
     const int64_t per_sm = (chunks + sms - 1) / sms;
@@ -628,10 +631,10 @@ int run_shape(int64_t T, int sms, int* warps) {
     return (int)((chunks + *warps - 1) / *warps);
 }
 
-template <int S_, bool kReact>
-cudaError_t launch_run_s(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int grid,
+template <int S_, bool kReact, int kBlocks>
+cudaError_t launch_run_b(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int grid,
                          int warps, int sms, cudaStream_t st) {
-    auto kern = k_run<S_, kReact>;
+    auto kern = k_run<S_, kReact, kBlocks>;
     const size_t smem = (size_t)warps * warp_words(mp.S, kReact) * sizeof(int32_t);
     if (smem > 48u * 1024u)
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -647,6 +650,13 @@ cudaError_t launch_run_s(const DevMesh& m, const ModelParams& mp, const DevState
     ce = cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(32 * warps), args, smem, st);
     if (ce == cudaSuccess) ++g_launches;
     return ce;
+}
+
+template <int S_, bool kReact>
+cudaError_t launch_run_s(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int grid,
+                         int warps, int sms, cudaStream_t st) {
+    if (grid <= 2 * sms) return launch_run_b<S_, kReact, 2>(m, mp, s, r, grid, warps, sms, st);
+    return launch_run_b<S_, kReact, 3>(m, mp, s, r, grid, warps, sms, st);
 }
 
 bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int sms, int* grid,

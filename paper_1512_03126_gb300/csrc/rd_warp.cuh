@@ -115,15 +115,21 @@ enum : int { kReactNone = 0, kReactDone = 1, kReactDoubt = 2 };
 // error does not grow with the counts.
 //
 // Bounds, in units of e = 2^-24 (the reference values are the double-precision
-// ones, whose own error is below 1e-12 of these): propensities 8, their sum
-// (at most 32 terms) 39, -log u1 by log1pf or logf (1 ulp each, condition
-// at most 1.45) 4, times tau and divided 3; so a waiting time is off by at
-// most 46 e of itself and, with one rounding per event, an event time by
-// (46 + k) e after k events.  Every comparison with tau_k or tau_k / 2 keeps
-// (128 + 4 k) e away from its limit, the choice of the reaction 128 e of the
-// total propensity, and the rounding of N-bar (256 + 8 k) e per molecule made
-// or consumed (+ 2^-20 for the double-precision sums of counts below 2^20);
-// inside a margin the function undoes its changes and answers kReactDoubt.
+// ones, whose own error is below 1e-10 of these), with m the largest number of
+// possible reactions met: propensities 8, their sum m - 1 more; -log u1 8: by
+// log1pf (1 ulp) of u1 - 1 above one half (condition at most 1.45), else of its
+// mantissa beside exponent times ln 2; times tau 2, __fdividef 4 (2 ulp).  So a
+// waiting time is off by at most (21 + m) e of itself and, with one rounding
+// per event, an event time by (21 + m + k) e after k events.  Comparisons with
+// tau_k or tau_k / 2 keep (26 + m + 2 k) e away from their limit, the choice of
+// the reaction (22 + 2 m) e of the total propensity (twice the sum's error,
+// and two roundings of the target), and the rounding of N-bar (30 + m + 3 k) e
+// per molecule made or consumed + 4 e (event times, products, the k sums, and
+// u) + 2^-20 (the double-precision sums, for counts below 2^20); inside a
+// margin the function undoes its changes and answers kReactDoubt.  The margins
+// matter for speed: at 128, 128 and 256 e one of the 68,034 tets of a
+// six-species box met one in most periods, and its double-precision repeat set
+// the period (29 us).
 // Waiting times beyond the period are first ruled out by -log u >= 1 - u
 // without a logarithm.
 // Replaces a double-precision chain of one logarithm (24 dependent operations
@@ -141,27 +147,37 @@ __device__ __forceinline__ int react_fast(const ModelParams& mp, const uint2* rx
     const uint32_t k0 = (uint32_t)v.seed, k1 = (uint32_t)(v.seed >> 32);
     float x = 0.0f, dsum = 0.0f;
     uint32_t touched = 0;
-    int k = 0;
+    int k = 0, m = 0;
+    // block k of the tet's reaction stream: u1 and u2 of event k; the next one
+    // is drawn beside the waiting time, off the chain from event to event
+    uint4 rw = rdd::philox_block(0u, (uint32_t)key, v.period, rdd::kPurposeReaction << 16, k0, k1);
     bool past = false, doubt = !(v.tau_kf < 1e6f);   // (keeps underflowed rates below 1e-13 a period)
     while (!doubt) {
         if (k > 0) poss = possible_by_presence(mp, pr, S, on);
         if (!poss) break;                          // total propensity 0
-        // block k of the tet's reaction stream: u1 and u2 of event k
-        const uint4 rw = rdd::philox_block((uint32_t)k, (uint32_t)key, v.period, rdd::kPurposeReaction << 16, k0, k1);
         const uint64_t x1 = ((uint64_t)(rw.x >> 5) << 26) | (rw.y >> 6);
         float a0 = 0.0f;
         for (uint32_t bits = poss; bits; bits &= bits - 1u) a0 += propensity_f(rx[__ffs(bits) - 1], Ncol, avf);
         const float at = a0 * v.tau_kf;
-        const float eps = (float)(128 + 4 * k) * e;
+        m = max(m, __popc(poss));
+        const float eps = (float)(26 + m + 2 * k) * e;
         const uint64_t y = 9007199254740991ull - x1;                    // (1 - u1) 2^53
         const float ylo = (float)(uint32_t)(y >> 29) * e;               // at most 1 - u1
         if (!(at < 1e30f)) { doubt = true; break; }
         if (ylo > 0.0f && ylo >= at * ((1.0f + eps) - x) * 1.0001f) break;   // no event before tau_k
         if (!(at > 1e-6f)) { doubt = true; break; }
-        float E;
-        if (y <= 4503599627370496ull) E = -log1pf(-(float)y * 1.1102230246251565e-16f);
-        else E = -logf((float)(x1 + 1ull) * 1.1102230246251565e-16f);
-        const float xn = x + E / at;
+        const uint4 rw_next =
+            rdd::philox_block((uint32_t)(k + 1), (uint32_t)key, v.period, rdd::kPurposeReaction << 16, k0, k1);
+        float arg = -(float)y * 1.1102230246251565e-16f, ex = 0.0f;     // u1 - 1
+        if (y > 4503599627370496ull) {
+            // u1 = 2^ex (1 + arg) below one half, arg in [-0.3, 0.42)
+            const uint32_t ub = __float_as_uint((float)(x1 + 1ull) * 1.1102230246251565e-16f);
+            const int ei = (int)((ub + 0x4afb0du) >> 23) - 127;
+            ex = (float)ei;
+            arg = __uint_as_float(ub - ((uint32_t)ei << 23)) - 1.0f;
+        }
+        const float E = -(log1pf(arg) + ex * 0.693147182f);
+        const float xn = x + __fdividef(E, at);
         if (xn >= 1.0f + eps) break;
         if (xn > 1.0f - eps) { doubt = true; break; }
         if (mid && !past) {
@@ -175,7 +191,7 @@ __device__ __forceinline__ int react_fast(const ModelParams& mp, const uint2* rx
         }
         // the first reaction whose cumulated propensity exceeds u2 a0
         const float target = (float)(((uint64_t)(rw.z >> 5) << 26) | (rw.w >> 6)) * 1.1102230246251565e-16f * a0;
-        const float margin = 128.0f * e * a0;
+        const float margin = (float)(22 + 2 * m) * e * a0;
         int mu = -1;
         float cum = 0.0f;
         for (uint32_t bits = poss; bits; bits &= bits - 1u) {
@@ -203,10 +219,11 @@ __device__ __forceinline__ int react_fast(const ModelParams& mp, const uint2* rx
         }
         dsum += dmax;
         x = xn;
+        rw = rw_next;
         if (++k > kMaxEvents) doubt = true;
     }
     if (!doubt && touched) {
-        const float eps = dsum * ((float)(256 + 8 * k) * e) + 9.5367431640625e-07f;
+        const float eps = dsum * ((float)(30 + m + 3 * k) * e) + (4.0f * e + 9.5367431640625e-07f);
         for (uint32_t bits = touched; bits; bits &= bits - 1u) {
             const int s = __ffs(bits) - 1;
             if (mid) {
@@ -232,36 +249,103 @@ __device__ __forceinline__ int react_fast(const ModelParams& mp, const uint2* rx
     return touched ? kReactDone : kReactNone;
 }
 
-// The same phase by the double-precision definition, for a tet whose
-// single-precision pass met a decision inside its error bound (or counts or
-// event numbers beyond it).  Returns the touched species, error bits in the
-// upper half.
+// The same phase by the double-precision definition (Algorithm 1, Step 2 and
+// 2.1: the first event at or past tau_k is discarded; before a species' count
+// changes, its occupancy integral advances by N * (t_event - t_last); under
+// the half-step rule N* is the count at tau_k / 2, that after every event
+// before it), for a tet whose single-precision pass met a decision inside its
+// error bound, or counts or event numbers beyond it.  Only reactions whose
+// reactants are present are evaluated (the others add exact zeros), each rate
+// constant once.  Returns the touched species, error bits in the upper half.
 static __device__ __noinline__ uint32_t react_exact(const ModelParams& mp, int key, uint32_t period, double tau_k,
-                                                    uint64_t seed, double vol_t, uint32_t on, float2 avf,
-                                                    int32_t* Ncol, int32_t* Dcol, uint32_t* err) {
-    int64_t N64[kMaxS], nmid[kMaxS];
-    double occ[kMaxS], tl[kMaxS];
-    for (int s = 0; s < mp.S; ++s) {
-        N64[s] = Ncol[32 * s];
+                                                    uint64_t seed, double vol_t, uint32_t on, int32_t* Ncol,
+                                                    int32_t* Dcol, uint32_t* err) {
+    const double avv = kAvogadro * (vol_t * 1000.0);
+    const bool want_mid = mp.rule == kRuleMid;
+    const double half = 0.5 * tau_k;
+    const int S = mp.S;
+    int64_t N[kMaxS], nmid[kMaxS];
+    double occ[kMaxS], tl[kMaxS], c[kMaxR], a[kMaxR];
+    for (int s = 0; s < S; ++s) {
+        N[s] = Ncol[32 * s];
         occ[s] = 0.0;
         tl[s] = 0.0;
     }
-    uint32_t touched = 0, bad = 0;
-    react_tet(mp, key, period, tau_k, seed, vol_t, on, avf, N64, occ, tl, touched, nmid, err);
-    for (int s = 0; s < mp.S; ++s) {
-        if (!((touched >> s) & 1u)) continue;
-        int64_t n = N64[s];
-        if (n < 0) { bad |= kErrNegative; n = 0; }
-        if (n > 2147483647) { bad |= kErrOverflow; n = 2147483647; }
-        Ncol[32 * s] = (int32_t)n;
-        int64_t star = nmid[s];
-        if (mp.rule != kRuleMid) {
+    uint32_t touched = 0, bad = 0, have = 0;
+    bool past_half = false;
+    rdd::Stream st(seed, (uint32_t)key, period, rdd::kPurposeReaction, 0);
+    double tc = 0.0;
+    for (int events = 0;;) {
+        uint32_t poss = on & mp.kpos;
+        for (int s = 0; s < S; ++s) {
+            if (N[s] <= 0) poss &= ~mp.needs[s];
+            else if (N[s] == 1) poss &= ~mp.needs2[s];
+        }
+        if (!poss) break;                          // a0 = 0
+        // propensity a_r = c_r h_r, h_r the number of reactant combinations
+        double a0 = 0.0;
+        for (uint32_t bits = poss; bits; bits &= bits - 1u) {
+            const int r = __ffs(bits) - 1, a1 = mp.rs1[r], a2 = mp.rs2[r];
+            if (!((have >> r) & 1u)) {
+                const double kr = mp.k[r];
+                const int o = mp.order[r];
+                c[r] = o == 0 ? kr * avv : (o == 1 ? kr : kr / avv);
+                have |= 1u << r;
+            }
+            int64_t h = 1;
+            if (a1 >= 0) {
+                if (a2 < 0) h = N[a1];
+                else if (a1 == a2) h = N[a1] * (N[a1] - 1) / 2;
+                else h = N[a1] * N[a2];
+            }
+            a[r] = c[r] * (double)h;
+            a0 = a0 + a[r];
+        }
+        if (!(a0 > 0.0)) break;
+        const double tn = tc + (-rdd::own_log(st.u01_open0())) / a0;
+        if (tn >= tau_k) break;
+        if (want_mid && !past_half && tn >= half) {
+            for (int s = 0; s < S; ++s) nmid[s] = N[s];
+            past_half = true;
+        }
+        const double target = st.u01() * a0;
+        int mu = -1, positive = -1;
+        double cum = 0.0;
+        for (uint32_t bits = poss; bits; bits &= bits - 1u) {
+            const int r = __ffs(bits) - 1;
+            cum = cum + a[r];
+            if (a[r] > 0.0) positive = r;
+            if (target < cum) { mu = r; break; }
+        }
+        if (mu < 0) mu = positive;
+        for (uint32_t bits = mp.rx[mu].y >> 16; bits; bits &= bits - 1u) {
+            const int s = __ffs(bits) - 1;
+            occ[s] = occ[s] + (double)N[s] * (tn - tl[s]);
+            tl[s] = tn;
+            touched |= 1u << s;
+            N[s] += mp.delta[mu][s];
+        }
+        tc = tn;
+        if (++events >= kEventCap) { atomicOr(err, kErrEventCap); break; }
+    }
+    if (want_mid && !past_half)
+        for (int s = 0; s < S; ++s) nmid[s] = N[s];
+    for (uint32_t bits = touched; bits; bits &= bits - 1u) {
+        const int s = __ffs(bits) - 1;
+        int64_t n = N[s], star = 0;
+        if (want_mid) {
+            star = nmid[s];
+        } else {
+            occ[s] = occ[s] + (double)N[s] * (tau_k - tl[s]);
             rdd::Stream rs(seed, (uint32_t)key, period, rdd::kPurposeRounding, (uint32_t)s);
             const double nbar = occ[s] / tau_k;
             const double fl = floor(nbar);
             star = (int64_t)fl + (rs.u01() < nbar - fl ? 1 : 0);
         }
+        if (n < 0) { bad |= kErrNegative; n = 0; }
+        if (n > 2147483647) { bad |= kErrOverflow; n = 2147483647; }
         if (star > 2147483647) star = 2147483647;
+        Ncol[32 * s] = (int32_t)n;
         Dcol[32 * s] = (int32_t)star;
     }
     return touched | (bad << 16);
@@ -368,8 +452,8 @@ __device__ __forceinline__ uint32_t draw_all(int S, int64_t T, const WarpMem& w,
         const unsigned hm = __ballot_sync(kAllLanes, heavy != 0u);
         if (hm == 0u) break;
         const int src = __ffs(hm) - 1;
-        const int sp_own = heavy ? __ffs(heavy) - 1 : 0;
-        const int sp = __shfl_sync(kAllLanes, sp_own, src);
+        const int sp_own = !kOne && heavy ? __ffs(heavy) - 1 : 0;
+        const int sp = kOne ? 0 : __shfl_sync(kAllLanes, sp_own, src);
         const int nn = __shfl_sync(kAllLanes, heavy ? draws_of(sp_own) : 0, src);
         if (lane == src) heavy &= heavy - 1u;
         if (nn >= (int)kMoleculeCut) {
@@ -483,8 +567,7 @@ __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParam
                 uint32_t tch = 0;
                 int r = react_fast(mp, w.rx, S, key, v, on, poss, avf, w.N + lane, w.D + lane, w.acc0 + lane, pr, &tch);
                 if (r == kReactDoubt) {
-                    tch = react_exact(mp, key, v.period, v.tau_k, v.seed, m.vol[t], mask, avf, w.N + lane, w.D + lane,
-                                      err);
+                    tch = react_exact(mp, key, v.period, v.tau_k, v.seed, m.vol[t], mask, w.N + lane, w.D + lane, err);
                     bad |= tch >> 16;
                     tch &= 0xffffu;
                     for (uint32_t bits = tch; bits; bits &= bits - 1u)

@@ -294,7 +294,7 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
                                 n[k] = 0;
                             }
                             w.N[32 * (s0 + k) + lane] = n[k];
-                            pr.set(s0 + k, n[k]);
+                            pr.add(s0 + k, n[k]);
                             if (kReact) held += n[k];
                         }
                     }

@@ -58,8 +58,14 @@ __global__ void k_mesh_setup(int32_t T, const int32_t* __restrict__ adj, const d
                              const double* __restrict__ area, const double* __restrict__ dist,
                              int4* __restrict__ src, double* __restrict__ g, double* __restrict__ G,
                              unsigned long long* gmax_bits, uint32_t* err) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
+    // the block's largest G first: one atomic a tet on one address took 1.4 of
+    // this kernel's 1.55 ms on 2.4 M tets
+    __shared__ unsigned long long block_max;
+    if (threadIdx.x == 0) block_max = 0ull;
+    __syncthreads();
+    const int t_ = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool live = t_ < T;
+    const int t = live ? t_ : T - 1;   // a lane past the end repeats the last tet, stores nothing
     uint32_t e = 0;
     double V = vol[t];
     if (!(V > 0.0) || !(V < HUGE_VAL)) e |= kErrVolume;
@@ -88,11 +94,22 @@ __global__ void k_mesh_setup(int32_t T, const int32_t* __restrict__ adj, const d
         }
         Gt = Gt + gf[f];
     }
-    src[t] = make_int4(s4[0], s4[1], s4[2], s4[3]);
-    for (int f = 0; f < 4; ++f) g[4 * t + f] = gf[f];
-    G[t] = Gt;
-    if (e) atomicOr(err, e);
-    else if (Gt < HUGE_VAL) atomicMax(gmax_bits, (unsigned long long)__double_as_longlong(Gt));
+    if (live) {
+        src[t] = make_int4(s4[0], s4[1], s4[2], s4[3]);
+        for (int f = 0; f < 4; ++f) g[4 * t + f] = gf[f];
+        G[t] = Gt;
+        if (e) atomicOr(err, e);
+    }
+    // G >= 0: bit order is value order
+    unsigned long long b = e == 0 && Gt < HUGE_VAL ? (unsigned long long)__double_as_longlong(Gt) : 0ull;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, b, d);
+        b = o > b ? o : b;
+    }
+    if ((threadIdx.x & 31) == 0 && b) atomicMax(&block_max, b);
+    __syncthreads();
+    if (threadIdx.x == 0 && block_max) atomicMax(gmax_bits, block_max);
 }
 
 void launch_mesh_setup(int32_t T, const int32_t* adj, const double* vol, const double* area,
@@ -170,15 +187,32 @@ static __device__ __noinline__ uint4 thresholds_by_definition(double tau_k, doub
     return make_uint4(C[0], C[1], C[2], C[3]);
 }
 
+// A positive double as hi + lo in single precision: its first 24 bits and the
+// 29 after them (lo rounded: off by at most 2^-24 of itself, 2^-48 of the
+// value).  By integer operations, since FP64 conversions run at FP64 speed.
+// hi is 0 or within (2^-100, 2^100), else *ok is cleared.
+__device__ __forceinline__ float2 split_double(double x, bool* ok) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int ex = (int)(b >> 52) - 1023;
+    if (b == 0ull) return make_float2(0.0f, 0.0f);
+    *ok = *ok && ex > -100 && ex < 100;
+    const uint32_t hi = ((uint32_t)(ex + 127) << 23) | ((uint32_t)(b >> 29) & 0x7fffffu);
+    const float unit = __uint_as_float((uint32_t)(ex - 52 + 127 > 0 ? ex - 52 + 127 : 1) << 23);
+    *ok = *ok && ex - 52 + 127 > 0;
+    return make_float2(__uint_as_float(hi), (float)((uint32_t)b & 0x1fffffffu) * unit);
+}
+
 // One tet a thread, all species.  Below zeta = 1 the G's cancel: 2^32 zeta
-// cum_f / G = (2^32 tau D) cum_f, off by at most 6 * 2^-53 of itself from the
-// definition's value (its five roundings and one here), so by less than
-// 2^-18.  Its floor is the definition's unless it lies within 4 * 2^-20 of a
-// whole number (8 are kept); such a face (one in 65,536), and every tet whose zeta is not
-// clearly below 1, takes the definition's operations.  FP64 (64 cycles an
-// operation, 562 a division) is what bounds this kernel: two operations a
-// face instead of a division and four.  2.4 M tets of 8 species: 2060 us with
-// one thread a (species, tet) and the divisions.
+// cum_f / G = (2^32 tau D) cum_f, in exact arithmetic; the definition's five
+// roundings move it by at most 6 * 2^-53 of itself.  The product of the two
+// factors' float pairs is off by at most 2^-45 of itself (2^-48 from each
+// split, 2^-48 for the dropped lo lo, 3 * 2^-48 in the two sums), so by 2^-13
+// at most: its floor is the definition's unless it lies within 2^-12 of a
+// whole number.  Such a face (one in 2,048), and every tet whose zeta is not
+// clearly below 1, takes the definition's operations.  2.4 M tets of 8 species
+// (403 MB, 59 us at the copy rate): 2060 us with one thread a (species, tet)
+// and FP64 divisions (64 cycles an FP64 operation, 562 a division), 467 with
+// one FP64 product and conversion a face.
 __global__ void k_thresholds(int32_t T, const __grid_constant__ ModelParams mp, const double* __restrict__ g,
                              const double* __restrict__ G, double tau_k, uint4* __restrict__ thr) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -190,22 +224,28 @@ __global__ void k_thresholds(int32_t T, const __grid_constant__ ModelParams mp, 
     cum[1] = cum[0] + g01.y;
     cum[2] = cum[1] + g23.x;
     cum[3] = cum[2] + g23.y;
-    const double Gt = G[t];
+    bool ok = true;
+    float2 c[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) c[f] = split_double(cum[f], &ok);
     for (int s = 0; s < mp.S; ++s) {
-        const double scale = tau_k * mp.D[s] * 4503599627370496.0;   // 2^52 tau D
+        bool sure = ok;
+        const float2 sc = split_double(tau_k * mp.D[s] * 4294967296.0, &sure);   // 2^32 tau D
         uint32_t C[4];
-        // 2^52 zeta, clearly below 2^52 (and finite)
-        bool sure = scale * Gt < 4503599627370496.0 * 0.999;
 #pragma unroll
         for (int f = 0; f < 4; ++f) {
-            const unsigned long long y = (unsigned long long)(scale * cum[f]);   // 2^20 units of a threshold step
-            const uint32_t frac = (uint32_t)y & 0xfffffu;
-            sure = sure && (y == 0ull || frac - 8u < 0xfffffu - 16u);
-            C[f] = (uint32_t)(y >> 20);
+            const float p = c[f].x * sc.x;
+            const float r = __fmaf_rn(c[f].x, sc.y, __fmaf_rn(c[f].y, sc.x, __fmaf_rn(c[f].x, sc.x, -p)));
+            const float whole = floorf(p);
+            const float rest = (p - whole) + r;
+            const float fl = floorf(rest);
+            const float frac = rest - fl;
+            sure = sure && p < 4294967296.0f * 0.999f && (p == 0.0f || (frac > 2.44140625e-4f && frac < 1.0f - 2.44140625e-4f));
+            C[f] = (uint32_t)whole + (uint32_t)(int)fl;
         }
-        uint4 c = make_uint4(C[0], C[1], C[2], C[3]);
-        if (!sure) c = thresholds_by_definition(tau_k, mp.D[s], Gt, cum);
-        thr[(int64_t)s * T + t] = c;
+        uint4 v = make_uint4(C[0], C[1], C[2], C[3]);
+        if (!sure) v = thresholds_by_definition(tau_k, mp.D[s], G[t], cum);
+        thr[(int64_t)s * T + t] = v;
     }
 }
 
@@ -455,7 +495,7 @@ enum { kPassAll = 0, kPassFirst = 1, kPassQueue = 2 };
 // tet reads or writes them) and are written back where they changed.
 // S_ > 0 fixes the species count at compile time.
 template <int S_, bool kReact, int kPass>
-__global__ void __launch_bounds__(kBlock, kPass == kPassFirst ? 4 : 3)
+__global__ void __launch_bounds__(kBlock, S_ == 1 ? 3 : (kPass == kPassAll ? 5 : 4))
 k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp, DevState s,
          const __grid_constant__ PeriodArgs a, int32_t* __restrict__ queue, int32_t* qcount, int32_t parity) {
     extern __shared__ int32_t sm[];
@@ -489,7 +529,7 @@ k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams 
                 for (int k = 0; k < 8; ++k)
                     if (s0 + k < S) {
                         w.N[32 * (s0 + k) + lane] = n[k];
-                        pr.set(s0 + k, n[k]);
+                        pr.add(s0 + k, n[k]);
                     }
             }
             if (kPass != kPassQueue && !a.first) bad |= take_inbox(a, t, S, lane, w.N, pr, &dirty);
@@ -584,7 +624,7 @@ k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp,
         for (int sp = 0; sp < S; ++sp) {
             const int32_t n = s.cnt[sp * T + t];
             w.N[32 * sp + lane] = n;
-            pr.set(sp, n);
+            pr.add(sp, n);
         }
     uint32_t bad = 0, dirty = 0, target = r.barrier_base;
     for (int q = 0; q <= r.periods; ++q) {

@@ -70,20 +70,30 @@ struct PeriodView {
     int thr_stride;
 };
 
-// Which species of a lane's tet have molecules, and which more than one: kept
-// beside the column, so that loops run over set bits only.
+// Which species of a lane's tet have molecules, which more than one and which
+// more than kCoopMin: kept beside the column, so that loops run over set bits
+// only.
 struct Presence {
-    uint32_t any = 0, two = 0;
+    uint32_t any = 0, two = 0, many = 0;
+    // a species not seen before
+    __device__ __forceinline__ void add(int s, int32_t n) {
+        if (n > 0) any |= 1u << s;
+        if (n > 1) two |= 1u << s;
+        if (n > kCoopMin) many |= 1u << s;
+    }
     __device__ __forceinline__ void set(int s, int32_t n) {
         const uint32_t bit = 1u << s;
-        any = n > 0 ? any | bit : any & ~bit;
-        two = n > 1 ? two | bit : two & ~bit;
+        any &= ~bit;
+        two &= ~bit;
+        many &= ~bit;
+        add(s, n);
     }
 };
 
 // Reactions of `on` whose reactants are present.
 __device__ __forceinline__ uint32_t possible_by_presence(const ModelParams& mp, const Presence& pr, int S, uint32_t on) {
     uint32_t m = on;
+#pragma unroll 4
     for (int s = 0; s < S; ++s) {
         if (!((pr.any >> s) & 1u)) m &= ~mp.needs[s];
         if (!((pr.two >> s) & 1u)) m &= ~mp.needs2[s];
@@ -432,7 +442,7 @@ __device__ __forceinline__ void count_block(const uint4& w, int m, const uint4& 
 // of species 0, when kPre says that they are loaded.
 template <bool kOne, bool kPre, class Big>
 __device__ __forceinline__ uint32_t draw_all(int S, int64_t T, const WarpMem& w, const PeriodView& v, int t, int key,
-                                             uint32_t present, uint32_t touched, uint4 pre, Big big) {
+                                             uint32_t present, uint32_t many, uint32_t touched, uint4 pre, Big big) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const uint32_t k0 = (uint32_t)v.seed, k1 = (uint32_t)(v.seed >> 32);
@@ -440,13 +450,14 @@ __device__ __forceinline__ uint32_t draw_all(int S, int64_t T, const WarpMem& w,
         return ((touched >> sp) & 1u) ? w.D[32 * sp + lane] : w.N[32 * sp + lane];
     };
     // the species of each lane with draws of a usual number, and the others
-    uint32_t drawn = 0, heavy = 0;
-    for (uint32_t bits = present; bits; bits &= bits - 1u) {
+    uint32_t heavy = present & many;
+    for (uint32_t bits = touched & present; bits; bits &= bits - 1u) {
         const int sp = __ffs(bits) - 1;
-        const int n = draws_of(sp);
-        if (n > kCoopMin) heavy |= 1u << sp;
-        else if (n > 0) drawn |= 1u << sp;
+        const int n = w.D[32 * sp + lane];
+        heavy = n > kCoopMin ? heavy | 1u << sp : heavy & ~(1u << sp);
+        if (n <= 0) present &= ~(1u << sp);
     }
+    uint32_t drawn = present & ~heavy;
     uint32_t todo = drawn;
     for (;;) {
         const unsigned hm = __ballot_sync(kAllLanes, heavy != 0u);
@@ -578,7 +589,7 @@ __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParam
             }
         }
     }
-    const uint32_t drawn = draw_all<kOne, kPre>(S, m.T, w, v, t, key, pr.any & mp.moves, touched, pre,
+    const uint32_t drawn = draw_all<kOne, kPre>(S, m.T, w, v, t, key, pr.any & mp.moves, pr.many, touched, pre,
                                                 [&](int sp, int32_t star) {
         const int32_t Nt = w.N[32 * sp + lane];
         const int4 o = diffuse_binomial(m.G, m.g, t, key, sp, mp.D[sp], v.period, v.tau_k, v.seed, Nt, star);

@@ -13,6 +13,7 @@
 //                  the tets whose reactions have to run in the second
 //   k_run          many periods in one cooperative launch, for a mesh whose
 //                  tets are all resident at once
+//   k_run_cluster  the same within one thread-block cluster, for small meshes
 //   k_gather       the closing synchronous transfer of a run
 //
 // Layout: counts are species-major int32 [S][T] (coalesced), updated in
@@ -656,6 +657,203 @@ k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp,
     if (bad) atomicOr(s.err, bad);
 }
 
+// The same for a mesh that one thread-block cluster holds: inboxes and masks
+// live in the cluster's shared memory, leavers are stores into the neighbour
+// tet's CTA, and the hardware cluster barrier takes the place of the grid
+// barrier, its memory fence and the polling of a counter in L2 (3 to 4 us of a
+// period together).
+__device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t cta) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(cta));
+    return r;
+}
+
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Leavers into the words of neighbours' slots; face f's slot is number
+// slot & 0xfff of CTA slot >> 12 (none: 0xffffffff).
+struct ClusterSender {
+    uint32_t slot[4];
+    uint32_t words, masks;      // shared addresses of this parity's words and masks
+    int S;
+    uint64_t bits;
+
+    __device__ __forceinline__ void operator()(int sp, const int4& o) {
+        const int n[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            if (n[f] <= 0 || slot[f] == 0xffffffffu) continue;
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
+                             map_to_cta(words + ((slot[f] & 0xfffu) * S + sp) * 4u, slot[f] >> 12)), "r"(n[f]) : "memory");
+            bits |= 1ull << (16 * f + sp);
+        }
+    }
+    __device__ __forceinline__ void finish() {
+        if (S <= 2 || bits == 0) return;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            const uint32_t b = (uint32_t)(bits >> (16 * f)) & 0xffffu;
+            if (b == 0u || slot[f] == 0xffffffffu) continue;
+            asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(
+                             map_to_cta(masks + (slot[f] & 0xfffu) * 2u, slot[f] >> 12)), "h"((uint16_t)b) : "memory");
+        }
+    }
+};
+
+// Dynamic shared memory of a CTA of `warps` warps, in words: the warps'
+// (rd_warp.cuh), then per tet two parities of four slots of S words and of
+// four 16-bit masks.
+__host__ __device__ inline int cluster_words(int S, bool react, int warps) {
+    return warps * warp_words(S, react) + 32 * warps * (8 * S + 4);
+}
+
+template <int S_, bool kReact>
+__global__ void __launch_bounds__(512, 1)
+k_run_cluster(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp, DevState s,
+              const __grid_constant__ RunArgs r) {
+    extern __shared__ __align__(16) int32_t sm[];
+    const int S = S_ > 0 ? S_ : mp.S;
+    const int lane = threadIdx.x & 31;
+    const int warps = blockDim.x >> 5, B = blockDim.x;
+    __shared__ uint2 rx[kReact ? kMaxR : 1];
+    const WarpMem w(sm + (threadIdx.x >> 5) * warp_words(S, kReact), S, kReact, rx);
+    if (kReact)
+        for (int i = threadIdx.x; i < kMaxR; i += B) rx[i] = mp.rx[i];
+    int32_t* words = sm + warps * warp_words(S, kReact);                      // [2][B][4][S]
+    unsigned long long* masks = reinterpret_cast<unsigned long long*>(words + 8 * S * B);   // [2][B]
+    for (int i = threadIdx.x; i < 8 * S * B; i += B) words[i] = 0;
+    for (int i = threadIdx.x; i < 2 * B; i += B) masks[i] = 0ull;
+    // Warp w of the cluster's W takes tets w, w + W, w + 2 W, ...: a compact
+    // cloud's crowded tets go to different warps (a warp's 32 consecutive tets
+    // around a point source made all others wait: 3,072-tet cube 4.7 us a
+    // period).
+    const int64_t T = m.T;
+    const int W = gridDim.x * warps;
+    const int64_t tt = (int64_t)lane * W + blockIdx.x * warps + (threadIdx.x >> 5);
+    const bool live = tt < T;
+    const int t = live ? (int)tt : 0;
+    Presence pr;
+    const uint32_t mask = kReact && mp.has_mask && live ? __ldg(m.mask + t) : 0xffffffffu;
+    ClusterSender send;
+    send.S = S;
+    {
+        const int4 sr = live ? __ldg(m.src + t) : make_int4(-1, -1, -1, -1);
+        const int f4[4] = {sr.x, sr.y, sr.z, sr.w};
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            send.slot[f] = 0xffffffffu;
+            if (f4[f] < 0) continue;
+            const int u = f4[f] >> 2, wu = u % W;   // its warp, and thread of the CTA
+            send.slot[f] = (uint32_t)(wu / warps) << 12 | (uint32_t)(((wu % warps) * 32 + u / W) * 4 + (f4[f] & 3));
+        }
+    }
+    if (live)
+        for (int sp = 0; sp < S; ++sp) {
+            const int32_t n = s.cnt[sp * T + t];
+            w.N[32 * sp + lane] = n;
+            pr.add(sp, n);
+        }
+    uint32_t bad = 0, dirty = 0;
+    cluster_sync_all();   // every CTA's words and masks are zero
+    const uint32_t words_at = (uint32_t)__cvta_generic_to_shared(words);
+    const uint32_t masks_at = (uint32_t)__cvta_generic_to_shared(masks);
+    for (int q = 0; q <= r.periods; ++q) {
+        const int p = q & 1;
+        if (q > 0) {
+            cluster_sync_all();
+            if (live) {
+                auto add = [&](int sp, int64_t v) {
+                    int64_t n = w.N[32 * sp + lane] + v;
+                    if (n > 2147483647) { bad |= kErrOverflow; n = 2147483647; }
+                    w.N[32 * sp + lane] = (int32_t)n;
+                    pr.set(sp, (int32_t)n);
+                    dirty |= 1u << sp;
+                };
+                int32_t* own = words + ((p ^ 1) * B + (int)threadIdx.x) * 4 * S;
+                if (S <= 2) {
+                    int4* a = reinterpret_cast<int4*>(own);
+                    for (int k = 0; k < S; ++k) {
+                        const int4 x = a[k];
+                        if ((x.x | x.y | x.z | x.w) == 0) continue;
+                        a[k] = make_int4(0, 0, 0, 0);
+                        if (S == 1) {
+                            add(0, (int64_t)x.x + x.y + x.z + x.w);
+                        } else {
+                            if (x.x | x.z) add(0, (int64_t)x.x + x.z);
+                            if (x.y | x.w) add(1, (int64_t)x.y + x.w);
+                        }
+                    }
+                } else {
+                    unsigned long long bits = masks[(p ^ 1) * B + threadIdx.x];
+                    if (bits) masks[(p ^ 1) * B + threadIdx.x] = 0ull;
+                    while (bits) {
+                        const int i = __ffsll((long long)bits) - 1;
+                        bits &= bits - 1ull;
+                        add(i & 15, own[(i >> 4) * S + (i & 15)]);
+                    }
+                }
+            }
+        }
+        if (q == r.periods) break;
+        const bool last = r.last_short && q == r.periods - 1;
+        const PeriodView v{r.period0 + (uint32_t)q, last ? r.tau_last : r.tau, last ? r.tau_lastf : r.tauf, r.seed,
+                           last ? r.thr_last : r.thr, 1};
+        send.bits = 0;
+        send.words = words_at + (uint32_t)(p * B * 16 * S);
+        send.masks = masks_at + (uint32_t)(p * B * 8);
+        bool deferred = false;
+        bad |= warp_step<S_ == 1, kReact, false>(m, mp, S, w, v, t, live, mask, pr, &dirty, &deferred, s.err, send);
+        if (live) send.finish();
+    }
+    if (live)
+        for (uint32_t bits = dirty; bits; bits &= bits - 1u) {
+            const int sp = __ffs(bits) - 1;
+            s.cnt[sp * T + t] = w.N[32 * sp + lane];
+        }
+    if (bad) atomicOr(s.err, bad);
+}
+
+// CTAs of k_run_cluster for T tets, at most `most`, and the warps of each (at
+// most 16: slot numbers below 4,096, registers; shared memory within 200 KB),
+// or 0.
+int cluster_shape(int64_t T, int S, bool react, int most, int* warps) {
+    const int64_t chunks = (T + 31) / 32;
+    int n = 1;
+    while (n < most && n < chunks) n <<= 1;
+    const int64_t per = (chunks + n - 1) / n;
+    *warps = (int)per;
+    if (per > 16 || (size_t)cluster_words(S, react, (int)per) * sizeof(int32_t) > 200u * 1024u) return 0;
+    return n;
+}
+
+template <int S_, bool kReact>
+cudaError_t launch_cluster_s(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int ctas,
+                             int warps, cudaStream_t st) {
+    auto kern = k_run_cluster<S_, kReact>;
+    const size_t smem = (size_t)cluster_words(mp.S, kReact, warps) * sizeof(int32_t);
+    cudaError_t ce = cudaSuccess;
+    if (smem > 48u * 1024u) ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (ce == cudaSuccess && ctas > 8) ce = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (ce != cudaSuccess) return ce;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas, 1, 1);
+    cfg.blockDim = dim3(32 * warps, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    ce = cudaLaunchKernelEx(&cfg, kern, m, mp, s, r);
+    if (ce == cudaSuccess) ++g_launches;
+    return ce;
+}
+
 // Warps a block and blocks of k_run for T tets, or 0 if they do not fit: the
 // 32-tet warps are spread over all SMs first (a warp that has an SM's issue
 // slots and caches to itself is fastest), in at most 3 blocks of 8 warps an SM.
@@ -702,9 +900,24 @@ cudaError_t launch_run_s(const DevMesh& m, const ModelParams& mp, const DevState
 bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int sms, int* grid,
                 cudaStream_t st) {
     int warps = 0;
+    cudaError_t ce = cudaErrorInvalidConfiguration;
+    // 16 CTAs are beyond the portable cluster size: where the device has no
+    // room for one, 8 (a launch that cannot be placed fails with no effect)
+    for (int most = 16; most >= 8; most >>= 1) {
+        const int ctas = cluster_shape(m.T, mp.S, mp.any_reaction != 0, most, &warps);
+        if (ctas == 0) break;
+        if (mp.S == 1)
+            ce = mp.any_reaction ? launch_cluster_s<1, true>(m, mp, s, r, ctas, warps, st)
+                                 : launch_cluster_s<1, false>(m, mp, s, r, ctas, warps, st);
+        else
+            ce = mp.any_reaction ? launch_cluster_s<0, true>(m, mp, s, r, ctas, warps, st)
+                                 : launch_cluster_s<0, false>(m, mp, s, r, ctas, warps, st);
+        *grid = 0;   // no grid barrier
+        if (ce == cudaSuccess) return true;
+        cudaGetLastError();
+    }
     *grid = run_shape(m.T, sms, &warps);
     if (*grid == 0) return false;
-    cudaError_t ce;
     if (mp.S == 1)
         ce = mp.any_reaction ? launch_run_s<1, true>(m, mp, s, r, *grid, warps, sms, st)
                              : launch_run_s<1, false>(m, mp, s, r, *grid, warps, sms, st);

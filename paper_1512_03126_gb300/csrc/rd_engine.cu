@@ -23,6 +23,8 @@
 #include <cmath>
 #include <mutex>
 #include <numeric>
+#include <queue>
+#include <type_traits>
 #include <vector>
 
 #include "rd_api_internal.h"
@@ -43,7 +45,8 @@ struct SlotDesc {
     const uint4* thr_last;   // thresholds for the shortened last period
     int32_t* N[2];           // count buffers [S][T]; the slice starts in N[0]
     uint32_t* bits[2];       // active-tet bitmaps of 2^wshift words, by period parity in the slice
-    int32_t wshift;          // tet t is bit t >> wshift of word t & (2^wshift - 1)
+    int32_t wshift;          // tet t is bit t >> wshift of word t & (2^wshift - 1); at least as many words
+                             // as the cluster has warps
     const uint4* packed;     // one species: {src, thr} per tet
     int32_t* N2;             // one species: counts of both parities interleaved
     uint64_t seed;
@@ -75,17 +78,37 @@ __device__ __forceinline__ void red_or(uint32_t* p, uint32_t v) {
     asm volatile("red.relaxed.gpu.global.or.b32 [%0], %1;" ::"l"(p), "r"(v));
 }
 
-// Fire-and-forget AND.
-__device__ __forceinline__ void red_and(uint32_t* p, uint32_t v) {
-    asm volatile("red.relaxed.gpu.global.and.b32 [%0], %1;" ::"l"(p), "r"(v));
+// The same into a word of a CTA of the cluster (shared::cluster address).
+__device__ __forceinline__ uint32_t cta_address(uint32_t addr, uint32_t cta) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(cta));
+    return r;
+}
+__device__ __forceinline__ void red_add_cluster(uint32_t addr, int32_t v) {
+    asm volatile("red.relaxed.cluster.shared::cluster.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void red_or_cluster(uint32_t addr, uint32_t v) {
+    asm volatile("red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
 constexpr int kWarps = kRunBlock / 32;
 constexpr int kGroup = 8;                   // bitmap columns (32 words each) a warp loads at once
 
-// Dynamic shared memory of a warp, in words: the step's (rd_warp.cuh) and the
-// bitmap words of its current batch.
-__host__ __device__ inline int engine_warp_words(int S, bool react) { return warp_words(S, react) + 32 * kGroup; }
+// Dynamic shared memory of a warp, in words: the step's (rd_warp.cuh) and,
+// unless the bitmaps are in shared memory themselves, the words of its current
+// batch.
+__host__ __device__ inline int engine_warp_words(int S, bool react, bool sm) {
+    return warp_words(S, react) + (sm ? 0 : 32 * kGroup);
+}
+
+// A simulation of one species in the cluster's shared memory (kSm): a CTA
+// keeps the words of its warps, wpc = W / kC of them, in both parities' bitmaps
+// and a pair of counts (both parities) for each tet of these words, row by row
+// (row i: the tets of bit i).  Bytes of one CTA:
+__host__ __device__ inline size_t sm_bytes(int64_t T, int wshift, int kC) {
+    const int64_t W = (int64_t)1 << wshift, wpc = W / kC, rows = (T + W - 1) / W;
+    return (size_t)(rows * wpc * 8 + wpc * 8);
+}
 
 // Position of set bit number k (from 0) of w, by halves.
 __device__ __forceinline__ int nth_set_bit(uint32_t w, int k) {
@@ -109,20 +132,68 @@ __shared__ unsigned long long s_mass[3];            // [0] molecules of the simu
                                                     // in periods of even / odd parity (two's complement)
 __shared__ SlotDesc s_desc;                         // the simulation's descriptor and chemistry
 __shared__ ModelParams s_mp;
-extern __shared__ int32_t s_warp[];                 // [kWarps][engine_warp_words]
+extern __shared__ __align__(16) int32_t s_warp[];   // [kWarps][engine_warp_words]; kSm: then bitmaps and counts
 
-// Counts of one period and the next: N[r] / N[r^1], or the two halves of the
-// interleaved pairs.
+// Counts and bitmaps of one period and the next, in global memory: N[r] /
+// N[r^1], or the two halves of the interleaved pairs.
 template <bool kOne>
-struct CountView {
+struct GlobalView {
     int32_t* cur;
     int32_t* next;
+    uint32_t* bcur;
+    uint32_t* bnext;
     int64_t T;
+    int ws;
     static constexpr int stride = kOne ? 2 : 1;
-    __device__ __forceinline__ CountView(const SlotDesc& d, int r) : T(d.m.T) {
+    __device__ __forceinline__ GlobalView(const SlotDesc& d, int r) : bcur(d.bits[r]), bnext(d.bits[r ^ 1]), T(d.m.T), ws(d.wshift) {
         cur = kOne ? d.N2 + r : d.N[r];
         next = kOne ? d.N2 + (r ^ 1) : d.N[r ^ 1];
     }
+    __device__ __forceinline__ int32_t load(int s, int t) const { return __ldcg(cur + (s * T + t) * stride); }
+    __device__ __forceinline__ void clear(int s, int t) const { cur[(s * T + t) * stride] = 0; }
+    __device__ __forceinline__ void add(int s, int t, int32_t n) const { red_add(next + (s * T + t) * stride, n); }
+    __device__ __forceinline__ void mark(int t) const { red_or(bnext + (t & ((1 << ws) - 1)), 1u << (t >> ws)); }
+    __device__ __forceinline__ void send(int t, int32_t n, bool more) const {
+        add(0, t, n);
+        if (more) mark(t);
+    }
+    // the tet's own CTA
+    __device__ __forceinline__ void keep(int s, int t, int32_t n) const { add(s, t, n); }
+    __device__ __forceinline__ void mark_own(int t) const { mark(t); }
+};
+
+// The same in the cluster's shared memory: load, clear, keep and mark_own are
+// of tets of the calling CTA.
+template <int kC>
+struct ClusterView {
+    int32_t* cnt;           // [rows][wpc][2] of this CTA
+    uint32_t* bcur;
+    uint32_t* bnext;
+    uint32_t next_at, bnext_at;   // shared addresses of the next period's counts and bits
+    int ws, wl, r;
+    static constexpr int kShift = kC == 1 ? 0 : (kC == 2 ? 1 : (kC == 4 ? 2 : 3));
+    __device__ __forceinline__ ClusterView(const SlotDesc& d, int r_, int32_t* data) : ws(d.wshift), wl(d.wshift - kShift), r(r_) {
+        const int wpc = 1 << wl;
+        uint32_t* bits = reinterpret_cast<uint32_t*>(data);
+        bcur = bits + r * wpc;
+        bnext = bits + (r ^ 1) * wpc;
+        cnt = data + 2 * wpc;
+        next_at = (uint32_t)__cvta_generic_to_shared(cnt + (r ^ 1));
+        bnext_at = (uint32_t)__cvta_generic_to_shared(bnext);
+    }
+    __device__ __forceinline__ int slot(int t) const { return ((t >> ws) << wl) | (t & ((1 << wl) - 1)); }
+    __device__ __forceinline__ int32_t load(int, int t) const { return cnt[2 * slot(t) + r]; }
+    __device__ __forceinline__ void clear(int, int t) const { cnt[2 * slot(t) + r] = 0; }
+    // one species: a leaver's add and bit together
+    __device__ __forceinline__ void send(int t, int32_t n, bool more) const {
+        const uint32_t word = (uint32_t)t & ((1u << ws) - 1u), loc = word & ((1u << wl) - 1u);
+        const uint32_t row = (uint32_t)t >> ws;
+        const uint32_t there = cta_address(bnext_at, word >> wl);
+        red_add_cluster(there + (next_at - bnext_at) + 8u * ((row << wl) | loc), n);
+        if (more) red_or_cluster(there + 4u * loc, 1u << row);
+    }
+    __device__ __forceinline__ void keep(int, int t, int32_t n) const { atomicAdd(cnt + 2 * slot(t) + (r ^ 1), n); }
+    __device__ __forceinline__ void mark_own(int t) const { atomicOr(bnext + (t & ((1 << wl) - 1)), 1u << (t >> ws)); }
 };
 
 // Leavers of a tet into the next period's counts (fire-and-forget integer
@@ -130,115 +201,230 @@ struct CountView {
 // simulation's molecule total is kept below 2^32 (checked every period), the
 // next read of the count, or the check at the end of the slice, sees it
 // negative and reports the overflow, exactly when the dense gather would.
-template <bool kOne>
+template <class View, bool kOne>
 struct Scatter {
-    const CountView<kOne>& c;
+    const View& c;
+    bool more;            // a further period follows in this slice
     const int4* src;
     int t;
     int4 sr;
     bool have;
-    uint32_t send;        // faces through which something leaves
+    uint32_t send;        // faces through which something leaves (several species)
     uint32_t bad;
     long long sent;       // molecules that leave
 
-    __device__ __forceinline__ Scatter(const CountView<kOne>& c_, const int4* src_, int t_, int4 sr_, bool have_)
-        : c(c_), src(src_), t(t_), sr(sr_), have(have_), send(0), bad(0), sent(0) {}
+    __device__ __forceinline__ Scatter(const View& c_, bool more_, const int4* src_, int t_, int4 sr_, bool have_)
+        : c(c_), more(more_), src(src_), t(t_), sr(sr_), have(have_), send(0), bad(0), sent(0) {}
 
     __device__ __forceinline__ void operator()(int sp, const int4& o) {
         if (!have) sr = __ldg(src + t);
         have = true;
         const int nbr[4] = {sr.x, sr.y, sr.z, sr.w}, n[4] = {o.x, o.y, o.z, o.w};
-        int32_t* Ns = kOne ? c.next : c.next + sp * c.T;
 #pragma unroll
         for (int f = 0; f < 4; ++f) {
             if (n[f] <= 0) continue;
             if (nbr[f] < 0) { bad |= kErrNegative; continue; }
-            red_add(Ns + (int64_t)(nbr[f] >> 2) * c.stride, n[f]);
-            send |= 1u << f;
+            if constexpr (kOne) {
+                c.send(nbr[f] >> 2, n[f], more);
+            } else {
+                c.add(sp, nbr[f] >> 2, n[f]);
+                send |= 1u << f;
+            }
         }
         sent += (long long)o.x + o.y + o.z + o.w;
     }
 };
+
+// One round: the tets t of the live lanes through the step, what stays and what
+// leaves into the next counts and bits.  Without kCalls a lane whose tet needs
+// the double-precision samplers is left undone (its counts too) and *deferred
+// set.
+template <bool kOne, bool kReact, bool kCalls, class View>
+__device__ __forceinline__ uint32_t engine_round(const SlotDesc& d, const ModelParams& mp, int S, const WarpMem& w,
+                                                 const PeriodView& v, const View& c, bool more, int t, bool live,
+                                                 uint32_t* err, unsigned long long* mass_delta, bool* deferred) {
+    const int lane = threadIdx.x & 31;
+    int4 sr = make_int4(-1, -1, -1, -1);
+    uint4 pre = make_uint4(0u, 0u, 0u, 0u);
+    long long held = 0;
+    uint32_t bad = 0;
+    Presence pr;
+    const uint32_t mask = kReact && mp.has_mask && live ? __ldg(d.m.mask + t) : 0xffffffffu;
+    if (live) {
+        if (kOne) {
+            // the record and the count, loaded together
+            sr = __ldg(reinterpret_cast<const int4*>(d.packed + 2 * (int64_t)t));
+            pre = __ldg(v.thr + (int64_t)t * v.thr_stride);
+        }
+        for (int s0 = 0; s0 < S; s0 += 4) {
+            int32_t n[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (s0 + k < S) n[k] = c.load(s0 + k, t);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (s0 + k >= S) continue;
+                if (n[k] < 0) {          // wrapped past 2^31-1 by the previous period's adds
+                    bad |= kErrOverflow;
+                    c.clear(s0 + k, t);
+                    n[k] = 0;
+                }
+                w.N[32 * (s0 + k) + lane] = n[k];
+                pr.add(s0 + k, n[k]);
+                if (kReact) held += n[k];
+            }
+        }
+    }
+    const uint32_t had = pr.any;
+    Scatter<View, kOne> scatter(c, more, d.m.src, t, sr, kOne);
+    uint32_t dirty = 0;
+    bad |= warp_step<kOne, kReact, false, kCalls, kOne>(d.m, mp, S, w, v, t, live, mask, pr, &dirty, deferred, err,
+                                                        scatter, pre);
+    bad |= scatter.bad;
+    long long delta = 0;
+    if (live && (kCalls || !*deferred)) {
+        bool keep = pr.any != 0u;
+        if (kReact && d.zero_order) keep = keep || (mask & d.zero_order) != 0u;
+        for (uint32_t bits = had; bits; bits &= bits - 1u) c.clear(__ffs(bits) - 1, t);
+        for (uint32_t bits = pr.any; bits; bits &= bits - 1u) {
+            const int s = __ffs(bits) - 1;
+            const int32_t n = w.N[32 * s + lane];
+            c.keep(s, t, n);
+            if (kReact) delta += n;
+        }
+        if (kReact) delta += scatter.sent - held;
+        if (more) {
+            if (keep) c.mark_own(t);
+            if constexpr (!kOne) {
+                const int nbr[4] = {scatter.sr.x, scatter.sr.y, scatter.sr.z, scatter.sr.w};
+#pragma unroll
+                for (int f = 0; f < 4; ++f)
+                    if ((scatter.send >> f) & 1u) c.mark(nbr[f] >> 2);
+            }
+        }
+    }
+    // net molecules made by reactions: all that stays and leaves minus what was
+    // held
+    if (kReact && delta != 0) atomicAdd(mass_delta, (unsigned long long)delta);
+    return bad;
+}
+
+// What a period's passes of one warp share.
+template <bool kOne, bool kReact, int kC, bool kSm>
+struct WarpPeriod {
+    using View = typename std::conditional<kSm, ClusterView<kC>, GlobalView<kOne>>::type;
+    static constexpr int kW = kC * kWarps;
+    static constexpr int kWShift = kC == 1 ? 4 : (kC == 2 ? 5 : (kC == 4 ? 6 : 7));
+    static_assert((1 << kWShift) == kW, "warps of a cluster");
+    int S, per, word0;         // this warp's words: `per` from word0 on
+    WarpMem w;
+    PeriodView v;
+    View c;
+    uint32_t* words;           // this warp's words of the period's bitmap
+    uint32_t* wb;              // global bitmaps: the current batch's
+    bool more;
+
+    static __device__ __forceinline__ View view(const SlotDesc& d, int r, int S) {
+        if constexpr (kSm) return View(d, r, s_warp + kWarps * engine_warp_words(S, kReact, true));
+        else return View(d, r);
+    }
+    static __device__ __forceinline__ PeriodView period_view(const SlotDesc& d, int q) {
+        const bool last = (q == d.P - 1) && d.last_short;
+        // thresholds: packed beside the reverse-face record (stride 2) except in
+        // a shortened last period
+        return PeriodView{d.period0 + (uint32_t)q, last ? d.tau_last : d.tau, last ? d.tau_lastf : d.tauf, d.seed,
+                          last ? d.thr_last : (kOne ? d.packed + 1 : d.thr), kOne && !last ? 2 : 1};
+    }
+    __device__ __forceinline__ WarpPeriod(const SlotDesc& d, int q)
+        : S(kOne ? 1 : d.S), per((1 << d.wshift) >> kWShift),
+          w(s_warp + (threadIdx.x >> 5) * engine_warp_words(S, kReact, kSm), S, kReact, s_mp.rx), v(period_view(d, q)),
+          c(view(d, (q - d.q0) & 1, S)), more(q + 1 < d.q1) {
+        const int warp = threadIdx.x >> 5;
+        const int rank = kC > 1 ? (int)cooperative_groups::this_cluster().block_rank() : 0;
+        word0 = (rank * kWarps + warp) * per;
+        words = c.bcur + (kSm ? warp * per : word0);
+        wb = reinterpret_cast<uint32_t*>(s_warp + warp * engine_warp_words(S, kReact, kSm) + warp_words(S, kReact));
+    }
+};
+
+// The tets of a batch whose bits the rounds set back, with the
+// double-precision samplers.
+template <bool kOne, bool kReact, int kC, bool kSm>
+__device__ __noinline__ uint32_t run_deferred(int q, int b, uint32_t* err, unsigned long long* mass_delta) {
+    const SlotDesc& d = s_desc;
+    const WarpPeriod<kOne, kReact, kC, kSm> p(d, q);
+    const int lane = threadIdx.x & 31;
+    uint32_t bad = 0;
+    for (int kk = 0; kk < kGroup; ++kk) {
+        const int at = (b * kGroup + kk) * 32 + lane;
+        const bool mine = at < p.per;
+        uint32_t word = 0u;
+        if (mine) {
+            uint32_t* from = kSm ? p.words + at : p.wb + kk * 32 + lane;
+            word = *from;
+            *from = 0u;
+        }
+        while (__ballot_sync(kAllLanes, word != 0u)) {
+            const bool live = word != 0u;
+            const int t = live ? ((__ffs(word) - 1) << d.wshift) + p.word0 + at : 0;
+            word &= word - 1u;
+            bool none = false;
+            bad |= engine_round<kOne, kReact, true>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta, &none);
+            __syncwarp();
+        }
+    }
+    return bad;
+}
 
 // One period of a simulation for one warp.  A bitmap word holds 32 tets a
 // power of two apart, so that every word has its share of a compact cloud of
 // molecules and of its crowded tets: dealing runs of 128 consecutive tets
 // left warps waiting at the period barrier for the one that held the source
 // (15 of 24 stall cycles an instruction).  The words go to the cluster's kW
-// warps in equal contiguous parts (fewer words than warps: several warps share
-// a word by bit position).  A column is 32 words, one per lane; a warp loads
+// warps in equal contiguous parts.  A column is 32 words, one per lane; a warp loads
 // kGroup of its columns at once and clears them for their next use.  With a
 // prefix sum of a column's popcounts each lane finds a set bit of its own (a
 // search over the sums and one inside the word: a fixed 60 instructions, where
 // writing the bits of a dense word into a list took 32 turns of one lane);
 // whenever 32 tets are at hand, one round steps them (warp_step), and adds
 // what stays and what leaves into the next counts.
-template <bool kOne, bool kReact, int kC>
+template <bool kOne, bool kReact, int kC, bool kSm>
 __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned long long* mass_delta,
                                                unsigned long long* done) {
-    constexpr int kW = kC * kWarps;
     const SlotDesc& d = s_desc;
-    const ModelParams& mp = s_mp;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rank = kC > 1 ? (int)cooperative_groups::this_cluster().block_rank() : 0;
-    const int gw = rank * kWarps + warp;
-    const int S = kOne ? 1 : d.S;
-    int32_t* base_mem = s_warp + warp * engine_warp_words(S, kReact);
-    const WarpMem w(base_mem, S, kReact, s_mp.rx);
-    uint32_t* wb = reinterpret_cast<uint32_t*>(base_mem + warp_words(S, kReact));
-    const int ws = d.wshift, W = 1 << ws;
-    // this warp's words: `per` from word0 on, or its bits of one shared word
-    constexpr int kWShift = kC == 1 ? 4 : (kC == 2 ? 5 : (kC == 4 ? 6 : 7));
-    static_assert((1 << kWShift) == kW, "warps of a cluster");
-    const bool shared = ws < kWShift;
-    const int per = shared ? 1 : W >> kWShift;
-    const int word0 = shared ? gw & (W - 1) : gw * per;
-    uint32_t part = 0xffffffffu;
-    if (shared) {
-        const int split = min(kW >> ws, 32), sub = gw >> ws;
-        part = 0u;
-        for (int i = sub; i < 32; i += split) part |= sub < split ? 1u << i : 0u;
-    }
-    const int r = (q - d.q0) & 1;
-    const bool last = (q == d.P - 1) && d.last_short;
-    // thresholds: packed beside the reverse-face record (stride 2) except in a
-    // shortened last period
-    const PeriodView v{d.period0 + (uint32_t)q, last ? d.tau_last : d.tau, last ? d.tau_lastf : d.tauf, d.seed,
-                       last ? d.thr_last : (kOne ? d.packed + 1 : d.thr), kOne && !last ? 2 : 1};
-    const CountView<kOne> c(d, r);
-    uint32_t* bcur = d.bits[r];
-    uint32_t* bnext = d.bits[r ^ 1];
-    const bool more = q + 1 < d.q1;
+    const int lane = threadIdx.x & 31;
+    const WarpPeriod<kOne, kReact, kC, kSm> p(d, q);
     uint32_t bad = 0;
-    int pend = 0, cnt = 0;      // tets not yet run: lane i < cnt holds one
     unsigned long long visited = 0;
-    for (int b = 0;; ++b) {
+    for (int b = 0; b * kGroup * 32 < p.per; ++b) {
         const int at = b * kGroup * 32 + lane;
-        const bool flush = b * kGroup * 32 >= per;   // past the last batch: run what is left
-        int columns = 1;
-        if (!flush) {
+        uint32_t any = 0;
+        if (kSm) {
+            for (int kk = 0; kk < kGroup && b * kGroup + kk < (p.per + 31) >> 5; ++kk)
+                if (at + kk * 32 < p.per && p.words[at + kk * 32]) any |= 1u << kk;
+        } else {
             uint32_t wds[kGroup];
 #pragma unroll
-            for (int kk = 0; kk < kGroup; ++kk) {
-                wds[kk] = at + kk * 32 < per ? __ldcg(bcur + word0 + at + kk * 32) & part : 0u;
-            }
-            uint32_t any = 0;
+            for (int kk = 0; kk < kGroup; ++kk) wds[kk] = at + kk * 32 < p.per ? __ldcg(p.words + at + kk * 32) : 0u;
 #pragma unroll
             for (int kk = 0; kk < kGroup; ++kk) {
-                if (wds[kk]) {
-                    if (shared) red_and(bcur + word0, ~part);
-                    else bcur[word0 + at + kk * 32] = 0u;
-                }
-                wb[kk * 32 + lane] = wds[kk];
+                if (wds[kk]) p.words[at + kk * 32] = 0u;
+                p.wb[kk * 32 + lane] = wds[kk];
                 any |= wds[kk] ? 1u << kk : 0u;
             }
-            columns = (int)__reduce_or_sync(kAllLanes, any);
         }
-        // the columns that hold a set bit (flush: one turn without any)
+        uint32_t columns = __reduce_or_sync(kAllLanes, any);   // those that hold a set bit
+        int pend = 0, cnt = 0;      // tets not yet run: lane i < cnt holds one
+        bool late = false;          // some tet was deferred
         while (columns) {
             const int kk = __ffs(columns) - 1;
             columns &= columns - 1;
-            const uint32_t word = flush ? 0u : wb[kk * 32 + lane];
+            uint32_t word = 0u;
+            if (at + kk * 32 < p.per) {
+                uint32_t* from = kSm ? p.words + at + kk * 32 : p.wb + kk * 32 + lane;
+                word = *from;
+                *from = 0u;
+            }
             const int own = __popc(word);
             int inc = own;
 #pragma unroll
@@ -258,9 +444,9 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
                     if (__shfl_sync(kAllLanes, inc, from + step - 1) <= e) from += step;
                 const int k = e - __shfl_sync(kAllLanes, inc - own, from);
                 const int bit = nth_set_bit(__shfl_sync(kAllLanes, word, from), k);
-                const int t_new = (bit << ws) + word0 + (b * kGroup + kk) * 32 + from;
+                const int t_new = (bit << d.wshift) + p.word0 + (b * kGroup + kk) * 32 + from;
                 const int t_lane = e < 0 ? pend : t_new;
-                if (avail < 32 && !(flush && avail > 0)) {
+                if (avail < 32 && columns) {
                     pend = t_lane;
                     cnt = avail;
                     break;
@@ -269,71 +455,22 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
                 const int t = live ? t_lane : 0;
                 off -= 32;
                 avail = max(avail - 32, 0);
-                int4 sr = make_int4(-1, -1, -1, -1);
-                uint4 pre = make_uint4(0u, 0u, 0u, 0u);
-                long long held = 0;
-                Presence pr;
-                const uint32_t mask = kReact && mp.has_mask && live ? __ldg(d.m.mask + t) : 0xffffffffu;
-                if (live) {
-                    if (kOne) {
-                        // the record and the count, loaded together
-                        sr = __ldg(reinterpret_cast<const int4*>(d.packed + 2 * (int64_t)t));
-                        pre = __ldg(v.thr + (int64_t)t * v.thr_stride);
-                    }
-                    for (int s0 = 0; s0 < S; s0 += 4) {
-                        int32_t n[4];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            if (s0 + k < S) n[k] = __ldcg(c.cur + ((s0 + k) * c.T + t) * c.stride);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            if (s0 + k >= S) continue;
-                            if (n[k] != 0) c.cur[((s0 + k) * c.T + t) * c.stride] = 0;
-                            if (n[k] < 0) {          // wrapped past 2^31-1 by the previous period's adds
-                                bad |= kErrOverflow;
-                                n[k] = 0;
-                            }
-                            w.N[32 * (s0 + k) + lane] = n[k];
-                            pr.add(s0 + k, n[k]);
-                            if (kReact) held += n[k];
-                        }
-                    }
-                }
-                Scatter<kOne> scatter(c, d.m.src, t, sr, kOne);
-                uint32_t dirty = 0;
                 bool deferred = false;
-                bad |= warp_step<kOne, kReact, false, kOne>(d.m, mp, S, w, v, t, live, mask, pr, &dirty, &deferred,
-                                                            err, scatter, pre);
-                bad |= scatter.bad;
-                long long delta = 0;
-                if (live) {
-                    bool keep = pr.any != 0u;
-                    if (kReact && d.zero_order) keep = keep || (mask & d.zero_order) != 0u;
-                    for (uint32_t bits = pr.any; bits; bits &= bits - 1u) {
-                        const int s = __ffs(bits) - 1;
-                        const int32_t n = w.N[32 * s + lane];
-                        red_add(c.next + (s * c.T + t) * c.stride, n);
-                        if (kReact) delta += n;
-                    }
-                    if (kReact) delta += scatter.sent - held;
-                    if (more) {
-                        if (keep) red_or(bnext + (t & (W - 1)), 1u << (t >> ws));
-                        const int nbr[4] = {scatter.sr.x, scatter.sr.y, scatter.sr.z, scatter.sr.w};
-#pragma unroll
-                        for (int f = 0; f < 4; ++f) {
-                            if (!((scatter.send >> f) & 1u)) continue;
-                            const int u = nbr[f] >> 2;
-                            red_or(bnext + (u & (W - 1)), 1u << (u >> ws));
-                        }
+                bad |= engine_round<kOne, kReact, false>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta,
+                                                         &deferred);
+                if (__ballot_sync(kAllLanes, deferred)) {
+                    late = true;
+                    if (deferred) {   // back into its word
+                        const int i = (t & ((1 << d.wshift) - 1)) - p.word0;
+                        atomicOr(kSm ? p.words + i : p.wb + (i - b * kGroup * 32), 1u << (t >> d.wshift));
                     }
                 }
-                // net molecules made by reactions: all that stays and leaves
-                // minus what was held
-                if (kReact && delta != 0) atomicAdd(mass_delta, (unsigned long long)delta);
                 __syncwarp();
+                if (avail == 0) break;   // (only the batch's last column gets here with none left)
             }
+            if (avail == 0) cnt = 0;
         }
-        if (flush) break;
+        if (late) bad |= run_deferred<kOne, kReact, kC, kSm>(q, b, err, mass_delta);
     }
     *done += visited;
     return bad;
@@ -355,7 +492,13 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
 // at the end of the slice); the molecule total of the simulation, tracked per
 // period (each round adds what its reactions make or consume), is kept
 // below 2^32 - 1 so that no count can wrap all the way round unseen.
-template <int S_, bool kReact, int kC>
+// With kSm (one species, a mesh whose counts fit, see sm_bytes) the counts and
+// bitmaps are in the cluster's shared memory for the slice, and every add and
+// OR goes to the owning CTA's.  In global memory a period of a 24^3-cell cube
+// on 8 CTAs took 18,700 cycles of which a warp worked 8,500 (2,000 to load its
+// words, 900 for the counts); the rest was the barrier's wait for the adds to
+// reach L2.
+template <int S_, bool kReact, int kC, bool kSm>
 __global__ void __launch_bounds__(kRunBlock, 2)
 k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__ mps, const int32_t* __restrict__ order,
              int32_t n_items, int32_t* head, uint32_t* err, unsigned long long* processed,
@@ -409,7 +552,10 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
         // (a thread a word; its tets are W apart, so a warp's loads are
         // contiguous); and the simulation's molecule total
         unsigned long long mine = 0;
-        for (int wi = rank * kRunBlock + threadIdx.x; wi < W; wi += kC * kRunBlock) {
+        const int wpc = W / kC;   // kSm: the words, and the tets, of this CTA
+        int32_t* const data = s_warp + kWarps * engine_warp_words(S, kReact, true);
+        for (int i = (kSm ? 0 : rank * kRunBlock) + threadIdx.x; i < (kSm ? wpc : W); i += kSm ? kRunBlock : kC * kRunBlock) {
+            const int wi = kSm ? rank * wpc + i : i;
             uint32_t word = 0;
             for (int t = wi, bit = 0; t < T; t += W, ++bit) {
                 bool occ = false;
@@ -420,11 +566,17 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
                     occ = occ || c > 0;
                     mine += (uint32_t)max(c, 0);
                     if (c < 0) bad |= kErrNegative;
-                    if (inter) reinterpret_cast<int2*>(d.N2)[t] = make_int2(c, 0);
+                    if (kSm) reinterpret_cast<int2*>(data + 2 * wpc)[bit * wpc + i] = make_int2(c, 0);
+                    else if (inter) reinterpret_cast<int2*>(d.N2)[t] = make_int2(c, 0);
                 }
                 if (occ) word |= 1u << bit;
             }
-            d.bits[0][wi] = word;
+            if (kSm) {
+                reinterpret_cast<uint32_t*>(data)[i] = word;
+                reinterpret_cast<uint32_t*>(data)[wpc + i] = 0u;
+            } else {
+                d.bits[0][wi] = word;
+            }
         }
 #pragma unroll
         for (int dd = 16; dd > 0; dd >>= 1) mine += __shfl_xor_sync(kAllLanes, mine, dd);
@@ -443,14 +595,22 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
         for (int q = d.q0; q < d.q1; ++q) {
             csync();   // the previous period's adds and bits are complete
             if (q > d.q0) account(q - 1);
-            bad |= run_period<kOne, kReact, kC>(q, err, &mass[1 + (q & 1)], &item_done);
+            bad |= run_period<kOne, kReact, kC, kSm>(q, err, &mass[1 + (q & 1)], &item_done);
         }
         csync();   // every add of the slice is complete
         account(d.q1 - 1);
         // a count the last period's adds took past 2^31-1 reads negative
         {
             const int half = (d.q1 - d.q0) & 1;
-            for (int t = rank * kRunBlock + threadIdx.x; t < T; t += kC * kRunBlock) {
+            if (kSm) {
+                for (int i = threadIdx.x; i < wpc; i += kRunBlock)
+                    for (int t = rank * wpc + i, bit = 0; t < T; t += W, ++bit) {
+                        const int32_t c = data[2 * wpc + 2 * (bit * wpc + i) + half];
+                        if (c < 0) bad |= kErrOverflow;
+                        d.N[0][t] = c;
+                    }
+            }
+            for (int t = rank * kRunBlock + threadIdx.x; !kSm && t < T; t += kC * kRunBlock) {
                 if (inter) {
                     // the slice's counts are in the pairs' half (q1 - q0) & 1;
                     // hand them back in N[0]
@@ -504,19 +664,32 @@ struct EngineLaunch {
     int sms;
     int clusters;
     int S;                // largest species count of the group's simulations
+    bool spread = false;  // one CTA an SM
+    size_t data = 0;      // bytes of counts and bitmaps in a CTA's shared memory (0: in global memory)
     int used = 0;         // clusters launched
     int max_active = 0;   // clusters resident at once (occupancy query)
     bool query_only = false;   // fill max_active, launch nothing
 };
 
-template <int SA, bool R, int C>
+// Shared memory of a CTA so that two of them fit on an SM, and what of it one
+// species' counts and bitmaps may take.
+constexpr size_t kCtaSmem = 112 * 1024;
+inline size_t sm_data_limit(bool react) {
+    return kCtaSmem - (sizeof(SlotDesc) + sizeof(ModelParams) + 256) -
+           (size_t)kWarps * engine_warp_words(1, react, true) * sizeof(int32_t);
+}
+
+template <int SA, bool R, int C, bool SM>
 cudaError_t launch_cluster(EngineLaunch& L) {
-    auto kern = k_engine_run<SA, R, C>;
+    auto kern = k_engine_run<SA, R, C, SM>;
     // the attribute covers every group of this kernel, whatever its species
-    const size_t most = (size_t)kWarps * engine_warp_words(SA == 1 ? 1 : kMaxS, R) * sizeof(int32_t);
-    cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    const size_t most = (size_t)kWarps * engine_warp_words(SA == 1 ? 1 : kMaxS, R, SM) * sizeof(int32_t) +
+                        (SM ? sm_data_limit(R) : 0) + kCtaSmem + 4096;
+    cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)std::min<size_t>(most, 220 * 1024));
     if (ce != cudaSuccess) return ce;
-    const size_t dyn = (size_t)kWarps * engine_warp_words(L.S, R) * sizeof(int32_t);
+    size_t dyn = (size_t)kWarps * engine_warp_words(L.S, R, SM) * sizeof(int32_t) + L.data;
+    if (L.spread) dyn = std::max<size_t>(dyn, kCtaSmem + 4096);   // more than half of an SM's
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C, 1, 1);
     cfg.blockDim = dim3(kRunBlock, 1, 1);
@@ -554,12 +727,35 @@ cudaError_t launch_cluster(EngineLaunch& L) {
                               L.times);
 }
 
-template <int SA>
+template <int SA, bool SM>
 cudaError_t launch_run_sa(bool react, int cluster, EngineLaunch& L) {
-    if (cluster >= 8) return react ? launch_cluster<SA, true, 8>(L) : launch_cluster<SA, false, 8>(L);
-    if (cluster == 4) return react ? launch_cluster<SA, true, 4>(L) : launch_cluster<SA, false, 4>(L);
-    if (cluster == 2) return react ? launch_cluster<SA, true, 2>(L) : launch_cluster<SA, false, 2>(L);
-    return react ? launch_cluster<SA, true, 1>(L) : launch_cluster<SA, false, 1>(L);
+    if (cluster >= 8) return react ? launch_cluster<SA, true, 8, SM>(L) : launch_cluster<SA, false, 8, SM>(L);
+    if (cluster == 4) return react ? launch_cluster<SA, true, 4, SM>(L) : launch_cluster<SA, false, 4, SM>(L);
+    if (cluster == 2) return react ? launch_cluster<SA, true, 2, SM>(L) : launch_cluster<SA, false, 2, SM>(L);
+    return react ? launch_cluster<SA, true, 1, SM>(L) : launch_cluster<SA, false, 1, SM>(L);
+}
+
+// log2 of a bitmap's words: at least T / 32 and the warps of a cluster.
+inline int words_shift(int64_t T, int cluster) {
+    int s = 4;
+    while ((1 << s) < cluster * kWarps || ((int64_t)32 << s) < T) ++s;
+    return s;
+}
+
+// Kernel groups of a step: by species class (1, 2, up to 4, up to 8, more: it
+// sets the shared memory of a warp) with and without reactions, and one
+// species in shared memory with and without.
+constexpr int kGroups = 12;
+inline int group_species(int g) {
+    constexpr int most[6] = {1, 2, 4, 8, kMaxS, 1};
+    return most[g >> 1];
+}
+cudaError_t launch_group(int g, int cluster, EngineLaunch& L) {
+    const bool react = (g & 1) != 0;
+    L.S = group_species(g);
+    if (g >= 10) return launch_run_sa<1, true>(react, cluster, L);
+    L.data = 0;
+    return g >> 1 ? launch_run_sa<0, false>(react, cluster, L) : launch_run_sa<1, false>(react, cluster, L);
 }
 
 // Every instantiation of the engine kernel is launched once, with no work
@@ -569,24 +765,6 @@ cudaError_t launch_run_sa(bool react, int cluster, EngineLaunch& L) {
 // streams, and on the serving mix a step whose groups included kernels not
 // launched before in the process ran the groups one after another (each
 // started when the previous one ended) instead of side by side.
-template <int SA, bool R, int C>
-void warm_kernel(EngineLaunch& W) {
-    if (launch_cluster<SA, R, C>(W) == cudaSuccess) note_launch();
-    cudaGetLastError();   // a failure here shows again, and is reported, at a real launch
-}
-
-template <int SA>
-void warm_kernels_sa(EngineLaunch& W) {
-    warm_kernel<SA, false, 1>(W);
-    warm_kernel<SA, true, 1>(W);
-    warm_kernel<SA, false, 2>(W);
-    warm_kernel<SA, true, 2>(W);
-    warm_kernel<SA, false, 4>(W);
-    warm_kernel<SA, true, 4>(W);
-    warm_kernel<SA, false, 8>(W);
-    warm_kernel<SA, true, 8>(W);
-}
-
 // head: int32[kGroups] of the engine being created (set to zero before, since a
 // fresh allocation may hold anything and a negative index would be taken for
 // an item, and left zero); err and
@@ -601,14 +779,17 @@ void warm_engine_kernels(int32_t* head, uint32_t* err, unsigned long long* proce
     }
     std::lock_guard<std::mutex> lock(mu);
     if (std::find(warmed.begin(), warmed.end(), dev) != warmed.end()) return;
-    if (cudaMemsetAsync(head, 0, sizeof(int32_t) * 10, (cudaStream_t)0) != cudaSuccess) {
+    if (cudaMemsetAsync(head, 0, sizeof(int32_t) * kGroups, (cudaStream_t)0) != cudaSuccess) {
         cudaGetLastError();
         return;
     }
     EngineLaunch W{nullptr, nullptr, nullptr, 0, head, err, processed, nullptr, (cudaStream_t)0, sms, 1, 1};
-    warm_kernels_sa<1>(W);
-    warm_kernels_sa<0>(W);
-    cudaMemsetAsync(head, 0, sizeof(int32_t) * 10, (cudaStream_t)0);
+    for (int g : {0, 1, 2, 3, 10, 11})   // every kernel: one species, several, one in shared memory
+        for (int c = 1; c <= 8; c <<= 1) {
+            if (launch_group(g, c, W) == cudaSuccess) note_launch();
+            cudaGetLastError();   // a failure here shows again, and is reported, at a real launch
+        }
+    cudaMemsetAsync(head, 0, sizeof(int32_t) * kGroups, (cudaStream_t)0);
     cudaStreamSynchronize((cudaStream_t)0);
     cudaGetLastError();
     warmed.push_back(dev);
@@ -639,11 +820,12 @@ struct rdsplit_engine {
     int32_t last_max_active = 0;              // clusters that fit at once in the last launch
     int64_t slice_work = 0;                   // tet-periods per simulation and step call (0: no limit)
     int32_t last_groups = 0;                  // kernel groups of the last launch
-    cudaStream_t aux[10] = {};                // one stream per kernel group
+    cudaStream_t aux[kGroups] = {};                // one stream per kernel group
     cudaEvent_t ev_fork = nullptr;
-    cudaEvent_t ev_join[10] = {};
+    cudaEvent_t ev_join[kGroups] = {};
     int32_t cluster = 2;                      // CTAs per simulation (1, 2, 4 or 8)
-    bool cluster_auto = false;                // chosen at each step by the number of simulations
+    bool cluster_auto = false;                // it and `spread` chosen at each step for the simulations at hand
+    bool spread = false;                      // one CTA an SM (else two)
     std::vector<rdsplit_mesh_t> slot_mesh;    // null = free
     std::vector<SlotDesc> h_desc;
     std::vector<int32_t> slot_q;              // local periods done
@@ -701,6 +883,60 @@ void plan_periods(double t, double tau, double t_end, int64_t* P, double* tau_la
     *P = n;
 }
 
+// CTAs per simulation, and per SM, for a whole ensemble: the choice whose
+// schedule (longest first, each simulation to the cluster that is free first)
+// ends soonest.  A period costs a part that no CTA takes off (its serial chain
+// and barrier) and one that they share: 36, 22, 14 and 10 us were measured on
+// 1, 2, 4 and 8 CTAs for 3,000 occupied tets; and a CTA that shares its SM with
+// another takes about 1.7 times as long.
+template <class Cls>
+void choose_cluster(rdsplit_engine* e, const std::vector<int32_t>& items, const Cls& cls_at) {
+    int best = 2;
+    bool best_spread = false;
+    double best_end = HUGE_VAL;
+    for (int c = 1; c <= 8; c <<= 1) {
+        std::vector<double> cost;
+        int32_t largest = items[0];
+        for (int32_t s : items) {
+            const rdsplit_mesh* h = e->slot_mesh[s];
+            if (h->T > e->slot_mesh[largest]->T) largest = s;
+            const double shared = std::min(1.0, (double)h->T / 8192.0) * h->S;
+            cost.push_back((double)(e->h_desc[s].q1 - e->h_desc[s].q0) * (0.25 + shared / c));
+        }
+        std::sort(cost.begin(), cost.end(), [](double a, double b) { return a > b; });
+        for (int spread = 0; spread < 2; ++spread) {
+            EngineLaunch Q{nullptr, nullptr, nullptr, 1, nullptr, nullptr, nullptr, nullptr, e->stream, e->sms, 0, 1};
+            Q.query_only = true;
+            Q.spread = spread != 0;
+            const int64_t T = e->slot_mesh[largest]->T;
+            const int g = cls_at(largest, c);
+            if (g >= 10) Q.data = sm_bytes(T, words_shift(T, c), c);
+            if (launch_group(g, c, Q) != cudaSuccess) {
+                cudaGetLastError();
+                continue;
+            }
+            std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+            for (int i = 0; i < Q.max_active; ++i) free_at.push(0.0);
+            // CTAs beyond one an SM share theirs
+            const double f = !spread && (int64_t)std::min<size_t>(items.size(), Q.max_active) * c > e->sms ? 1.7 : 1.0;
+            double end = 0.0;
+            for (double w : cost) {
+                const double t = free_at.top() + w * f;
+                free_at.pop();
+                free_at.push(t);
+                end = std::max(end, t);
+            }
+            if (end < best_end) {
+                best_end = end;
+                best = c;
+                best_spread = spread != 0;
+            }
+        }
+    }
+    e->cluster = best;
+    e->spread = best_spread;
+}
+
 void finish_slot(rdsplit_engine* e, int slot) {
     rdsplit_mesh* h = e->slot_mesh[slot];
     const SlotDesc& d = e->h_desc[slot];
@@ -728,7 +964,7 @@ int rdsplit_engine_create(int32_t max_slots, int64_t max_active_tets, rdsplit_en
     e->d_desc = (SlotDesc*)rdapi::dev_alloc(sizeof(SlotDesc) * max_slots);
     e->d_mp = (ModelParams*)rdapi::dev_alloc(sizeof(ModelParams) * max_slots);
     e->d_order = (int32_t*)rdapi::dev_alloc(sizeof(int32_t) * max_slots);
-    e->d_head = (int32_t*)rdapi::dev_alloc(sizeof(int32_t) * 10);
+    e->d_head = (int32_t*)rdapi::dev_alloc(sizeof(int32_t) * kGroups);
     e->err = (uint32_t*)rdapi::dev_alloc(sizeof(uint32_t));
     e->processed = (unsigned long long*)rdapi::dev_alloc(sizeof(unsigned long long));
     e->d_times = (unsigned long long*)rdapi::dev_alloc(sizeof(unsigned long long) * 4 * max_slots);
@@ -781,9 +1017,7 @@ int rdsplit_engine_add(rdsplit_engine_t e, rdsplit_mesh_t h, double t_end, uint6
     if (h->period + P > (int64_t)0xffffffffll) return rdapi::fail(RDSPLIT_EOVERFLOW, "%s: period index exceeds 2^32-1", where);
     if (P > 0x7fffffffll) return rdapi::fail(RDSPLIT_EINVAL, "%s: too many periods", where);
     const size_t T = (size_t)h->T;
-    int wshift = 0;
-    while (((size_t)32 << wshift) < T) ++wshift;
-    const size_t W = (size_t)1 << wshift;
+    const size_t W = (size_t)1 << words_shift(h->T, 8);   // for any cluster size
     if (!h->bits[0]) {
         h->bits[0] = (uint32_t*)rdapi::dev_alloc(4 * W);
         h->bits[1] = (uint32_t*)rdapi::dev_alloc(4 * W);
@@ -815,7 +1049,7 @@ int rdsplit_engine_add(rdsplit_engine_t e, rdsplit_mesh_t h, double t_end, uint6
     d.N[1] = h->rem;
     d.bits[0] = h->bits[0];
     d.bits[1] = h->bits[1];
-    d.wshift = wshift;
+    d.wshift = 0;   // set at each step
     d.packed = pack ? h->packed : nullptr;
     d.N2 = pack ? reinterpret_cast<int32_t*>(h->N2) : nullptr;
     d.seed = seed;
@@ -873,17 +1107,26 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
         max_adv = std::max<int64_t>(max_adv, d.q1 - d.q0);
     }
     if (items.empty()) return engine_err(e, where);
-    // Simulations are launched in groups by species class (1, 2, up to 4, up
-    // to 8, more: it sets the shared memory of a warp) and with or without
-    // reactions.  Groups run concurrently on their own streams, the
-    // resident clusters shared among them by work; largest first in each.
-    auto cls_of = [&](int s) {
+    // Simulations are launched in groups of one kernel and shared-memory size
+    // each.  Groups run concurrently on their own streams, the resident
+    // clusters shared among them by work; largest first in each.
+    auto cls_at = [&](int s, int cluster) {
         const rdsplit_mesh* h = e->slot_mesh[s];
-        const int S = h->S;
+        const int S = h->S, react = h->R > 0 ? 1 : 0;
+        if (S == 1 && sm_bytes(h->T, words_shift(h->T, cluster), cluster) <= sm_data_limit(react != 0)) return 10 + react;
         const int c = S <= 1 ? 0 : (S <= 2 ? 1 : (S <= 4 ? 2 : (S <= 8 ? 3 : 4)));
-        return 2 * c + (h->R > 0 ? 1 : 0);
+        return 2 * c + react;
     };
-    constexpr int kGroups = 10;
+    if (e->cluster_auto) choose_cluster(e, items, cls_at);
+    const int csize = e->cluster;
+    auto cls_of = [&](int s) { return cls_at(s, csize); };
+    size_t g_data[kGroups] = {0};
+    for (int32_t s : items) {
+        const rdsplit_mesh* h = e->slot_mesh[s];
+        e->h_desc[s].wshift = words_shift(h->T, csize);
+        const int g = cls_of(s);
+        if (g >= 10) g_data[g] = std::max(g_data[g], sm_bytes(h->T, e->h_desc[s].wshift, csize));
+    }
     std::vector<size_t> idx(items.size());
     std::iota(idx.begin(), idx.end(), 0);
     std::stable_sort(idx.begin(), idx.end(), [&](size_t a, size_t b) {
@@ -913,32 +1156,11 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
         cudaGetLastError();
         return rdapi::fail(RDSPLIT_ECUDA, "%s: upload failed: %s", where, cudaGetErrorString(ce));
     }
-    // The largest cluster of which as many fit as there are simulations: an
-    // ensemble of fewer than the GPU's clusters would leave SMs idle.
-    if (e->cluster_auto) {
-        for (int c = 8; c >= 1; c >>= 1) {
-            e->cluster = c;
-            EngineLaunch Q{e->d_desc, e->d_mp, e->d_order, 1, e->d_head, e->err, e->processed, nullptr, st, e->sms, 0, 1};
-            Q.query_only = true;
-            const int g = cls_of(order.back());
-            Q.S = g >> 1 ? (g >> 1 == 1 ? 2 : g >> 1 == 2 ? 4 : g >> 1 == 3 ? 8 : kMaxS) : 1;
-            const cudaError_t qe = g >> 1 ? launch_run_sa<0>((g & 1) != 0, c, Q) : launch_run_sa<1>((g & 1) != 0, c, Q);
-            if (qe == cudaSuccess && Q.max_active >= (int)items.size()) break;
-        }
-        if (e->cluster == 1) e->cluster = 2;
-    }
-    const int csize = e->cluster;
     if (e->timing && !e->ev[0]) {
         cudaEventCreate(&e->ev[0]);
         cudaEventCreate(&e->ev[1]);
     }
     if (e->timing) cudaEventRecord(e->ev[0], st);
-    auto launch_group = [&](int g, EngineLaunch& L) -> cudaError_t {
-        const bool react = (g & 1) != 0;
-        const int most[5] = {1, 2, 4, 8, kMaxS};
-        L.S = most[g >> 1];
-        return g >> 1 ? launch_run_sa<0>(react, csize, L) : launch_run_sa<1>(react, csize, L);
-    };
     int used = 0, fit = 0;
     if (n_groups == 1) {
         int g = 0;
@@ -947,14 +1169,17 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
         // SM where the GPCs allow it)
         EngineLaunch L{e->d_desc, e->d_mp, e->d_order, g_count[g], e->d_head, e->err, e->processed,
                        e->timing ? e->d_times : nullptr, st, e->sms, e->concurrency, 1};
-        ce = launch_group(g, L);
+        L.data = g_data[g];
+        L.spread = e->spread;
+        ce = launch_group(g, csize, L);
         used = L.used;
         fit = L.max_active;
     } else {
         // the clusters that fit, shared by work (at least one per group)
         EngineLaunch Q{e->d_desc, e->d_mp, e->d_order, 1, e->d_head, e->err, e->processed, nullptr, st, e->sms, 0, 1};
         Q.query_only = true;
-        ce = launch_group(7, Q);
+        Q.spread = e->spread;
+        ce = launch_group(7, csize, Q);
         fit = Q.max_active;
         const int budget = e->concurrency > 0 ? std::min(e->concurrency, fit) : fit;
         double total = 0.0;
@@ -988,7 +1213,9 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
             ce = cudaStreamWaitEvent(e->aux[g], e->ev_fork, 0);
             EngineLaunch L{e->d_desc, e->d_mp, e->d_order + g_begin[g], g_count[g], e->d_head + g, e->err,
                            e->processed, e->timing ? e->d_times : nullptr, e->aux[g], e->sms, share[g], 1};
-            if (ce == cudaSuccess) ce = launch_group(g, L);
+            L.data = g_data[g];
+            L.spread = e->spread;
+            if (ce == cudaSuccess) ce = launch_group(g, csize, L);
             used += L.used;
             if (ce == cudaSuccess) ce = cudaEventRecord(e->ev_join[g], e->aux[g]);
             if (ce == cudaSuccess) ce = cudaStreamWaitEvent(st, e->ev_join[g], 0);

@@ -486,6 +486,34 @@ struct Sender {
     }
 };
 
+// The deferred tets of a warp (warp_step without calls), one a lane, with the
+// double-precision samplers: rare, and kept out of line so that the kernels'
+// registers and loops are free of them.  Returns the species whose count
+// changed, error bits in the upper half.
+template <bool kReact>
+static __device__ __noinline__ uint32_t step_deferred(const DevMesh& m, const ModelParams& mp, int32_t* column0,
+                                                      const uint2* rx, uint32_t period, double tau_k, uint64_t seed,
+                                                      const uint4* thr, int32_t* in_cur, uint8_t* mask_cur, int t,
+                                                      bool live, bool tried, bool dense, uint32_t* err) {
+    const int S = mp.S, lane = threadIdx.x & 31;
+    const WarpMem w(column0, S, kReact, rx);
+    const PeriodView v{period, tau_k, (float)tau_k, seed, thr, 1};
+    PeriodArgs a{};
+    a.in_cur = in_cur;
+    a.mask_cur = mask_cur;
+    Presence pr;
+    if (live) pr = presence_of(w.N + lane, S);
+    const uint32_t mask = kReact && mp.has_mask && live ? __ldg(m.mask + t) : 0xffffffffu;
+    Sender send(a, m.src, t, S);
+    if (live && dense) send.load();
+    uint32_t dirty = 0;
+    bool none = false;
+    const uint32_t bad = warp_step<false, kReact, false, true>(m, mp, S, w, v, t, live, mask, pr, &dirty, &none, err, send,
+                                                               make_uint4(0u, 0u, 0u, 0u), tried);
+    if (live) send.finish(dense);
+    return (live ? dirty : 0u) | (bad << 16);
+}
+
 // Passes of a period: all in one kernel, or a first pass that defers the tets
 // whose reaction phase has to run to a queue and a second one over the queue.
 enum { kPassAll = 0, kPassFirst = 1, kPassQueue = 2 };
@@ -496,7 +524,7 @@ enum { kPassAll = 0, kPassFirst = 1, kPassQueue = 2 };
 // tet reads or writes them) and are written back where they changed.
 // S_ > 0 fixes the species count at compile time.
 template <int S_, bool kReact, int kPass>
-__global__ void __launch_bounds__(kBlock, S_ == 1 ? 3 : (kPass == kPassAll ? 5 : 4))
+__global__ void __launch_bounds__(kBlock, S_ == 1 ? 3 : 4)
 k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp, DevState s,
          const __grid_constant__ PeriodArgs a, int32_t* __restrict__ queue, int32_t* qcount, int32_t parity) {
     extern __shared__ int32_t sm[];
@@ -538,8 +566,20 @@ k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams 
         Sender send(a, m.src, t, S);
         if (a.dense && live) send.clear_all();
         bool deferred = false;
-        bad |= warp_step<S_ == 1, kReact, kPass == kPassFirst>(m, mp, S, w, v, t, live, mask, pr, &dirty, &deferred, s.err, send);
-        if (live && !deferred) send.finish(a.dense != 0);
+        if (kPass == kPassQueue) {
+            deferred = live;
+        } else {
+            bad |= warp_step<S_ == 1, kReact, kPass == kPassFirst, false>(m, mp, S, w, v, t, live, mask, pr, &dirty,
+                                                                          &deferred, s.err, send);
+            if (live && !deferred) send.finish(a.dense != 0);
+        }
+        if (kPass != kPassFirst && __ballot_sync(0xffffffffu, deferred)) {
+            const uint32_t x = step_deferred<kReact>(m, mp, w.N, w.rx, a.period, a.tau_k, a.seed, a.thr, a.in_cur,
+                                                     a.mask_cur, t, deferred, kPass == kPassAll && (pr.many >> 16) == 0u,
+                                                     a.dense != 0, s.err);
+            dirty |= x & 0xffffu;
+            bad |= x >> 16;
+        }
         if (kPass == kPassFirst) {
             const unsigned dm = __ballot_sync(0xffffffffu, deferred);
             if (dm) {
@@ -646,8 +686,16 @@ k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp,
                            last ? r.thr_last : r.thr, 1};
         Sender send(a, m.src, t, S);
         bool deferred = false;
-        bad |= warp_step<S_ == 1, kReact, false>(m, mp, S, w, v, t, live, mask, pr, &dirty, &deferred, s.err, send);
-        if (live) send.finish(false);
+        bad |= warp_step<S_ == 1, kReact, false, false>(m, mp, S, w, v, t, live, mask, pr, &dirty, &deferred, s.err,
+                                                        send);
+        if (live && !deferred) send.finish(false);
+        if (__ballot_sync(0xffffffffu, deferred)) {
+            const uint32_t x = step_deferred<kReact>(m, mp, w.N, w.rx, v.period, v.tau_k, v.seed, v.thr, a.in_cur,
+                                                     a.mask_cur, t, deferred, (pr.many >> 16) == 0u, false, s.err);
+            dirty |= x & 0xffffu;
+            bad |= x >> 16;
+            if (deferred) pr = presence_of(w.N + lane, S);
+        }
     }
     if (live)
         for (uint32_t bits = dirty; bits; bits &= bits - 1u) {
@@ -701,6 +749,27 @@ struct ClusterSender {
         }
     }
 };
+
+template <bool kReact>
+static __device__ __noinline__ uint32_t step_deferred_in_cluster(const DevMesh& m, const ModelParams& mp,
+                                                                 int32_t* column0, const uint2* rx, uint32_t period,
+                                                                 double tau_k, uint64_t seed, const uint4* thr,
+                                                                 uint4 slot, uint32_t words, uint32_t masks, int t,
+                                                                 bool live, bool tried, uint32_t* err) {
+    const int S = mp.S, lane = threadIdx.x & 31;
+    const WarpMem w(column0, S, kReact, rx);
+    const PeriodView v{period, tau_k, (float)tau_k, seed, thr, 1};
+    Presence pr;
+    if (live) pr = presence_of(w.N + lane, S);
+    const uint32_t mask = kReact && mp.has_mask && live ? __ldg(m.mask + t) : 0xffffffffu;
+    ClusterSender send{{slot.x, slot.y, slot.z, slot.w}, words, masks, S, 0};
+    uint32_t dirty = 0;
+    bool none = false;
+    const uint32_t bad = warp_step<false, kReact, false, true>(m, mp, S, w, v, t, live, mask, pr, &dirty, &none, err, send,
+                                                               make_uint4(0u, 0u, 0u, 0u), tried);
+    if (live) send.finish();
+    return (live ? dirty : 0u) | (bad << 16);
+}
 
 // Dynamic shared memory of a CTA of `warps` warps, in words: the warps'
 // (rd_warp.cuh), then per tet two parities of four slots of S words and of
@@ -804,8 +873,18 @@ k_run_cluster(const __grid_constant__ DevMesh m, const __grid_constant__ ModelPa
         send.words = words_at + (uint32_t)(p * B * 16 * S);
         send.masks = masks_at + (uint32_t)(p * B * 8);
         bool deferred = false;
-        bad |= warp_step<S_ == 1, kReact, false>(m, mp, S, w, v, t, live, mask, pr, &dirty, &deferred, s.err, send);
-        if (live) send.finish();
+        bad |= warp_step<S_ == 1, kReact, false, false>(m, mp, S, w, v, t, live, mask, pr, &dirty, &deferred, s.err,
+                                                        send);
+        if (live && !deferred) send.finish();
+        if (__ballot_sync(0xffffffffu, deferred)) {
+            const uint32_t x = step_deferred_in_cluster<kReact>(
+                m, mp, w.N, w.rx, v.period, v.tau_k, v.seed, v.thr,
+                make_uint4(send.slot[0], send.slot[1], send.slot[2], send.slot[3]), send.words, send.masks, t, deferred,
+                (pr.many >> 16) == 0u, s.err);
+            dirty |= x & 0xffffu;
+            bad |= x >> 16;
+            if (deferred) pr = presence_of(w.N + lane, S);
+        }
     }
     if (live)
         for (uint32_t bits = dirty; bits; bits &= bits - 1u) {
@@ -944,7 +1023,7 @@ void launch_period_s(const DevMesh& m, const ModelParams& mp, const DevState& s,
     const int64_t n = (a.t_hi > 0 ? a.t_hi : m.T) - a.t_lo;
     const int grid = (int)((n + block - 1) / block);
     if (!mp.any_reaction) {
-        // nothing to defer: without reactions one pass is both
+        // no reaction phase to defer: without reactions one pass is both
         launch_pass<S_, false, kPassAll>(m, mp, s, a, nullptr, nullptr, 0, grid, block, st);
     } else if (!split) {
         launch_pass<S_, true, kPassAll>(m, mp, s, a, nullptr, nullptr, 0, grid, block, st);

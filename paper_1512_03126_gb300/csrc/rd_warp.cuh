@@ -37,6 +37,10 @@ constexpr unsigned kAllLanes = 0xffffffffu;
 // (at least a full round of 32 Philox blocks); below it its blocks go to the
 // shared list.
 constexpr int32_t kCoopMin = 128;
+// A tet with this many molecules of a species is deferred to the pass with the
+// double-precision samplers: below it, with at most kMoleculeCut / 2 made or
+// consumed in the period, N* stays below kMoleculeCut.
+constexpr int32_t kDeferMin = (int32_t)kMoleculeCut / 2;
 constexpr int kListWords = 64;   // draw list of a warp (a round takes 32 entries)
 
 // Shared memory of one warp: N, D (draws of species a reaction touched) and
@@ -70,25 +74,32 @@ struct PeriodView {
     int thr_stride;
 };
 
-// Which species of a lane's tet have molecules, which more than one and which
-// more than kCoopMin: kept beside the column, so that loops run over set bits
+// Which species of a lane's tet have molecules, which more than one, which
+// more than kCoopMin or kDeferMin: kept beside the column, so that loops run over set bits
 // only.
 struct Presence {
-    uint32_t any = 0, two = 0, many = 0;
+    uint32_t any = 0, two = 0;
+    uint32_t many = 0;   // lower half: more than kCoopMin; upper half: kDeferMin or more
     // a species not seen before
     __device__ __forceinline__ void add(int s, int32_t n) {
         if (n > 0) any |= 1u << s;
         if (n > 1) two |= 1u << s;
-        if (n > kCoopMin) many |= 1u << s;
+        if (n > kCoopMin) many |= (n >= kDeferMin ? 0x10001u : 1u) << s;
     }
     __device__ __forceinline__ void set(int s, int32_t n) {
         const uint32_t bit = 1u << s;
         any &= ~bit;
         two &= ~bit;
-        many &= ~bit;
+        many &= ~(bit * 0x10001u);
         add(s, n);
     }
 };
+
+__device__ __forceinline__ Presence presence_of(const int32_t* Ncol, int S) {
+    Presence pr;
+    for (int s = 0; s < S; ++s) pr.add(s, Ncol[32 * s]);
+    return pr;
+}
 
 // Reactions of `on` whose reactants are present.
 __device__ __forceinline__ uint32_t possible_by_presence(const ModelParams& mp, const Presence& pr, int S, uint32_t on) {
@@ -230,7 +241,7 @@ __device__ __forceinline__ int react_fast(const ModelParams& mp, const uint2* rx
         dsum += dmax;
         x = xn;
         rw = rw_next;
-        if (++k > kMaxEvents) doubt = true;
+        if (++k > kMaxEvents || dsum > (float)(kMoleculeCut - kDeferMin - 1)) doubt = true;
     }
     if (!doubt && touched) {
         const float eps = dsum * ((float)(30 + m + 3 * k) * e) + (4.0f * e + 9.5367431640625e-07f);
@@ -392,7 +403,7 @@ static __device__ __noinline__ int4 diffuse_binomial(const double* __restrict__ 
 
 // The molecule-by-molecule draw that stops once all Nt molecules have left:
 // only where N* exceeds the count and more than Nt of the N* draws leave.
-static __device__ __noinline__ int4 draw_capped(uint64_t seed, uint32_t period, int key, int s, int32_t Nstar,
+__device__ __forceinline__ int4 draw_capped(uint64_t seed, uint32_t period, int key, int s, int32_t Nstar,
                                                 int32_t Nt, uint4 C) {
     int4 o = make_int4(0, 0, 0, 0);
     rdd::Stream ds(seed, (uint32_t)key, period, rdd::kPurposeDiffusion, (uint32_t)s);
@@ -433,14 +444,14 @@ __device__ __forceinline__ void count_block(const uint4& w, int m, const uint4& 
 // make a round with one block a lane.  The cost follows the number of blocks,
 // not the largest count of a lane or the species present in any lane.
 // Species with more than kCoopMin draws are drawn by the whole warp first,
-// and those from kMoleculeCut on by big(sp, N*).  Returns the species whose
+// and (kCalls) those from kMoleculeCut on by big(sp, N*).  Returns the species whose
 // acc words hold leavers-to-be.  All lanes must call it.  The per-lane loop
 // with a whole-warp pass per species and tet from 10 molecules on took one
 // serial pass a tet: 600 cycles each, up to 32 a warp.
 // With one species (kOne) every lane draws its own first block, without the
 // list, and only counts above four go on to it.  pre: the lane's thresholds
 // of species 0, when kPre says that they are loaded.
-template <bool kOne, bool kPre, class Big>
+template <bool kOne, bool kPre, bool kCalls, class Big>
 __device__ __forceinline__ uint32_t draw_all(int S, int64_t T, const WarpMem& w, const PeriodView& v, int t, int key,
                                              uint32_t present, uint32_t many, uint32_t touched, uint4 pre, Big big) {
     const int lane = threadIdx.x & 31;
@@ -450,7 +461,7 @@ __device__ __forceinline__ uint32_t draw_all(int S, int64_t T, const WarpMem& w,
         return ((touched >> sp) & 1u) ? w.D[32 * sp + lane] : w.N[32 * sp + lane];
     };
     // the species of each lane with draws of a usual number, and the others
-    uint32_t heavy = present & many;
+    uint32_t heavy = present & many & 0xffffu;
     for (uint32_t bits = touched & present; bits; bits &= bits - 1u) {
         const int sp = __ffs(bits) - 1;
         const int n = w.D[32 * sp + lane];
@@ -467,7 +478,7 @@ __device__ __forceinline__ uint32_t draw_all(int S, int64_t T, const WarpMem& w,
         const int sp = kOne ? 0 : __shfl_sync(kAllLanes, sp_own, src);
         const int nn = __shfl_sync(kAllLanes, heavy ? draws_of(sp_own) : 0, src);
         if (lane == src) heavy &= heavy - 1u;
-        if (nn >= (int)kMoleculeCut) {
+        if (kCalls && nn >= (int)kMoleculeCut) {
             if (lane == src) big(sp, nn);
             __syncwarp();
             continue;
@@ -546,21 +557,30 @@ __device__ __forceinline__ uint32_t draw_all(int S, int64_t T, const WarpMem& w,
 // counts and `pr` says which are not zero (all clear for a lane that is not
 // live); mask: the tet's reaction mask.  After it N and pr hold what stays;
 // emit(sp, o) was called by a lane for each species of which molecules leave
-// (o: per face).  Bits of the species whose count changed are added to
-// *dirty.  With kDefer, a lane whose tet needs the reaction phase leaves it
-// undone and answers true in *deferred.  Returns error bits.  All lanes must
-// call it.
-template <bool kOne, bool kReact, bool kDefer, bool kPre = false, class Emit>
+// (o: per face).  Bits of the species whose count changed are added to *dirty.
+// Returns error bits.  All lanes must call it.
+//
+// kCalls = false leaves out what is rare and needs a function call (the
+// double-precision repeat of a reaction phase, the binomial sampler): such a
+// tet is left as it was and *deferred set; its lane goes through the form
+// with kCalls afterwards (tried: its single-precision pass met a doubt
+// before and is not repeated).  A call in the hot loop costs every turn of it: what
+// lives across the call is spilled (80 to 100 local-memory instructions per 32
+// tets with three calls inside).  With kDefer every tet whose first waiting
+// time may fall inside the period is deferred, too.
+template <bool kOne, bool kReact, bool kDefer, bool kCalls, bool kPre = false, class Emit>
 __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParams& mp, int S, const WarpMem& w,
                                               const PeriodView& v, int t, bool live, uint32_t mask, Presence& pr,
                                               uint32_t* dirty, bool* deferred, uint32_t* err, Emit& emit,
-                                              uint4 pre = make_uint4(0u, 0u, 0u, 0u)) {
+                                              uint4 pre = make_uint4(0u, 0u, 0u, 0u), bool tried = false) {
     const int lane = threadIdx.x & 31;
     const int key = live ? key_of(m, t) : 0;
     uint32_t bad = 0, touched = 0;
+    uint32_t present = pr.any & mp.moves;
+    if (!kCalls && (pr.many >> 16)) *deferred = true;
     if (kReact) {
         const uint32_t on = mask & mp.kpos;
-        const uint32_t poss = live ? possible_by_presence(mp, pr, S, on) : 0u;
+        const uint32_t poss = live && (kCalls || !*deferred) ? possible_by_presence(mp, pr, S, on) : 0u;
         if (poss) {
             const float2 avf = __ldg(m.avv + t);
             if (kDefer) {
@@ -573,32 +593,42 @@ __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParam
                 const float need = a0 * v.tau_kf * 1.0001f * 1.0001f;
                 *deferred = !(need < 3.0e38f) || !((float)(uint32_t)(y >> 29) * 5.9604644775390625e-08f >= need) ||
                             (y >> 29) == 0ull;
-                if (*deferred) pr = Presence{};
             } else {
                 uint32_t tch = 0;
-                int r = react_fast(mp, w.rx, S, key, v, on, poss, avf, w.N + lane, w.D + lane, w.acc0 + lane, pr, &tch);
+                int r = kReactDoubt;
+                if (!kCalls || !tried)
+                    r = react_fast(mp, w.rx, S, key, v, on, poss, avf, w.N + lane, w.D + lane, w.acc0 + lane, pr, &tch);
                 if (r == kReactDoubt) {
-                    tch = react_exact(mp, key, v.period, v.tau_k, v.seed, m.vol[t], mask, w.N + lane, w.D + lane, err);
-                    bad |= tch >> 16;
-                    tch &= 0xffffu;
-                    for (uint32_t bits = tch; bits; bits &= bits - 1u)
-                        pr.set(__ffs(bits) - 1, w.N[32 * (__ffs(bits) - 1) + lane]);
+                    if constexpr (kCalls) {
+                        tch = react_exact(mp, key, v.period, v.tau_k, v.seed, m.vol[t], mask, w.N + lane, w.D + lane,
+                                          err);
+                        bad |= tch >> 16;
+                        tch &= 0xffffu;
+                        for (uint32_t bits = tch; bits; bits &= bits - 1u)
+                            pr.set(__ffs(bits) - 1, w.N[32 * (__ffs(bits) - 1) + lane]);
+                    } else {
+                        *deferred = true;
+                    }
                 }
                 *dirty |= tch;
                 if (mp.rule != kRuleEnd) touched = tch;   // first order: the draw uses N(tau_k)
+                present = pr.any & mp.moves;
             }
         }
     }
-    const uint32_t drawn = draw_all<kOne, kPre>(S, m.T, w, v, t, key, pr.any & mp.moves, pr.many, touched, pre,
-                                                [&](int sp, int32_t star) {
-        const int32_t Nt = w.N[32 * sp + lane];
-        const int4 o = diffuse_binomial(m.G, m.g, t, key, sp, mp.D[sp], v.period, v.tau_k, v.seed, Nt, star);
-        const int32_t all = o.x + o.y + o.z + o.w;
-        if (all > 0) {
-            w.N[32 * sp + lane] = Nt - all;
-            pr.set(sp, Nt - all);
-            *dirty |= 1u << sp;
-            emit(sp, o);
+    if (!kCalls && *deferred) present = 0u;
+    const uint32_t drawn = draw_all<kOne, kPre, kCalls>(S, m.T, w, v, t, key, present, pr.many, touched, pre,
+                                                        [&](int sp, int32_t star) {
+        if constexpr (kCalls) {
+            const int32_t Nt = w.N[32 * sp + lane];
+            const int4 o = diffuse_binomial(m.G, m.g, t, key, sp, mp.D[sp], v.period, v.tau_k, v.seed, Nt, star);
+            const int32_t all = o.x + o.y + o.z + o.w;
+            if (all > 0) {
+                w.N[32 * sp + lane] = Nt - all;
+                pr.set(sp, Nt - all);
+                *dirty |= 1u << sp;
+                emit(sp, o);
+            }
         }
     });
     for (uint32_t bits = drawn; bits; bits &= bits - 1u) {

@@ -45,8 +45,9 @@ struct SlotDesc {
     const uint4* thr_last;   // thresholds for the shortened last period
     int32_t* N[2];           // count buffers [S][T]; the slice starts in N[0]
     uint32_t* bits[2];       // active-tet bitmaps of 2^wshift words, by period parity in the slice
-    int32_t wshift;          // tet t is bit t >> wshift of word t & (2^wshift - 1); at least as many words
-                             // as the cluster has warps
+    int32_t wshift;          // at least as many words as the cluster has warps
+    int32_t sm;              // counts and bitmaps in the cluster's shared memory
+    int32_t gshift;          // runs of 2^gshift consecutive tets share a word (see word_of)
     const uint4* packed;     // one species: {src, thr} per tet
     int32_t* N2;             // one species: counts of both parities interleaved
     uint64_t seed;
@@ -93,13 +94,11 @@ __device__ __forceinline__ void red_or_cluster(uint32_t addr, uint32_t v) {
 
 constexpr int kWarps = kRunBlock / 32;
 constexpr int kGroup = 8;                   // bitmap columns (32 words each) a warp loads at once
+constexpr int kSmCols = 2;                  // of a simulation in shared memory: all of them
 
-// Dynamic shared memory of a warp, in words: the step's (rd_warp.cuh) and,
-// unless the bitmaps are in shared memory themselves, the words of its current
-// batch.
-__host__ __device__ inline int engine_warp_words(int S, bool react, bool sm) {
-    return warp_words(S, react) + (sm ? 0 : 32 * kGroup);
-}
+// Dynamic shared memory of a warp, in words: the step's (rd_warp.cuh) and the
+// bitmap words of its current batch.
+__host__ __device__ inline int engine_warp_words(int S, bool react) { return warp_words(S, react) + 32 * kGroup; }
 
 // A simulation of one species in the cluster's shared memory (kSm): a CTA
 // keeps the words of its warps, wpc = W / kC of them, in both parities' bitmaps
@@ -125,6 +124,17 @@ __device__ __forceinline__ int nth_set_bit(uint32_t w, int k) {
     return p;
 }
 
+// The place of tet t in a bitmap of 2^ws words: run t >> gs of consecutive tets
+// goes to word (t >> gs) mod 2^ws, so that a word holds 32 / 2^gs runs far
+// apart.
+__device__ __forceinline__ int word_of(int t, int ws, int gs) { return (t >> gs) & ((1 << ws) - 1); }
+__device__ __forceinline__ int bit_of(int t, int ws, int gs) {
+    return ((t >> (gs + ws)) << gs) | (t & ((1 << gs) - 1));
+}
+__device__ __forceinline__ int tet_of(int word, int bit, int ws, int gs) {
+    return ((bit >> gs) << (gs + ws)) | (word << gs) | (bit & ((1 << gs) - 1));
+}
+
 // Shared memory of the engine kernel.
 __shared__ int32_t s_item;                          // work-item index (first CTA of the cluster)
 __shared__ unsigned long long s_mass[3];            // [0] molecules of the simulation (all species) at the
@@ -143,16 +153,17 @@ struct GlobalView {
     uint32_t* bcur;
     uint32_t* bnext;
     int64_t T;
-    int ws;
+    int ws, gs;
     static constexpr int stride = kOne ? 2 : 1;
-    __device__ __forceinline__ GlobalView(const SlotDesc& d, int r) : bcur(d.bits[r]), bnext(d.bits[r ^ 1]), T(d.m.T), ws(d.wshift) {
+    __device__ __forceinline__ GlobalView(const SlotDesc& d, int r)
+        : bcur(d.bits[r]), bnext(d.bits[r ^ 1]), T(d.m.T), ws(d.wshift), gs(d.gshift) {
         cur = kOne ? d.N2 + r : d.N[r];
         next = kOne ? d.N2 + (r ^ 1) : d.N[r ^ 1];
     }
     __device__ __forceinline__ int32_t load(int s, int t) const { return __ldcg(cur + (s * T + t) * stride); }
     __device__ __forceinline__ void clear(int s, int t) const { cur[(s * T + t) * stride] = 0; }
     __device__ __forceinline__ void add(int s, int t, int32_t n) const { red_add(next + (s * T + t) * stride, n); }
-    __device__ __forceinline__ void mark(int t) const { red_or(bnext + (t & ((1 << ws) - 1)), 1u << (t >> ws)); }
+    __device__ __forceinline__ void mark(int t) const { red_or(bnext + word_of(t, ws, gs), 1u << bit_of(t, ws, gs)); }
     __device__ __forceinline__ void send(int t, int32_t n, bool more) const {
         add(0, t, n);
         if (more) mark(t);
@@ -285,12 +296,21 @@ __device__ __forceinline__ uint32_t engine_round(const SlotDesc& d, const ModelP
     if (live && (kCalls || !*deferred)) {
         bool keep = pr.any != 0u;
         if (kReact && d.zero_order) keep = keep || (mask & d.zero_order) != 0u;
-        for (uint32_t bits = had; bits; bits &= bits - 1u) c.clear(__ffs(bits) - 1, t);
-        for (uint32_t bits = pr.any; bits; bits &= bits - 1u) {
-            const int s = __ffs(bits) - 1;
-            const int32_t n = w.N[32 * s + lane];
-            c.keep(s, t, n);
-            if (kReact) delta += n;
+        if (kOne) {
+            if (had) c.clear(0, t);
+            if (pr.any) {
+                const int32_t n = w.N[lane];
+                c.keep(0, t, n);
+                if (kReact) delta += n;
+            }
+        } else {
+            for (uint32_t bits = had; bits; bits &= bits - 1u) c.clear(__ffs(bits) - 1, t);
+            for (uint32_t bits = pr.any; bits; bits &= bits - 1u) {
+                const int s = __ffs(bits) - 1;
+                const int32_t n = w.N[32 * s + lane];
+                c.keep(s, t, n);
+                if (kReact) delta += n;
+            }
         }
         if (kReact) delta += scatter.sent - held;
         if (more) {
@@ -316,7 +336,9 @@ struct WarpPeriod {
     static constexpr int kW = kC * kWarps;
     static constexpr int kWShift = kC == 1 ? 4 : (kC == 2 ? 5 : (kC == 4 ? 6 : 7));
     static_assert((1 << kWShift) == kW, "warps of a cluster");
-    int S, per, word0;         // this warp's words: `per` from word0 on
+    int S, per;                // this warp's words: `per`, number k is word0 + k * step (kSm: of the CTA's)
+    int word0;
+    static constexpr int step = kSm ? 1 : kW;
     WarpMem w;
     PeriodView v;
     View c;
@@ -325,7 +347,7 @@ struct WarpPeriod {
     bool more;
 
     static __device__ __forceinline__ View view(const SlotDesc& d, int r, int S) {
-        if constexpr (kSm) return View(d, r, s_warp + kWarps * engine_warp_words(S, kReact, true));
+        if constexpr (kSm) return View(d, r, s_warp + kWarps * engine_warp_words(S, kReact));
         else return View(d, r);
     }
     static __device__ __forceinline__ PeriodView period_view(const SlotDesc& d, int q) {
@@ -337,36 +359,34 @@ struct WarpPeriod {
     }
     __device__ __forceinline__ WarpPeriod(const SlotDesc& d, int q)
         : S(kOne ? 1 : d.S), per((1 << d.wshift) >> kWShift),
-          w(s_warp + (threadIdx.x >> 5) * engine_warp_words(S, kReact, kSm), S, kReact, s_mp.rx), v(period_view(d, q)),
+          w(s_warp + (threadIdx.x >> 5) * engine_warp_words(S, kReact), S, kReact, s_mp.rx), v(period_view(d, q)),
           c(view(d, (q - d.q0) & 1, S)), more(q + 1 < d.q1) {
         const int warp = threadIdx.x >> 5;
         const int rank = kC > 1 ? (int)cooperative_groups::this_cluster().block_rank() : 0;
-        word0 = (rank * kWarps + warp) * per;
+        word0 = (rank * kWarps + warp) * (kSm ? per : 1);
         words = c.bcur + (kSm ? warp * per : word0);
-        wb = reinterpret_cast<uint32_t*>(s_warp + warp * engine_warp_words(S, kReact, kSm) + warp_words(S, kReact));
+        wb = reinterpret_cast<uint32_t*>(s_warp + warp * engine_warp_words(S, kReact) + warp_words(S, kReact));
     }
 };
 
-// The tets of a batch whose bits the rounds set back, with the
-// double-precision samplers.
+// The warp's tets whose bits the rounds set back, with the double-precision
+// samplers.
 template <bool kOne, bool kReact, int kC, bool kSm>
-__device__ __noinline__ uint32_t run_deferred(int q, int b, uint32_t* err, unsigned long long* mass_delta) {
+__device__ __noinline__ uint32_t run_deferred(int q, uint32_t* err, unsigned long long* mass_delta) {
     const SlotDesc& d = s_desc;
     const WarpPeriod<kOne, kReact, kC, kSm> p(d, q);
     const int lane = threadIdx.x & 31;
     uint32_t bad = 0;
-    for (int kk = 0; kk < kGroup; ++kk) {
-        const int at = (b * kGroup + kk) * 32 + lane;
-        const bool mine = at < p.per;
+    for (int w0 = 0; w0 < p.per; w0 += 32) {
+        const int at = w0 + lane;
         uint32_t word = 0u;
-        if (mine) {
-            uint32_t* from = kSm ? p.words + at : p.wb + kk * 32 + lane;
-            word = *from;
-            *from = 0u;
+        if (at < p.per) {
+            word = kSm ? p.words[at] : __ldcg(p.words + at * p.step);
+            if (word) p.words[at * p.step] = 0u;
         }
         while (__ballot_sync(kAllLanes, word != 0u)) {
             const bool live = word != 0u;
-            const int t = live ? ((__ffs(word) - 1) << d.wshift) + p.word0 + at : 0;
+            const int t = live ? tet_of(p.word0 + at * p.step, __ffs(word) - 1, d.wshift, kSm ? 0 : d.gshift) : 0;
             word &= word - 1u;
             bool none = false;
             bad |= engine_round<kOne, kReact, true>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta, &none);
@@ -381,99 +401,96 @@ __device__ __noinline__ uint32_t run_deferred(int q, int b, uint32_t* err, unsig
 // molecules and of its crowded tets: dealing runs of 128 consecutive tets
 // left warps waiting at the period barrier for the one that held the source
 // (15 of 24 stall cycles an instruction).  The words go to the cluster's kW
-// warps in equal contiguous parts.  A column is 32 words, one per lane; a warp loads
-// kGroup of its columns at once and clears them for their next use.  With a
-// prefix sum of a column's popcounts each lane finds a set bit of its own (a
-// search over the sums and one inside the word: a fixed 60 instructions, where
-// writing the bits of a dense word into a list took 32 turns of one lane);
-// whenever 32 tets are at hand, one round steps them (warp_step), and adds
-// what stays and what leaves into the next counts.
+// warps in equal contiguous parts.  A warp loads a batch of up to kGroup
+// columns (32 words, one per lane) at once and clears them for their next use.
+// One prefix sum over the lanes' set bits of the whole batch lets each lane
+// find a tet of its own (a search over the sums, the column, the bit in the
+// word: a fixed 110 instructions a round; a sum and a search for every column,
+// nearly all of which hold a few bits of a sparse mesh, made the 512-cube
+// ensemble three times slower); 32 tets make a round (engine_round).
+//
+// Out of line and free of calls, like run_deferred beside it: with the round
+// in the kernel's own loop, what it keeps across the call of run_deferred
+// (addresses and descriptor fields lifted out of the loops) sat in local
+// memory, 110 loads a round.
+struct PeriodResult {
+    uint32_t bad, done, late;   // error bits, tets visited, whether some were deferred
+};
 template <bool kOne, bool kReact, int kC, bool kSm>
-__device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned long long* mass_delta,
-                                               unsigned long long* done) {
+__device__ __noinline__ PeriodResult run_period(int q, uint32_t* err, unsigned long long* mass_delta) {
     const SlotDesc& d = s_desc;
     const int lane = threadIdx.x & 31;
     const WarpPeriod<kOne, kReact, kC, kSm> p(d, q);
-    uint32_t bad = 0;
-    unsigned long long visited = 0;
-    for (int b = 0; b * kGroup * 32 < p.per; ++b) {
-        const int at = b * kGroup * 32 + lane;
-        uint32_t any = 0;
-        if (kSm) {
-            for (int kk = 0; kk < kGroup && b * kGroup + kk < (p.per + 31) >> 5; ++kk)
-                if (at + kk * 32 < p.per && p.words[at + kk * 32]) any |= 1u << kk;
-        } else {
-            uint32_t wds[kGroup];
+    constexpr int kCols = kSm ? kSmCols : kGroup;
+    uint32_t bad = 0, done = 0;
+    bool late = false;              // some tet was deferred
+    for (int w0 = 0; w0 < p.per; w0 += 32 * kCols) {
+        int own = 0;
+        {
+            uint32_t wds[kCols];
 #pragma unroll
-            for (int kk = 0; kk < kGroup; ++kk) wds[kk] = at + kk * 32 < p.per ? __ldcg(p.words + at + kk * 32) : 0u;
+            for (int kk = 0; kk < kCols; ++kk) {
+                const int i = w0 + kk * 32 + lane;
+                wds[kk] = i < p.per ? (kSm ? p.words[i] : __ldcg(p.words + i * p.step)) : 0u;
+            }
 #pragma unroll
-            for (int kk = 0; kk < kGroup; ++kk) {
-                if (wds[kk]) p.words[at + kk * 32] = 0u;
+            for (int kk = 0; kk < kCols; ++kk) {
+                if (wds[kk]) p.words[(w0 + kk * 32 + lane) * p.step] = 0u;
                 p.wb[kk * 32 + lane] = wds[kk];
-                any |= wds[kk] ? 1u << kk : 0u;
+                own += __popc(wds[kk]);
             }
         }
-        uint32_t columns = __reduce_or_sync(kAllLanes, any);   // those that hold a set bit
-        int pend = 0, cnt = 0;      // tets not yet run: lane i < cnt holds one
-        bool late = false;          // some tet was deferred
-        while (columns) {
-            const int kk = __ffs(columns) - 1;
-            columns &= columns - 1;
-            uint32_t word = 0u;
-            if (at + kk * 32 < p.per) {
-                uint32_t* from = kSm ? p.words + at + kk * 32 : p.wb + kk * 32 + lane;
-                word = *from;
-                *from = 0u;
-            }
-            const int own = __popc(word);
-            int inc = own;
+        int inc = own;
 #pragma unroll
-            for (int dd = 1; dd < 32; dd <<= 1) {
-                const int y = __shfl_up_sync(kAllLanes, inc, dd);
-                if (lane >= dd) inc += y;
-            }
-            const int total = __shfl_sync(kAllLanes, inc, 31);
-            int off = cnt, avail = cnt + total;
-            visited += (unsigned long long)total;
-            for (;;) {
-                // the lane's tet: one that was left over, or the column's set bit number lane - off
-                const int e = lane - off;
-                int from = 0;
+        for (int dd = 1; dd < 32; dd <<= 1) {
+            const int y = __shfl_up_sync(kAllLanes, inc, dd);
+            if (lane >= dd) inc += y;
+        }
+        const int total = __shfl_sync(kAllLanes, inc, 31);
+        done += (uint32_t)total;
+        __syncwarp();
+        for (int e0 = 0; e0 < total; e0 += 32) {
+            // the lane's tet: the batch's set bit number e0 + lane
+            const int e = e0 + lane;
+            const bool live = e < total;
+            int from = 0;
 #pragma unroll
-                for (int step = 16; step > 0; step >>= 1)
-                    if (__shfl_sync(kAllLanes, inc, from + step - 1) <= e) from += step;
-                const int k = e - __shfl_sync(kAllLanes, inc - own, from);
-                const int bit = nth_set_bit(__shfl_sync(kAllLanes, word, from), k);
-                const int t_new = (bit << d.wshift) + p.word0 + (b * kGroup + kk) * 32 + from;
-                const int t_lane = e < 0 ? pend : t_new;
-                if (avail < 32 && columns) {
-                    pend = t_lane;
-                    cnt = avail;
-                    break;
-                }
-                const bool live = lane < avail;
-                const int t = live ? t_lane : 0;
-                off -= 32;
-                avail = max(avail - 32, 0);
-                bool deferred = false;
-                bad |= engine_round<kOne, kReact, false>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta,
-                                                         &deferred);
-                if (__ballot_sync(kAllLanes, deferred)) {
-                    late = true;
-                    if (deferred) {   // back into its word
-                        const int i = (t & ((1 << d.wshift) - 1)) - p.word0;
-                        atomicOr(kSm ? p.words + i : p.wb + (i - b * kGroup * 32), 1u << (t >> d.wshift));
+            for (int step = 16; step > 0; step >>= 1)
+                if (__shfl_sync(kAllLanes, inc, from + step - 1) <= e) from += step;
+            int k = e - __shfl_sync(kAllLanes, inc - own, from);
+            uint32_t word = p.wb[from];
+            int col = 0;
+            {
+#pragma unroll
+                for (int kk = 1; kk < kCols; ++kk) {
+                    const int c = __popc(word);
+                    if (col == kk - 1 && k >= c) {
+                        k -= c;
+                        col = kk;
+                        word = p.wb[kk * 32 + from];
                     }
                 }
-                __syncwarp();
-                if (avail == 0) break;   // (only the batch's last column gets here with none left)
             }
-            if (avail == 0) cnt = 0;
+            const int i = w0 + col * 32 + from;
+            const int bit = nth_set_bit(word, k);
+            const int t = live ? tet_of(p.word0 + i * p.step, bit, d.wshift, kSm ? 0 : d.gshift) : 0;
+            bool deferred = false;
+            bad |= engine_round<kOne, kReact, false>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta,
+                                                     &deferred);
+            if (__ballot_sync(kAllLanes, deferred)) {
+                // back into the bitmap, for the pass after the batch
+                late = true;
+                if (deferred) {
+                    if (kSm) atomicOr(p.words + i, 1u << bit);
+                    else red_or(p.words + i * p.step, 1u << bit);
+                }
+            }
+            __syncwarp();
         }
-        if (late) bad |= run_deferred<kOne, kReact, kC, kSm>(q, b, err, mass_delta);
     }
-    *done += visited;
-    return bad;
+    if (late && !kSm) __threadfence();   // the bits set back are read by other lanes
+    __syncwarp();
+    return PeriodResult{bad, done, late ? 1u : 0u};
 }
 
 // One simulation per cluster of kC CTAs (kC = 1: per CTA).  The cluster's
@@ -492,14 +509,15 @@ __device__ __forceinline__ uint32_t run_period(int q, uint32_t* err, unsigned lo
 // at the end of the slice); the molecule total of the simulation, tracked per
 // period (each round adds what its reactions make or consume), is kept
 // below 2^32 - 1 so that no count can wrap all the way round unseen.
-// With kSm (one species, a mesh whose counts fit, see sm_bytes) the counts and
+// Where a simulation's descriptor says so (one species, a mesh whose counts
+// fit, see sm_bytes) the counts and
 // bitmaps are in the cluster's shared memory for the slice, and every add and
 // OR goes to the owning CTA's.  In global memory a period of a 24^3-cell cube
 // on 8 CTAs took 18,700 cycles of which a warp worked 8,500 (2,000 to load its
 // words, 900 for the counts); the rest was the barrier's wait for the adds to
 // reach L2.
-template <int S_, bool kReact, int kC, bool kSm>
-__global__ void __launch_bounds__(kRunBlock, 2)
+template <int S_, bool kReact, int kC>
+__global__ void __launch_bounds__(kRunBlock, 1)
 k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__ mps, const int32_t* __restrict__ order,
              int32_t n_items, int32_t* head, uint32_t* err, unsigned long long* processed,
              unsigned long long* times) {
@@ -547,17 +565,20 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
         const int S = kOne ? 1 : d.S;
         const int W = 1 << d.wshift;
         constexpr bool inter = kOne;   // interleaved counts
+        const bool sm = kOne && d.sm != 0;
         uint32_t bad = 0;
         // initial bitmap: occupied tets and tets with a zero-order reaction on
         // (a thread a word; its tets are W apart, so a warp's loads are
         // contiguous); and the simulation's molecule total
         unsigned long long mine = 0;
-        const int wpc = W / kC;   // kSm: the words, and the tets, of this CTA
-        int32_t* const data = s_warp + kWarps * engine_warp_words(S, kReact, true);
-        for (int i = (kSm ? 0 : rank * kRunBlock) + threadIdx.x; i < (kSm ? wpc : W); i += kSm ? kRunBlock : kC * kRunBlock) {
-            const int wi = kSm ? rank * wpc + i : i;
+        const int wpc = W / kC;   // in shared memory: the words, and the tets, of this CTA
+        int32_t* const data = s_warp + kWarps * engine_warp_words(S, kReact);
+        for (int i = (sm ? 0 : rank * kRunBlock) + threadIdx.x; i < (sm ? wpc : W); i += sm ? kRunBlock : kC * kRunBlock) {
+            const int wi = sm ? rank * wpc + i : i;
             uint32_t word = 0;
-            for (int t = wi, bit = 0; t < T; t += W, ++bit) {
+            for (int bit = 0; bit < 32; ++bit) {
+                const int t = tet_of(wi, bit, d.wshift, sm ? 0 : d.gshift);
+                if (t >= T) continue;
                 bool occ = false;
                 if (kReact && d.zero_order)
                     occ = ((s_mp.has_mask ? d.m.mask[t] : 0xffffffffu) & d.zero_order) != 0u;
@@ -566,12 +587,12 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
                     occ = occ || c > 0;
                     mine += (uint32_t)max(c, 0);
                     if (c < 0) bad |= kErrNegative;
-                    if (kSm) reinterpret_cast<int2*>(data + 2 * wpc)[bit * wpc + i] = make_int2(c, 0);
+                    if (sm) reinterpret_cast<int2*>(data + 2 * wpc)[bit * wpc + i] = make_int2(c, 0);
                     else if (inter) reinterpret_cast<int2*>(d.N2)[t] = make_int2(c, 0);
                 }
                 if (occ) word |= 1u << bit;
             }
-            if (kSm) {
+            if (sm) {
                 reinterpret_cast<uint32_t*>(data)[i] = word;
                 reinterpret_cast<uint32_t*>(data)[wpc + i] = 0u;
             } else {
@@ -595,14 +616,26 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
         for (int q = d.q0; q < d.q1; ++q) {
             csync();   // the previous period's adds and bits are complete
             if (q > d.q0) account(q - 1);
-            bad |= run_period<kOne, kReact, kC, kSm>(q, err, &mass[1 + (q & 1)], &item_done);
+            unsigned long long* made = &mass[1 + (q & 1)];
+            PeriodResult r;
+            if (sm) {
+                if constexpr (kOne) {
+                    r = run_period<true, kReact, kC, true>(q, err, made);
+                    if (r.late) bad |= run_deferred<true, kReact, kC, true>(q, err, made);
+                }
+            } else {
+                r = run_period<kOne, kReact, kC, false>(q, err, made);
+                if (r.late) bad |= run_deferred<kOne, kReact, kC, false>(q, err, made);
+            }
+            bad |= r.bad;
+            item_done += r.done;
         }
         csync();   // every add of the slice is complete
         account(d.q1 - 1);
         // a count the last period's adds took past 2^31-1 reads negative
         {
             const int half = (d.q1 - d.q0) & 1;
-            if (kSm) {
+            if (sm) {
                 for (int i = threadIdx.x; i < wpc; i += kRunBlock)
                     for (int t = rank * wpc + i, bit = 0; t < T; t += W, ++bit) {
                         const int32_t c = data[2 * wpc + 2 * (bit * wpc + i) + half];
@@ -610,7 +643,7 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
                         d.N[0][t] = c;
                     }
             }
-            for (int t = rank * kRunBlock + threadIdx.x; !kSm && t < T; t += kC * kRunBlock) {
+            for (int t = rank * kRunBlock + threadIdx.x; !sm && t < T; t += kC * kRunBlock) {
                 if (inter) {
                     // the slice's counts are in the pairs' half (q1 - q0) & 1;
                     // hand them back in N[0]
@@ -664,32 +697,29 @@ struct EngineLaunch {
     int sms;
     int clusters;
     int S;                // largest species count of the group's simulations
-    bool spread = false;  // one CTA an SM
     size_t data = 0;      // bytes of counts and bitmaps in a CTA's shared memory (0: in global memory)
     int used = 0;         // clusters launched
     int max_active = 0;   // clusters resident at once (occupancy query)
     bool query_only = false;   // fill max_active, launch nothing
 };
 
-// Shared memory of a CTA so that two of them fit on an SM, and what of it one
-// species' counts and bitmaps may take.
-constexpr size_t kCtaSmem = 112 * 1024;
+// What of a CTA's shared memory one species' counts and bitmaps may take: the rest
+// of the SM's 256 KB caches the records of simulations that stay in global memory.
 inline size_t sm_data_limit(bool react) {
-    return kCtaSmem - (sizeof(SlotDesc) + sizeof(ModelParams) + 256) -
-           (size_t)kWarps * engine_warp_words(1, react, true) * sizeof(int32_t);
+    return 128 * 1024 - (sizeof(SlotDesc) + sizeof(ModelParams) + 256) -
+           (size_t)kWarps * engine_warp_words(1, react) * sizeof(int32_t);
 }
 
-template <int SA, bool R, int C, bool SM>
+template <int SA, bool R, int C>
 cudaError_t launch_cluster(EngineLaunch& L) {
-    auto kern = k_engine_run<SA, R, C, SM>;
+    auto kern = k_engine_run<SA, R, C>;
     // the attribute covers every group of this kernel, whatever its species
-    const size_t most = (size_t)kWarps * engine_warp_words(SA == 1 ? 1 : kMaxS, R, SM) * sizeof(int32_t) +
-                        (SM ? sm_data_limit(R) : 0) + kCtaSmem + 4096;
+    const size_t most = (size_t)kWarps * engine_warp_words(SA == 1 ? 1 : kMaxS, R) * sizeof(int32_t) +
+                        (SA == 1 ? sm_data_limit(R) : 0);
     cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)std::min<size_t>(most, 220 * 1024));
+                                          (int)most);
     if (ce != cudaSuccess) return ce;
-    size_t dyn = (size_t)kWarps * engine_warp_words(L.S, R, SM) * sizeof(int32_t) + L.data;
-    if (L.spread) dyn = std::max<size_t>(dyn, kCtaSmem + 4096);   // more than half of an SM's
+    const size_t dyn = (size_t)kWarps * engine_warp_words(L.S, R) * sizeof(int32_t) + L.data;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C, 1, 1);
     cfg.blockDim = dim3(kRunBlock, 1, 1);
@@ -727,12 +757,12 @@ cudaError_t launch_cluster(EngineLaunch& L) {
                               L.times);
 }
 
-template <int SA, bool SM>
+template <int SA>
 cudaError_t launch_run_sa(bool react, int cluster, EngineLaunch& L) {
-    if (cluster >= 8) return react ? launch_cluster<SA, true, 8, SM>(L) : launch_cluster<SA, false, 8, SM>(L);
-    if (cluster == 4) return react ? launch_cluster<SA, true, 4, SM>(L) : launch_cluster<SA, false, 4, SM>(L);
-    if (cluster == 2) return react ? launch_cluster<SA, true, 2, SM>(L) : launch_cluster<SA, false, 2, SM>(L);
-    return react ? launch_cluster<SA, true, 1, SM>(L) : launch_cluster<SA, false, 1, SM>(L);
+    if (cluster >= 8) return react ? launch_cluster<SA, true, 8>(L) : launch_cluster<SA, false, 8>(L);
+    if (cluster == 4) return react ? launch_cluster<SA, true, 4>(L) : launch_cluster<SA, false, 4>(L);
+    if (cluster == 2) return react ? launch_cluster<SA, true, 2>(L) : launch_cluster<SA, false, 2>(L);
+    return react ? launch_cluster<SA, true, 1>(L) : launch_cluster<SA, false, 1>(L);
 }
 
 // log2 of a bitmap's words: at least T / 32 and the warps of a cluster.
@@ -743,19 +773,26 @@ inline int words_shift(int64_t T, int cluster) {
 }
 
 // Kernel groups of a step: by species class (1, 2, up to 4, up to 8, more: it
-// sets the shared memory of a warp) with and without reactions, and one
-// species in shared memory with and without.
-constexpr int kGroups = 12;
-inline int group_species(int g) {
-    constexpr int most[6] = {1, 2, 4, 8, kMaxS, 1};
-    return most[g >> 1];
+// sets the shared memory of a warp), with and without reactions.
+constexpr int kGroups = 10;
+inline int group_of(int S, int R) {
+    const int c = S <= 1 ? 0 : (S <= 2 ? 1 : (S <= 4 ? 2 : (S <= 8 ? 3 : 4)));
+    return 2 * c + (R > 0 ? 1 : 0);
 }
 cudaError_t launch_group(int g, int cluster, EngineLaunch& L) {
-    const bool react = (g & 1) != 0;
-    L.S = group_species(g);
-    if (g >= 10) return launch_run_sa<1, true>(react, cluster, L);
-    L.data = 0;
-    return g >> 1 ? launch_run_sa<0, false>(react, cluster, L) : launch_run_sa<1, false>(react, cluster, L);
+    constexpr int most[5] = {1, 2, 4, 8, kMaxS};
+    L.S = most[g >> 1];
+    return g >> 1 ? launch_run_sa<0>((g & 1) != 0, cluster, L) : launch_run_sa<1>((g & 1) != 0, cluster, L);
+}
+
+// Bytes of a CTA's shared memory that a simulation's counts and bitmaps take,
+// or 0 where they stay in global memory: one species, all its words in a
+// warp's kSmCols columns, and room.
+inline size_t sm_need(int64_t T, int S, int R, int cluster) {
+    const int shift = words_shift(T, cluster);
+    if (S != 1 || (1 << shift) > 32 * kSmCols * cluster * kWarps) return 0;
+    const size_t b = sm_bytes(T, shift, cluster);
+    return b <= sm_data_limit(R > 0) ? b : 0;
 }
 
 // Every instantiation of the engine kernel is launched once, with no work
@@ -784,7 +821,7 @@ void warm_engine_kernels(int32_t* head, uint32_t* err, unsigned long long* proce
         return;
     }
     EngineLaunch W{nullptr, nullptr, nullptr, 0, head, err, processed, nullptr, (cudaStream_t)0, sms, 1, 1};
-    for (int g : {0, 1, 2, 3, 10, 11})   // every kernel: one species, several, one in shared memory
+    for (int g = 0; g < 4; ++g)   // every kernel: one species or several, with or without reactions
         for (int c = 1; c <= 8; c <<= 1) {
             if (launch_group(g, c, W) == cudaSuccess) note_launch();
             cudaGetLastError();   // a failure here shows again, and is reported, at a real launch
@@ -824,8 +861,7 @@ struct rdsplit_engine {
     cudaEvent_t ev_fork = nullptr;
     cudaEvent_t ev_join[kGroups] = {};
     int32_t cluster = 2;                      // CTAs per simulation (1, 2, 4 or 8)
-    bool cluster_auto = false;                // it and `spread` chosen at each step for the simulations at hand
-    bool spread = false;                      // one CTA an SM (else two)
+    bool cluster_auto = false;                // chosen at each step for the simulations at hand
     std::vector<rdsplit_mesh_t> slot_mesh;    // null = free
     std::vector<SlotDesc> h_desc;
     std::vector<int32_t> slot_q;              // local periods done
@@ -883,58 +919,46 @@ void plan_periods(double t, double tau, double t_end, int64_t* P, double* tau_la
     *P = n;
 }
 
-// CTAs per simulation, and per SM, for a whole ensemble: the choice whose
-// schedule (longest first, each simulation to the cluster that is free first)
-// ends soonest.  A period costs a part that no CTA takes off (its serial chain
-// and barrier) and one that they share: 36, 22, 14 and 10 us were measured on
-// 1, 2, 4 and 8 CTAs for 3,000 occupied tets; and a CTA that shares its SM with
-// another takes about 1.7 times as long.
-template <class Cls>
-void choose_cluster(rdsplit_engine* e, const std::vector<int32_t>& items, const Cls& cls_at) {
+// What a simulation costs a cluster of c CTAs, in arbitrary units: a period has
+// a part that no CTA takes off (its serial chain and barrier) and one that they
+// share (36, 22, 14 and 10 us were measured on 1, 2, 4 and 8 CTAs for 3,000
+// occupied tets).
+inline double slice_cost(const rdsplit_engine* e, int32_t s, int c) {
+    const rdsplit_mesh* h = e->slot_mesh[s];
+    return (double)(e->h_desc[s].q1 - e->h_desc[s].q0) * (0.25 + std::min(1.0, (double)h->T / 8192.0) * h->S / c);
+}
+
+// CTAs per simulation for a whole ensemble: the size whose schedule (longest
+// first, each simulation to the cluster that is free first) ends soonest.
+int choose_cluster(rdsplit_engine* e, const std::vector<int32_t>& items) {
     int best = 2;
-    bool best_spread = false;
     double best_end = HUGE_VAL;
     for (int c = 1; c <= 8; c <<= 1) {
+        EngineLaunch Q{nullptr, nullptr, nullptr, 1, nullptr, nullptr, nullptr, nullptr, e->stream, e->sms, 0, 1};
+        Q.query_only = true;
         std::vector<double> cost;
-        int32_t largest = items[0];
-        for (int32_t s : items) {
-            const rdsplit_mesh* h = e->slot_mesh[s];
-            if (h->T > e->slot_mesh[largest]->T) largest = s;
-            const double shared = std::min(1.0, (double)h->T / 8192.0) * h->S;
-            cost.push_back((double)(e->h_desc[s].q1 - e->h_desc[s].q0) * (0.25 + shared / c));
+        for (int32_t s : items) cost.push_back(slice_cost(e, s, c));
+        const rdsplit_mesh* first = e->slot_mesh[items[0]];
+        if (launch_group(group_of(first->S, first->R), c, Q) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
         }
         std::sort(cost.begin(), cost.end(), [](double a, double b) { return a > b; });
-        for (int spread = 0; spread < 2; ++spread) {
-            EngineLaunch Q{nullptr, nullptr, nullptr, 1, nullptr, nullptr, nullptr, nullptr, e->stream, e->sms, 0, 1};
-            Q.query_only = true;
-            Q.spread = spread != 0;
-            const int64_t T = e->slot_mesh[largest]->T;
-            const int g = cls_at(largest, c);
-            if (g >= 10) Q.data = sm_bytes(T, words_shift(T, c), c);
-            if (launch_group(g, c, Q) != cudaSuccess) {
-                cudaGetLastError();
-                continue;
-            }
-            std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
-            for (int i = 0; i < Q.max_active; ++i) free_at.push(0.0);
-            // CTAs beyond one an SM share theirs
-            const double f = !spread && (int64_t)std::min<size_t>(items.size(), Q.max_active) * c > e->sms ? 1.7 : 1.0;
-            double end = 0.0;
-            for (double w : cost) {
-                const double t = free_at.top() + w * f;
-                free_at.pop();
-                free_at.push(t);
-                end = std::max(end, t);
-            }
-            if (end < best_end) {
-                best_end = end;
-                best = c;
-                best_spread = spread != 0;
-            }
+        std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+        for (int i = 0; i < Q.max_active; ++i) free_at.push(0.0);
+        double end = 0.0;
+        for (double w : cost) {
+            const double t = free_at.top() + w;
+            free_at.pop();
+            free_at.push(t);
+            end = std::max(end, t);
+        }
+        if (end < best_end) {
+            best_end = end;
+            best = c;
         }
     }
-    e->cluster = best;
-    e->spread = best_spread;
+    return best;
 }
 
 void finish_slot(rdsplit_engine* e, int slot) {
@@ -1110,22 +1134,17 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
     // Simulations are launched in groups of one kernel and shared-memory size
     // each.  Groups run concurrently on their own streams, the resident
     // clusters shared among them by work; largest first in each.
-    auto cls_at = [&](int s, int cluster) {
-        const rdsplit_mesh* h = e->slot_mesh[s];
-        const int S = h->S, react = h->R > 0 ? 1 : 0;
-        if (S == 1 && sm_bytes(h->T, words_shift(h->T, cluster), cluster) <= sm_data_limit(react != 0)) return 10 + react;
-        const int c = S <= 1 ? 0 : (S <= 2 ? 1 : (S <= 4 ? 2 : (S <= 8 ? 3 : 4)));
-        return 2 * c + react;
-    };
-    if (e->cluster_auto) choose_cluster(e, items, cls_at);
+    auto cls_of = [&](int s) { return group_of(e->slot_mesh[s]->S, e->slot_mesh[s]->R); };
+    if (e->cluster_auto) e->cluster = choose_cluster(e, items);
     const int csize = e->cluster;
-    auto cls_of = [&](int s) { return cls_at(s, csize); };
     size_t g_data[kGroups] = {0};
     for (int32_t s : items) {
         const rdsplit_mesh* h = e->slot_mesh[s];
+        const size_t need = sm_need(h->T, h->S, h->R, csize);
         e->h_desc[s].wshift = words_shift(h->T, csize);
-        const int g = cls_of(s);
-        if (g >= 10) g_data[g] = std::max(g_data[g], sm_bytes(h->T, e->h_desc[s].wshift, csize));
+        e->h_desc[s].gshift = 5;
+        e->h_desc[s].sm = need > 0 ? 1 : 0;
+        g_data[cls_of(s)] = std::max(g_data[cls_of(s)], need);
     }
     std::vector<size_t> idx(items.size());
     std::iota(idx.begin(), idx.end(), 0);
@@ -1170,7 +1189,6 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
         EngineLaunch L{e->d_desc, e->d_mp, e->d_order, g_count[g], e->d_head, e->err, e->processed,
                        e->timing ? e->d_times : nullptr, st, e->sms, e->concurrency, 1};
         L.data = g_data[g];
-        L.spread = e->spread;
         ce = launch_group(g, csize, L);
         used = L.used;
         fit = L.max_active;
@@ -1178,7 +1196,6 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
         // the clusters that fit, shared by work (at least one per group)
         EngineLaunch Q{e->d_desc, e->d_mp, e->d_order, 1, e->d_head, e->err, e->processed, nullptr, st, e->sms, 0, 1};
         Q.query_only = true;
-        Q.spread = e->spread;
         ce = launch_group(7, csize, Q);
         fit = Q.max_active;
         const int budget = e->concurrency > 0 ? std::min(e->concurrency, fit) : fit;
@@ -1214,8 +1231,7 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
             EngineLaunch L{e->d_desc, e->d_mp, e->d_order + g_begin[g], g_count[g], e->d_head + g, e->err,
                            e->processed, e->timing ? e->d_times : nullptr, e->aux[g], e->sms, share[g], 1};
             L.data = g_data[g];
-            L.spread = e->spread;
-            if (ce == cudaSuccess) ce = launch_group(g, csize, L);
+                if (ce == cudaSuccess) ce = launch_group(g, csize, L);
             used += L.used;
             if (ce == cudaSuccess) ce = cudaEventRecord(e->ev_join[g], e->aux[g]);
             if (ce == cudaSuccess) ce = cudaStreamWaitEvent(st, e->ev_join[g], 0);

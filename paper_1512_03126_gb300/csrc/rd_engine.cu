@@ -336,9 +336,17 @@ struct WarpPeriod {
     static constexpr int kW = kC * kWarps;
     static constexpr int kWShift = kC == 1 ? 4 : (kC == 2 ? 5 : (kC == 4 ? 6 : 7));
     static_assert((1 << kWShift) == kW, "warps of a cluster");
-    int S, per;                // this warp's words: `per`, number k is word0 + k * step (kSm: of the CTA's)
-    int word0;
-    static constexpr int step = kSm ? 1 : kW;
+    int S, per;                // this warp's words: `per` of them
+    int word0, used;           // global: the words that hold tets
+    // Word number k of the warp.  Global bitmaps: runs of 4 words (128 tets, 16
+    // bytes) dealt round-robin, so that a load takes 8 sectors instead of 32
+    // (192 cubes of up to 384,000 tets, 0.1 s: 1.37 -> 0.83 s).
+    __device__ __forceinline__ int word(int k) const {
+        if (kSm) return word0 + k;
+        return per >= 4 ? ((((k >> 2) << kWShift) + word0) << 2) | (k & 3) : (k << kWShift) + word0;
+    }
+    __device__ __forceinline__ bool has(int k) const { return k < per && (kSm || word(k) < used); }
+    __device__ __forceinline__ uint32_t* at(int k) const { return kSm ? words + k : words + word(k); }
     WarpMem w;
     PeriodView v;
     View c;
@@ -364,7 +372,8 @@ struct WarpPeriod {
         const int warp = threadIdx.x >> 5;
         const int rank = kC > 1 ? (int)cooperative_groups::this_cluster().block_rank() : 0;
         word0 = (rank * kWarps + warp) * (kSm ? per : 1);
-        words = c.bcur + (kSm ? warp * per : word0);
+        used = d.gshift == 5 ? (d.m.T + 31) >> 5 : 1 << d.wshift;
+        words = c.bcur + (kSm ? warp * per : 0);
         wb = reinterpret_cast<uint32_t*>(s_warp + warp * engine_warp_words(S, kReact) + warp_words(S, kReact));
     }
 };
@@ -380,13 +389,13 @@ __device__ __noinline__ uint32_t run_deferred(int q, uint32_t* err, unsigned lon
     for (int w0 = 0; w0 < p.per; w0 += 32) {
         const int at = w0 + lane;
         uint32_t word = 0u;
-        if (at < p.per) {
-            word = kSm ? p.words[at] : __ldcg(p.words + at * p.step);
-            if (word) p.words[at * p.step] = 0u;
+        if (p.has(at)) {
+            word = kSm ? *p.at(at) : __ldcg(p.at(at));
+            if (word) *p.at(at) = 0u;
         }
         while (__ballot_sync(kAllLanes, word != 0u)) {
             const bool live = word != 0u;
-            const int t = live ? tet_of(p.word0 + at * p.step, __ffs(word) - 1, d.wshift, kSm ? 0 : d.gshift) : 0;
+            const int t = live ? tet_of(p.word(at), __ffs(word) - 1, d.wshift, kSm ? 0 : d.gshift) : 0;
             word &= word - 1u;
             bool none = false;
             bad |= engine_round<kOne, kReact, true>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta, &none);
@@ -431,11 +440,11 @@ __device__ __noinline__ PeriodResult run_period(int q, uint32_t* err, unsigned l
 #pragma unroll
             for (int kk = 0; kk < kCols; ++kk) {
                 const int i = w0 + kk * 32 + lane;
-                wds[kk] = i < p.per ? (kSm ? p.words[i] : __ldcg(p.words + i * p.step)) : 0u;
+                wds[kk] = p.has(i) ? (kSm ? *p.at(i) : __ldcg(p.at(i))) : 0u;
             }
 #pragma unroll
             for (int kk = 0; kk < kCols; ++kk) {
-                if (wds[kk]) p.words[(w0 + kk * 32 + lane) * p.step] = 0u;
+                if (wds[kk]) *p.at(w0 + kk * 32 + lane) = 0u;
                 p.wb[kk * 32 + lane] = wds[kk];
                 own += __popc(wds[kk]);
             }
@@ -473,7 +482,7 @@ __device__ __noinline__ PeriodResult run_period(int q, uint32_t* err, unsigned l
             }
             const int i = w0 + col * 32 + from;
             const int bit = nth_set_bit(word, k);
-            const int t = live ? tet_of(p.word0 + i * p.step, bit, d.wshift, kSm ? 0 : d.gshift) : 0;
+            const int t = live ? tet_of(p.word(i), bit, d.wshift, kSm ? 0 : d.gshift) : 0;
             bool deferred = false;
             bad |= engine_round<kOne, kReact, false>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta,
                                                      &deferred);
@@ -481,8 +490,8 @@ __device__ __noinline__ PeriodResult run_period(int q, uint32_t* err, unsigned l
                 // back into the bitmap, for the pass after the batch
                 late = true;
                 if (deferred) {
-                    if (kSm) atomicOr(p.words + i, 1u << bit);
-                    else red_or(p.words + i * p.step, 1u << bit);
+                    if (kSm) atomicOr(p.at(i), 1u << bit);
+                    else red_or(p.at(i), 1u << bit);
                 }
             }
             __syncwarp();

@@ -43,7 +43,7 @@ struct rdsplit_mesh {
     uint32_t* bits[2] = {nullptr, nullptr};   // active-tet bitmaps by period parity (batched engine)
     uint4* packed = nullptr;   // one species: {reverse-face record, thresholds} per tet (batched engine)
     int2* N2 = nullptr;        // one species: {count, count} of two period parities (batched engine)
-    int32_t* dq = nullptr;     // [T] tets deferred to the slow pass (two-pass period)
+    int32_t* dq = nullptr;     // [T] tets deferred to the second pass (two-pass period)
     int32_t* dqn = nullptr;    // [2] deferred-tet counters by period parity
     int32_t period_mode = 0;   // 0 auto (one pass), 1 one pass (k_period), 2 two passes (light + slow)
     int32_t period_block = 0;  // threads per block of the period kernel (0: by mesh size)

@@ -8,7 +8,7 @@
 // grid-wide synchronisation and no spin-wait is needed.  Per period the
 // cluster visits the tets whose bit is set in that period's activity bitmap
 // (tets that hold molecules or have a zero-order reaction on), runs the same
-// per-tet work as the dense kernel (step_tet, warp_split), and adds the
+// per-tet work as the dense kernels (warp_step), and adds the
 // molecules that stay or leave into the next count buffer with integer atomic
 // adds — exact and independent of order, so the counts equal those of the
 // dense gather.  A tet that keeps or receives molecules sets its bit in the

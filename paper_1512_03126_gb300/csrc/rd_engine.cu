@@ -725,8 +725,7 @@ cudaError_t launch_cluster(EngineLaunch& L) {
     // the attribute covers every group of this kernel, whatever its species
     const size_t most = (size_t)kWarps * engine_warp_words(SA == 1 ? 1 : kMaxS, R) * sizeof(int32_t) +
                         (SA == 1 ? sm_data_limit(R) : 0);
-    cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)most);
+    const cudaError_t ce = allow_shared((const void*)kern, most);
     if (ce != cudaSuccess) return ce;
     const size_t dyn = (size_t)kWarps * engine_warp_words(L.S, R) * sizeof(int32_t) + L.data;
     cudaLaunchConfig_t cfg = {};

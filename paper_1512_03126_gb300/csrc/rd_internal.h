@@ -172,6 +172,15 @@ bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, cons
                 cudaStream_t st);
 int run_shape(int64_t T, int sms, int* warps);
 
+// Lets a kernel take up to `most` bytes of dynamic shared memory a block on the
+// current device (and, on request, clusters of more than 8 CTAs).  Called
+// before every launch of such a kernel with the most that any mesh and model
+// ask of it; the first call raises the limit, which belongs to the function
+// and not to a launch: set to each launch's own size, one thread's smaller
+// mesh lowered it between another's setting and its launch (two threads of 12
+// and 16 species: counts wrong within some thousand launches).
+cudaError_t allow_shared(const void* kern, size_t most, bool wide_clusters = false);
+
 int64_t launches();
 int sm_count();       // multiprocessors of the current device
 void note_launch();   // count a launch issued outside this file's launchers

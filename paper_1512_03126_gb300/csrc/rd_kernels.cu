@@ -26,6 +26,9 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <mutex>
+#include <utility>
+#include <vector>
 
 #include "rd_device.cuh"
 #include "rd_internal.h"
@@ -39,7 +42,26 @@ std::atomic<int64_t> g_launches{0};
 constexpr int kBlock = 256;
 
 inline int grid_for(int64_t n) { return (int)((n + kBlock - 1) / kBlock); }
+
+// The most that a block of kBlock threads asks for (k_period, k_run).
+constexpr size_t block_shared_most(bool react) { return (size_t)(kBlock / 32) * warp_words(kMaxS, react) * sizeof(int32_t); }
+// The most that a CTA of k_run_cluster may take.
+constexpr size_t kClusterShared = 200u * 1024u;
 }  // namespace
+
+cudaError_t allow_shared(const void* kern, size_t most, bool wide_clusters) {
+    static std::mutex mu;
+    static std::vector<std::pair<const void*, int>> raised;
+    int dev = 0;
+    cudaError_t ce = cudaGetDevice(&dev);
+    if (ce != cudaSuccess) return ce;
+    std::lock_guard<std::mutex> lock(mu);
+    if (std::find(raised.begin(), raised.end(), std::make_pair(kern, dev)) != raised.end()) return cudaSuccess;
+    ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (ce == cudaSuccess && wide_clusters) ce = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (ce == cudaSuccess) raised.emplace_back(kern, dev);
+    return ce;
+}
 
 int sm_count() {
     int dev = 0, n = 0;
@@ -903,7 +925,7 @@ int cluster_shape(int64_t T, int S, bool react, int most, int* warps) {
     while (n < most && n < chunks) n <<= 1;
     const int64_t per = (chunks + n - 1) / n;
     *warps = (int)per;
-    if (per > 16 || (size_t)cluster_words(S, react, (int)per) * sizeof(int32_t) > 200u * 1024u) return 0;
+    if (per > 16 || (size_t)cluster_words(S, react, (int)per) * sizeof(int32_t) > kClusterShared) return 0;
     return n;
 }
 
@@ -912,9 +934,7 @@ cudaError_t launch_cluster_s(const DevMesh& m, const ModelParams& mp, const DevS
                              int warps, cudaStream_t st) {
     auto kern = k_run_cluster<S_, kReact>;
     const size_t smem = (size_t)cluster_words(mp.S, kReact, warps) * sizeof(int32_t);
-    cudaError_t ce = cudaSuccess;
-    if (smem > 48u * 1024u) ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (ce == cudaSuccess && ctas > 8) ce = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaError_t ce = allow_shared((const void*)kern, kClusterShared, true);
     if (ce != cudaSuccess) return ce;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas, 1, 1);
@@ -953,10 +973,9 @@ cudaError_t launch_run_b(const DevMesh& m, const ModelParams& mp, const DevState
                          int warps, int sms, cudaStream_t st) {
     auto kern = k_run<S_, kReact, kBlocks>;
     const size_t smem = (size_t)warps * warp_words(mp.S, kReact) * sizeof(int32_t);
-    if (smem > 48u * 1024u)
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t ce = allow_shared((const void*)kern, block_shared_most(kReact));
     int fit = 0;
-    cudaError_t ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, 32 * warps, smem);
+    if (ce == cudaSuccess) ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, 32 * warps, smem);
     if (ce == cudaSuccess && (int64_t)fit * sms < grid) ce = cudaErrorCooperativeLaunchTooLarge;
     if (ce != cudaSuccess) return ce;
     DevMesh m_ = m;
@@ -1011,8 +1030,8 @@ template <int S_, bool kReact, int kPass>
 void launch_pass(const DevMesh& m, const ModelParams& mp, const DevState& s, const PeriodArgs& a, int32_t* queue,
                  int32_t* qcount, int32_t parity, int grid, int block, cudaStream_t st) {
     const size_t smem = (size_t)(block / 32) * warp_words(mp.S, kReact) * sizeof(int32_t);
-    if (smem > 48u * 1024u)   // large blocks of many species
-        cudaFuncSetAttribute(k_period<S_, kReact, kPass>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // large blocks of many species; a failure is reported as the launch's (last error)
+    if (S_ != 1 && allow_shared((const void*)k_period<S_, kReact, kPass>, block_shared_most(kReact)) != cudaSuccess) return;
     k_period<S_, kReact, kPass><<<grid, block, smem, st>>>(m, mp, s, a, queue, qcount, parity);
     ++g_launches;
 }

@@ -43,8 +43,10 @@ extern "C" {
 #define RDSPLIT_EINVAL (-1)    /* bad argument, malformed mesh or model */
 #define RDSPLIT_ENOMEM (-2)    /* device allocation failed or budget exceeded */
 #define RDSPLIT_ECUDA (-3)     /* a CUDA runtime call failed */
-#define RDSPLIT_ETIMEOUT (-4)  /* a run's grid barrier was waited for in vain (two
-                                  minutes; not expected: its blocks are resident) */
+#define RDSPLIT_ETIMEOUT (-4)  /* a run's grid barrier saw no progress for too long
+                                  (rdsplit_set_wait_limit; not expected: its blocks
+                                  are resident).  The handle's counts, time and
+                                  period index are those of before the call */
 #define RDSPLIT_EOVERFLOW (-5) /* a count would exceed INT32_MAX, or a
                                   period would exceed the per-tet event cap */
 #define RDSPLIT_ESTATE (-6)    /* call out of order (e.g. run before set_model) */
@@ -219,6 +221,13 @@ int rdsplit_get_shape(rdsplit_mesh_t mesh, int32_t* n_tets, int32_t* n_species);
  */
 int rdsplit_set_period_kernel(rdsplit_mesh_t mesh, int32_t mode, int32_t block);
 int rdsplit_get_period_kernel(rdsplit_mesh_t mesh, int32_t* two_passes, int32_t* block);
+
+/*
+ * How long a grid barrier of the handle's runs may see no progress before the
+ * run gives up with RDSPLIT_ETIMEOUT: seconds > 0, 120 by default.  A tet with
+ * many reaction events in one period counts as progress every 2^16 of them.
+ */
+int rdsplit_set_wait_limit(rdsplit_mesh_t mesh, double seconds);
 
 /*
  * Domain decomposition (Sec. III.D: each process advances its own tets to

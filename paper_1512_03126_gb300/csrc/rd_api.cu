@@ -172,6 +172,9 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
     if (h->inbox_dirty) CUDA_TRY(clear_inboxes(h));
     int64_t j = 0;        // periods done
     int64_t jl = 0;       // of them in single launches since the last closing transfer
+    const double t_start = h->t;
+    const int64_t period_start = h->period;
+    bool saved = false;   // the counts of the start are in h->staging (see launch_run)
     while (h->t < t_end && (max_periods < 0 || j < max_periods)) {
         h->inbox_dirty = true;   // until the closing transfer
         // the next stretch: one period, or as many as a resident launch takes
@@ -196,9 +199,10 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
         if (resident) {
             RunArgs r{(uint32_t)h->period, n, last ? 1 : 0, h->tau, tau_k, (float)h->tau, (float)tau_k, seed, h->thr,
                       h->thr_last, {h->inbox[0], h->inbox[1]}, {h->imask[0], h->imask[1]}, h->barrier,
-                      h->barrier_base};
+                      h->barrier_base, h->wait_limit_ns};
             int grid = 0;
-            if (launch_run(m, h->mp, s, r, sms, &grid, h->stream)) {
+            if (launch_run(m, h->mp, s, r, sms, &grid, saved ? nullptr : h->staging, h->stream)) {
+                saved = saved || grid > 0;
                 h->barrier_base += (uint32_t)grid * (uint32_t)n;
                 h->inbox_dirty = false;
                 h->t = t;
@@ -238,10 +242,15 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
     if (rc) return rc;
     h->inbox_dirty = false;
     rc = check_err(h, "rdsplit_run");
-    if (rc == RDSPLIT_ETIMEOUT) {   // blocks left the launch early
+    if (rc == RDSPLIT_ETIMEOUT) {   // blocks left a launch early: back to where the call began
         h->inbox_dirty = true;
         CUDA_TRY(cudaMemsetAsync(h->barrier, 0, sizeof(uint32_t), h->stream));
         h->barrier_base = 0;
+        if (saved)
+            CUDA_TRY(cudaMemcpyAsync(h->cnt, h->staging, sizeof(int32_t) * (size_t)h->T * h->S,
+                                     cudaMemcpyDeviceToDevice, h->stream));
+        h->t = t_start;
+        h->period = period_start;
     }
     collect_timing(h);
     return rc;
@@ -364,7 +373,7 @@ int mesh_create_impl(const char* where, int32_t n_tets, const int32_t* adj, cons
         (rc = alloc_into(&d_dist, 4 * T, "dist")) || (rc = alloc_into(&h->vol, T, "vol")) ||
         (rc = alloc_into(&h->src, T, "src")) || (rc = alloc_into(&h->g, 4 * T, "g")) ||
         (rc = alloc_into(&h->G, T, "G")) || (rc = alloc_into(&h->gmax, 1, "gmax")) ||
-        (rc = alloc_into(&h->err, 1, "err")) || (rc = alloc_into(&h->barrier, 1, "barrier")) || (reorder && (rc = alloc_into(&h->perm, T, "order"))))
+        (rc = alloc_into(&h->err, kErrWords, "err")) || (rc = alloc_into(&h->barrier, 1, "barrier")) || (reorder && (rc = alloc_into(&h->perm, T, "order"))))
         return cleanup(rc);
     cudaStream_t st = h->stream;
     cudaError_t ce = cudaSuccess;
@@ -374,7 +383,7 @@ int mesh_create_impl(const char* where, int32_t n_tets, const int32_t* adj, cons
     ce = ce ? ce : cudaMemcpyAsync(d_dist, centroid_dist, 32 * T, cudaMemcpyHostToDevice, st);
     if (reorder) ce = ce ? ce : cudaMemcpyAsync(h->perm, perm.data(), 4 * T, cudaMemcpyHostToDevice, st);
     ce = ce ? ce : cudaMemsetAsync(h->gmax, 0, sizeof(unsigned long long), st);
-    ce = ce ? ce : cudaMemsetAsync(h->err, 0, sizeof(uint32_t), st);
+    ce = ce ? ce : cudaMemsetAsync(h->err, 0, sizeof(uint32_t) * kErrWords, st);
     ce = ce ? ce : cudaMemsetAsync(h->barrier, 0, sizeof(uint32_t), st);
     if (ce != cudaSuccess) {
         cudaGetLastError();
@@ -647,7 +656,7 @@ static int get_counts_impl(rdsplit_mesh_t h, int32_t* out, bool device) {
     if (!h->has_model) return fail(RDSPLIT_ESTATE, "rdsplit_get_counts: no model attached");
     const size_t n = (size_t)h->T * h->S;
     int32_t* dst = device ? out : h->staging;
-    launch_counts_out(h->T, h->S, h->cnt, dst, h->perm, h->stream);
+    launch_counts_out(h->T, h->S, h->cnt, dst, h->perm, nullptr, h->stream);
     int rc = launch_check("rdsplit_get_counts");
     if (rc) return rc;
     if (!device) CUDA_TRY(cudaMemcpyAsync(out, h->staging, n * 4, cudaMemcpyDeviceToHost, h->stream));
@@ -814,6 +823,13 @@ int rdsplit_get_period_kernel(rdsplit_mesh_t h, int32_t* two_passes, int32_t* bl
     if (!h) return fail(RDSPLIT_EINVAL, "rdsplit_get_period_kernel: NULL handle");
     if (two_passes) *two_passes = two_pass(h) ? 1 : 0;
     if (block) *block = period_block(h, sm_count());
+    return RDSPLIT_OK;
+}
+
+int rdsplit_set_wait_limit(rdsplit_mesh_t h, double seconds) {
+    if (!h) return fail(RDSPLIT_EINVAL, "rdsplit_set_wait_limit: NULL handle");
+    if (!(seconds > 0.0)) return fail(RDSPLIT_EINVAL, "rdsplit_set_wait_limit: seconds must be > 0");
+    h->wait_limit_ns = (unsigned long long)std::min(std::max(seconds * 1e9, 1.0), 1e18);
     return RDSPLIT_OK;
 }
 

@@ -997,7 +997,7 @@ int rdsplit_engine_create(int32_t max_slots, int64_t max_active_tets, rdsplit_en
     e->d_mp = (ModelParams*)rdapi::dev_alloc(sizeof(ModelParams) * max_slots);
     e->d_order = (int32_t*)rdapi::dev_alloc(sizeof(int32_t) * max_slots);
     e->d_head = (int32_t*)rdapi::dev_alloc(sizeof(int32_t) * kGroups);
-    e->err = (uint32_t*)rdapi::dev_alloc(sizeof(uint32_t));
+    e->err = (uint32_t*)rdapi::dev_alloc(sizeof(uint32_t) * kErrWords);
     e->processed = (unsigned long long*)rdapi::dev_alloc(sizeof(unsigned long long));
     e->d_times = (unsigned long long*)rdapi::dev_alloc(sizeof(unsigned long long) * 4 * max_slots);
     if (!e->d_desc || !e->d_mp || !e->d_order || !e->d_head || !e->err || !e->processed || !e->d_times) {
@@ -1014,7 +1014,7 @@ int rdsplit_engine_create(int32_t max_slots, int64_t max_active_tets, rdsplit_en
     warm_engine_kernels(e->d_head, e->err, e->processed, e->sms);
     if (cudaMemsetAsync(e->processed, 0, sizeof(unsigned long long), e->stream) != cudaSuccess ||
         cudaMemsetAsync(e->d_times, 0, sizeof(unsigned long long) * 4 * max_slots, e->stream) != cudaSuccess ||
-        cudaMemsetAsync(e->err, 0, sizeof(uint32_t), e->stream) != cudaSuccess) {
+        cudaMemsetAsync(e->err, 0, sizeof(uint32_t) * kErrWords, e->stream) != cudaSuccess) {
         cudaGetLastError();
         delete e;
         return rdapi::fail(RDSPLIT_ECUDA, "rdsplit_engine_create: memset failed");

@@ -20,6 +20,14 @@ enum : uint32_t {
     kErrEventCap = 1u << 6,      // more SSA events in one tet-period than the cap
     kErrTimeout = 1u << 7,       // a grid barrier's wait ran out
 };
+// Words of an error buffer: the bits above, and a count that a tet with very
+// many events in one period bumps as it goes (see grid_barrier).
+constexpr int kErrWords = 2;
+// A grid barrier gives up after this long without a bump: 20 times what the
+// events between two bumps take at their slowest (2^16 events of up to 30,000
+// cycles each, six warps sharing a multiprocessor's FP64 unit).
+constexpr unsigned long long kWaitLimitNs = 120ull * 1000000000ull;
+constexpr int kBumpEvents = 1 << 16;
 
 // Chemistry, passed by value to kernels (lives in the constant bank).
 struct ModelParams {
@@ -78,7 +86,7 @@ __device__ __forceinline__ int key_of(const DevMesh& m, int t) { return m.perm ?
 
 struct DevState {
     int32_t* cnt;           // [S][T] counts, in place over the periods of a run
-    uint32_t* err;          // error word
+    uint32_t* err;          // error words [kErrWords]
 };
 
 // ---- setup --------------------------------------------------------------
@@ -98,8 +106,9 @@ void launch_pack_mask(int32_t T, int32_t R, const uint8_t* mask8, uint32_t* mask
                       cudaStream_t st);
 void launch_counts_in(int32_t T, int32_t S, const int32_t* ts, int32_t* st_major, uint32_t* err,
                       const int32_t* perm, cudaStream_t st);
+// err: writes nothing if a run before it on the stream gave up waiting (or null).
 void launch_counts_out(int32_t T, int32_t S, const int32_t* st_major, int32_t* ts, const int32_t* perm,
-                       cudaStream_t st);
+                       const uint32_t* err, cudaStream_t st);
 
 // ---- one period (gather of the previous period fused with reactions and
 // diffusion of this one) and the closing gather --------------------------
@@ -164,12 +173,15 @@ struct RunArgs {
     uint8_t* mask[2];
     uint32_t* barrier;      // grid-barrier counter; holds barrier_base before the launch
     uint32_t barrier_base;  // and barrier_base + grid * periods after it
+    unsigned long long wait_limit_ns = kWaitLimitNs;   // of a grid barrier without progress
 };
 // Launches it if the mesh's tets fit on the device at once (else, or when a
 // cooperative launch is refused, answers false with nothing launched); *grid
-// receives its blocks.
+// receives its blocks.  A launch that ends with kErrTimeout leaves counts of
+// different periods: unless `save` is null, a form that can end so copies the
+// counts there first.
 bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int sms, int* grid,
-                cudaStream_t st);
+                int32_t* save, cudaStream_t st);
 int run_shape(int64_t T, int sms, int* warps);
 
 // Lets a kernel take up to `most` bytes of dynamic shared memory a block on the

@@ -326,8 +326,9 @@ __global__ void k_counts_in(int32_t T, int32_t S, const int32_t* __restrict__ ts
 }
 
 __global__ void k_counts_out(int32_t T, int32_t S, const int32_t* __restrict__ sm, int32_t* __restrict__ ts,
-                             const int32_t* __restrict__ perm) {
+                             const int32_t* __restrict__ perm, const uint32_t* __restrict__ err) {
     extern __shared__ int32_t tile[];
+    if (err && (*err & kErrTimeout)) return;
     const int ld = S | 1;
     const int64_t t0 = (int64_t)blockIdx.x * kBlock;
     const int n = (int)min((int64_t)kBlock, T - t0);
@@ -354,8 +355,9 @@ void launch_counts_in(int32_t T, int32_t S, const int32_t* ts, int32_t* sm, uint
     ++g_launches;
 }
 
-void launch_counts_out(int32_t T, int32_t S, const int32_t* sm, int32_t* ts, const int32_t* perm, cudaStream_t st) {
-    k_counts_out<<<grid_for(T), kBlock, kBlock * (S | 1) * sizeof(int32_t), st>>>(T, S, sm, ts, perm);
+void launch_counts_out(int32_t T, int32_t S, const int32_t* sm, int32_t* ts, const int32_t* perm, const uint32_t* err,
+                       cudaStream_t st) {
+    k_counts_out<<<grid_for(T), kBlock, kBlock * (S | 1) * sizeof(int32_t), st>>>(T, S, sm, ts, perm, err);
     ++g_launches;
 }
 
@@ -625,15 +627,19 @@ k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams 
 // Grid barrier of a cooperative launch: the counter only grows, by one per
 // block and barrier; the wait ends when it reaches `target` (modulo 2^32).
 // The launch holds every block resident, so the wait is as long as the slowest
-// block's period; past the limit (a period at the event cap takes seconds)
-// the block sets kErrTimeout and gives up, and the others follow it.
-__device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target, uint32_t* err, volatile int* gave_up) {
-    constexpr unsigned long long kLimitNs = 120ull * 1000000000ull;
+// block's period.  That can be minutes (a tet's period goes up to 2^22 events
+// of some microseconds, and the warps of a multiprocessor share its FP64 unit),
+// so the limit is on the time without progress: a tet at work on many events
+// bumps err[1] every kBumpEvents of them.  Past the limit the block sets
+// kErrTimeout and gives up, and the others follow it.
+__device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target, uint32_t* err,
+                                             unsigned long long limit_ns, volatile int* gave_up) {
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();   // the block's inbox words before its arrival
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
         unsigned long long start = 0ull;
+        uint32_t bumps = 0u;
         for (uint32_t i = 1;; ++i) {
             uint32_t c;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(counter) : "memory");
@@ -641,8 +647,10 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target,
             if ((i & 1023u) == 0u) {
                 unsigned long long now;
                 asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-                if (start == 0ull) start = now;
-                if (now - start > kLimitNs || (__ldcg(err) & kErrTimeout)) {
+                const uint32_t b = __ldcg(err + 1);
+                if (start == 0ull || b != bumps) start = now;
+                bumps = b;
+                if (now - start > limit_ns || (__ldcg(err) & kErrTimeout)) {
                     atomicOr(err, kErrTimeout);
                     *gave_up = 1;
                     break;
@@ -699,7 +707,7 @@ k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp,
         a.mask_cur = r.mask[p];
         if (q > 0) {
             target += gridDim.x;
-            if (!grid_barrier(r.barrier, target, s.err, &gave_up)) return;
+            if (!grid_barrier(r.barrier, target, s.err, r.wait_limit_ns, &gave_up)) return;
             if (live) bad |= take_inbox(a, t, S, lane, w.N, pr, &dirty);
         }
         if (q == r.periods) break;
@@ -996,7 +1004,7 @@ cudaError_t launch_run_s(const DevMesh& m, const ModelParams& mp, const DevState
 }
 
 bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int sms, int* grid,
-                cudaStream_t st) {
+                int32_t* save, cudaStream_t st) {
     int warps = 0;
     cudaError_t ce = cudaErrorInvalidConfiguration;
     // 16 CTAs are beyond the portable cluster size: where the device has no
@@ -1016,6 +1024,9 @@ bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, cons
     }
     *grid = run_shape(m.T, sms, &warps);
     if (*grid == 0) return false;
+    if (save && cudaMemcpyAsync(save, s.cnt, sizeof(int32_t) * (size_t)m.T * mp.S, cudaMemcpyDeviceToDevice, st) !=
+                    cudaSuccess)
+        return false;   // the caller's next launch reports it
     if (mp.S == 1)
         ce = mp.any_reaction ? launch_run_s<1, true>(m, mp, s, r, *grid, warps, sms, st)
                              : launch_run_s<1, false>(m, mp, s, r, *grid, warps, sms, st);

@@ -259,7 +259,7 @@ extern "C" int rdsplit_run_static(int32_t n_tets, const int32_t* d_adj, const do
             RunArgs r{(uint32_t)pk, n, 0, tau_k, tau_k, (float)tau_k, (float)tau_k, seed, thr, thr,
                       {out[0], out[1]}, {mask[0], mask[1]}, barrier, barrier_base};
             int grid = 0;
-            if (!launch_run(m, mp, s, r, sms, &grid, st)) {
+            if (!launch_run(m, mp, s, r, sms, &grid, nullptr, st)) {   // d_counts still holds the counts
                 resident = false;
                 continue;
             }
@@ -281,7 +281,7 @@ extern "C" int rdsplit_run_static(int32_t n_tets, const int32_t* d_adj, const do
         a.mask_prev = mask[q];
         launch_gather(m, n_species, s, a, st);
     }
-    launch_counts_out(n_tets, n_species, cnt, d_counts, nullptr, st);
+    launch_counts_out(n_tets, n_species, cnt, d_counts, nullptr, err, st);
     ce = cudaGetLastError();
     if (ce != cudaSuccess) return rdapi::fail(RDSPLIT_ECUDA, "%s: launch failed: %s", where, cudaGetErrorString(ce));
     if ((rc = read_err(base, L, st, where))) return rc;

@@ -348,6 +348,7 @@ static __device__ __noinline__ uint32_t react_exact(const ModelParams& mp, int k
         }
         tc = tn;
         if (++events >= kEventCap) { atomicOr(err, kErrEventCap); break; }
+        if (events % kBumpEvents == 0) atomicAdd(err + 1, 1u);   // still at work (see grid_barrier)
     }
     if (want_mid && !past_half)
         for (int s = 0; s < S; ++s) nmid[s] = N[s];

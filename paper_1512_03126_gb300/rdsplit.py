@@ -54,6 +54,7 @@ def _declare(L):
         "rdsplit_set_stream": ([vp, vp], C.c_int),
         "rdsplit_mesh_destroy": ([vp], C.c_int),
         "rdsplit_set_allocator": ([vp, vp, vp], C.c_int),
+        "rdsplit_set_wait_limit": ([vp, dbl], C.c_int),
         "rdsplit_set_timing": ([vp, i32], C.c_int),
         "rdsplit_set_period_kernel": ([vp, i32, i32], C.c_int),
         "rdsplit_partition_set": ([vp, i32, i32], C.c_int),
@@ -275,6 +276,10 @@ def rdsplit_get_period_kernel(h):
     a, b = C.c_int32(), C.c_int32()
     _check(lib().rdsplit_get_period_kernel(h, C.byref(a), C.byref(b)))
     return a.value, b.value
+
+
+def rdsplit_set_wait_limit(h, seconds: float):
+    _check(lib().rdsplit_set_wait_limit(h, float(seconds)))
 
 
 def rdsplit_set_timing(h, stride: int):

@@ -1,0 +1,70 @@
+"""A run whose grid barrier sees no progress for the handle's limit ends with
+RDSPLIT_ETIMEOUT and leaves counts, time and period index as they were before
+the call; within the limit a long period is no error.  One tet has some tens of
+thousands of reaction events in a period while all others wait for it."""
+import numpy as np
+import pytest
+
+from paper_1512_03126_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rd():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_1512_03126_gb300 import build
+    build.build()
+    from paper_1512_03126_gb300 import rdsplit
+    return rdsplit
+
+
+def one_busy_tet(events):
+    """12,000 tets (more than one cluster holds); A <-> B, `events` a period
+    for the 1,000 molecules of one tet, diffusion a thousandth of it."""
+    mesh = I.kuhn_box(10, 10, 20, (1e-6, 1e-6, 2e-6), 0.2, 5)
+    tau = 1e-7 ** 2 / 1e-12 / 100.0
+    k = np.array([events / 1000.0 / tau] * 2)
+    model = I.Model(D=np.array([1e-12, 1e-15]), lhs=np.array([[1, 0], [0, 1]], np.int32),
+                    rhs=np.array([[0, 1], [1, 0]], np.int32), k=k)
+    counts = np.zeros((mesh.n_tets, 2), np.int32)
+    counts[4321, 1] = 1000
+    return mesh, model, counts
+
+
+def test_running_out_leaves_the_state_of_before_the_call(rd, oracle):
+    mesh, model, counts = one_busy_tet(3e4)
+    ref = oracle.run(mesh, model, counts, np.inf, 9, max_periods=3)[0]
+    with rd.Simulation(mesh, model, counts) as sim:
+        sim.run_periods(1, 9)
+        first, when = sim.counts(), sim.time
+        rd.rdsplit_set_wait_limit(sim.h, 1e-3)
+        for _ in range(2):
+            with pytest.raises(rd.RdsplitError) as e:
+                sim.run_periods(2, 9)
+            assert e.value.code == rd.RDSPLIT_ETIMEOUT
+            assert np.array_equal(sim.counts(), first) and sim.time == when
+        rd.rdsplit_set_wait_limit(sim.h, 120.0)
+        sim.run_periods(2, 9)
+        assert np.array_equal(sim.counts(), ref)
+
+
+def test_progress_restarts_the_limit(rd, oracle):
+    """About 400,000 events, some seconds, under a limit that covers 2^16 of
+    them at the slowest (30,000 cycles each) but not all."""
+    mesh, model, counts = one_busy_tet(4e5)
+    ref = oracle.run(mesh, model, counts, np.inf, 9, max_periods=1)[0]
+    with rd.Simulation(mesh, model, counts) as sim:
+        rd.rdsplit_set_wait_limit(sim.h, 1.0)
+        sim.run_periods(1, 9)
+        assert np.array_equal(sim.counts(), ref)
+
+
+def test_limits_that_are_not_positive_are_rejected(rd):
+    mesh, model, counts = one_busy_tet(1e3)
+    with rd.Simulation(mesh, model, counts) as sim:
+        for bad in (0.0, -1.0, float("nan")):
+            with pytest.raises(rd.RdsplitError) as e:
+                rd.rdsplit_set_wait_limit(sim.h, bad)
+            assert e.value.code == rd.RDSPLIT_EINVAL

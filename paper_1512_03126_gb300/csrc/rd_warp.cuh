@@ -444,9 +444,9 @@ __device__ __forceinline__ void count_block(const uint4& w, int m, const uint4& 
 // done), so neighbouring entries belong to different lanes, and 32 entries
 // make a round with one block a lane.  The cost follows the number of blocks,
 // not the largest count of a lane or the species present in any lane.
-// Species with more than kCoopMin draws are drawn by the whole warp first,
-// and (kCalls) those from kMoleculeCut on by big(sp, N*).  Returns the species whose
-// acc words hold leavers-to-be.  All lanes must call it.  The per-lane loop
+// Before the list, (kCalls) species with kMoleculeCut draws or more are drawn by
+// big(sp, N*), and those with more than kCoopMin by the whole warp.  Returns the
+// species whose acc words hold leavers-to-be.  All lanes must call it.  The per-lane loop
 // with a whole-warp pass per species and tet from 10 molecules on took one
 // serial pass a tet: 600 cycles each, up to 32 a warp.
 // With one species (kOne) every lane draws its own first block, without the
@@ -471,6 +471,25 @@ __device__ __forceinline__ uint32_t draw_all(int S, int64_t T, const WarpMem& w,
     }
     uint32_t drawn = present & ~heavy;
     uint32_t todo = drawn;
+    if (kCalls) {
+        // the binomials of all lanes side by side, one species of each lane a
+        // turn (one lane at a time, a mesh of 5,000 molecules a tet took up to
+        // 14 times as long)
+        uint32_t binom = 0;
+        for (uint32_t bits = heavy; bits; bits &= bits - 1u) {
+            const int sp = __ffs(bits) - 1;
+            if (draws_of(sp) >= (int)kMoleculeCut) binom |= 1u << sp;
+        }
+        heavy &= ~binom;
+        while (__ballot_sync(kAllLanes, binom != 0u)) {
+            if (binom) {
+                const int sp = __ffs(binom) - 1;
+                binom &= binom - 1u;
+                big(sp, draws_of(sp));
+            }
+            __syncwarp();
+        }
+    }
     for (;;) {
         const unsigned hm = __ballot_sync(kAllLanes, heavy != 0u);
         if (hm == 0u) break;
@@ -479,11 +498,6 @@ __device__ __forceinline__ uint32_t draw_all(int S, int64_t T, const WarpMem& w,
         const int sp = kOne ? 0 : __shfl_sync(kAllLanes, sp_own, src);
         const int nn = __shfl_sync(kAllLanes, heavy ? draws_of(sp_own) : 0, src);
         if (lane == src) heavy &= heavy - 1u;
-        if (kCalls && nn >= (int)kMoleculeCut) {
-            if (lane == src) big(sp, nn);
-            __syncwarp();
-            continue;
-        }
         const int tt = __shfl_sync(kAllLanes, t, src), kk = __shfl_sync(kAllLanes, key, src);
         const uint4 C = __ldg(v.thr + ((int64_t)sp * T + tt) * v.thr_stride);
         uint32_t a0 = 0, a1 = 0;

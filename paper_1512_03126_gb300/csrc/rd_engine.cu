@@ -378,61 +378,21 @@ struct WarpPeriod {
     }
 };
 
-// The warp's tets whose bits the rounds set back, with the double-precision
-// samplers.
-template <bool kOne, bool kReact, int kC, bool kSm>
-__device__ __noinline__ uint32_t run_deferred(int q, uint32_t* err, unsigned long long* mass_delta) {
-    const SlotDesc& d = s_desc;
-    const WarpPeriod<kOne, kReact, kC, kSm> p(d, q);
-    const int lane = threadIdx.x & 31;
-    uint32_t bad = 0;
-    for (int w0 = 0; w0 < p.per; w0 += 32) {
-        const int at = w0 + lane;
-        uint32_t word = 0u;
-        if (p.has(at)) {
-            word = kSm ? *p.at(at) : __ldcg(p.at(at));
-            if (word) *p.at(at) = 0u;
-        }
-        while (__ballot_sync(kAllLanes, word != 0u)) {
-            const bool live = word != 0u;
-            const int t = live ? tet_of(p.word(at), __ffs(word) - 1, d.wshift, kSm ? 0 : d.gshift) : 0;
-            word &= word - 1u;
-            bool none = false;
-            bad |= engine_round<kOne, kReact, true>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta, &none);
-            __syncwarp();
-        }
-    }
-    return bad;
-}
-
-// One period of a simulation for one warp.  A bitmap word holds 32 tets a
-// power of two apart, so that every word has its share of a compact cloud of
-// molecules and of its crowded tets: dealing runs of 128 consecutive tets
-// left warps waiting at the period barrier for the one that held the source
-// (15 of 24 stall cycles an instruction).  The words go to the cluster's kW
-// warps in equal contiguous parts.  A warp loads a batch of up to kGroup
-// columns (32 words, one per lane) at once and clears them for their next use.
-// One prefix sum over the lanes' set bits of the whole batch lets each lane
+// The set bits of the warp's words, in rounds of 32: visit(i, bit, t, live) once
+// a round, with the lane's word number, bit and tet.  Words are cleared for
+// their next use when they are loaded.  Returns the number of set bits.
+//
+// A warp loads a batch of up to kGroup columns (32 words, one per lane) at
+// once.  One prefix sum over the lanes' set bits of the whole batch lets each lane
 // find a tet of its own (a search over the sums, the column, the bit in the
 // word: a fixed 110 instructions a round; a sum and a search for every column,
 // nearly all of which hold a few bits of a sparse mesh, made the 512-cube
-// ensemble three times slower); 32 tets make a round (engine_round).
-//
-// Out of line and free of calls, like run_deferred beside it: with the round
-// in the kernel's own loop, what it keeps across the call of run_deferred
-// (addresses and descriptor fields lifted out of the loops) sat in local
-// memory, 110 loads a round.
-struct PeriodResult {
-    uint32_t bad, done, late;   // error bits, tets visited, whether some were deferred
-};
-template <bool kOne, bool kReact, int kC, bool kSm>
-__device__ __noinline__ PeriodResult run_period(int q, uint32_t* err, unsigned long long* mass_delta) {
-    const SlotDesc& d = s_desc;
+// ensemble three times slower).
+template <bool kSm, class Period, class Visit>
+__device__ __forceinline__ uint32_t visit_set_bits(const SlotDesc& d, const Period& p, Visit visit) {
     const int lane = threadIdx.x & 31;
-    const WarpPeriod<kOne, kReact, kC, kSm> p(d, q);
     constexpr int kCols = kSm ? kSmCols : kGroup;
-    uint32_t bad = 0, done = 0;
-    bool late = false;              // some tet was deferred
+    uint32_t done = 0;
     for (int w0 = 0; w0 < p.per; w0 += 32 * kCols) {
         int own = 0;
         {
@@ -482,21 +442,62 @@ __device__ __noinline__ PeriodResult run_period(int q, uint32_t* err, unsigned l
             }
             const int i = w0 + col * 32 + from;
             const int bit = nth_set_bit(word, k);
-            const int t = live ? tet_of(p.word(i), bit, d.wshift, kSm ? 0 : d.gshift) : 0;
-            bool deferred = false;
-            bad |= engine_round<kOne, kReact, false>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta,
-                                                     &deferred);
-            if (__ballot_sync(kAllLanes, deferred)) {
-                // back into the bitmap, for the pass after the batch
-                late = true;
-                if (deferred) {
-                    if (kSm) atomicOr(p.at(i), 1u << bit);
-                    else red_or(p.at(i), 1u << bit);
-                }
-            }
+            visit(i, bit, live ? tet_of(p.word(i), bit, d.wshift, kSm ? 0 : d.gshift) : 0, live);
             __syncwarp();
         }
     }
+    return done;
+}
+
+// The warp's tets whose bits the rounds set back, with the double-precision
+// samplers, 32 of them side by side (with a round for each bit of the lanes'
+// own words, 24,576 tets of 5,000 molecules on 8 CTAs kept 6 lanes of 32 busy:
+// 48 ms where this takes 17).
+template <bool kOne, bool kReact, int kC, bool kSm>
+__device__ __noinline__ uint32_t run_deferred(int q, uint32_t* err, unsigned long long* mass_delta) {
+    const SlotDesc& d = s_desc;
+    const WarpPeriod<kOne, kReact, kC, kSm> p(d, q);
+    uint32_t bad = 0;
+    visit_set_bits<kSm>(d, p, [&](int, int, int t, bool live) {
+        bool none = false;
+        bad |= engine_round<kOne, kReact, true>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta, &none);
+    });
+    return bad;
+}
+
+// One period of a simulation for one warp: its tets in rounds of 32
+// (engine_round).  In shared memory a bitmap word holds 32 tets a power of two
+// apart, so that every word has its share of a compact cloud of molecules and of
+// its crowded tets, and the words go to the cluster's kW warps in equal
+// contiguous parts; in global memory a word holds 32 consecutive tets and
+// words are dealt in runs of four (WarpPeriod::word).
+//
+// Out of line and free of calls, like run_deferred beside it: with the round
+// in the kernel's own loop, what it keeps across the call of run_deferred
+// (addresses and descriptor fields lifted out of the loops) sat in local
+// memory, 110 loads a round.
+struct PeriodResult {
+    uint32_t bad, done, late;   // error bits, tets visited, whether some were deferred
+};
+template <bool kOne, bool kReact, int kC, bool kSm>
+__device__ __noinline__ PeriodResult run_period(int q, uint32_t* err, unsigned long long* mass_delta) {
+    const SlotDesc& d = s_desc;
+    const WarpPeriod<kOne, kReact, kC, kSm> p(d, q);
+    uint32_t bad = 0;
+    bool late = false;              // some tet was deferred
+    const uint32_t done = visit_set_bits<kSm>(d, p, [&](int i, int bit, int t, bool live) {
+        bool deferred = false;
+        bad |= engine_round<kOne, kReact, false>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta,
+                                                 &deferred);
+        if (__ballot_sync(kAllLanes, deferred)) {
+            // back into the bitmap, for the pass after these rounds
+            late = true;
+            if (deferred) {
+                if (kSm) atomicOr(p.at(i), 1u << bit);
+                else red_or(p.at(i), 1u << bit);
+            }
+        }
+    });
     if (late && !kSm) __threadfence();   // the bits set back are read by other lanes
     __syncwarp();
     return PeriodResult{bad, done, late ? 1u : 0u};

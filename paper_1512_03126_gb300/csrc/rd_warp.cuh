@@ -347,8 +347,10 @@ static __device__ __noinline__ uint32_t react_exact(const ModelParams& mp, int k
             N[s] += mp.delta[mu][s];
         }
         tc = tn;
-        if (++events >= kEventCap) { atomicOr(err, kErrEventCap); break; }
-        if (events % kBumpEvents == 0) atomicAdd(err + 1, 1u);   // still at work (see grid_barrier)
+        if (++events % kBumpEvents == 0) {
+            if (events >= kEventCap) { atomicOr(err, kErrEventCap); break; }
+            atomicAdd(err + 1, 1u);   // still at work (see grid_barrier)
+        }
     }
     if (want_mid && !past_half)
         for (int s = 0; s < S; ++s) nmid[s] = N[s];
@@ -588,6 +590,10 @@ __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParam
                                               const PeriodView& v, int t, bool live, uint32_t mask, Presence& pr,
                                               uint32_t* dirty, bool* deferred, uint32_t* err, Emit& emit,
                                               uint4 pre = make_uint4(0u, 0u, 0u, 0u), bool tried = false) {
+    // The lanes come from loops over their own inbox words: unless they are brought
+    // together here, each goes through the reaction phase by itself (10,368 tets
+    // of eleven species, up to 475 events a period, 60 periods: 82 ms instead of 43).
+    __syncwarp();
     const int lane = threadIdx.x & 31;
     const int key = live ? key_of(m, t) : 0;
     uint32_t bad = 0, touched = 0;

@@ -43,10 +43,10 @@ extern "C" {
 #define RDSPLIT_EINVAL (-1)    /* bad argument, malformed mesh or model */
 #define RDSPLIT_ENOMEM (-2)    /* device allocation failed or budget exceeded */
 #define RDSPLIT_ECUDA (-3)     /* a CUDA runtime call failed */
-#define RDSPLIT_ETIMEOUT (-4)  /* a run's grid barrier saw no progress for too long
-                                  (rdsplit_set_wait_limit; not expected: its blocks
-                                  are resident).  The handle's counts, time and
-                                  period index are those of before the call */
+#define RDSPLIT_ETIMEOUT (-4)  /* a run's grid barrier was waited for longer than
+                                  its limit (rdsplit_set_wait_limit; not expected:
+                                  its blocks are resident).  Counts, time and period
+                                  index are those of before the call */
 #define RDSPLIT_EOVERFLOW (-5) /* a count would exceed INT32_MAX, or a
                                   period would exceed the per-tet event cap */
 #define RDSPLIT_ESTATE (-6)    /* call out of order (e.g. run before set_model) */
@@ -223,9 +223,10 @@ int rdsplit_set_period_kernel(rdsplit_mesh_t mesh, int32_t mode, int32_t block);
 int rdsplit_get_period_kernel(rdsplit_mesh_t mesh, int32_t* two_passes, int32_t* block);
 
 /*
- * How long a grid barrier of the handle's runs may see no progress before the
- * run gives up with RDSPLIT_ETIMEOUT: seconds > 0, 120 by default.  A tet with
- * many reaction events in one period counts as progress every 2^16 of them.
+ * How long a block of the handle's runs may wait at a grid barrier before the
+ * run gives up with RDSPLIT_ETIMEOUT: seconds > 0.  By default as long as a
+ * period may take: about a minute for a model of two reactions, up to half an
+ * hour for 32 reactions of 16 species on a mesh that fills the GPU.
  */
 int rdsplit_set_wait_limit(rdsplit_mesh_t mesh, double seconds);
 

@@ -174,7 +174,7 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
     int64_t jl = 0;       // of them in single launches since the last closing transfer
     const double t_start = h->t;
     const int64_t period_start = h->period;
-    bool saved = false;   // the counts of the start are in h->staging (see launch_run)
+    bool saved = false;   // the counts of the start are in h->staging (RunArgs::save)
     while (h->t < t_end && (max_periods < 0 || j < max_periods)) {
         h->inbox_dirty = true;   // until the closing transfer
         // the next stretch: one period, or as many as a resident launch takes
@@ -199,9 +199,9 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
         if (resident) {
             RunArgs r{(uint32_t)h->period, n, last ? 1 : 0, h->tau, tau_k, (float)h->tau, (float)tau_k, seed, h->thr,
                       h->thr_last, {h->inbox[0], h->inbox[1]}, {h->imask[0], h->imask[1]}, h->barrier,
-                      h->barrier_base, h->wait_limit_ns};
+                      h->barrier_base, h->wait_limit_ns, saved ? nullptr : h->staging};
             int grid = 0;
-            if (launch_run(m, h->mp, s, r, sms, &grid, saved ? nullptr : h->staging, h->stream)) {
+            if (launch_run(m, h->mp, s, r, sms, &grid, h->stream)) {
                 saved = saved || grid > 0;
                 h->barrier_base += (uint32_t)grid * (uint32_t)n;
                 h->inbox_dirty = false;
@@ -373,7 +373,7 @@ int mesh_create_impl(const char* where, int32_t n_tets, const int32_t* adj, cons
         (rc = alloc_into(&d_dist, 4 * T, "dist")) || (rc = alloc_into(&h->vol, T, "vol")) ||
         (rc = alloc_into(&h->src, T, "src")) || (rc = alloc_into(&h->g, 4 * T, "g")) ||
         (rc = alloc_into(&h->G, T, "G")) || (rc = alloc_into(&h->gmax, 1, "gmax")) ||
-        (rc = alloc_into(&h->err, kErrWords, "err")) || (rc = alloc_into(&h->barrier, 1, "barrier")) || (reorder && (rc = alloc_into(&h->perm, T, "order"))))
+        (rc = alloc_into(&h->err, 1, "err")) || (rc = alloc_into(&h->barrier, 1, "barrier")) || (reorder && (rc = alloc_into(&h->perm, T, "order"))))
         return cleanup(rc);
     cudaStream_t st = h->stream;
     cudaError_t ce = cudaSuccess;
@@ -383,7 +383,7 @@ int mesh_create_impl(const char* where, int32_t n_tets, const int32_t* adj, cons
     ce = ce ? ce : cudaMemcpyAsync(d_dist, centroid_dist, 32 * T, cudaMemcpyHostToDevice, st);
     if (reorder) ce = ce ? ce : cudaMemcpyAsync(h->perm, perm.data(), 4 * T, cudaMemcpyHostToDevice, st);
     ce = ce ? ce : cudaMemsetAsync(h->gmax, 0, sizeof(unsigned long long), st);
-    ce = ce ? ce : cudaMemsetAsync(h->err, 0, sizeof(uint32_t) * kErrWords, st);
+    ce = ce ? ce : cudaMemsetAsync(h->err, 0, sizeof(uint32_t), st);
     ce = ce ? ce : cudaMemsetAsync(h->barrier, 0, sizeof(uint32_t), st);
     if (ce != cudaSuccess) {
         cudaGetLastError();

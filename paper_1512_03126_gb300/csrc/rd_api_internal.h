@@ -37,7 +37,7 @@ struct rdsplit_mesh {
     uint32_t* barrier = nullptr;              // grid-barrier counter of a run's launches
     uint32_t barrier_base = 0;                // its value between runs
     bool inbox_dirty = false;                 // a run or partition run left inbox words or masks set
-    unsigned long long wait_limit_ns = rdk::kWaitLimitNs;   // of a run's grid barriers
+    unsigned long long wait_limit_ns = 0;     // of a run's grid barriers (0: derived from the model)
     uint4* thr = nullptr;
     uint4* thr_last = nullptr;
     int32_t* staging = nullptr;

@@ -726,9 +726,9 @@ cudaError_t launch_cluster(EngineLaunch& L) {
     // the attribute covers every group of this kernel, whatever its species
     const size_t most = (size_t)kWarps * engine_warp_words(SA == 1 ? 1 : kMaxS, R) * sizeof(int32_t) +
                         (SA == 1 ? sm_data_limit(R) : 0);
-    const cudaError_t ce = allow_shared((const void*)kern, most);
-    if (ce != cudaSuccess) return ce;
     const size_t dyn = (size_t)kWarps * engine_warp_words(L.S, R) * sizeof(int32_t) + L.data;
+    const cudaError_t ce = allow_shared((const void*)kern, dyn, most);
+    if (ce != cudaSuccess) return ce;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C, 1, 1);
     cfg.blockDim = dim3(kRunBlock, 1, 1);
@@ -998,7 +998,7 @@ int rdsplit_engine_create(int32_t max_slots, int64_t max_active_tets, rdsplit_en
     e->d_mp = (ModelParams*)rdapi::dev_alloc(sizeof(ModelParams) * max_slots);
     e->d_order = (int32_t*)rdapi::dev_alloc(sizeof(int32_t) * max_slots);
     e->d_head = (int32_t*)rdapi::dev_alloc(sizeof(int32_t) * kGroups);
-    e->err = (uint32_t*)rdapi::dev_alloc(sizeof(uint32_t) * kErrWords);
+    e->err = (uint32_t*)rdapi::dev_alloc(sizeof(uint32_t));
     e->processed = (unsigned long long*)rdapi::dev_alloc(sizeof(unsigned long long));
     e->d_times = (unsigned long long*)rdapi::dev_alloc(sizeof(unsigned long long) * 4 * max_slots);
     if (!e->d_desc || !e->d_mp || !e->d_order || !e->d_head || !e->err || !e->processed || !e->d_times) {
@@ -1015,7 +1015,7 @@ int rdsplit_engine_create(int32_t max_slots, int64_t max_active_tets, rdsplit_en
     warm_engine_kernels(e->d_head, e->err, e->processed, e->sms);
     if (cudaMemsetAsync(e->processed, 0, sizeof(unsigned long long), e->stream) != cudaSuccess ||
         cudaMemsetAsync(e->d_times, 0, sizeof(unsigned long long) * 4 * max_slots, e->stream) != cudaSuccess ||
-        cudaMemsetAsync(e->err, 0, sizeof(uint32_t) * kErrWords, e->stream) != cudaSuccess) {
+        cudaMemsetAsync(e->err, 0, sizeof(uint32_t), e->stream) != cudaSuccess) {
         cudaGetLastError();
         delete e;
         return rdapi::fail(RDSPLIT_ECUDA, "rdsplit_engine_create: memset failed");

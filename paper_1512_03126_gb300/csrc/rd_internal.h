@@ -20,14 +20,6 @@ enum : uint32_t {
     kErrEventCap = 1u << 6,      // more SSA events in one tet-period than the cap
     kErrTimeout = 1u << 7,       // a grid barrier's wait ran out
 };
-// Words of an error buffer: the bits above, and a count that a tet with very
-// many events in one period bumps as it goes (see grid_barrier).
-constexpr int kErrWords = 2;
-// A grid barrier gives up after this long without a bump: 20 times what the
-// events between two bumps take at their slowest (2^16 events of up to 30,000
-// cycles each, six warps sharing a multiprocessor's FP64 unit).
-constexpr unsigned long long kWaitLimitNs = 120ull * 1000000000ull;
-constexpr int kBumpEvents = 1 << 16;
 
 // Chemistry, passed by value to kernels (lives in the constant bank).
 struct ModelParams {
@@ -86,7 +78,7 @@ __device__ __forceinline__ int key_of(const DevMesh& m, int t) { return m.perm ?
 
 struct DevState {
     int32_t* cnt;           // [S][T] counts, in place over the periods of a run
-    uint32_t* err;          // error words [kErrWords]
+    uint32_t* err;          // error word
 };
 
 // ---- setup --------------------------------------------------------------
@@ -173,25 +165,26 @@ struct RunArgs {
     uint8_t* mask[2];
     uint32_t* barrier;      // grid-barrier counter; holds barrier_base before the launch
     uint32_t barrier_base;  // and barrier_base + grid * periods after it
-    unsigned long long wait_limit_ns = kWaitLimitNs;   // of a grid barrier without progress
+    unsigned long long wait_limit_ns = 0;   // of a grid barrier; 0: what the longest period may take
+    // A launch that ends with kErrTimeout leaves counts of different periods: the
+    // form with a grid barrier stores those it starts from here, unless null.
+    int32_t* save = nullptr;
 };
 // Launches it if the mesh's tets fit on the device at once (else, or when a
 // cooperative launch is refused, answers false with nothing launched); *grid
-// receives its blocks.  A launch that ends with kErrTimeout leaves counts of
-// different periods: unless `save` is null, a form that can end so copies the
-// counts there first.
+// receives its blocks (0: no grid barrier).
 bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int sms, int* grid,
-                int32_t* save, cudaStream_t st);
+                cudaStream_t st);
 int run_shape(int64_t T, int sms, int* warps);
 
-// Lets a kernel take up to `most` bytes of dynamic shared memory a block on the
-// current device (and, on request, clusters of more than 8 CTAs).  Called
-// before every launch of such a kernel with the most that any mesh and model
-// ask of it; the first call raises the limit, which belongs to the function
-// and not to a launch: set to each launch's own size, one thread's smaller
-// mesh lowered it between another's setting and its launch (two threads of 12
-// and 16 species: counts wrong within some thousand launches).
-cudaError_t allow_shared(const void* kern, size_t most, bool wide_clusters = false);
+// Called before a launch with `bytes` of dynamic shared memory a block, with the
+// most that any mesh and model ask of the kernel.  The limit beyond the default
+// 48 KB belongs to the function on a device, not to a launch, so the first
+// launch that needs it raises it to `most` for good: set to each launch's own
+// size, one thread's smaller mesh lowered it between another's setting and its
+// launch (two threads of 12 and 16 species: counts wrong within some thousand
+// launches).
+cudaError_t allow_shared(const void* kern, size_t bytes, size_t most);
 
 int64_t launches();
 int sm_count();       // multiprocessors of the current device

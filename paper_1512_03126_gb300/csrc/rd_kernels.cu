@@ -49,18 +49,26 @@ constexpr size_t block_shared_most(bool react) { return (size_t)(kBlock / 32) * 
 constexpr size_t kClusterShared = 200u * 1024u;
 }  // namespace
 
-cudaError_t allow_shared(const void* kern, size_t most, bool wide_clusters) {
+namespace {
+// Sets an attribute of a kernel once on each device.
+cudaError_t set_once(const void* kern, cudaFuncAttribute attr, int value) {
     static std::mutex mu;
-    static std::vector<std::pair<const void*, int>> raised;
+    static std::vector<std::pair<std::pair<const void*, int>, int>> done;
     int dev = 0;
     cudaError_t ce = cudaGetDevice(&dev);
     if (ce != cudaSuccess) return ce;
+    const auto what = std::make_pair(std::make_pair(kern, (int)attr), dev);
     std::lock_guard<std::mutex> lock(mu);
-    if (std::find(raised.begin(), raised.end(), std::make_pair(kern, dev)) != raised.end()) return cudaSuccess;
-    ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
-    if (ce == cudaSuccess && wide_clusters) ce = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (ce == cudaSuccess) raised.emplace_back(kern, dev);
+    if (std::find(done.begin(), done.end(), what) != done.end()) return cudaSuccess;
+    ce = cudaFuncSetAttribute(kern, attr, value);
+    if (ce == cudaSuccess) done.push_back(what);
     return ce;
+}
+}  // namespace
+
+cudaError_t allow_shared(const void* kern, size_t bytes, size_t most) {
+    if (bytes <= 48u * 1024u) return cudaSuccess;
+    return set_once(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
 int sm_count() {
@@ -627,11 +635,8 @@ k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams 
 // Grid barrier of a cooperative launch: the counter only grows, by one per
 // block and barrier; the wait ends when it reaches `target` (modulo 2^32).
 // The launch holds every block resident, so the wait is as long as the slowest
-// block's period.  That can be minutes (a tet's period goes up to 2^22 events
-// of some microseconds, and the warps of a multiprocessor share its FP64 unit),
-// so the limit is on the time without progress: a tet at work on many events
-// bumps err[1] every kBumpEvents of them.  Past the limit the block sets
-// kErrTimeout and gives up, and the others follow it.
+// block's period, which can be minutes (see longest_period_ns).  Past the limit
+// the block sets kErrTimeout and gives up, and the others follow it.
 __device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target, uint32_t* err,
                                              unsigned long long limit_ns, volatile int* gave_up) {
     __syncthreads();
@@ -639,7 +644,6 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target,
         __threadfence();   // the block's inbox words before its arrival
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
         unsigned long long start = 0ull;
-        uint32_t bumps = 0u;
         for (uint32_t i = 1;; ++i) {
             uint32_t c;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(counter) : "memory");
@@ -647,9 +651,7 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target,
             if ((i & 1023u) == 0u) {
                 unsigned long long now;
                 asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-                const uint32_t b = __ldcg(err + 1);
-                if (start == 0ull || b != bumps) start = now;
-                bumps = b;
+                if (start == 0ull) start = now;
                 if (now - start > limit_ns || (__ldcg(err) & kErrTimeout)) {
                     atomicOr(err, kErrTimeout);
                     *gave_up = 1;
@@ -696,6 +698,7 @@ k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp,
             const int32_t n = s.cnt[sp * T + t];
             w.N[32 * sp + lane] = n;
             pr.add(sp, n);
+            if (r.save) r.save[sp * T + t] = n;
         }
     uint32_t bad = 0, dirty = 0, target = r.barrier_base;
     for (int q = 0; q <= r.periods; ++q) {
@@ -942,7 +945,8 @@ cudaError_t launch_cluster_s(const DevMesh& m, const ModelParams& mp, const DevS
                              int warps, cudaStream_t st) {
     auto kern = k_run_cluster<S_, kReact>;
     const size_t smem = (size_t)cluster_words(mp.S, kReact, warps) * sizeof(int32_t);
-    cudaError_t ce = allow_shared((const void*)kern, kClusterShared, true);
+    cudaError_t ce = allow_shared((const void*)kern, smem, kClusterShared);
+    if (ce == cudaSuccess && ctas > 8) ce = set_once((const void*)kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (ce != cudaSuccess) return ce;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas, 1, 1);
@@ -976,12 +980,22 @@ int run_shape(int64_t T, int sms, int* warps) {
     return (int)((chunks + *warps - 1) / *warps);
 }
 
+// What a period of k_run may take at most, doubled: the event cap, at 12,000
+// cycles an event and 1,000 for each reaction and species of the model (10,000
+// measured with two of each, 16,000 with 30 reactions and eleven species), a
+// clock of half the usual 2 GHz, and the warps of a multiprocessor sharing its
+// FP64 unit, which four of them keep busy.
+unsigned long long longest_period_ns(const ModelParams& mp, int warps_per_sm) {
+    const unsigned long long cycles = 12000ull + 1000ull * (unsigned)(mp.R + mp.S);
+    return (unsigned long long)kEventCap * cycles * (unsigned)std::max(4, warps_per_sm) / 4ull;
+}
+
 template <int S_, bool kReact, int kBlocks>
 cudaError_t launch_run_b(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int grid,
                          int warps, int sms, cudaStream_t st) {
     auto kern = k_run<S_, kReact, kBlocks>;
     const size_t smem = (size_t)warps * warp_words(mp.S, kReact) * sizeof(int32_t);
-    cudaError_t ce = allow_shared((const void*)kern, block_shared_most(kReact));
+    cudaError_t ce = allow_shared((const void*)kern, smem, block_shared_most(kReact));
     int fit = 0;
     if (ce == cudaSuccess) ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, 32 * warps, smem);
     if (ce == cudaSuccess && (int64_t)fit * sms < grid) ce = cudaErrorCooperativeLaunchTooLarge;
@@ -990,6 +1004,7 @@ cudaError_t launch_run_b(const DevMesh& m, const ModelParams& mp, const DevState
     ModelParams mp_ = mp;
     DevState s_ = s;
     RunArgs r_ = r;
+    if (r_.wait_limit_ns == 0) r_.wait_limit_ns = longest_period_ns(mp, warps * ((grid + sms - 1) / sms));
     void* args[] = {&m_, &mp_, &s_, &r_};
     ce = cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(32 * warps), args, smem, st);
     if (ce == cudaSuccess) ++g_launches;
@@ -1004,7 +1019,7 @@ cudaError_t launch_run_s(const DevMesh& m, const ModelParams& mp, const DevState
 }
 
 bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int sms, int* grid,
-                int32_t* save, cudaStream_t st) {
+                cudaStream_t st) {
     int warps = 0;
     cudaError_t ce = cudaErrorInvalidConfiguration;
     // 16 CTAs are beyond the portable cluster size: where the device has no
@@ -1024,9 +1039,6 @@ bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, cons
     }
     *grid = run_shape(m.T, sms, &warps);
     if (*grid == 0) return false;
-    if (save && cudaMemcpyAsync(save, s.cnt, sizeof(int32_t) * (size_t)m.T * mp.S, cudaMemcpyDeviceToDevice, st) !=
-                    cudaSuccess)
-        return false;   // the caller's next launch reports it
     if (mp.S == 1)
         ce = mp.any_reaction ? launch_run_s<1, true>(m, mp, s, r, *grid, warps, sms, st)
                              : launch_run_s<1, false>(m, mp, s, r, *grid, warps, sms, st);
@@ -1042,7 +1054,7 @@ void launch_pass(const DevMesh& m, const ModelParams& mp, const DevState& s, con
                  int32_t* qcount, int32_t parity, int grid, int block, cudaStream_t st) {
     const size_t smem = (size_t)(block / 32) * warp_words(mp.S, kReact) * sizeof(int32_t);
     // large blocks of many species; a failure is reported as the launch's (last error)
-    if (S_ != 1 && allow_shared((const void*)k_period<S_, kReact, kPass>, block_shared_most(kReact)) != cudaSuccess) return;
+    if (allow_shared((const void*)k_period<S_, kReact, kPass>, smem, block_shared_most(kReact)) != cudaSuccess) return;
     k_period<S_, kReact, kPass><<<grid, block, smem, st>>>(m, mp, s, a, queue, qcount, parity);
     ++g_launches;
 }

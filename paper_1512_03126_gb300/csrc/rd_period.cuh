@@ -7,7 +7,6 @@
 namespace rdk {
 
 constexpr int kEventCap = 1 << 22;   // SSA events per tet and period
-static_assert(kEventCap % kBumpEvents == 0, "the cap is looked at where a tet says that it is at work");
 // Below this N* the diffusion draw is one uniform per molecule (the paper's
 // per-molecule form, Sec. II.B); at or above it, Binomial + conditional
 // binomials in double precision.

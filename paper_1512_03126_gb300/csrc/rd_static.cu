@@ -259,7 +259,7 @@ extern "C" int rdsplit_run_static(int32_t n_tets, const int32_t* d_adj, const do
             RunArgs r{(uint32_t)pk, n, 0, tau_k, tau_k, (float)tau_k, (float)tau_k, seed, thr, thr,
                       {out[0], out[1]}, {mask[0], mask[1]}, barrier, barrier_base};
             int grid = 0;
-            if (!launch_run(m, mp, s, r, sms, &grid, nullptr, st)) {   // d_counts still holds the counts
+            if (!launch_run(m, mp, s, r, sms, &grid, st)) {   // (d_counts still holds the counts)
                 resident = false;
                 continue;
             }

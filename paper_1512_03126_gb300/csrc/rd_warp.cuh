@@ -296,66 +296,58 @@ static __device__ __noinline__ uint32_t react_exact(const ModelParams& mp, int k
     bool past_half = false;
     rdd::Stream st(seed, (uint32_t)key, period, rdd::kPurposeReaction, 0);
     double tc = 0.0;
-    // in stretches of kBumpEvents (an atomic in the events' own loop made it
-    // 4 % slower)
     for (int events = 0;;) {
-        bool more = false;
-        for (;;) {
-            uint32_t poss = on & mp.kpos;
-            for (int s = 0; s < S; ++s) {
-                if (N[s] <= 0) poss &= ~mp.needs[s];
-                else if (N[s] == 1) poss &= ~mp.needs2[s];
-            }
-            if (!poss) break;                          // a0 = 0
-            // propensity a_r = c_r h_r, h_r the number of reactant combinations
-            double a0 = 0.0;
-            for (uint32_t bits = poss; bits; bits &= bits - 1u) {
-                const int r = __ffs(bits) - 1, a1 = mp.rs1[r], a2 = mp.rs2[r];
-                if (!((have >> r) & 1u)) {
-                    const double kr = mp.k[r];
-                    const int o = mp.order[r];
-                    c[r] = o == 0 ? kr * avv : (o == 1 ? kr : kr / avv);
-                    have |= 1u << r;
-                }
-                int64_t h = 1;
-                if (a1 >= 0) {
-                    if (a2 < 0) h = N[a1];
-                    else if (a1 == a2) h = N[a1] * (N[a1] - 1) / 2;
-                    else h = N[a1] * N[a2];
-                }
-                a[r] = c[r] * (double)h;
-                a0 = a0 + a[r];
-            }
-            if (!(a0 > 0.0)) break;
-            const double tn = tc + (-rdd::own_log(st.u01_open0())) / a0;
-            if (tn >= tau_k) break;
-            if (want_mid && !past_half && tn >= half) {
-                for (int s = 0; s < S; ++s) nmid[s] = N[s];
-                past_half = true;
-            }
-            const double target = st.u01() * a0;
-            int mu = -1, positive = -1;
-            double cum = 0.0;
-            for (uint32_t bits = poss; bits; bits &= bits - 1u) {
-                const int r = __ffs(bits) - 1;
-                cum = cum + a[r];
-                if (a[r] > 0.0) positive = r;
-                if (target < cum) { mu = r; break; }
-            }
-            if (mu < 0) mu = positive;
-            for (uint32_t bits = mp.rx[mu].y >> 16; bits; bits &= bits - 1u) {
-                const int s = __ffs(bits) - 1;
-                occ[s] = occ[s] + (double)N[s] * (tn - tl[s]);
-                tl[s] = tn;
-                touched |= 1u << s;
-                N[s] += mp.delta[mu][s];
-            }
-            tc = tn;
-            if (++events % kBumpEvents == 0) { more = true; break; }
+        uint32_t poss = on & mp.kpos;
+        for (int s = 0; s < S; ++s) {
+            if (N[s] <= 0) poss &= ~mp.needs[s];
+            else if (N[s] == 1) poss &= ~mp.needs2[s];
         }
-        if (!more) break;
-        if (events >= kEventCap) { atomicOr(err, kErrEventCap); break; }
-        atomicAdd(err + 1, 1u);   // still at work (see grid_barrier)
+        if (!poss) break;                          // a0 = 0
+        // propensity a_r = c_r h_r, h_r the number of reactant combinations
+        double a0 = 0.0;
+        for (uint32_t bits = poss; bits; bits &= bits - 1u) {
+            const int r = __ffs(bits) - 1, a1 = mp.rs1[r], a2 = mp.rs2[r];
+            if (!((have >> r) & 1u)) {
+                const double kr = mp.k[r];
+                const int o = mp.order[r];
+                c[r] = o == 0 ? kr * avv : (o == 1 ? kr : kr / avv);
+                have |= 1u << r;
+            }
+            int64_t h = 1;
+            if (a1 >= 0) {
+                if (a2 < 0) h = N[a1];
+                else if (a1 == a2) h = N[a1] * (N[a1] - 1) / 2;
+                else h = N[a1] * N[a2];
+            }
+            a[r] = c[r] * (double)h;
+            a0 = a0 + a[r];
+        }
+        if (!(a0 > 0.0)) break;
+        const double tn = tc + (-rdd::own_log(st.u01_open0())) / a0;
+        if (tn >= tau_k) break;
+        if (want_mid && !past_half && tn >= half) {
+            for (int s = 0; s < S; ++s) nmid[s] = N[s];
+            past_half = true;
+        }
+        const double target = st.u01() * a0;
+        int mu = -1, positive = -1;
+        double cum = 0.0;
+        for (uint32_t bits = poss; bits; bits &= bits - 1u) {
+            const int r = __ffs(bits) - 1;
+            cum = cum + a[r];
+            if (a[r] > 0.0) positive = r;
+            if (target < cum) { mu = r; break; }
+        }
+        if (mu < 0) mu = positive;
+        for (uint32_t bits = mp.rx[mu].y >> 16; bits; bits &= bits - 1u) {
+            const int s = __ffs(bits) - 1;
+            occ[s] = occ[s] + (double)N[s] * (tn - tl[s]);
+            tl[s] = tn;
+            touched |= 1u << s;
+            N[s] += mp.delta[mu][s];
+        }
+        tc = tn;
+        if (++events >= kEventCap) { atomicOr(err, kErrEventCap); break; }
     }
     if (want_mid && !past_half)
         for (int s = 0; s < S; ++s) nmid[s] = N[s];
@@ -595,10 +587,6 @@ __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParam
                                               const PeriodView& v, int t, bool live, uint32_t mask, Presence& pr,
                                               uint32_t* dirty, bool* deferred, uint32_t* err, Emit& emit,
                                               uint4 pre = make_uint4(0u, 0u, 0u, 0u), bool tried = false) {
-    // The lanes come from loops over their own inbox words: unless they are brought
-    // together here, each goes through the reaction phase by itself (10,368 tets
-    // of eleven species, up to 475 events a period, 60 periods: 82 ms instead of 43).
-    __syncwarp();
     const int lane = threadIdx.x & 31;
     const int key = live ? key_of(m, t) : 0;
     uint32_t bad = 0, touched = 0;
@@ -607,7 +595,11 @@ __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParam
     if (kReact) {
         const uint32_t on = mask & mp.kpos;
         const uint32_t poss = live && (kCalls || !*deferred) ? possible_by_presence(mp, pr, S, on) : 0u;
-        if (poss) {
+        // The lanes come from loops over their own inbox words: unless they are
+        // brought together here, each goes through the reaction phase by itself
+        // (10,368 tets of eleven species, up to 475 events a period, 60 periods: 82
+        // ms instead of 42).
+        if (__ballot_sync(kAllLanes, poss != 0u) && poss) {
             const float2 avf = __ldg(m.avv + t);
             if (kDefer) {
                 // only the first waiting time, by its bound

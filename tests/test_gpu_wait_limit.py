@@ -1,4 +1,4 @@
-"""A run whose grid barrier sees no progress for the handle's limit ends with
+"""A run whose grid barrier is waited for longer than the handle's limit ends with
 RDSPLIT_ETIMEOUT and leaves counts, time and period index as they were before
 the call; within the limit a long period is no error.  One tet has some tens of
 thousands of reaction events in a period while all others wait for it."""
@@ -45,18 +45,16 @@ def test_running_out_leaves_the_state_of_before_the_call(rd, oracle):
                 sim.run_periods(2, 9)
             assert e.value.code == rd.RDSPLIT_ETIMEOUT
             assert np.array_equal(sim.counts(), first) and sim.time == when
-        rd.rdsplit_set_wait_limit(sim.h, 120.0)
+        rd.rdsplit_set_wait_limit(sim.h, 60.0)
         sim.run_periods(2, 9)
         assert np.array_equal(sim.counts(), ref)
 
 
-def test_progress_restarts_the_limit(rd, oracle):
-    """About 400,000 events, some seconds, under a limit that covers 2^16 of
-    them at the slowest (30,000 cycles each) but not all."""
+def test_a_long_period_is_no_error(rd, oracle):
+    """About 300,000 events of one tet, a second and more, within the default limit."""
     mesh, model, counts = one_busy_tet(4e5)
     ref = oracle.run(mesh, model, counts, np.inf, 9, max_periods=1)[0]
     with rd.Simulation(mesh, model, counts) as sim:
-        rd.rdsplit_set_wait_limit(sim.h, 1.0)
         sim.run_periods(1, 9)
         assert np.array_equal(sim.counts(), ref)
 

@@ -164,6 +164,10 @@ __device__ __forceinline__ int react_fast(const ModelParams& mp, const uint2* rx
                                           uint32_t* scratch, Presence& pr, uint32_t* touched_out) {
     constexpr float e = 5.9604644775390625e-08f;   // 2^-24
     constexpr int kMaxEvents = 64;
+    // A tet that expects more events than this at the start of the period would
+    // go past kMaxEvents, mostly (162 tets of two species, about 75 events a
+    // period, 20 periods: 12.5 ms with the attempt, 11.5 without).
+    float longest = 72.0f;
     const bool mid = mp.rule == kRuleMid;
     const uint32_t k0 = (uint32_t)v.seed, k1 = (uint32_t)(v.seed >> 32);
     float x = 0.0f, dsum = 0.0f;
@@ -184,7 +188,7 @@ __device__ __forceinline__ int react_fast(const ModelParams& mp, const uint2* rx
         const float eps = (float)(26 + m + 2 * k) * e;
         const uint64_t y = 9007199254740991ull - x1;                    // (1 - u1) 2^53
         const float ylo = (float)(uint32_t)(y >> 29) * e;               // at most 1 - u1
-        if (!(at < 1e30f)) { doubt = true; break; }
+        if (!(at < longest)) { doubt = true; break; }
         if (ylo > 0.0f && ylo >= at * ((1.0f + eps) - x) * 1.0001f) break;   // no event before tau_k
         if (!(at > 1e-6f)) { doubt = true; break; }
         const uint4 rw_next =
@@ -239,6 +243,7 @@ __device__ __forceinline__ int react_fast(const ModelParams& mp, const uint2* rx
             dmax = fmaxf(dmax, fabsf((float)dn));
         }
         dsum += dmax;
+        longest = 1e30f;
         x = xn;
         rw = rw_next;
         if (++k > kMaxEvents || dsum > (float)(kMoleculeCut - kDeferMin - 1)) doubt = true;

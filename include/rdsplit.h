@@ -46,7 +46,9 @@ extern "C" {
 #define RDSPLIT_ETIMEOUT (-4)  /* a run's grid barrier was waited for longer than
                                   its limit (rdsplit_set_wait_limit; not expected:
                                   its blocks are resident).  Counts, time and period
-                                  index are those of before the call */
+                                  index are those of before the call (or of the
+                                  period, before the wait, from which on the call
+                                  spread a small mesh over the whole device) */
 #define RDSPLIT_EOVERFLOW (-5) /* a count would exceed INT32_MAX, or a
                                   period would exceed the per-tet event cap */
 #define RDSPLIT_ESTATE (-6)    /* call out of order (e.g. run before set_model) */
@@ -209,8 +211,10 @@ int rdsplit_get_shape(rdsplit_mesh_t mesh, int32_t* n_tets, int32_t* n_species);
  *           more warps per SM) and defers the others to the second
  *   mode 0  automatic (default): while all tets of the mesh are resident on
  *           the GPU at once (up to 24 warps of 32 tets per multiprocessor),
- *           many periods per launch with a grid barrier between them; else
- *           one pass per period
+ *           many periods per launch: within one cluster of 16 multiprocessors
+ *           for small meshes while most tets need no double-precision sampler,
+ *           else with a grid barrier between them; for larger meshes one pass
+ *           per period
  *   block   threads per block of the period kernel (of the first pass in
  *           mode 2): a multiple of 32 in 32..256, or 0 (default) for a size
  *           chosen from the mesh (smaller blocks for small meshes, so that

@@ -80,11 +80,15 @@ int alloc_into(T** p, size_t count, const char* what) {
     return RDSPLIT_OK;
 }
 
-// Read and clear the device error word; translate kernel error bits.
-int check_err_impl(rdsplit_mesh* h, const char* where) {
-    uint32_t e = 0;
-    CUDA_TRY(cudaMemcpyAsync(&e, h->err, sizeof e, cudaMemcpyDeviceToHost, h->stream));
+// Read and clear the device error word; translate kernel error bits.  left:
+// receives, and clears, the word after it (RunArgs::left).
+int check_err_impl(rdsplit_mesh* h, const char* where, uint32_t* left = nullptr) {
+    uint32_t w[2] = {0, 0};
+    CUDA_TRY(cudaMemcpyAsync(w, h->err, left ? 2 * sizeof(uint32_t) : sizeof(uint32_t), cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
+    const uint32_t e = w[0];
+    if (left) *left = w[1];
+    if (w[1]) CUDA_TRY(cudaMemsetAsync(h->err + 1, 0, sizeof(uint32_t), h->stream));
     if (e == 0) return RDSPLIT_OK;
     CUDA_TRY(cudaMemsetAsync(h->err, 0, sizeof(uint32_t), h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
@@ -172,9 +176,13 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
     if (h->inbox_dirty) CUDA_TRY(clear_inboxes(h));
     int64_t j = 0;        // periods done
     int64_t jl = 0;       // of them in single launches since the last closing transfer
-    const double t_start = h->t;
-    const int64_t period_start = h->period;
-    bool saved = false;   // the counts of the start are in h->staging (RunArgs::save)
+    bool saved = false;   // the counts of t_saved are in h->staging (RunArgs::save)
+    double t_saved = h->t;
+    int64_t period_saved = h->period;
+    int spread = 0;       // periods to go with the mesh spread over the device
+    bool unchecked = true;
+    uint32_t left = 0;
+    int rc = RDSPLIT_OK;
     while (h->t < t_end && (max_periods < 0 || j < max_periods)) {
         h->inbox_dirty = true;   // until the closing transfer
         // the next stretch: one period, or as many as a resident launch takes
@@ -185,6 +193,7 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
         if (room <= 0) return fail(RDSPLIT_EOVERFLOW, "rdsplit_run: period index exceeds 2^32-1");
         int64_t most = std::min<int64_t>(resident ? kRunPeriods : 1, room);
         if (max_periods >= 0) most = std::min<int64_t>(most, max_periods - j);
+        if (spread > 0) most = std::min<int64_t>(most, spread);
         while (n < most && t < t_end) {
             if (t + h->tau > t_end) {
                 tau_k = t_end - t;
@@ -199,15 +208,32 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
         if (resident) {
             RunArgs r{(uint32_t)h->period, n, last ? 1 : 0, h->tau, tau_k, (float)h->tau, (float)tau_k, seed, h->thr,
                       h->thr_last, {h->inbox[0], h->inbox[1]}, {h->imask[0], h->imask[1]}, h->barrier,
-                      h->barrier_base, h->wait_limit_ns, saved ? nullptr : h->staging};
+                      h->barrier_base, h->wait_limit_ns, saved ? nullptr : h->staging, h->err + 1, spread > 0 ? 1 : 0};
             int grid = 0;
             if (launch_run(m, h->mp, s, r, sms, &grid, h->stream)) {
-                saved = saved || grid > 0;
+                if (grid > 0 && !saved) {
+                    saved = true;
+                    t_saved = h->t;
+                    period_saved = h->period;
+                }
                 h->barrier_base += (uint32_t)grid * (uint32_t)n;
                 h->inbox_dirty = false;
+                const double t0 = h->t;
                 h->t = t;
                 h->period += n;
                 j += n;
+                spread = std::max(0, spread - n);
+                unchecked = grid > 0;
+                if (grid == 0) {   // within one cluster: done, or left early?
+                    if ((rc = launch_check("rdsplit_run")) || (rc = check_err_impl(h, "rdsplit_run", &left))) break;
+                    if (left > 0) {
+                        h->t = t0;
+                        for (uint32_t i = 1; i < left; ++i) h->t += h->tau;
+                        h->period -= n - (int64_t)(left - 1u);
+                        j -= n - (int64_t)(left - 1u);
+                        spread = kSpreadPeriods;
+                    }
+                }
                 continue;
             }
             resident = false;
@@ -230,7 +256,9 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
         h->period += 1;
         j += 1;
         jl += 1;
+        unchecked = true;
     }
+    if (rc || !unchecked) return rc;
     if (jl > 0) {
         const int q = (int)((jl - 1) & 1);
         PeriodArgs a{};
@@ -238,19 +266,18 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
         a.mask_prev = h->imask[q];
         launch_gather(m, h->S, s, a, h->stream);
     }
-    int rc = launch_check("rdsplit_run");
-    if (rc) return rc;
+    if ((rc = launch_check("rdsplit_run"))) return rc;
     h->inbox_dirty = false;
     rc = check_err(h, "rdsplit_run");
-    if (rc == RDSPLIT_ETIMEOUT) {   // blocks left a launch early: back to where the call began
+    if (rc == RDSPLIT_ETIMEOUT) {   // blocks left a launch early: back to the counts saved
         h->inbox_dirty = true;
         CUDA_TRY(cudaMemsetAsync(h->barrier, 0, sizeof(uint32_t), h->stream));
         h->barrier_base = 0;
         if (saved)
             CUDA_TRY(cudaMemcpyAsync(h->cnt, h->staging, sizeof(int32_t) * (size_t)h->T * h->S,
                                      cudaMemcpyDeviceToDevice, h->stream));
-        h->t = t_start;
-        h->period = period_start;
+        h->t = t_saved;
+        h->period = period_saved;
     }
     collect_timing(h);
     return rc;
@@ -373,7 +400,7 @@ int mesh_create_impl(const char* where, int32_t n_tets, const int32_t* adj, cons
         (rc = alloc_into(&d_dist, 4 * T, "dist")) || (rc = alloc_into(&h->vol, T, "vol")) ||
         (rc = alloc_into(&h->src, T, "src")) || (rc = alloc_into(&h->g, 4 * T, "g")) ||
         (rc = alloc_into(&h->G, T, "G")) || (rc = alloc_into(&h->gmax, 1, "gmax")) ||
-        (rc = alloc_into(&h->err, 1, "err")) || (rc = alloc_into(&h->barrier, 1, "barrier")) || (reorder && (rc = alloc_into(&h->perm, T, "order"))))
+        (rc = alloc_into(&h->err, 2, "err")) || (rc = alloc_into(&h->barrier, 1, "barrier")) || (reorder && (rc = alloc_into(&h->perm, T, "order"))))
         return cleanup(rc);
     cudaStream_t st = h->stream;
     cudaError_t ce = cudaSuccess;
@@ -383,7 +410,7 @@ int mesh_create_impl(const char* where, int32_t n_tets, const int32_t* adj, cons
     ce = ce ? ce : cudaMemcpyAsync(d_dist, centroid_dist, 32 * T, cudaMemcpyHostToDevice, st);
     if (reorder) ce = ce ? ce : cudaMemcpyAsync(h->perm, perm.data(), 4 * T, cudaMemcpyHostToDevice, st);
     ce = ce ? ce : cudaMemsetAsync(h->gmax, 0, sizeof(unsigned long long), st);
-    ce = ce ? ce : cudaMemsetAsync(h->err, 0, sizeof(uint32_t), st);
+    ce = ce ? ce : cudaMemsetAsync(h->err, 0, 2 * sizeof(uint32_t), st);
     ce = ce ? ce : cudaMemsetAsync(h->barrier, 0, sizeof(uint32_t), st);
     if (ce != cudaSuccess) {
         cudaGetLastError();

@@ -105,6 +105,10 @@ inline int period_block(const rdsplit_mesh* h, int sms) {
 }
 // Periods a launch of k_run takes at most (some milliseconds to tens of them).
 constexpr int kRunPeriods = 4096;
+// Periods that a run spreads over the device when the form within one cluster
+// has left (RunArgs::left), before it goes back to it: a launch and a wait for
+// them cost less than a hundredth of that.
+constexpr int kSpreadPeriods = 128;
 int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed);
 int check_err(rdsplit_mesh* h, const char* where);
 }  // namespace rdapi

@@ -169,10 +169,15 @@ struct RunArgs {
     // A launch that ends with kErrTimeout leaves counts of different periods: the
     // form with a grid barrier stores those it starts from here, unless null.
     int32_t* save = nullptr;
+    // The form within one cluster may leave before its last period (see
+    // k_run_cluster) and then stores here the periods done, plus 1, unless null.
+    // It is skipped where the mesh is to be spread over the whole device.
+    uint32_t* left = nullptr;
+    int32_t spread = 0;
 };
 // Launches it if the mesh's tets fit on the device at once (else, or when a
 // cooperative launch is refused, answers false with nothing launched); *grid
-// receives its blocks (0: no grid barrier).
+// receives its blocks (0: the form within one cluster).
 bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, const RunArgs& r, int sms, int* grid,
                 cudaStream_t st);
 int run_shape(int64_t T, int sms, int* warps);

@@ -336,7 +336,7 @@ __global__ void k_counts_in(int32_t T, int32_t S, const int32_t* __restrict__ ts
 __global__ void k_counts_out(int32_t T, int32_t S, const int32_t* __restrict__ sm, int32_t* __restrict__ ts,
                              const int32_t* __restrict__ perm, const uint32_t* __restrict__ err) {
     extern __shared__ int32_t tile[];
-    if (err && (*err & kErrTimeout)) return;
+    if (err && ((err[0] & kErrTimeout) || err[1])) return;   // gave up, or left early
     const int ld = S | 1;
     const int64_t t0 = (int64_t)blockIdx.x * kBlock;
     const int n = (int)min((int64_t)kBlock, T - t0);
@@ -677,6 +677,7 @@ __global__ void __launch_bounds__(kBlock, kBlocks)
 k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp, DevState s,
       const __grid_constant__ RunArgs r) {
     extern __shared__ int32_t sm[];
+    if (r.left && __ldcg(r.left)) return;   // queued behind a launch that left early
     __shared__ int gave_up;
     const int S = S_ > 0 ? S_ : mp.S;
     const int lane = threadIdx.x & 31;
@@ -783,12 +784,23 @@ struct ClusterSender {
     }
 };
 
+// At most 16 multiprocessors hold the mesh.  Where most tets need the
+// double-precision samplers their FP64 units set the period, and the whole
+// device would share that work: a warp that left kLeaveLanes or more of its tets
+// to them asks all CTAs to leave after the period, and the caller goes on with
+// the mesh spread over the device (k_run) for a while.  7,986 tets of 5,000
+// molecules, 12 periods: 6.9 ms within the cluster, 2.7 so.  (Up to four warps a
+// CTA the FP64 units of 16 multiprocessors serve as well: RunArgs::left is null.)
+constexpr int kLeaveLanes = 16;
+constexpr int kLeaveWarps = 4;
+
 template <bool kReact>
 static __device__ __noinline__ uint32_t step_deferred_in_cluster(const DevMesh& m, const ModelParams& mp,
                                                                  int32_t* column0, const uint2* rx, uint32_t period,
                                                                  double tau_k, uint64_t seed, const uint4* thr,
                                                                  uint4 slot, uint32_t words, uint32_t masks, int t,
-                                                                 bool live, bool tried, uint32_t* err) {
+                                                                 bool live, bool tried, uint32_t* err,
+                                                                 uint32_t stop_at, uint32_t after) {
     const int S = mp.S, lane = threadIdx.x & 31;
     const WarpMem w(column0, S, kReact, rx);
     const PeriodView v{period, tau_k, (float)tau_k, seed, thr, 1};
@@ -801,14 +813,16 @@ static __device__ __noinline__ uint32_t step_deferred_in_cluster(const DevMesh& 
     const uint32_t bad = warp_step<false, kReact, false, true>(m, mp, S, w, v, t, live, mask, pr, &dirty, &none, err, send,
                                                                make_uint4(0u, 0u, 0u, 0u), tried);
     if (live) send.finish();
+    if (stop_at != 0u && __popc(__ballot_sync(kAllLanes, live)) >= kLeaveLanes && lane < (int)gridDim.x)
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(map_to_cta(stop_at, (uint32_t)lane)), "r"(after) : "memory");
     return (live ? dirty : 0u) | (bad << 16);
 }
 
 // Dynamic shared memory of a CTA of `warps` warps, in words: the warps'
 // (rd_warp.cuh), then per tet two parities of four slots of S words and of
-// four 16-bit masks.
+// four 16-bit masks, and a word that says when to leave.
 __host__ __device__ inline int cluster_words(int S, bool react, int warps) {
-    return warps * warp_words(S, react) + 32 * warps * (8 * S + 4);
+    return warps * warp_words(S, react) + 32 * warps * (8 * S + 4) + 4;
 }
 
 template <int S_, bool kReact>
@@ -816,6 +830,7 @@ __global__ void __launch_bounds__(512, 1)
 k_run_cluster(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp, DevState s,
               const __grid_constant__ RunArgs r) {
     extern __shared__ __align__(16) int32_t sm[];
+    if (r.left && __ldcg(r.left)) return;   // queued behind a launch that left early
     const int S = S_ > 0 ? S_ : mp.S;
     const int lane = threadIdx.x & 31;
     const int warps = blockDim.x >> 5, B = blockDim.x;
@@ -826,7 +841,7 @@ k_run_cluster(const __grid_constant__ DevMesh m, const __grid_constant__ ModelPa
     int32_t* words = sm + warps * warp_words(S, kReact);                      // [2][B][4][S]
     unsigned long long* masks = reinterpret_cast<unsigned long long*>(words + 8 * S * B);   // [2][B]
     for (int i = threadIdx.x; i < 8 * S * B; i += B) words[i] = 0;
-    for (int i = threadIdx.x; i < 2 * B; i += B) masks[i] = 0ull;
+    for (int i = threadIdx.x; i < 2 * B + 1; i += B) masks[i] = 0ull;   // and the word to leave
     // Warp w of the cluster's W takes tets w, w + W, w + 2 W, ...: a compact
     // cloud's crowded tets go to different warps (a warp's 32 consecutive tets
     // around a point source made all others wait: 3,072-tet cube 4.7 us a
@@ -861,10 +876,17 @@ k_run_cluster(const __grid_constant__ DevMesh m, const __grid_constant__ ModelPa
     cluster_sync_all();   // every CTA's words and masks are zero
     const uint32_t words_at = (uint32_t)__cvta_generic_to_shared(words);
     const uint32_t masks_at = (uint32_t)__cvta_generic_to_shared(masks);
+    const uint32_t stop_at = masks_at + (uint32_t)(B * 16);   // the period after which a warp asked to leave, plus 1
     for (int q = 0; q <= r.periods; ++q) {
         const int p = q & 1;
+        bool leave = false;
         if (q > 0) {
             cluster_sync_all();
+            // all CTAs agree: nobody starts period q before all have finished
+            // q - 1, and a request made in period q itself reads q + 1
+            uint32_t asked;
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(asked) : "r"(stop_at) : "memory");
+            leave = asked != 0u && asked <= (uint32_t)q;
             if (live) {
                 auto add = [&](int sp, int64_t v) {
                     int64_t n = w.N[32 * sp + lane] + v;
@@ -898,7 +920,8 @@ k_run_cluster(const __grid_constant__ DevMesh m, const __grid_constant__ ModelPa
                 }
             }
         }
-        if (q == r.periods) break;
+        if (leave && q < r.periods && blockIdx.x == 0 && threadIdx.x == 0) *r.left = (uint32_t)q + 1u;
+        if (leave || q == r.periods) break;
         const bool last = r.last_short && q == r.periods - 1;
         const PeriodView v{r.period0 + (uint32_t)q, last ? r.tau_last : r.tau, last ? r.tau_lastf : r.tauf, r.seed,
                            last ? r.thr_last : r.thr, 1};
@@ -913,7 +936,7 @@ k_run_cluster(const __grid_constant__ DevMesh m, const __grid_constant__ ModelPa
             const uint32_t x = step_deferred_in_cluster<kReact>(
                 m, mp, w.N, w.rx, v.period, v.tau_k, v.seed, v.thr,
                 make_uint4(send.slot[0], send.slot[1], send.slot[2], send.slot[3]), send.words, send.masks, t, deferred,
-                (pr.many >> 16) == 0u, s.err);
+                (pr.many >> 16) == 0u, s.err, r.left ? stop_at : 0u, (uint32_t)q + 1u);
             dirty |= x & 0xffffu;
             bad |= x >> 16;
             if (deferred) pr = presence_of(w.N + lane, S);
@@ -960,7 +983,9 @@ cudaError_t launch_cluster_s(const DevMesh& m, const ModelParams& mp, const DevS
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    ce = cudaLaunchKernelEx(&cfg, kern, m, mp, s, r);
+    RunArgs r_ = r;
+    if (warps <= kLeaveWarps) r_.left = nullptr;
+    ce = cudaLaunchKernelEx(&cfg, kern, m, mp, s, r_);
     if (ce == cudaSuccess) ++g_launches;
     return ce;
 }
@@ -1004,6 +1029,7 @@ cudaError_t launch_run_b(const DevMesh& m, const ModelParams& mp, const DevState
     ModelParams mp_ = mp;
     DevState s_ = s;
     RunArgs r_ = r;
+    if (r.periods > 1) r_.left = nullptr;   // nothing that may leave is queued before it
     if (r_.wait_limit_ns == 0) r_.wait_limit_ns = longest_period_ns(mp, warps * ((grid + sms - 1) / sms));
     void* args[] = {&m_, &mp_, &s_, &r_};
     ce = cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(32 * warps), args, smem, st);
@@ -1024,7 +1050,7 @@ bool launch_run(const DevMesh& m, const ModelParams& mp, const DevState& s, cons
     cudaError_t ce = cudaErrorInvalidConfiguration;
     // 16 CTAs are beyond the portable cluster size: where the device has no
     // room for one, 8 (a launch that cannot be placed fails with no effect)
-    for (int most = 16; most >= 8; most >>= 1) {
+    for (int most = r.spread ? 0 : 16; most >= 8; most >>= 1) {
         const int ctas = cluster_shape(m.T, mp.S, mp.any_reaction != 0, most, &warps);
         if (ctas == 0) break;
         if (mp.S == 1)

@@ -127,10 +127,14 @@ int model_params(int32_t S, const double* D, int32_t R, const int32_t* lhs, cons
     return RDSPLIT_OK;
 }
 
-int read_err(unsigned char* base, const Layout& L, cudaStream_t st, const char* where) {
-    uint32_t e = 0;
-    cudaError_t ce = cudaMemcpyAsync(&e, base + L.err, sizeof e, cudaMemcpyDeviceToHost, st);
+// left: receives, and clears, the word after the error word (RunArgs::left).
+int read_err(unsigned char* base, const Layout& L, cudaStream_t st, const char* where, uint32_t* left = nullptr) {
+    uint32_t w[2] = {0, 0};
+    cudaError_t ce = cudaMemcpyAsync(w, base + L.err, sizeof w, cudaMemcpyDeviceToHost, st);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+    const uint32_t e = w[0];
+    if (left) *left = w[1];
+    if (ce == cudaSuccess && w[1]) ce = cudaMemsetAsync(base + L.err + 4, 0, sizeof(uint32_t), st);
     if (ce != cudaSuccess) {
         cudaGetLastError();
         return rdapi::fail(RDSPLIT_ECUDA, "%s: %s", where, cudaGetErrorString(ce));
@@ -236,9 +240,16 @@ extern "C" int rdsplit_run_static(int32_t n_tets, const int32_t* d_adj, const do
     uint32_t barrier_base = 0;
     int warps = 0;
     bool resident = run_shape(n_tets, sms, &warps) > 0;
+    int spread = 0;   // periods to go with the mesh spread over the device (see run_loop)
+    // the launch within one cluster that may have left early and has not been asked
+    double t0 = tn;
+    int64_t p0 = pk;
+    uint32_t left = 0;
+again:
     while (tn < t_end) {
         if (pk >= (int64_t)0xffffffffll) return rdapi::fail(RDSPLIT_EOVERFLOW, "%s: period index exceeds 2^32-1", where);
-        const int64_t most = std::min<int64_t>(resident ? rdapi::kRunPeriods : 1, 0xffffffffll - pk);
+        int64_t most = std::min<int64_t>(resident ? rdapi::kRunPeriods : 1, 0xffffffffll - pk);
+        if (spread > 0) most = std::min<int64_t>(most, spread);
         int n = 0;
         bool last = false;
         double te = tn, tau_k = tau;
@@ -257,13 +268,24 @@ extern "C" int rdsplit_run_static(int32_t n_tets, const int32_t* d_adj, const do
         if (last) launch_thresholds(n_tets, mp, g, G, tau_k, thr, st);
         if (resident) {
             RunArgs r{(uint32_t)pk, n, 0, tau_k, tau_k, (float)tau_k, (float)tau_k, seed, thr, thr,
-                      {out[0], out[1]}, {mask[0], mask[1]}, barrier, barrier_base};
+                      {out[0], out[1]}, {mask[0], mask[1]}, barrier, barrier_base, 0, nullptr, err + 1,
+                      spread > 0 ? 1 : 0};
             int grid = 0;
             if (!launch_run(m, mp, s, r, sms, &grid, st)) {   // (d_counts still holds the counts)
                 resident = false;
                 continue;
             }
             barrier_base += (uint32_t)grid * (uint32_t)n;
+            spread = std::max(0, spread - n);
+            if (!last) {
+                t0 = tn;
+                p0 = pk;
+                // a shortened last period is queued behind it and does nothing if it left
+                if (grid == 0 && te + tau <= t_end) {
+                    if ((rc = read_err(base, L, st, where, &left))) return rc;
+                    if (left > 0) break;
+                }
+            }
         } else {
             const int q = (int)(jl & 1);
             PeriodArgs a{(uint32_t)pk, tau_k, (float)tau_k, seed, jl == 0 ? 1 : 0, thr, out[q ^ 1], out[q],
@@ -274,17 +296,35 @@ extern "C" int rdsplit_run_static(int32_t n_tets, const int32_t* d_adj, const do
         tn = te;
         pk += n;
     }
-    if (jl > 0) {
+    if (left == 0 && jl > 0) {
         const int q = (int)((jl - 1) & 1);
         PeriodArgs a{};
         a.in_prev = out[q];
         a.mask_prev = mask[q];
         launch_gather(m, n_species, s, a, st);
     }
-    launch_counts_out(n_tets, n_species, cnt, d_counts, nullptr, err, st);
-    ce = cudaGetLastError();
-    if (ce != cudaSuccess) return rdapi::fail(RDSPLIT_ECUDA, "%s: launch failed: %s", where, cudaGetErrorString(ce));
-    if ((rc = read_err(base, L, st, where))) return rc;
+    if (left == 0) {
+        launch_counts_out(n_tets, n_species, cnt, d_counts, nullptr, err, st);
+        ce = cudaGetLastError();
+        if (ce != cudaSuccess) return rdapi::fail(RDSPLIT_ECUDA, "%s: launch failed: %s", where, cudaGetErrorString(ce));
+        if ((rc = read_err(base, L, st, where, &left))) return rc;
+    }
+    if (left > 0) {
+        // from the period after which it left, with the thresholds of a full one
+        tn = t0;
+        pk = p0;
+        for (uint32_t i = left - 1u; i > 0; --i, ++pk) tn += tau;
+        left = 0;
+        spread = rdapi::kSpreadPeriods;
+        ce = cudaMemsetAsync(barrier, 0, sizeof(uint32_t), st);   // (a launch queued behind it may not have counted)
+        if (ce != cudaSuccess) {
+            cudaGetLastError();
+            return rdapi::fail(RDSPLIT_ECUDA, "%s: %s", where, cudaGetErrorString(ce));
+        }
+        barrier_base = 0;
+        launch_thresholds(n_tets, mp, g, G, tau, thr, st);
+        goto again;
+    }
     *t = tn;
     *period = pk;
     return RDSPLIT_OK;

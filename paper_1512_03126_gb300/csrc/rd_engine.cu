@@ -44,10 +44,9 @@ struct SlotDesc {
     const uint4* thr;        // thresholds for tau
     const uint4* thr_last;   // thresholds for the shortened last period
     int32_t* N[2];           // count buffers [S][T]; the slice starts in N[0]
-    uint32_t* bits[2];       // active-tet bitmaps of 2^wshift words, by period parity in the slice
-    int32_t wshift;          // at least as many words as the cluster has warps
+    uint32_t* bits[2];       // active-tet bitmaps, by period parity in the slice
+    int32_t wshift;          // of 2^wshift words, at least as many as the cluster has warps
     int32_t sm;              // counts and bitmaps in the cluster's shared memory
-    int32_t gshift;          // runs of 2^gshift consecutive tets share a word (see word_of)
     const uint4* packed;     // one species: {src, thr} per tet
     int32_t* N2;             // one species: counts of both parities interleaved
     uint64_t seed;
@@ -95,6 +94,11 @@ __device__ __forceinline__ void red_or_cluster(uint32_t addr, uint32_t v) {
 constexpr int kWarps = kRunBlock / 32;
 constexpr int kGroup = 8;                   // bitmap columns (32 words each) a warp loads at once
 constexpr int kSmCols = 2;                  // of a simulation in shared memory: all of them
+// A warp's list of tets to visit (a simulation in global memory): up to 31 left
+// over, and what is appended at once.  The lists are where a simulation in
+// shared memory has its counts.
+constexpr int kListMost = 256;
+constexpr size_t kListBytes = (size_t)kWarps * (32 + kListMost) * sizeof(int32_t);
 
 // Dynamic shared memory of a warp, in words: the step's (rd_warp.cuh) and the
 // bitmap words of its current batch.
@@ -124,16 +128,9 @@ __device__ __forceinline__ int nth_set_bit(uint32_t w, int k) {
     return p;
 }
 
-// The place of tet t in a bitmap of 2^ws words: run t >> gs of consecutive tets
-// goes to word (t >> gs) mod 2^ws, so that a word holds 32 / 2^gs runs far
-// apart.
-__device__ __forceinline__ int word_of(int t, int ws, int gs) { return (t >> gs) & ((1 << ws) - 1); }
-__device__ __forceinline__ int bit_of(int t, int ws, int gs) {
-    return ((t >> (gs + ws)) << gs) | (t & ((1 << gs) - 1));
-}
-__device__ __forceinline__ int tet_of(int word, int bit, int ws, int gs) {
-    return ((bit >> gs) << (gs + ws)) | (word << gs) | (bit & ((1 << gs) - 1));
-}
+// A simulation in the cluster's shared memory: tet t is bit t >> ws of word
+// t mod 2^ws (one in global memory: bit t & 31 of word t >> 5).
+__device__ __forceinline__ int tet_in_shared(int word, int bit, int ws) { return (bit << ws) | word; }
 
 // Shared memory of the engine kernel.
 __shared__ int32_t s_item;                          // work-item index (first CTA of the cluster)
@@ -153,21 +150,21 @@ struct GlobalView {
     uint32_t* bcur;
     uint32_t* bnext;
     int64_t T;
-    int ws, gs;
     static constexpr int stride = kOne ? 2 : 1;
     __device__ __forceinline__ GlobalView(const SlotDesc& d, int r)
-        : bcur(d.bits[r]), bnext(d.bits[r ^ 1]), T(d.m.T), ws(d.wshift), gs(d.gshift) {
+        : bcur(d.bits[r]), bnext(d.bits[r ^ 1]), T(d.m.T) {
         cur = kOne ? d.N2 + r : d.N[r];
         next = kOne ? d.N2 + (r ^ 1) : d.N[r ^ 1];
     }
     __device__ __forceinline__ int32_t load(int s, int t) const { return __ldcg(cur + (s * T + t) * stride); }
     __device__ __forceinline__ void clear(int s, int t) const { cur[(s * T + t) * stride] = 0; }
     __device__ __forceinline__ void add(int s, int t, int32_t n) const { red_add(next + (s * T + t) * stride, n); }
-    __device__ __forceinline__ void mark(int t) const { red_or(bnext + word_of(t, ws, gs), 1u << bit_of(t, ws, gs)); }
+    __device__ __forceinline__ void mark(int t) const { red_or(bnext + (t >> 5), 1u << (t & 31)); }
     __device__ __forceinline__ void send(int t, int32_t n, bool more) const {
         add(0, t, n);
         if (more) mark(t);
     }
+    __device__ __forceinline__ void unvisit(int t) const { red_or(bcur + (t >> 5), 1u << (t & 31)); }
     // the tet's own CTA
     __device__ __forceinline__ void keep(int s, int t, int32_t n) const { add(s, t, n); }
     __device__ __forceinline__ void mark_own(int t) const { mark(t); }
@@ -205,6 +202,7 @@ struct ClusterView {
     }
     __device__ __forceinline__ void keep(int, int t, int32_t n) const { atomicAdd(cnt + 2 * slot(t) + (r ^ 1), n); }
     __device__ __forceinline__ void mark_own(int t) const { atomicOr(bnext + (t & ((1 << wl) - 1)), 1u << (t >> ws)); }
+    __device__ __forceinline__ void unvisit(int t) const { atomicOr(bcur + (t & ((1 << wl) - 1)), 1u << (t >> ws)); }
 };
 
 // Leavers of a tet into the next period's counts (fire-and-forget integer
@@ -351,7 +349,8 @@ struct WarpPeriod {
     PeriodView v;
     View c;
     uint32_t* words;           // this warp's words of the period's bitmap
-    uint32_t* wb;              // global bitmaps: the current batch's
+    uint32_t* wb;              // the current batch's
+    int32_t* list;             // global bitmaps: tets to visit
     bool more;
 
     static __device__ __forceinline__ View view(const SlotDesc& d, int r, int S) {
@@ -372,66 +371,82 @@ struct WarpPeriod {
         const int warp = threadIdx.x >> 5;
         const int rank = kC > 1 ? (int)cooperative_groups::this_cluster().block_rank() : 0;
         word0 = (rank * kWarps + warp) * (kSm ? per : 1);
-        used = d.gshift == 5 ? (d.m.T + 31) >> 5 : 1 << d.wshift;
+        used = (d.m.T + 31) >> 5;
         words = c.bcur + (kSm ? warp * per : 0);
         wb = reinterpret_cast<uint32_t*>(s_warp + warp * engine_warp_words(S, kReact) + warp_words(S, kReact));
+        list = s_warp + kWarps * engine_warp_words(S, kReact) + warp * (32 + kListMost);
     }
 };
 
-// The set bits of the warp's words, in rounds of 32: visit(i, bit, t, live) once
-// a round, with the lane's word number, bit and tet.  Words are cleared for
-// their next use when they are loaded.  Returns the number of set bits.
+// The warp's words of a batch: up to kGroup columns (32 words, one per lane)
+// loaded at once and cleared for their next use.  Returns the lane's set bits.
+template <bool kSm, class Period>
+__device__ __forceinline__ int load_batch(const Period& p, int w0) {
+    const int lane = threadIdx.x & 31;
+    constexpr int kCols = kSm ? kSmCols : kGroup;
+    uint32_t wds[kCols];
+    int own = 0;
+#pragma unroll
+    for (int kk = 0; kk < kCols; ++kk) {
+        const int i = w0 + kk * 32 + lane;
+        wds[kk] = p.has(i) ? (kSm ? *p.at(i) : __ldcg(p.at(i))) : 0u;
+    }
+#pragma unroll
+    for (int kk = 0; kk < kCols; ++kk) {
+        if (wds[kk]) *p.at(w0 + kk * 32 + lane) = 0u;
+        p.wb[kk * 32 + lane] = wds[kk];
+        own += __popc(wds[kk]);
+    }
+    return own;
+}
+
+__device__ __forceinline__ int sum_to_lane(int x) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int dd = 1; dd < 32; dd <<= 1) {
+        const int y = __shfl_up_sync(kAllLanes, x, dd);
+        if (lane >= dd) x += y;
+    }
+    return x;
+}
+
+// The tets of the set bits of the warp's words, in rounds of 32: visit(t, live)
+// once a round.  Words are cleared when they are loaded.  Returns the number of
+// set bits.
 //
-// A warp loads a batch of up to kGroup columns (32 words, one per lane) at
-// once.  One prefix sum over the lanes' set bits of the whole batch lets each lane
-// find a tet of its own (a search over the sums, the column, the bit in the
-// word: a fixed 110 instructions a round; a sum and a search for every column,
-// nearly all of which hold a few bits of a sparse mesh, made the 512-cube
-// ensemble three times slower).
+// In shared memory a simulation has two columns a warp at most: one prefix sum
+// over the lanes' set bits lets each lane find a tet of its own (a search over
+// the sums, the column, the bit in the word: a fixed 110 instructions a round).
+//
+// In global memory the columns' set bits are appended to a list, column by column,
+// and every 32 of them make a round, so that only a period's last one is not
+// full.  A word holds 32 consecutive tets, of which a cloud of molecules has
+// several: writing them out costs less than the search (the 512-cube ensemble on
+// 2 CTAs: 1.92 -> 1.86 s).
 template <bool kSm, class Period, class Visit>
 __device__ __forceinline__ uint32_t visit_set_bits(const SlotDesc& d, const Period& p, Visit visit) {
     const int lane = threadIdx.x & 31;
-    constexpr int kCols = kSm ? kSmCols : kGroup;
     uint32_t done = 0;
-    for (int w0 = 0; w0 < p.per; w0 += 32 * kCols) {
-        int own = 0;
-        {
-            uint32_t wds[kCols];
+    if constexpr (kSm) {
+        for (int w0 = 0; w0 < p.per; w0 += 32 * kSmCols) {
+            const int own = load_batch<true>(p, w0);
+            const int inc = sum_to_lane(own);
+            const int total = __shfl_sync(kAllLanes, inc, 31);
+            done += (uint32_t)total;
+            __syncwarp();
+            for (int e0 = 0; e0 < total; e0 += 32) {
+                // the lane's tet: the batch's set bit number e0 + lane
+                const int e = e0 + lane;
+                const bool live = e < total;
+                int from = 0;
 #pragma unroll
-            for (int kk = 0; kk < kCols; ++kk) {
-                const int i = w0 + kk * 32 + lane;
-                wds[kk] = p.has(i) ? (kSm ? *p.at(i) : __ldcg(p.at(i))) : 0u;
-            }
+                for (int step = 16; step > 0; step >>= 1)
+                    if (__shfl_sync(kAllLanes, inc, from + step - 1) <= e) from += step;
+                int k = e - __shfl_sync(kAllLanes, inc - own, from);
+                uint32_t word = p.wb[from];
+                int col = 0;
 #pragma unroll
-            for (int kk = 0; kk < kCols; ++kk) {
-                if (wds[kk]) *p.at(w0 + kk * 32 + lane) = 0u;
-                p.wb[kk * 32 + lane] = wds[kk];
-                own += __popc(wds[kk]);
-            }
-        }
-        int inc = own;
-#pragma unroll
-        for (int dd = 1; dd < 32; dd <<= 1) {
-            const int y = __shfl_up_sync(kAllLanes, inc, dd);
-            if (lane >= dd) inc += y;
-        }
-        const int total = __shfl_sync(kAllLanes, inc, 31);
-        done += (uint32_t)total;
-        __syncwarp();
-        for (int e0 = 0; e0 < total; e0 += 32) {
-            // the lane's tet: the batch's set bit number e0 + lane
-            const int e = e0 + lane;
-            const bool live = e < total;
-            int from = 0;
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1)
-                if (__shfl_sync(kAllLanes, inc, from + step - 1) <= e) from += step;
-            int k = e - __shfl_sync(kAllLanes, inc - own, from);
-            uint32_t word = p.wb[from];
-            int col = 0;
-            {
-#pragma unroll
-                for (int kk = 1; kk < kCols; ++kk) {
+                for (int kk = 1; kk < kSmCols; ++kk) {
                     const int c = __popc(word);
                     if (col == kk - 1 && k >= c) {
                         k -= c;
@@ -439,10 +454,54 @@ __device__ __forceinline__ uint32_t visit_set_bits(const SlotDesc& d, const Peri
                         word = p.wb[kk * 32 + from];
                     }
                 }
+                const int i = w0 + col * 32 + from;
+                visit(live ? tet_in_shared(p.word(i), nth_set_bit(word, k), d.wshift) : 0, live);
+                __syncwarp();
             }
-            const int i = w0 + col * 32 + from;
-            const int bit = nth_set_bit(word, k);
-            visit(i, bit, live ? tet_of(p.word(i), bit, d.wshift, kSm ? 0 : d.gshift) : 0, live);
+        }
+    } else {
+        int32_t* const list = p.list;
+        int cnt = 0, col = kGroup, w0 = -32 * kGroup;
+        uint32_t word = 0u;   // what is left of the lane's word in the current column
+        for (;;) {
+            while (cnt < 32) {
+                if (!__any_sync(kAllLanes, word != 0u)) {
+                    // the next column, or batch
+                    if (col == kGroup) {
+                        w0 += 32 * kGroup;
+                        if (w0 >= p.per) break;
+                        load_batch<false>(p, w0);
+                        __syncwarp();
+                        col = 0;
+                    }
+                    word = p.wb[col * 32 + lane];
+                    ++col;
+                    continue;
+                }
+                int n = __popc(word);
+                int inc = sum_to_lane(n);
+                int total = __shfl_sync(kAllLanes, inc, 31);
+                if (total > kListMost) {   // as much as the list holds: eight bits of each lane
+                    n = min(n, kListMost / 32);
+                    inc = sum_to_lane(n);
+                    total = __shfl_sync(kAllLanes, inc, 31);
+                }
+                const int base = p.word(w0 + (col - 1) * 32 + lane) << 5;
+                for (int at = cnt + inc - n; n > 0; --n) {
+                    list[at++] = base + __ffs(word) - 1;
+                    word &= word - 1u;
+                }
+                cnt += total;
+                done += (uint32_t)total;
+                __syncwarp();
+            }
+            if (cnt == 0) break;
+            const int take = min(cnt, 32);
+            cnt -= take;
+            const bool live = lane < take;
+            const int t = live ? list[cnt + lane] : 0;
+            __syncwarp();
+            visit(t, live);
             __syncwarp();
         }
     }
@@ -458,7 +517,7 @@ __device__ __noinline__ uint32_t run_deferred(int q, uint32_t* err, unsigned lon
     const SlotDesc& d = s_desc;
     const WarpPeriod<kOne, kReact, kC, kSm> p(d, q);
     uint32_t bad = 0;
-    visit_set_bits<kSm>(d, p, [&](int, int, int t, bool live) {
+    visit_set_bits<kSm>(d, p, [&](int t, bool live) {
         bool none = false;
         bad |= engine_round<kOne, kReact, true>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta, &none);
     });
@@ -485,7 +544,7 @@ __device__ __noinline__ PeriodResult run_period(int q, uint32_t* err, unsigned l
     const WarpPeriod<kOne, kReact, kC, kSm> p(d, q);
     uint32_t bad = 0;
     bool late = false;              // some tet was deferred
-    const uint32_t done = visit_set_bits<kSm>(d, p, [&](int i, int bit, int t, bool live) {
+    const uint32_t done = visit_set_bits<kSm>(d, p, [&](int t, bool live) {
         bool deferred = false;
         bad |= engine_round<kOne, kReact, false>(d, s_mp, p.S, p.w, p.v, p.c, p.more, t, live, err, mass_delta,
                                                  &deferred);
@@ -493,8 +552,7 @@ __device__ __noinline__ PeriodResult run_period(int q, uint32_t* err, unsigned l
             // back into the bitmap, for the pass after these rounds
             late = true;
             if (deferred) {
-                if (kSm) atomicOr(p.at(i), 1u << bit);
-                else red_or(p.at(i), 1u << bit);
+                p.c.unvisit(t);
             }
         }
     });
@@ -577,36 +635,41 @@ k_engine_run(const SlotDesc* __restrict__ descs, const ModelParams* __restrict__
         constexpr bool inter = kOne;   // interleaved counts
         const bool sm = kOne && d.sm != 0;
         uint32_t bad = 0;
-        // initial bitmap: occupied tets and tets with a zero-order reaction on
-        // (a thread a word; its tets are W apart, so a warp's loads are
-        // contiguous); and the simulation's molecule total
+        // initial bitmap: occupied tets and tets with a zero-order reaction on;
+        // and the simulation's molecule total.  A lane a tet: in shared memory
+        // word by word of this CTA, 32 tets W apart (a row of the counts at a
+        // time), in global memory 32 consecutive tets a warp.
         unsigned long long mine = 0;
         const int wpc = W / kC;   // in shared memory: the words, and the tets, of this CTA
         int32_t* const data = s_warp + kWarps * engine_warp_words(S, kReact);
-        for (int i = (sm ? 0 : rank * kRunBlock) + threadIdx.x; i < (sm ? wpc : W); i += sm ? kRunBlock : kC * kRunBlock) {
-            const int wi = sm ? rank * wpc + i : i;
-            uint32_t word = 0;
-            for (int bit = 0; bit < 32; ++bit) {
-                const int t = tet_of(wi, bit, d.wshift, sm ? 0 : d.gshift);
-                if (t >= T) continue;
-                bool occ = false;
-                if (kReact && d.zero_order)
-                    occ = ((s_mp.has_mask ? d.m.mask[t] : 0xffffffffu) & d.zero_order) != 0u;
-                for (int s = 0; s < S; ++s) {
-                    const int32_t c = d.N[0][(int64_t)s * T + t];
-                    occ = occ || c > 0;
-                    mine += (uint32_t)max(c, 0);
-                    if (c < 0) bad |= kErrNegative;
-                    if (sm) reinterpret_cast<int2*>(data + 2 * wpc)[bit * wpc + i] = make_int2(c, 0);
-                    else if (inter) reinterpret_cast<int2*>(d.N2)[t] = make_int2(c, 0);
-                }
-                if (occ) word |= 1u << bit;
+        auto look = [&](int t) {
+            bool occ = false;
+            if (kReact && d.zero_order) occ = ((s_mp.has_mask ? d.m.mask[t] : 0xffffffffu) & d.zero_order) != 0u;
+            for (int s = 0; s < S; ++s) {
+                const int32_t c = d.N[0][(int64_t)s * T + t];
+                occ = occ || c > 0;
+                mine += (uint32_t)max(c, 0);
+                if (c < 0) bad |= kErrNegative;
+                if (sm) reinterpret_cast<int2*>(data + 2 * wpc)[(t >> d.wshift) * wpc + (t & (wpc - 1))] = make_int2(c, 0);
+                else if (inter) reinterpret_cast<int2*>(d.N2)[t] = make_int2(c, 0);
             }
-            if (sm) {
+            return occ;
+        };
+        if (sm) {
+            for (int i = threadIdx.x; i < wpc; i += kRunBlock) {
+                uint32_t word = 0;
+                for (int bit = 0; bit < 32; ++bit) {
+                    const int t = tet_in_shared(rank * wpc + i, bit, d.wshift);
+                    if (t < T && look(t)) word |= 1u << bit;
+                }
                 reinterpret_cast<uint32_t*>(data)[i] = word;
                 reinterpret_cast<uint32_t*>(data)[wpc + i] = 0u;
-            } else {
-                d.bits[0][wi] = word;
+            }
+        } else {
+            for (int base = rank * kRunBlock; base < T; base += kC * kRunBlock) {
+                const int t = base + threadIdx.x;
+                const uint32_t word = __ballot_sync(kAllLanes, t < T && look(t));
+                if (lane == 0 && t < T) d.bits[0][t >> 5] = word;
             }
         }
 #pragma unroll
@@ -725,7 +788,7 @@ cudaError_t launch_cluster(EngineLaunch& L) {
     auto kern = k_engine_run<SA, R, C>;
     // the attribute covers every group of this kernel, whatever its species
     const size_t most = (size_t)kWarps * engine_warp_words(SA == 1 ? 1 : kMaxS, R) * sizeof(int32_t) +
-                        (SA == 1 ? sm_data_limit(R) : 0);
+                        (SA == 1 ? sm_data_limit(R) : kListBytes);
     const size_t dyn = (size_t)kWarps * engine_warp_words(L.S, R) * sizeof(int32_t) + L.data;
     const cudaError_t ce = allow_shared((const void*)kern, dyn, most);
     if (ce != cudaSuccess) return ce;
@@ -1151,9 +1214,8 @@ int rdsplit_engine_step(rdsplit_engine_t e, int64_t n_steps) {
         const rdsplit_mesh* h = e->slot_mesh[s];
         const size_t need = sm_need(h->T, h->S, h->R, csize);
         e->h_desc[s].wshift = words_shift(h->T, csize);
-        e->h_desc[s].gshift = 5;
         e->h_desc[s].sm = need > 0 ? 1 : 0;
-        g_data[cls_of(s)] = std::max(g_data[cls_of(s)], need);
+        g_data[cls_of(s)] = std::max(g_data[cls_of(s)], need > 0 ? need : kListBytes);
     }
     std::vector<size_t> idx(items.size());
     std::iota(idx.begin(), idx.end(), 0);

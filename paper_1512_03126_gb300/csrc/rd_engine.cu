@@ -259,12 +259,44 @@ __device__ __forceinline__ uint32_t engine_round(const SlotDesc& d, const ModelP
     uint32_t bad = 0;
     Presence pr;
     const uint32_t mask = kReact && mp.has_mask && live ? __ldg(d.m.mask + t) : 0xffffffffu;
-    if (live) {
-        if (kOne) {
-            // the record and the count, loaded together
-            sr = __ldg(reinterpret_cast<const int4*>(d.packed + 2 * (int64_t)t));
-            pre = __ldg(v.thr + (int64_t)t * v.thr_stride);
+    if (kOne && live) {
+        // the record and the count, loaded together
+        sr = __ldg(reinterpret_cast<const int4*>(d.packed + 2 * (int64_t)t));
+        pre = __ldg(v.thr + (int64_t)t * v.thr_stride);
+    }
+    if constexpr (kOne && !kReact && !kCalls) {
+        // At most eight molecules in each tet: two Philox blocks of its own draw
+        // them, and everything stays in registers (most rounds of a mesh with
+        // more tets than molecules).  With this and one sum a batch a round takes
+        // 584 instructions in all, 711 with warp_step and a sum a column: 64 cubes of
+        // 20 to 40 cells, 100 periods from the 2,500th on, 2.42 -> 1.90 ms (2.22
+        // before the warp step); the 512-cube ensemble 1.86 -> 1.43 s.
+        const int32_t n = live ? c.load(0, t) : 0;
+        if (!__any_sync(kAllLanes, n < 0 || n > 8)) {
+            if (n == 0) return 0u;
+            const uint32_t key = (uint32_t)key_of(d.m, t), k0 = (uint32_t)v.seed, k1 = (uint32_t)(v.seed >> 32);
+            uint32_t a0 = 0, a1 = 0;
+            for (int b = 0; 4 * b < n; ++b)
+                count_block(rdd::philox_block((uint32_t)b, key, v.period, rdd::kPurposeDiffusion << 16, k0, k1),
+                            min(4, n - 4 * b), pre, a0, a1);
+            c.clear(0, t);
+            const int nbr[4] = {sr.x, sr.y, sr.z, sr.w};
+            const int o[4] = {(int)(a0 & 0xffffu), (int)(a0 >> 16), (int)(a1 & 0xffffu), (int)(a1 >> 16)};
+#pragma unroll
+            for (int f = 0; f < 4; ++f) {
+                if (o[f] == 0) continue;
+                if (nbr[f] < 0) bad |= kErrNegative;
+                else c.send(nbr[f] >> 2, o[f], more);
+            }
+            const int32_t stay = n - (o[0] + o[1] + o[2] + o[3]);
+            if (stay > 0) {
+                c.keep(0, t, stay);
+                if (more) c.mark_own(t);
+            }
+            return bad;
         }
+    }
+    if (live) {
         for (int s0 = 0; s0 < S; s0 += 4) {
             int32_t n[4];
 #pragma unroll
@@ -418,11 +450,9 @@ __device__ __forceinline__ int sum_to_lane(int x) {
 // over the lanes' set bits lets each lane find a tet of its own (a search over
 // the sums, the column, the bit in the word: a fixed 110 instructions a round).
 //
-// In global memory the columns' set bits are appended to a list, column by column,
-// and every 32 of them make a round, so that only a period's last one is not
-// full.  A word holds 32 consecutive tets, of which a cloud of molecules has
-// several: writing them out costs less than the search (the 512-cube ensemble on
-// 2 CTAs: 1.92 -> 1.86 s).
+// In global memory the lanes append their set bits to a list, and every 32 of
+// them make a round, so that only a period's last one is not full.  One prefix
+// sum serves a whole batch, and a lane goes through its words at its own pace.
 template <bool kSm, class Period, class Visit>
 __device__ __forceinline__ uint32_t visit_set_bits(const SlotDesc& d, const Period& p, Visit visit) {
     const int lane = threadIdx.x & 31;
@@ -461,24 +491,20 @@ __device__ __forceinline__ uint32_t visit_set_bits(const SlotDesc& d, const Peri
         }
     } else {
         int32_t* const list = p.list;
-        int cnt = 0, col = kGroup, w0 = -32 * kGroup;
-        uint32_t word = 0u;   // what is left of the lane's word in the current column
+        int cnt = 0, own = 0, col = 0, w0 = -32 * kGroup, base = 0;
+        uint32_t word = 0u;   // of the lane: bits left in the batch (own), in its current word
         for (;;) {
             while (cnt < 32) {
-                if (!__any_sync(kAllLanes, word != 0u)) {
-                    // the next column, or batch
-                    if (col == kGroup) {
-                        w0 += 32 * kGroup;
-                        if (w0 >= p.per) break;
-                        load_batch<false>(p, w0);
-                        __syncwarp();
-                        col = 0;
-                    }
-                    word = p.wb[col * 32 + lane];
-                    ++col;
+                if (!__any_sync(kAllLanes, own > 0)) {
+                    w0 += 32 * kGroup;
+                    if (w0 >= p.per) break;
+                    own = load_batch<false>(p, w0);
+                    word = 0u;
+                    col = 0;
+                    __syncwarp();
                     continue;
                 }
-                int n = __popc(word);
+                int n = own;
                 int inc = sum_to_lane(n);
                 int total = __shfl_sync(kAllLanes, inc, 31);
                 if (total > kListMost) {   // as much as the list holds: eight bits of each lane
@@ -486,8 +512,13 @@ __device__ __forceinline__ uint32_t visit_set_bits(const SlotDesc& d, const Peri
                     inc = sum_to_lane(n);
                     total = __shfl_sync(kAllLanes, inc, 31);
                 }
-                const int base = p.word(w0 + (col - 1) * 32 + lane) << 5;
+                own -= n;
                 for (int at = cnt + inc - n; n > 0; --n) {
+                    while (word == 0u) {
+                        word = p.wb[col * 32 + lane];
+                        base = p.word(w0 + col * 32 + lane) << 5;
+                        ++col;
+                    }
                     list[at++] = base + __ffs(word) - 1;
                     word &= word - 1u;
                 }

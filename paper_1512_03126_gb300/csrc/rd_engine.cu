@@ -139,6 +139,7 @@ __shared__ unsigned long long s_mass[3];            // [0] molecules of the simu
                                                     // in periods of even / odd parity (two's complement)
 __shared__ SlotDesc s_desc;                         // the simulation's descriptor and chemistry
 __shared__ ModelParams s_mp;
+static_assert(sizeof(SlotDesc) + sizeof(ModelParams) + 64 <= 48u * 1024u - kDefaultShared, "static shared memory");
 extern __shared__ __align__(16) int32_t s_warp[];   // [kWarps][engine_warp_words]; kSm: then bitmaps and counts
 
 // Counts and bitmaps of one period and the next, in global memory: N[r] /

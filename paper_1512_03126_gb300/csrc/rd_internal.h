@@ -190,6 +190,9 @@ int run_shape(int64_t T, int sms, int* warps);
 // launch (two threads of 12 and 16 species: counts wrong within some thousand
 // launches).
 cudaError_t allow_shared(const void* kern, size_t bytes, size_t most);
+// Dynamic shared memory that needs no raise: the default 48 KB include a
+// kernel's static shared memory, here allowed 8 KB.
+constexpr size_t kDefaultShared = 40u * 1024u;
 
 int64_t launches();
 int sm_count();       // multiprocessors of the current device

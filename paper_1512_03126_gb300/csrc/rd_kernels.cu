@@ -67,7 +67,7 @@ cudaError_t set_once(const void* kern, cudaFuncAttribute attr, int value) {
 }  // namespace
 
 cudaError_t allow_shared(const void* kern, size_t bytes, size_t most) {
-    if (bytes <= 48u * 1024u) return cudaSuccess;
+    if (bytes <= kDefaultShared) return cudaSuccess;
     return set_once(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 

@@ -43,9 +43,19 @@ import numpy as np
 def device_bytes(n_tets: int, n_species: int) -> int:
     """Device memory a simulation holds in the library (mesh, model state and
     the engine's per-simulation lists), used for admission."""
-    per_tet = 16 + 32 + 8 + 8 + 4 + 8 + 8 + 8 + 32 + 8
-    per_tet_species = 4 + 4 + 32 + 32 + 4
-    return int(n_tets) * per_tet + int(n_tets) * int(n_species) * per_tet_species
+    T, S = int(n_tets), int(n_species)
+    stride = S if S <= 2 else (S + 3) // 4 * 4          # species words of an inbox slot
+    masks = 0 if S <= 2 else (1 if S <= 8 else 2)       # bytes of its mask
+    per_tet = 16 + 32 + 8 + 8                           # reverse faces, face rates and their sum, volume
+    per_tet += 4 + 8 + 4                                # reaction mask, unit factors, queue
+    per_tet += 2 * 4 * (4 * stride + masks)             # inboxes of both parities
+    per_tet += S * (4 + 4 + 4 + 16 + 16)                # counts, their copies, thresholds (tau, last period)
+    if S == 1:
+        per_tet += 32 + 8                               # the engine's records and count pairs
+    words = 128                                         # the engine's bitmaps
+    while 32 * words < T:
+        words *= 2
+    return T * per_tet + 2 * 4 * words + 4096           # (small arrays)
 
 
 @dataclass

@@ -64,12 +64,41 @@ def make_workload(name: str):
 
 
 def algorithmic_bytes_per_tet_period(S: int, R: int, masked: bool) -> int:
-    """Bytes the fused period kernel must move per tet and period: the
-    reverse-face table (16 B) and, per species, the remaining count (read 4,
-    write 4), the four incoming out-slots (16), the four outgoing out-slots
+    """Bytes of a tet and period with dense transfers, every slot written and
+    read: the reverse-face table (16 B) and, per species, the remaining count
+    (read 4, write 4), the four incoming slots (16), the four outgoing slots
     (16) and the cumulative face thresholds (16); with reactions the tet
-    volume (8) and, with a reaction mask, its bits (4)."""
+    volume (8) and, with a reaction mask, its bits (4).  The kernels move far
+    less (sparse_bytes_per_tet_period)."""
     return 16 + 56 * S + (8 if R > 0 else 0) + (4 if masked else 0)
+
+
+def sparse_bytes_per_tet_period(S: int, R: int, masked: bool) -> int:
+    """Bytes that k_period reads for every tet and period, whether anything
+    happens or not: the counts (4 per species), the inbox words (16 per
+    species, one or two species) or the masks that say which are valid (4, from
+    nine species on 8) and, with reactions, the unit factors (8) and the
+    reaction mask (4).  Thresholds, reverse faces, transfers and changed
+    counts come on top where molecules are."""
+    inbox = 16 * S if S <= 2 else (4 if S <= 8 else 8)
+    return 4 * S + inbox + (8 if R > 0 else 0) + (4 if masked else 0)
+
+
+def dense_roofline(T: int, S: int, R: int, masked: bool, periods: int, steps: int, ms_per_step: float, launches: int,
+                   launch_us: float, sampled: int, kernel: str) -> dict:
+    """Roofline line of a dense run: the time of a period in the timed steps and,
+    beside it, the time of one period in a launch of its own (sampled in a
+    further step: timing asks for that form)."""
+    resident = launches < periods * steps
+    period_us = ms_per_step * 1e3 / periods
+    bytes_ = sparse_bytes_per_tet_period(S, R, masked)
+    achieved = bytes_ * T / (period_us * 1e-6) / 1e9
+    peak, peak_kind = measured_peaks()
+    return {"kernel": "k_run or k_run_cluster (many periods a launch)" if resident else kernel,
+            "bound": "instruction issue and the chain of a period, not HBM", "achieved": round(achieved, 1), "peak": peak,
+            "unit": "GB/s", "frac": round(achieved / peak, 4), "traffic": None, "bytes_per_tet_period": bytes_,
+            "period_us": round(period_us, 3), "one_period_launch": kernel, "launch_us": round(launch_us, 3),
+            "sampled_launches": sampled, "peak_source": f"{peak_kind} hbm_gbs"}
 
 
 def host_cores() -> int:
@@ -220,17 +249,10 @@ def run_ours(args, rank, world, local_rank):
     seconds = total_ms / 1e3
     value = units_per_step * args.steps * world / seconds
 
-    # roofline of the period kernel
-    bpt = algorithmic_bytes_per_tet_period(S, R, w.model.mask is not None)
-    per_launch_s = (kms / kn) / 1e3 if kn else float("nan")
-    achieved = bpt * T / per_launch_s / 1e9
-    peak, peak_kind = measured_peaks()
     two, blk = rd.rdsplit_get_period_kernel(sim.h)
     kname = f"k_period in two passes (block {blk})" if two else f"k_period (block {blk})"
-    roofline = {"kernel": kname, "bound": "hbm", "achieved": round(achieved, 1), "peak": peak,
-                "unit": "GB/s", "frac": round(achieved / peak, 4), "traffic": None,
-                "bytes_per_tet_period": bpt, "launch_us": round(per_launch_s * 1e6, 3),
-                "sampled_launches": kn, "peak_source": f"{peak_kind} hbm_gbs"}
+    roofline = dense_roofline(T, S, R, w.model.mask is not None, periods, args.steps, total_ms / args.steps, launches,
+                              kms / kn * 1e3 if kn else float("nan"), kn, kname)
 
     # end to end through the C ABI with host buffers (pinned)
     e2e = None
@@ -655,18 +677,12 @@ def time_dense(rd, w, steps: int, warmup: int, stream, flush, mode: int = 0, blo
     rd.rdsplit_set_timing(sim.h, 0)
     two, blk = rd.rdsplit_get_period_kernel(sim.h)
     sim.close()
-    bpt = algorithmic_bytes_per_tet_period(S, R, w.model.mask is not None)
-    per_launch_s = (kms / kn) / 1e3 if kn else float("nan")
-    achieved = bpt * T / per_launch_s / 1e9
-    peak, peak_kind = measured_peaks()
     return {"value": T * periods * steps / (total / 1e3), "unit": UNIT, "ms_per_step": total / steps,
             "steps": steps, "periods": periods, "n_tets": T, "species": S, "reactions": R,
             "gpu_launches": launches,
-            "roofline": {"kernel": f"k_period in two passes (block {blk})" if two else f"k_period (block {blk})",
-                         "bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
-                         "frac": round(achieved / peak, 4), "traffic": None, "bytes_per_tet_period": bpt,
-                         "launch_us": round(per_launch_s * 1e6, 3), "sampled_launches": kn,
-                         "peak_source": f"{peak_kind} hbm_gbs"}}
+            "roofline": dense_roofline(T, S, R, w.model.mask is not None, periods, steps, total / steps, launches,
+                                       kms / kn * 1e3 if kn else float("nan"), kn,
+                                       f"k_period in two passes (block {blk})" if two else f"k_period (block {blk})")}
 
 
 def oracle_one_core(w, seconds: float):

@@ -554,7 +554,10 @@ enum { kPassAll = 0, kPassFirst = 1, kPassQueue = 2 };
 // reaction phase, the diffusion draws, leavers pushed to the neighbours'
 // inboxes (rd_warp.cuh).  Counts stay in place in cnt (only their own
 // tet reads or writes them) and are written back where they changed.
-// S_ > 0 fixes the species count at compile time.
+// S_ > 0 fixes the species count at compile time.  Blocks an SM, that is
+// registers against warps in flight: several species 4, 64 registers (2.4 M-tet
+// bar, 24 periods: 3.36 ms; 3 blocks 4.00, 5 blocks 3.75); one species 3, 80
+// registers (384,000-tet cube, 100 periods: 2, 3 and 4 blocks 1.86, 1.84, 1.80 ms).
 template <int S_, bool kReact, int kPass>
 __global__ void __launch_bounds__(kBlock, S_ == 1 ? 3 : 4)
 k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp, DevState s,
@@ -668,10 +671,9 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* counter, uint32_t target,
 // at once (one lane each): counts stay in shared memory, the code, the
 // thresholds and the neighbour records in the SM's caches, and a grid barrier
 // takes the place of the launch between two periods.  Started alone, a
-// period of a small mesh is mostly cold instruction and constant fetches: the
-// 3,072-tet cube's took 10.2 us a launch and takes 6.5 here (217 periods, 2.21 ->
-// 1.40 ms; 48,000-tet A/B/C cube, 200 periods, 2.91 -> 2.20 ms).  Ends with the closing transfer, all
-// inbox words and masks cleared.
+// period of a small mesh is mostly cold instruction and constant fetches
+// (48,000-tet A/B/C cube, 48 periods: 0.63 ms one launch a period, 0.42 here).
+// Ends with the closing transfer, all inbox words and masks cleared.
 template <int S_, bool kReact, int kBlocks>
 __global__ void __launch_bounds__(kBlock, kBlocks)
 k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp, DevState s,
@@ -789,10 +791,14 @@ struct ClusterSender {
 // device would share that work: a warp that left kLeaveLanes or more of its tets
 // to them asks all CTAs to leave after the period, and the caller goes on with
 // the mesh spread over the device (k_run) for a while.  7,986 tets of 5,000
-// molecules, 12 periods: 6.9 ms within the cluster, 2.7 so.  (Up to four warps a
-// CTA the FP64 units of 16 multiprocessors serve as well: RunArgs::left is null.)
+// molecules, 12 periods: 6.9 ms within the cluster, 2.7 so.  Up to four
+// warps a CTA the FP64 units of 16 multiprocessors serve as well, and with many
+// reactions, most of whose work is not theirs, up to eight: RunArgs::left is null
+// there (2 reactions, 6 warps a CTA, 100 events: 17.2 ms within the cluster, 14.3
+// spread; 30 reactions of eleven species, 7 warps: 36.9 and 40.5; 21 of eight, 12
+// warps: 114 and 96).
 constexpr int kLeaveLanes = 16;
-constexpr int kLeaveWarps = 4;
+inline int leave_above_warps(const ModelParams& mp) { return mp.any_reaction && mp.R + mp.S > 8 ? 8 : 4; }
 
 template <bool kReact>
 static __device__ __noinline__ uint32_t step_deferred_in_cluster(const DevMesh& m, const ModelParams& mp,
@@ -984,7 +990,7 @@ cudaError_t launch_cluster_s(const DevMesh& m, const ModelParams& mp, const DevS
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     RunArgs r_ = r;
-    if (warps <= kLeaveWarps) r_.left = nullptr;
+    if (warps <= leave_above_warps(mp)) r_.left = nullptr;
     ce = cudaLaunchKernelEx(&cfg, kern, m, mp, s, r_);
     if (ce == cudaSuccess) ++g_launches;
     return ce;

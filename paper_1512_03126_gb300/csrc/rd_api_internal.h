@@ -46,7 +46,7 @@ struct rdsplit_mesh {
     int2* N2 = nullptr;        // one species: {count, count} of two period parities (batched engine)
     int32_t* dq = nullptr;     // [T] tets deferred to the second pass (two-pass period)
     int32_t* dqn = nullptr;    // [2] deferred-tet counters by period parity
-    int32_t period_mode = 0;   // 0 auto (one pass), 1 one pass (k_period), 2 two passes (light + slow)
+    int32_t period_mode = 0;   // 0 auto (one pass), 1 one pass (k_period), 2 two passes
     int32_t period_block = 0;  // threads per block of the period kernel (0: by mesh size)
     int32_t part_lo = 0, part_hi = 0;  // partition steps advance stored tets [part_lo, part_hi)
     int64_t part_j = 0;                // periods done since the partition run began
@@ -91,10 +91,10 @@ namespace rdapi {
 // asked for: one pass measured faster on every workload here).
 inline bool two_pass(const rdsplit_mesh* h) { return h->period_mode == 2; }
 
-// Threads per block of the period kernel: as set, or 128 (measured fastest on
-// the 2.4 M-tet bar: 310 us per period against 339 us with 256), smaller
-// for a small mesh so that it still spreads over the SMs (at least 4 blocks
-// per SM when the tets allow it; a power of two down to 32).
+// Threads per block of the period kernel: as set, or 128 (2.4 M-tet bar, 48
+// periods: 6.07, 5.93, 6.10 and 6.41 ms with 32, 64, 128 and 256), smaller for a
+// small mesh so that it still spreads over the SMs (at least 4 blocks per SM
+// when the tets allow it; a power of two down to 32).
 inline int period_block(int64_t T, int sms) {
     int b = 128;
     while (b > 32 && T < (int64_t)4 * sms * b) b >>= 1;

@@ -1033,7 +1033,11 @@ inline double slice_cost(const rdsplit_engine* e, int32_t s, int c) {
 }
 
 // CTAs per simulation for a whole ensemble: the size whose schedule (longest
-// first, each simulation to the cluster that is free first) ends soonest.
+// first, each simulation to the cluster that is free first) ends soonest.  Its
+// choice was the fastest of the four sizes for 512 cubes of 6 to 40 cells a side
+// (2 CTAs: 1.42 s; 2.54, 1.63, 2.69 on 1, 4, 8), 40 cubes of 6 to 24 (8: 14 ms;
+// 52, 37, 30 on 1, 2, 4), 24 of them with A/B/C (8: 5.0 ms; 26, 16, 9.0) and 152
+// tubes of 960 tets (1: 5.7 ms; 9.4, 20, 43 on 2, 4, 8).
 int choose_cluster(rdsplit_engine* e, const std::vector<int32_t>& items) {
     int best = 2;
     double best_end = HUGE_VAL;

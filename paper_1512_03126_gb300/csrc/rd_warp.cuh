@@ -16,12 +16,12 @@
 //    certify every decision (react_fast); only a decision inside its bound
 //    repeats the tet in double precision (react_exact).
 //
-// Measured on GB300 against a kernel with the counts in registers, one
-// whole-warp pass per tet of ten molecules or more, and the reaction phase in
-// double precision (a run of periods, counts in and out): 3,072-tet point
-// source, 217 periods, 5.09 -> 2.21 ms; 48,000-tet A/B/C cube, 200 periods,
-// 4.15 -> 2.91 ms; six species, 68,034 tets, 100 periods, 9.29 -> 3.55 ms;
-// 2.4 M-tet bar, 24 periods, 9.48 -> 7.12 ms.
+// Against kernels with the counts in registers, one whole-warp pass per tet of
+// ten molecules or more, the reaction phase in double precision and one launch a
+// period, this step and the kernels around it take, on GB300 (a run of periods,
+// counts in and out): 3,072-tet point source, 217 periods, 5.0 -> 0.8 ms;
+// 48,000-tet A/B/C cube, 200 periods, 4.1 -> 1.8 ms; six species, 68,034 tets,
+// 100 periods, 9.3 -> 2.0 ms; 2.4 M-tet bar, 24 periods, 9.5 -> 3.4 ms.
 //
 // Every draw uses the words of the same keyed stream as the sequential
 // definition, so the counts are the same whole numbers.

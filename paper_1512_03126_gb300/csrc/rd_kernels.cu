@@ -418,9 +418,11 @@ void launch_avv(int32_t T, const double* vol, float2* avv, cudaStream_t st) {
 // from nine species on) a face says which species' words are valid, so a tet
 // reads 4 or 8 bytes unless something came: 256 of the 356 bytes a
 // tet-period of eight species moved were inbox words, nearly all zero.
-// Returns error bits.
+// Returns error bits.  first: the words of one species, if the caller has loaded
+// them (kLoaded).
+template <bool kLoaded = false>
 __device__ __forceinline__ uint32_t take_inbox(const PeriodArgs& a, int t, int S, int lane, int32_t* N,
-                                               Presence& pr, uint32_t* dirty) {
+                                               Presence& pr, uint32_t* dirty, int4 first = make_int4(0, 0, 0, 0)) {
     const int Sp = inbox_stride(S);
     uint32_t bad = 0;
     auto add = [&](int sp, int64_t v) {
@@ -433,7 +435,7 @@ __device__ __forceinline__ uint32_t take_inbox(const PeriodArgs& a, int t, int S
     };
     if (S <= 2) {
         int4* p = reinterpret_cast<int4*>(a.in_prev + (int64_t)t * 4 * Sp);
-        const int4 x = __ldcg(p);
+        const int4 x = kLoaded ? first : __ldcg(p);
         int4 y = make_int4(0, 0, 0, 0);
         if (S == 2) y = __ldcg(p + 1);
         if (x.x | x.y | x.z | x.w) {
@@ -554,12 +556,15 @@ enum { kPassAll = 0, kPassFirst = 1, kPassQueue = 2 };
 // reaction phase, the diffusion draws, leavers pushed to the neighbours'
 // inboxes (rd_warp.cuh).  Counts stay in place in cnt (only their own
 // tet reads or writes them) and are written back where they changed.
-// S_ > 0 fixes the species count at compile time.  Blocks an SM, that is
-// registers against warps in flight: several species 4, 64 registers (2.4 M-tet
-// bar, 24 periods: 3.36 ms; 3 blocks 4.00, 5 blocks 3.75); one species 3, 80
-// registers (384,000-tet cube, 100 periods: 2, 3 and 4 blocks 1.86, 1.84, 1.80 ms).
+// S_ > 0 fixes the species count at compile time.  Four blocks an SM (64
+// registers): 2.4 M-tet bar, 24 periods, 3.36 ms, with 3 blocks 4.00 and 5 blocks
+// 3.75; one species, 384,000-tet cube, 100 periods, 1.80, with 3 blocks 1.84, 2
+// blocks 1.86.  One species loads its inbox words beside the count, and the
+// reverse faces beside the thresholds where it holds molecules, instead of one
+// after the other (162,000 tets of one molecule, 100 periods: 0.84 -> 0.66 ms; for
+// several species the words held in registers cost the bar 18 %).
 template <int S_, bool kReact, int kPass>
-__global__ void __launch_bounds__(kBlock, S_ == 1 ? 3 : 4)
+__global__ void __launch_bounds__(kBlock, 4)
 k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp, DevState s,
          const __grid_constant__ PeriodArgs a, int32_t* __restrict__ queue, int32_t* qcount, int32_t parity) {
     extern __shared__ int32_t sm[];
@@ -584,6 +589,8 @@ k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams 
         Presence pr;
         const uint32_t mask = kReact && mp.has_mask && live ? __ldg(m.mask + t) : 0xffffffffu;
         if (live) {
+            int4 words = make_int4(0, 0, 0, 0);
+            if (S_ == 1 && kPass != kPassQueue && !a.first) words = __ldcg(reinterpret_cast<const int4*>(a.in_prev) + t);
             for (int s0 = 0; s0 < S; s0 += 8) {
                 int32_t n[8];
 #pragma unroll
@@ -596,16 +603,17 @@ k_period(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams 
                         pr.add(s0 + k, n[k]);
                     }
             }
-            if (kPass != kPassQueue && !a.first) bad |= take_inbox(a, t, S, lane, w.N, pr, &dirty);
+            if (kPass != kPassQueue && !a.first) bad |= take_inbox<S_ == 1>(a, t, S, lane, w.N, pr, &dirty, words);
         }
         Sender send(a, m.src, t, S);
+        if (S_ == 1 && !kReact && pr.any) send.load();   // beside the thresholds
         if (a.dense && live) send.clear_all();
         bool deferred = false;
         if (kPass == kPassQueue) {
             deferred = live;
         } else {
-            bad |= warp_step<S_ == 1, kReact, kPass == kPassFirst, false>(m, mp, S, w, v, t, live, mask, pr, &dirty,
-                                                                          &deferred, s.err, send);
+            bad |= warp_step<S_ == 1, kReact, kPass == kPassFirst, false, false, true>(m, mp, S, w, v, t, live, mask, pr,
+                                                                                       &dirty, &deferred, s.err, send);
             if (live && !deferred) send.finish(a.dense != 0);
         }
         if (kPass != kPassFirst && __ballot_sync(0xffffffffu, deferred)) {
@@ -722,8 +730,8 @@ k_run(const __grid_constant__ DevMesh m, const __grid_constant__ ModelParams mp,
                            last ? r.thr_last : r.thr, 1};
         Sender send(a, m.src, t, S);
         bool deferred = false;
-        bad |= warp_step<S_ == 1, kReact, false, false>(m, mp, S, w, v, t, live, mask, pr, &dirty, &deferred, s.err,
-                                                        send);
+        bad |= warp_step<S_ == 1, kReact, false, false, false, true>(m, mp, S, w, v, t, live, mask, pr, &dirty, &deferred,
+                                                                     s.err, send);
         if (live && !deferred) send.finish(false);
         if (__ballot_sync(0xffffffffu, deferred)) {
             const uint32_t x = step_deferred<kReact>(m, mp, w.N, w.rx, v.period, v.tau_k, v.seed, v.thr, a.in_cur,

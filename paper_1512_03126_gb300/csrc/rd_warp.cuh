@@ -587,7 +587,8 @@ __device__ __forceinline__ uint32_t draw_all(int S, int64_t T, const WarpMem& w,
 // lives across the call is spilled (80 to 100 local-memory instructions per 32
 // tets with three calls inside).  With kDefer every tet whose first waiting
 // time may fall inside the period is deferred, too.
-template <bool kOne, bool kReact, bool kDefer, bool kCalls, bool kPre = false, class Emit>
+// kLean: one species without reactions draws a warp's few molecules in registers.
+template <bool kOne, bool kReact, bool kDefer, bool kCalls, bool kPre = false, bool kLean = false, class Emit>
 __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParams& mp, int S, const WarpMem& w,
                                               const PeriodView& v, int t, bool live, uint32_t mask, Presence& pr,
                                               uint32_t* dirty, bool* deferred, uint32_t* err, Emit& emit,
@@ -637,6 +638,30 @@ __device__ __forceinline__ uint32_t warp_step(const DevMesh& m, const ModelParam
                 if (mp.rule != kRuleEnd) touched = tch;   // first order: the draw uses N(tau_k)
                 present = pr.any & mp.moves;
             }
+        }
+    }
+    if constexpr (kLean && kOne && !kReact && !kCalls) {
+        // At most eight molecules in each tet: no list, no leavers in shared
+        // memory (a point source in 279,936 tets, 2,000 periods: 16.2 -> 14.1 ms;
+        // within one cluster it gains nothing and costs 1 %).
+        const int32_t n = present ? w.N[lane] : 0;
+        if (!__any_sync(kAllLanes, n > 8)) {
+            if (n == 0) return 0u;
+            const uint4 C = __ldg(v.thr + (int64_t)t * v.thr_stride);
+            uint32_t a0 = 0, a1 = 0;
+            for (int b = 0; 4 * b < n; ++b)
+                count_block(rdd::philox_block((uint32_t)b, (uint32_t)key, v.period, rdd::kPurposeDiffusion << 16,
+                                              (uint32_t)v.seed, (uint32_t)(v.seed >> 32)),
+                            min(4, n - 4 * b), C, a0, a1);
+            if (a0 | a1) {
+                const int4 o = make_int4((int)(a0 & 0xffffu), (int)(a0 >> 16), (int)(a1 & 0xffffu), (int)(a1 >> 16));
+                const int32_t left = n - (o.x + o.y + o.z + o.w);
+                w.N[lane] = left;
+                pr.set(0, left);
+                *dirty |= 1u;
+                emit(0, o);
+            }
+            return 0u;
         }
     }
     if (!kCalls && *deferred) present = 0u;

@@ -891,16 +891,16 @@ k_run_cluster(const __grid_constant__ DevMesh m, const __grid_constant__ ModelPa
     const uint32_t words_at = (uint32_t)__cvta_generic_to_shared(words);
     const uint32_t masks_at = (uint32_t)__cvta_generic_to_shared(masks);
     const uint32_t stop_at = masks_at + (uint32_t)(B * 16);   // the period after which a warp asked to leave, plus 1
+    int end = r.periods;
     for (int q = 0; q <= r.periods; ++q) {
         const int p = q & 1;
-        bool leave = false;
         if (q > 0) {
             cluster_sync_all();
-            // all CTAs agree: nobody starts period q before all have finished
-            // q - 1, and a request made in period q itself reads q + 1
+            // all CTAs agree: a request made in period q - 1 reads q, nobody starts
+            // period q before all have finished that, and one made in it reads q + 1
             uint32_t asked;
             asm volatile("ld.shared.u32 %0, [%1];" : "=r"(asked) : "r"(stop_at) : "memory");
-            leave = asked != 0u && asked <= (uint32_t)q;
+            if (asked == (uint32_t)q) end = q;
             if (live) {
                 auto add = [&](int sp, int64_t v) {
                     int64_t n = w.N[32 * sp + lane] + v;
@@ -934,8 +934,7 @@ k_run_cluster(const __grid_constant__ DevMesh m, const __grid_constant__ ModelPa
                 }
             }
         }
-        if (leave && q < r.periods && blockIdx.x == 0 && threadIdx.x == 0) *r.left = (uint32_t)q + 1u;
-        if (leave || q == r.periods) break;
+        if (q == end) break;
         const bool last = r.last_short && q == r.periods - 1;
         const PeriodView v{r.period0 + (uint32_t)q, last ? r.tau_last : r.tau, last ? r.tau_lastf : r.tauf, r.seed,
                            last ? r.thr_last : r.thr, 1};
@@ -956,6 +955,7 @@ k_run_cluster(const __grid_constant__ DevMesh m, const __grid_constant__ ModelPa
             if (deferred) pr = presence_of(w.N + lane, S);
         }
     }
+    if (end < r.periods && blockIdx.x == 0 && threadIdx.x == 0) *r.left = (uint32_t)end + 1u;
     if (live)
         for (uint32_t bits = dirty; bits; bits &= bits - 1u) {
             const int sp = __ffs(bits) - 1;

@@ -258,17 +258,18 @@ int run_loop(rdsplit_mesh* h, double t_end, int64_t max_periods, uint64_t seed) 
         jl += 1;
         unchecked = true;
     }
-    if (rc || !unchecked) return rc;
-    if (jl > 0) {
-        const int q = (int)((jl - 1) & 1);
-        PeriodArgs a{};
-        a.in_prev = h->inbox[q];
-        a.mask_prev = h->imask[q];
-        launch_gather(m, h->S, s, a, h->stream);
+    if (rc == RDSPLIT_OK && unchecked) {
+        if (jl > 0) {
+            const int q = (int)((jl - 1) & 1);
+            PeriodArgs a{};
+            a.in_prev = h->inbox[q];
+            a.mask_prev = h->imask[q];
+            launch_gather(m, h->S, s, a, h->stream);
+        }
+        if ((rc = launch_check("rdsplit_run"))) return rc;
+        h->inbox_dirty = false;
+        rc = check_err(h, "rdsplit_run");
     }
-    if ((rc = launch_check("rdsplit_run"))) return rc;
-    h->inbox_dirty = false;
-    rc = check_err(h, "rdsplit_run");
     if (rc == RDSPLIT_ETIMEOUT) {   // blocks left a launch early: back to the counts saved
         h->inbox_dirty = true;
         CUDA_TRY(cudaMemsetAsync(h->barrier, 0, sizeof(uint32_t), h->stream));

@@ -59,6 +59,30 @@ def test_a_long_period_is_no_error(rd, oracle):
         assert np.array_equal(sim.counts(), ref)
 
 
+def test_running_out_between_two_forms(rd, oracle):
+    """3,072 tets that leave their cluster after a period, one of them busy for
+    tenths of a second in the next: the wait over the device runs out with the
+    cluster's next launch queued behind it.  The handle is at a point of the call
+    (its counts are the oracle's there) and goes on from it."""
+    mesh = I.kuhn_box(8, 8, 8, (8e-7, 8e-7, 8e-7), 0.2, 5)
+    tau = 1e-7 ** 2 / 1e-12 / 100.0
+    model = I.Model(D=np.array([1e-14]), lhs=np.ones((1, 1), np.int32), rhs=np.zeros((1, 1), np.int32),
+                    k=np.array([0.01 / tau]))
+    counts = np.full((mesh.n_tets, 1), 4500, np.int32)
+    counts[777] = 200000
+    with rd.Simulation(mesh, model, counts) as sim:
+        rd.rdsplit_set_wait_limit(sim.h, 1e-6)
+        with pytest.raises(rd.RdsplitError) as e:
+            sim.run_periods(140, 9)
+        assert e.value.code == rd.RDSPLIT_ETIMEOUT
+        done = sim.time[1]
+        assert 0 < done < 140
+        assert np.array_equal(sim.counts(), oracle.run(mesh, model, counts, np.inf, 9, max_periods=done)[0])
+        rd.rdsplit_set_wait_limit(sim.h, 60.0)
+        sim.run_periods(3, 9)
+        assert np.array_equal(sim.counts(), oracle.run(mesh, model, counts, np.inf, 9, max_periods=done + 3)[0])
+
+
 def test_limits_that_are_not_positive_are_rejected(rd):
     mesh, model, counts = one_busy_tet(1e3)
     with rd.Simulation(mesh, model, counts) as sim:
